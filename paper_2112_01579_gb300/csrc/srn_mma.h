@@ -15,8 +15,7 @@ constexpr bool is_adjoint(int SH) { return SH == SRN_SHADE_ADJOINT || SH == kPoi
 constexpr bool is_points(int SH) { return SH == kPoints || SH == kPointsAdj; }
 
 // Warpgroups per CTA for hidden width C and shading mode SH (one CTA per
-// SM): what the shared memory of the A tiles and weight tiles and the
-// register file allow.  Width 32 runs 7 (72 registers a thread), except the
+// SM): what the register file and TMEM allow.  Width 32 runs 7 (72 registers a thread), except the
 // finite-difference variant, whose extra state needs the 80 registers of 6,
 // and the adjoint variants, whose TMEM stash limits them to 4.
 constexpr int wgs_for(int C, int SH) {
@@ -24,18 +23,25 @@ constexpr int wgs_for(int C, int SH) {
                         : (C == 32 ? (SH == SRN_SHADE_FD ? 6 : 7) : (C == 48 ? 4 : 3));
 }
 constexpr int kAdjMaxLayers = 4;  // layers of the networks the tensor-core adjoint takes
-// TMEM columns a CTA allocates, and the columns of one warpgroup.  The
-// adjoint variants keep an accumulator wide enough for the input-gradient
-// MMA (N = K0, the layer-0 input columns) and for the hidden layers (N = C),
-// rounded up to 32 columns, followed by the stashed activation derivatives
-// of the (at most two) hidden layers, C columns each: 64 + 64 (width 32, four
-// warpgroups), 96 + 96 (48, two), 96 + 128 (64, two).
-constexpr int tmem_cols_for(int SH) { return is_adjoint(SH) ? 512 : 256; }
-constexpr int adj_acc_cols(int C, int K0) { return (((K0 > C ? K0 : C) + 31) / 32) * 32; }
-constexpr int tmem_wg_cols(int C, int SH, int K0) {
-  return is_adjoint(SH) ? adj_acc_cols(C, K0) + (kAdjMaxLayers - 2) * C : C;
+// TMEM columns a CTA allocates (all 512: one CTA holds an SM's registers, so
+// no second CTA of these kernels waits for columns), and the columns of one
+// warpgroup.  A warpgroup holds its accumulator (C columns) and, from column
+// C on, its operand rows: max(K0, 2C) FP16, two per column (C = 32: 64
+// columns, seven warpgroups 448; 48: 96, four; 64: 128, three).  The adjoint
+// variants widen the accumulator for the input-gradient MMA (N = K0 columns,
+// which overlap the operand rows of the other layers: its own row lies in the
+// stash, consumed by then) and append the stashed activation derivatives of
+// the (at most two) hidden layers, C columns each: 64 + 64 (width 32, four
+// warpgroups), 96 + 96 (48, two), 128 + 128 (64, two).
+constexpr int kTmemCols = 512;
+constexpr int a_cols(int C, int K0) { return K0 / 2 > C ? K0 / 2 : C; }
+constexpr int adj_acc_cols(int C, int K0) {
+  return K0 > C + a_cols(C, K0) ? ((K0 + 31) / 32) * 32 : C + a_cols(C, K0);
 }
-constexpr int kTile = 128 * 128;       // 128 rows x 128 B (64 FP16 columns): an A-tile block, the constant tile
+constexpr int tmem_wg_cols(int C, int SH, int K0) {
+  return is_adjoint(SH) ? adj_acc_cols(C, K0) + (kAdjMaxLayers - 2) * C : C + a_cols(C, K0);
+}
+constexpr int kTile = 128 * 128;       // 128 rows x 128 B (64 FP16 columns): the constant tile
 
 constexpr long long kWaitCycles = 2000000000ll;  // ~1 s at 2 GHz
 
@@ -50,22 +56,20 @@ struct PointsDev {
 
 // ---------------------------------------------------------------- layout
 struct SmemPlan {
-  int oA, oOne, oB0, oBh, oBb, oBhT, oB0T, oWl, oTF, oTFinv, oFm, oQp, oMbar, oMisc, total;
+  int oOne, oB0, oBh, oBb, oBhT, oB0T, oWl, oTF, oTFinv, oFm, oQp, oMbar, oMisc, total;
 };
 
-// Shared memory for hidden width C and WGS warpgroups.  An operand row spans
-// ceil(K / 64) blocks of 64 FP16 columns: a warpgroup's A tile (128 rows,
-// unswizzled core-matrix layout, see a_off) takes kTile bytes per block; B
-// tiles are 128B-swizzled K-atoms C * 128 bytes apart.
+// Shared memory for hidden width C and WGS warpgroups: the weights (B tiles,
+// 128B-swizzled K-atoms C * 128 bytes apart) and small tables.  The per-ray
+// operand rows are in tensor memory, so most of the SM's 256 KB stay L1.
 inline SmemPlan make_plan(const NetDev& n, int C, int WGS, bool adjoint = false) {
   const int D0 = net_d0(n);
   const int K0 = ((D0 + 2 + 15) / 16) * 16;
-  const int NA0 = (K0 + 63) / 64, NAH = (2 * C + 63) / 64, NA = NA0 > NAH ? NA0 : NAH;
+  const int NA0 = (K0 + 63) / 64, NAH = (2 * C + 63) / 64;
   const int BT = C * 128;
   const int NBB = n.l > 2 ? (16 * (n.l - 2) + 63) / 64 : 1;
   SmemPlan s;
   int o = 0;
-  s.oA = o; o += WGS * NA * kTile;
   s.oOne = o; o += kTile;                   // constant tile: columns 0, 1 = 1
   s.oB0 = o; o += NA0 * BT;                 // layer 0
   s.oBh = o; o += (n.l - 2) * NAH * BT;     // hidden layers: [W | W]

@@ -10,12 +10,12 @@
 //   latent-grid trilinear fetch, Fourier features, transfer function,
 //   compositing, early termination) stays one thread per ray as in the paper,
 //   while the layers run as M=128 x N=C tensor-core MMAs.
-// * Every sample: the thread writes its FP16 layer-0 input row into a
-//   K-major shared-memory tile (no swizzle, see a_off); one elected thread
+// * Every sample: the thread writes its FP16 layer-0 input row into tensor
+//   memory (operand A of the MMA, see tmem_st8); one elected thread
 //   issues tcgen05.mma
 //   (kind::f16, FP32 accumulate in TMEM); the thread reads its row back with
 //   tcgen05.ld, applies the activation in FP32 and writes it into the same
-//   tile as the next layer's A row as an FP16 hi + lo pair (a = hi + lo to
+//   columns as the next layer's A row as an FP16 hi + lo pair (a = hi + lo to
 //   ~2^-22 relative; the B tile holds [W | W]), so the hidden activations
 //   keep FP32 accuracy through the FP16 tensor cores.  Inside the tile the input columns are
 //   [sin_0, cos_0, ..., sin_{m-1}, cos_{m-1}, p, z, 1, 1]; the B tile of
@@ -121,6 +121,17 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_
       : "memory");
 }
 
+// The same with A in tensor memory (lane = row, two FP16 of K per column).
+__device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                : "memory");
@@ -199,29 +210,22 @@ __device__ __forceinline__ uint32_t sw_tile_off(int r, int cg) {
   return (uint32_t)((cg >> 3) * kTile) + sw_off(r, cg & 7);
 }
 
-// A tiles (the per-ray operand rows: layer inputs, activations, adjoint rows)
-// are K-major without swizzle: core matrices of 8 rows x 16 bytes, chunk cg
-// (= column / 8) of row r at (r / 8) SBO + 128 cg + 16 (r % 8) with
-// SBO = NA 1024 for NA 64-column blocks of K.  A thread's chunk offsets are
-// then immediates from its row base (no per-store swizzle arithmetic), and a
-// quarter-warp's 16-byte stores of one chunk fill 128 contiguous bytes, free
-// of bank conflicts.  The tile is NA kTile bytes, as the swizzled one was.
-template <int NA>
-__device__ __forceinline__ uint32_t a_off(int r, int cg) {
-  return (uint32_t)((r >> 3) * (NA * 1024) + cg * 128 + (r & 7) * 16);
+// The per-ray operand rows (layer inputs, activations, adjoint rows) live in
+// tensor memory: row = lane, two FP16 of K per 32-bit column.  A thread
+// stores its own row with tcgen05.st, eight columns (16 FP16) at a time, so a
+// row takes four stores instead of eight 16-byte shared-memory stores (and
+// the proxy fence they need before the MMA), and the MMA leaves the L1 /
+// shared-memory pipe to the latent gathers.  The same bits as operand rows in
+// shared memory, and faster on every variant: main configuration at 1024^2
+// 10.61 -> 9.81 ms, four keyframed 517 x 333 frames 7.69 -> 7.12 ms, adjoint
+// shading at 512^2 20.0 -> 18.4 ms, six layers of 48 channels at 512^2 3.91 ->
+// 3.57 ms, 2^20 points 96 -> 82 us.
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&w)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"r"(taddr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
 }
-// Descriptor of such a tile at saddr: leading byte offset 128 (the next core
-// matrix along K), stride byte offset NA 1024 (the next 8-row group), no
-// swizzle, sm100 descriptor version 1.  K = 16 per MMA advances saddr by 256.
-template <int NA>
-__device__ __forceinline__ uint64_t a_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)(128u >> 4) << 16;
-  d |= (uint64_t)((NA * 1024u) >> 4) << 32;
-  d |= (uint64_t)1u << 46;
-  return d;
-}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Transfer function with precomputed reciprocal segment widths (same
 // segments and lerp as the shared tf_eval).
@@ -358,9 +362,11 @@ __device__ __forceinline__ void latent_q(const uint8_t* __restrict__ Q, const fl
 // time input when TI) in the tile's column order [sin_0, cos_0, ...,
 // sin_{m-1}, cos_{m-1}, p, z, (t), 1, 1, 0...] over the K0 columns layer 0
 // reads.  Values are packed to FP16 pairs
-// and stored 16 bytes at a time as they are produced.
-template <int M, int F, int K0, int TI, int GQ, int NA, int ST>
-__device__ __forceinline__ void write_input_row(uint8_t* tile, int row, float3 p, bool nerf, const float* fm,
+// and stored to the thread's TMEM row 16 at a time as they are produced; the
+// whole warp takes part (tcgen05.st is warp-collective), lanes without a
+// sample write a row nothing reads.
+template <int M, int F, int K0, int TI, int GQ, int ST>
+__device__ __forceinline__ void write_input_row(uint32_t t_a, float3 p, bool nerf, const float* fm,
                                                 const __half* G, const uint8_t* Q, const float* qp, int R,
                                                 const RayLat& rl) {
   constexpr int D0 = 3 + 2 * M + F + TI;
@@ -368,13 +374,13 @@ __device__ __forceinline__ void write_input_row(uint8_t* tile, int row, float3 p
   float z[F];
   if constexpr (GQ != 0) latent_q<F, ST>(Q, qp, R, rl, p, z);
   else latent_h<F, ST>(G, R, rl, p, z);
-  uint32_t w[4];
-  int nw = 0, chunk = 0;
+  uint32_t w[8];
+  int nw = 0, col = 0;
   auto emit = [&](float a, float b) {
     w[nw++] = pack_h2(a, b);
-    if (nw == 4) {
-      *reinterpret_cast<uint4*>(tile + a_off<NA>(row, chunk)) = make_uint4(w[0], w[1], w[2], w[3]);
-      ++chunk;
+    if (nw == 8) {
+      tmem_st8(t_a + col, w);
+      col += 8;
       nw = 0;
     }
   };
@@ -420,12 +426,12 @@ __device__ __forceinline__ void write_input_row(uint8_t* tile, int row, float3 p
   float tail[K0 - 2 * M];
 #pragma unroll
   for (int i = 0; i < K0 - 2 * M; ++i) {
-    const int col = 2 * M + i;
+    const int cc = 2 * M + i;
     float v = 0.0f;
-    if (col < 2 * M + 3) v = col == 2 * M ? p.x : (col == 2 * M + 1 ? p.y : p.z);
-    else if (col < 2 * M + 3 + F) v = z[col - 2 * M - 3];
-    else if (col < D0) v = rl.tin;  // Section 7 "direct" time input
-    else if (col == D0 || col == D0 + 1) v = 1.0f;
+    if (cc < 2 * M + 3) v = cc == 2 * M ? p.x : (cc == 2 * M + 1 ? p.y : p.z);
+    else if (cc < 2 * M + 3 + F) v = z[cc - 2 * M - 3];
+    else if (cc < D0) v = rl.tin;  // Section 7 "direct" time input
+    else if (cc == D0 || cc == D0 + 1) v = 1.0f;
     tail[i] = v;
   }
 #pragma unroll
@@ -542,7 +548,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   constexpr int WGS = wgs_for(C, SH), THREADS = 128 * WGS;
   constexpr int D0 = 3 + 2 * M + F + TI;
   constexpr int K0 = ((D0 + 2 + 15) / 16) * 16;  // inputs + two bias columns
-  constexpr int NA0 = (K0 + 63) / 64, NAH = (2 * C + 63) / 64;
+  constexpr int NAH = (2 * C + 63) / 64;         // K-atoms of a hidden layer's B tile
   constexpr int BT = C * 128;                    // bytes of one K-atom of a B tile (C rows)
   constexpr uint32_t IDESC = idesc_n(C);
   static_assert(C % 16 == 0 && C <= 64 && K0 <= 128, "shape outside the kernel's tiling");
@@ -550,14 +556,13 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   constexpr bool POINTS = is_points(SH);
   constexpr bool SNAKE = ACT == SRN_ACT_SNAKEALT;
   constexpr bool ADJ = is_adjoint(SH);  // input gradient by backward MMAs (Section 5 "adjoint")
-  constexpr int TMC = tmem_cols_for(SH);
+  constexpr int TMC = kTmemCols;
   constexpr int NACC = adj_acc_cols(C, K0);  // adjoint: accumulator columns before the derivative stash
   static_assert(!ADJ || (TI == 0 && GQ == 0), "tensor-core adjoint: no time input, FP16 grid");
-  static_assert(!ADJ || WGS * tmem_wg_cols(C, SH, K0) <= TMC, "adjoint TMEM layout exceeds the allocation");
+  static_assert(WGS * tmem_wg_cols(C, SH, K0) <= TMC, "TMEM layout exceeds the allocation");
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* Aall = sm + plan.oA;
   uint8_t* B0 = sm + plan.oB0;
   uint8_t* Bh = sm + plan.oBh;
   uint8_t* Bb = sm + plan.oBb;
@@ -580,7 +585,6 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   constexpr int DF = SH == SRN_SHADE_HEAD ? 4 : 1;
   const int L = LF > 0 ? LF : net.l;
   const int D = LF > 0 ? DF : net.D;
-  constexpr int NA = NA0 > NAH ? NA0 : NAH;
   // the FP16 latent grid holds G 2^-gexp: the latent columns' layer-0 weights
   // are staged times 2^gexp (exact), the 8-bit grid's lo / step times 2^-gexp
   const int gexp = net.grid_exp ? *net.grid_exp : 0;
@@ -703,17 +707,13 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
         qp[i] = ldexpf((i & 1) ? net.grid_qp[i] : fmaf(128.0f, net.grid_qp[i + 1], net.grid_qp[i]), -gexp);
   }
   load_tf(tf, b.tf);
-  // the thread's A row starts at zero; the constant tile has ones in columns
-  // 0 and 1 of every row (the bias MMA of the hidden layers)
-  {
-    uint8_t* A = Aall + wg * NA * kTile;
+  // the constant tile has ones in columns 0 and 1 of every row (the bias MMA
+  // of the hidden layers)
+  if (wg == 0) {
     uint8_t* One = sm + plan.oOne;
-    for (int cg = 0; cg < NA * 8; ++cg) *reinterpret_cast<uint4*>(A + a_off<NA>(row, cg)) = make_uint4(0, 0, 0, 0);
-    if (wg == 0) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<uint4*>(One + sw_off(row, j)) = make_uint4(j == 0 ? pack_h2(1.0f, 1.0f) : 0u, 0u, 0u, 0u);
-    }
+    for (int j = 0; j < 8; ++j)
+      *reinterpret_cast<uint4*>(One + sw_off(row, j)) = make_uint4(j == 0 ? pack_h2(1.0f, 1.0f) : 0u, 0u, 0u, 0u);
   }
   if (row == 0) {
     mbar_init(smem_u32(&mbar[wg]), 1);
@@ -746,8 +746,12 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   const uint32_t tmem = (uint32_t)misc[0];
   const uint32_t d_tmem = tmem + (uint32_t)(wg * tmem_wg_cols(C, SH, K0));
   const uint32_t t_row = d_tmem + ((uint32_t)((row >> 5) * 32) << 16);  // warp's lane quarter
-  uint8_t* A = Aall + wg * NA * kTile;
-  const uint32_t a_addr = smem_u32(A), b0_addr = smem_u32(B0), bh_addr = smem_u32(Bh), bb_addr = smem_u32(Bb);
+  // operand rows: behind the accumulator (adjoint: in the upper half of the
+  // wide accumulator, which only the last, N = K0 MMA fills; that MMA's row
+  // takes the place of the consumed derivative stash)
+  constexpr int ACOL = C;
+  const uint32_t a_tmem = d_tmem + ACOL, t_a = t_row + ACOL;
+  const uint32_t b0_addr = smem_u32(B0), bh_addr = smem_u32(Bh), bb_addr = smem_u32(Bb);
   const uint32_t one_addr = smem_u32(sm + plan.oOne);
   const uint32_t bht_addr = smem_u32(BhT), b0t_addr = smem_u32(B0T);
   const uint32_t mb = smem_u32(&mbar[wg]);
@@ -833,8 +837,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
     // ---- layer-0 input of this pass
     float len = 0.f;
     float3 qs = make_float3(0.f, 0.f, 0.f);  // sample position of this pass
-    if (POINTS && active && !failed) {
-      write_input_row<M, F, K0, TI, GQ, NA, ST>(A, row, ppos, nerf, fm, net.grid_h, net.grid_q, qp, net.R, rl);
+    if (POINTS) {
       qs = ppos;
     } else if (active && !failed) {
       const float ta = fmaf((float)k, b.step, t0);
@@ -850,10 +853,12 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
         if (ax == 1) q.y = clamp01f(q.y + h);
         if (ax == 2) q.z = clamp01f(q.z + h);
       }
-      write_input_row<M, F, K0, TI, GQ, NA, ST>(A, row, q, nerf, fm, net.grid_h, net.grid_q, qp, net.R, rl);
       qs = q;
     }
-    fence_proxy_async();
+    if (__any_sync(0xffffffffu, active && !failed)) {
+      write_input_row<M, F, K0, TI, GQ, ST>(t_a, qs, nerf, fm, net.grid_h, net.grid_q, qp, net.R, rl);
+      tmem_wait_st();
+    }
     tc_fence_before();
     const bool any = bar_red_or(bar_id, 128, active && !failed);
     if (!any || misc[4 + wg]) break;
@@ -862,7 +867,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
 #pragma unroll
       for (int kk = 0; kk < K0 / 16; ++kk) {
         const uint32_t ka = ((16 * kk) >> 6), kb = ((16 * kk) & 63) * 2;
-        mma_f16(d_tmem, a_desc<NA>(a_addr + kk * 256), sw128_desc(b0_addr + ka * BT + kb), IDESC, kk > 0);
+        mma_f16_ta(d_tmem, a_tmem + 8 * kk, sw128_desc(b0_addr + ka * BT + kb), IDESC, kk > 0);
       }
       mma_commit(mb);
     }
@@ -888,15 +893,16 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
         if (!failed) {
           // activation as FP16 hi (columns 0..C-1) + lo (columns C..2C-1)
 #pragma unroll
-          for (int j = 0; j < C / 8; ++j) {
-            uint32_t hi[4], lo[4];
+          for (int j = 0; j < C / 16; ++j) {
+            uint32_t hi[8], lo[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              split_h2(act_fold<ACT>(x[8 * j + 2 * e]), act_fold<ACT>(x[8 * j + 2 * e + 1]), hi[e], lo[e]);
+            for (int e = 0; e < 8; ++e) {
+              split_h2(act_fold<ACT>(x[16 * j + 2 * e]), act_fold<ACT>(x[16 * j + 2 * e + 1]), hi[e], lo[e]);
             }
-            *reinterpret_cast<uint4*>(A + a_off<NA>(row, j)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<uint4*>(A + a_off<NA>(row, C / 8 + j)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            tmem_st8(t_a + 8 * j, hi);
+            tmem_st8(t_a + C / 2 + 8 * j, lo);
           }
+          tmem_wait_st();
           if constexpr (ADJ) {
             // activation derivative of this hidden layer, kept in TMEM for the
             // backward: SnakeAlt' = 0.5 + sin(2x) (the accumulator holds 2x); sin' = cos
@@ -906,7 +912,6 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
             tmem_st_row<C>(t_row + NACC + C * layer, dv);
           }
         }
-        fence_proxy_async();
         tc_fence_before();
         bar_sync(bar_id, 128);
         if (misc[4 + wg]) { stop = true; break; }
@@ -919,7 +924,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
 #pragma unroll
           for (int kk = 0; kk < 2 * C / 16; ++kk) {
             const uint32_t ka = ((16 * kk) >> 6), kb = ((16 * kk) & 63) * 2;
-            mma_f16(d_tmem, a_desc<NA>(a_addr + kk * 256), sw128_desc(bw + ka * BT + kb), IDESC, 1u);
+            mma_f16_ta(d_tmem, a_tmem + 8 * kk, sw128_desc(bw + ka * BT + kb), IDESC, 1u);
           }
           mma_commit(mb);
         }
@@ -951,19 +956,20 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
     float3 gadj = make_float3(0.f, 0.f, 0.f);
     if constexpr (ADJ) {
       for (int h = L - 2; h >= 0; --h) {
+        const int acol = h >= 1 ? ACOL : NACC;
         if (!failed) {
 #pragma unroll
-          for (int j = 0; j < C / 8; ++j) {
-            uint32_t hi[4], lo[4];
+          for (int j = 0; j < C / 16; ++j) {
+            uint32_t hi[8], lo[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              split_h2(dl[8 * j + 2 * e], dl[8 * j + 2 * e + 1], hi[e], lo[e]);
+            for (int e = 0; e < 8; ++e) {
+              split_h2(dl[16 * j + 2 * e], dl[16 * j + 2 * e + 1], hi[e], lo[e]);
             }
-            *reinterpret_cast<uint4*>(A + a_off<NA>(row, j)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<uint4*>(A + a_off<NA>(row, C / 8 + j)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            tmem_st8(t_row + acol + 8 * j, hi);
+            tmem_st8(t_row + acol + C / 2 + 8 * j, lo);
           }
+          tmem_wait_st();
         }
-        fence_proxy_async();
         tc_fence_before();
         bar_sync(bar_id, 128);
         if (misc[4 + wg]) { stop = true; break; }
@@ -972,11 +978,11 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
 #pragma unroll
           for (int kk = 0; kk < 2 * C / 16; ++kk) {
             const uint32_t ka = ((16 * kk) >> 6), kb = ((16 * kk) & 63) * 2;
-            const uint64_t ad = a_desc<NA>(a_addr + kk * 256);
+            const uint32_t ad = d_tmem + acol + 8 * kk;
             if (h >= 1)
-              mma_f16(d_tmem, ad, sw128_desc(bht_addr + (h - 1) * NAH * BT + ka * BT + kb), IDESC, kk > 0);
+              mma_f16_ta(d_tmem, ad, sw128_desc(bht_addr + (h - 1) * NAH * BT + ka * BT + kb), IDESC, kk > 0);
             else
-              mma_f16(d_tmem, ad, sw128_desc(b0t_addr + ka * (K0 * 128) + kb), idesc_n(K0), kk > 0);
+              mma_f16_ta(d_tmem, ad, sw128_desc(b0t_addr + ka * (K0 * 128) + kb), idesc_n(K0), kk > 0);
           }
           mma_commit(mb);
         }
