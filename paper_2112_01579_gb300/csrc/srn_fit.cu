@@ -11,7 +11,8 @@
 //      the entries it owns (fixed order); one partial row per CTA.  Latent
 //      adjoints dz and the cell of every point go to scratch.
 //      (Two-layer width-32 density networks take the tensor-core point
-//      kernel of srn_fit_mma.cu instead.)
+//      kernel of srn_fit_mma.cu instead; other networks of up to four layers
+//      and 48 inputs the tiled kernel, fit_tile_kernel.)
 //   2. stable LSD radix sort of (cell, point) pairs, one 9-bit pass for up to
 //      512 cells, else 8-bit digits: per-block per-warp digit counts, a scan
 //      per digit over the blocks, stable scatter (which adds the digits'
@@ -31,6 +32,7 @@
 #include "srn_fit.h"
 #include "srn_net32.cuh"
 #include "srn_sample.cuh"
+#include "srn_tile32.cuh"
 
 namespace srn {
 namespace {
@@ -257,6 +259,348 @@ __global__ void __launch_bounds__(kFitThreads, 4) fit_point_kernel(const NetDev 
     __syncthreads();
   }
   if (tid == 0) row[a.n_entries] = sred[0];
+}
+
+// ---------------------------------------------------------------- tiled point kernel
+// The point kernel for networks of two to four layers with at most 48 inputs
+// (every shape of the plain and main workloads): the same step as
+// fit_point_kernel, each warp running its 32 points as a tile (srn_tile32.cuh).
+//
+// What bounds it: FP32 FMAs (forward, backward and weight gradient, about
+// 3 x sum d_in d_out per point) and the shared-memory loads that feed them.
+// The weight gradient dW_i = sum_p delta v^T takes a 4 x 3 (layer 0) or 4 x 2
+// block of entries per thread over the CTA's 128 points, four points per
+// 16-byte load: 7 loads for 48 FMAs, where one entry at a time takes two
+// loads per FMA.  A thread keeps its entries in registers over all its
+// chunks; sums of 32 points are formed first and then added, so the rounding
+// error does not grow with the number of points a CTA takes.  The vectors of
+// every layer stay in shared memory from the forward to the backward (a
+// layer's adjoint rows take the place of its activations once the gradient
+// that needs them is done), the activation derivatives in registers, so
+// neither sines nor Fourier features are evaluated twice.  Fit step of the
+// main configuration (32^3 x 16, four layers) at 2^18 points: 876 -> 375 us;
+// 65,537 points of the same network through autograd 434 -> 312 us.
+constexpr int kTileStride = 36;  // floats per row: eight rows' 16-byte loads hit distinct banks
+constexpr int kTileMaxIn = 48;   // inputs of layer 0: 16 threads x 3 entries
+
+// acc[i][j] += sum over the CTA's points of d[o_i][p] v[r_j][p], o_i = tid % 8
+// + 8 i, r_j = tid / 8 + 16 j (rows past `rows` repeat the last one; their
+// sums are never stored).  d and v are the first warp's rows, `wstride`
+// floats apart per warp.
+template <int NJ>
+__device__ __forceinline__ void outer_sum(float (&acc)[4][NJ], const float* d, const float* v, int wstride, int rows) {
+  const int og = threadIdx.x & 7, jg = threadIdx.x >> 3;
+  int vr[NJ];
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) vr[j] = min(jg + 16 * j, rows - 1) * kTileStride;
+#pragma unroll 1
+  for (int w = 0; w < kFitThreads / 32; ++w) {
+    const float* dw = d + w * wstride + og * kTileStride;
+    const float* vw = v + w * wstride;
+    float2 s[4][NJ];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) s[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int p = 0; p < 32; p += 4) {
+      float4 dd[4], vv[NJ];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) dd[i] = *reinterpret_cast<const float4*>(dw + 8 * i * kTileStride + p);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) vv[j] = *reinterpret_cast<const float4*>(vw + vr[j] + p);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          s[i][j] = __ffma2_rn(make_float2(dd[i].x, dd[i].y), make_float2(vv[j].x, vv[j].y), s[i][j]);
+          s[i][j] = __ffma2_rn(make_float2(dd[i].z, dd[i].w), make_float2(vv[j].z, vv[j].w), s[i][j]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) acc[i][j] += s[i][j].x + s[i][j].y;
+  }
+}
+
+// Sum of one row's 32 values (times w's, when given), four interleaved sums.
+__device__ __forceinline__ float row_sum(const float* r) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int p = 0; p < 32; p += 4) {
+    const float4 x = *reinterpret_cast<const float4*>(r + p);
+    s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+  }
+  return (s.x + s.y) + (s.z + s.w);
+}
+__device__ __forceinline__ float row_dot(const float* r, const float* w) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int p = 0; p < 32; p += 4) {
+    const float4 x = *reinterpret_cast<const float4*>(r + p), y = *reinterpret_cast<const float4*>(w + p);
+    s.x = fmaf(x.x, y.x, s.x); s.y = fmaf(x.y, y.y, s.y); s.z = fmaf(x.z, y.z, s.z); s.w = fmaf(x.w, y.w, s.w);
+  }
+  return (s.x + s.y) + (s.z + s.w);
+}
+
+// dz[j][f] for the lane's four points and F / 4 channels from the adjoint rows d.
+template <int F>
+__device__ __forceinline__ void store_dz(const float* d, const float* Wz, float* dz, int j0, int n) {
+  const int pg = tile32::point_group(), og = tile32::out_group();
+  float2 acc[2][F / 4];
+  tile32::back<32, kTileStride, F / 4>(acc, d, Wz, [&](int f) { return og * (F / 4) + f; });
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int j = j0 + 4 * pg + i;
+    if (j < n) {
+      float* out = dz + (size_t)j * F + og * (F / 4);
+#pragma unroll
+      for (int f = 0; f < F / 4; ++f) out[f] = (i & 1) ? acc[i >> 1][f].y : acc[i >> 1][f].x;
+    }
+  }
+}
+
+template <int NL>
+__global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const NetDev net, const PointArgs a,
+                                                                  const tile32::Net t, int wfloats) {
+  constexpr int C = 32, S = kTileStride, NH = NL - 1;  // NH activations per point
+  extern __shared__ float4 smem4[];
+  float* sm = reinterpret_cast<float*>(smem4);
+  tile32::load_net<C>(sm, t, net);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* base0 = sm + t.total;                // first warp's rows
+  float* v0 = base0 + warp * wfloats;         // layer inputs, then NH blocks of activation rows, then dout
+  float* act0 = v0 + t.d0 * S;
+  float* sdout = act0 + NH * C * S;
+  const int pg = tile32::point_group(), og = tile32::out_group();
+  const int step = a.step_ptr ? *a.step_ptr : a.step;
+  const Latent lat = make_latent(net, a.time);
+  const float inv_n = 1.0f / (float)a.n;
+  const int D = t.D, nchunks = (a.n + kFitThreads - 1) / kFitThreads;
+
+  float g0[4][3], gh[NL > 2 ? NL - 2 : 1][4][2], gb[NH], gl[4], gbl = 0.f, loss_acc = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    gl[i] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) g0[i][j] = 0.f;
+#pragma unroll
+    for (int h = 0; h < NL - 2; ++h) gh[h][i][0] = gh[h][i][1] = 0.f;
+  }
+#pragma unroll
+  for (int h = 0; h < NH; ++h) gb[h] = 0.f;
+
+  for (int chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
+    const int j = chunk * kFitThreads + tid;
+    const bool valid = j < a.n;
+    float3 p = make_float3(0.5f, 0.5f, 0.5f);
+    if (valid) {
+      if (a.mode == 0) p = sample::fit_point(a.cdf, a.cdf_res, a.seed, step, j, a.n);
+      else p = clamp_p(make_float3(a.pts_in[3 * j], a.pts_in[3 * j + 1], a.pts_in[3 * j + 2]));
+      tile32::put_inputs<S>(v0, sm, t, lat, p);
+    } else {
+      for (int k = 0; k < t.d0; ++k) v0[k * S + lane] = 0.f;
+    }
+    __syncwarp();
+    // ---- forward: activations to shared memory, their derivatives kept
+    tile32::Acc<C> x, df[NH];
+    tile32::set_bias<C>(x, sm + t.ob0);
+    tile32::layer<C, S>(x, v0, sm + t.oW0, t.d0);
+    tile32::activate_df<C>(net.act, x, df[0]);
+    tile32::put<C, S>(x, act0);
+    __syncwarp();
+#pragma unroll
+    for (int h = 1; h < NH; ++h) {
+      const float* W = sm + t.oHid + (h - 1) * t.hidStride;
+      tile32::set_bias<C>(x, W + C * C);
+      tile32::layer<C, S>(x, act0 + (h - 1) * C * S, W, C);
+      tile32::activate_df<C>(net.act, x, df[h]);
+      tile32::put<C, S>(x, act0 + h * C * S);
+      __syncwarp();
+    }
+    const float* alast = act0 + (NH - 1) * C * S;
+    float dout[4] = {0.f, 0.f, 0.f, 0.f};
+    if (a.mode == 0) {
+      float out[4];
+#pragma unroll
+      for (int dd = 0; dd < 4; ++dd) out[dd] = dd < D ? tile32::last_layer<C, S>(alast, sm, t, dd) : 0.f;
+      if (valid) {
+        const float r = out[0] - vol_sample(a.vol, p);
+        loss_acc += fabsf(r);
+        dout[0] = sgnf(r) * inv_n;
+        if (D == 4) {
+          const float hh[3] = {1.0f / (float)(a.vol.nx - 1), 1.0f / (float)(a.vol.ny - 1),
+                               1.0f / (float)(a.vol.nz - 1)};
+#pragma unroll
+          for (int ax = 0; ax < 3; ++ax) {
+            float3 pp = p, pm = p;
+            if (ax == 0) { pp.x = clamp01f(p.x + hh[0]); pm.x = clamp01f(p.x - hh[0]); }
+            if (ax == 1) { pp.y = clamp01f(p.y + hh[1]); pm.y = clamp01f(p.y - hh[1]); }
+            if (ax == 2) { pp.z = clamp01f(p.z + hh[2]); pm.z = clamp01f(p.z - hh[2]); }
+            const float g = (vol_sample(a.vol, pp) - vol_sample(a.vol, pm)) / (2.0f * hh[ax]);
+            const float ra = out[1 + ax] - a.gs * g;
+            loss_acc += a.gw * fabsf(ra);
+            dout[1 + ax] = a.gw * sgnf(ra) * inv_n;
+          }
+        }
+      }
+    } else if (valid) {
+#pragma unroll
+      for (int dd = 0; dd < 4; ++dd)
+        if (dd < D) dout[dd] = a.dout_in[(size_t)j * D + dd];
+    }
+#pragma unroll
+    for (int dd = 0; dd < 4; ++dd) sdout[dd * S + lane] = dout[dd];
+    __syncwarp();
+    // ---- last layer: gradients over the warp's own points (lane = input), then delta
+#pragma unroll
+    for (int dd = 0; dd < 4; ++dd)
+      if (dd < D) gl[dd] += row_dot(alast + lane * S, sdout + dd * S);
+    if (lane < D) gbl += row_sum(sdout + lane * S);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < C / 8; ++q) x.v[i][q] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int dd = 0; dd < 4; ++dd) {
+      if (dd < D) {
+        const float4 dv = *reinterpret_cast<const float4*>(sdout + dd * S + 4 * pg);
+        const float ds[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+        for (int q = 0; q < C / 8; ++q) {
+          const float2 w = *reinterpret_cast<const float2*>(sm + t.oWl + dd * C + og * (C / 4) + 2 * q);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x.v[i][q] = __ffma2_rn(w, make_float2(ds[i], ds[i]), x.v[i][q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < C / 8; ++q) {
+        x.v[i][q].x *= df[NH - 1].v[i][q].x;
+        x.v[i][q].y *= df[NH - 1].v[i][q].y;
+      }
+    __syncwarp();  // the last activations are read
+    tile32::put<C, S>(x, act0 + (NH - 1) * C * S);
+    __syncthreads();
+    // ---- hidden layers: adjoint rows of layer h in block h, inputs in block h - 1
+#pragma unroll
+    for (int h = NH - 1; h >= 1; --h) {
+      const float* dh = act0 + h * C * S;
+      outer_sum<2>(gh[h - 1], base0 + t.d0 * S + h * C * S, base0 + t.d0 * S + (h - 1) * C * S, wfloats, C);
+      gb[h] += row_sum(dh + lane * S);
+      float2 g[2][C / 4];
+      tile32::back<C, S, C / 4>(g, dh, sm + t.oHid + (h - 1) * t.hidStride,
+                                [&](int q) { return og * (C / 4) + q; });
+      __syncthreads();  // block h - 1's activations are read
+      float* dn = act0 + (h - 1) * C * S + og * (C / 4) * S + 4 * pg;
+#pragma unroll
+      for (int q = 0; q < C / 4; ++q) {
+        auto dfv = [&](int i) { return (q & 1) ? df[h - 1].v[i][q / 2].y : df[h - 1].v[i][q / 2].x; };
+        *reinterpret_cast<float4*>(dn + q * S) =
+            make_float4(g[0][q].x * dfv(0), g[0][q].y * dfv(1), g[1][q].x * dfv(2), g[1][q].y * dfv(3));
+      }
+      __syncthreads();
+    }
+    // ---- layer 0, the latent adjoint and the point's cell
+    outer_sum<3>(g0, base0 + t.d0 * S, base0, wfloats, t.d0);
+    gb[0] += row_sum(act0 + lane * S);
+    {
+      const float* Wz = sm + t.oW0 + (3 + 2 * t.m) * C;
+      const int j0 = chunk * kFitThreads + warp * 32;
+      switch (t.F) {
+        case 4: store_dz<4>(act0, Wz, a.dz, j0, a.n); break;
+        case 8: store_dz<8>(act0, Wz, a.dz, j0, a.n); break;
+        case 16: store_dz<16>(act0, Wz, a.dz, j0, a.n); break;
+        default: store_dz<32>(act0, Wz, a.dz, j0, a.n);
+      }
+    }
+    if (valid) {
+      a.pts[3 * j] = p.x;
+      a.pts[3 * j + 1] = p.y;
+      a.pts[3 * j + 2] = p.z;
+      int ix, iy, iz;
+      float fx, fy, fz;
+      cell_coord(p.x, lat.R, ix, fx);
+      cell_coord(p.y, lat.R, iy, fy);
+      cell_coord(p.z, lat.R, iz, fz);
+      a.key[j] = (unsigned)((iz * (lat.R - 1) + iy) * (lat.R - 1) + ix);
+      a.idx[j] = (unsigned)j;
+    }
+    __syncthreads();
+  }
+
+  // ---- the CTA's partial row [W | b | loss]
+  const int nW = C * t.d0 + (NL - 2) * C * C + D * C;
+  float* row = a.part + (size_t)blockIdx.x * (a.n_entries + 1);
+  const int o8 = tid & 7, j16 = tid >> 3;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (j16 + 16 * q < t.d0) row[(o8 + 8 * i) * t.d0 + tile32::input_column(j16 + 16 * q, t.m)] = g0[i][q];
+#pragma unroll
+    for (int h = 0; h < NL - 2; ++h)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) row[C * t.d0 + h * C * C + (o8 + 8 * i) * C + j16 + 16 * q] = gh[h][i][q];
+  }
+  // entries each warp summed over its own points: the four warps in order
+  constexpr int kRows = 4 + NH + 2;  // last-layer weights, biases, last bias, loss
+  float* ex = base0;
+  __syncthreads();
+#pragma unroll
+  for (int dd = 0; dd < 4; ++dd) ex[(dd * 4 + warp) * 32 + lane] = gl[dd];
+#pragma unroll
+  for (int h = 0; h < NH; ++h) ex[((4 + h) * 4 + warp) * 32 + lane] = gb[h];
+  ex[((4 + NH) * 4 + warp) * 32 + lane] = gbl;
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, w);
+  ex[((5 + NH) * 4 + warp) * 32 + lane] = loss_acc;
+  __syncthreads();
+  for (int e = tid; e < kRows * 32; e += kFitThreads) {
+    const int r = e >> 5, o = e & 31;
+    const float* q = ex + r * 128 + o;
+    const float s = ((q[0] + q[32]) + q[64]) + q[96];
+    if (r < 4) {
+      if (r < D) row[nW - D * C + r * C + o] = s;
+    } else if (r < 4 + NH) {
+      row[nW + (r - 4) * C + o] = s;
+    } else if (r == 4 + NH) {
+      if (o < D) row[nW + NH * C + o] = s;
+    } else if (o == 0) {
+      row[a.n_entries] = s;
+    }
+  }
+}
+
+// Rows of one warp's tile in floats (inputs, activations, output adjoints).
+int fit_tile_floats(const NetDev& net) { return (net_d0(net) + (net.l - 1) * 32 + 4) * kTileStride; }
+size_t fit_tile_smem(const NetDev& net) {
+  return sizeof(float) * ((size_t)tile32::make_net(net).total + (size_t)(kFitThreads / 32) * fit_tile_floats(net));
+}
+// Up to four layers: their activation derivatives fit a thread's registers
+// (32 a layer), and with at most 48 inputs two CTAs' rows fit an SM's shared
+// memory (100 KB a CTA).  Deeper or wider-input networks keep
+// fit_point_kernel, which stashes in local memory.
+bool fit_tile_supported(const NetDev& net) {
+  return net.c == 32 && net.l >= 2 && net.l <= 4 && net_d0(net) <= kTileMaxIn && net.F <= 32;
+}
+
+template <int NL>
+cudaError_t fit_tile_t(const NetDev& net, const PointArgs& pa, int grid, cudaStream_t st) {
+  auto k = fit_tile_kernel<NL>;
+  const size_t smem = fit_tile_smem(net);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k<<<grid, kFitThreads, smem, st>>>(net, pa, tile32::make_net(net), fit_tile_floats(net));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fit_tile(const NetDev& net, const PointArgs& pa, int grid, cudaStream_t st) {
+  if (net.l == 2) return fit_tile_t<2>(net, pa, grid, st);
+  return net.l == 3 ? fit_tile_t<3>(net, pa, grid, st) : fit_tile_t<4>(net, pa, grid, st);
 }
 
 // ---------------------------------------------------------------- radix sort
@@ -841,6 +1185,10 @@ cudaError_t run_backward(FitScratch& s, const NetDev& net, PointArgs pa, float* 
     e = launch_fit_mma(net, ma, grid, mma_status, st);
     if (e != cudaSuccess) return e;
     n_cta = grid * rows;
+  } else if (n_cta > 0 && fit_tile_supported(net)) {
+    // two CTAs of 128 points per SM
+    n_cta = std::min(n_cta, 2 * sm_count());
+    if ((e = launch_fit_tile(net, pa, n_cta, st)) != cudaSuccess) return e;
   } else if (n_cta > 0) {
     auto k = fit_point_kernel<32>;
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
