@@ -1,9 +1,9 @@
 // Section 6.2 adaptive resampling: the prediction-error grid and the
 // error-proportional point distribution the fit draws from.
 //
-// Error grid: one thread per voxel evaluates the FP32 network (the fused
-// layer code of the FP32 path, weights staged in shared memory) at the
-// voxel's Philox positions and averages |rho - V| in a fixed order.
+// Error grid: one lane per voxel draws the voxel's Philox positions, its warp
+// evaluates the FP32 network for 32 voxels at a time (srn_tile32.cuh), and
+// the lane averages |rho - V| in a fixed order.
 //
 // Distribution: every decision that turns floating point into an integer is
 // an IEEE round-to-nearest operation (FP32 multiply / divide, floor), the
@@ -12,8 +12,8 @@
 // offset pass), and a binary search per point in the fit's point kernel.
 // The result is exact and identical on every run.
 #include "srn_fit.h"
-#include "srn_net32.cuh"
 #include "srn_sample.cuh"
+#include "srn_tile32.cuh"
 
 namespace srn {
 namespace {
@@ -24,41 +24,52 @@ constexpr int kErrThreads = 128;
 constexpr int kCdfThreads = kCdfBlock / 2;  // two weights per thread
 
 template <int C>
-__global__ void __launch_bounds__(kErrThreads) error_grid_kernel(const NetDev net, const VolDev vol, int res, int spv,
-                                                                 unsigned long long seed, float time,
-                                                                 float* __restrict__ E, const Layout L) {
+__global__ void __launch_bounds__(kErrThreads, C == 32 ? 4 : 2)
+    error_grid_kernel(const NetDev net, const VolDev vol, int res, int spv, unsigned long long seed, float time,
+                      float* __restrict__ E, const tile32::Net t, int rows) {
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
-  load_net<C>(sm, L, net);
+  tile32::load_net<C>(sm, t, net);
+  const tile32::Ctx ctx{sm, &t, net.act, tile32::nerf_rows(sm + t.oF, t.m)};
+  const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* x = sm + t.total + warp * rows * tile32::kPts;
   const long long nvox = (long long)res * res * res;
-  const long long v = (long long)blockIdx.x * kErrThreads + threadIdx.x;
-  if (v >= nvox) return;
   const Latent lat = make_latent(net, time);
-  const int vx = (int)(v % res), vy = (int)((v / res) % res), vz = (int)(v / ((long long)res * res));
   const uint2 key = sample::seed_key(seed);
-  float acc = 0.0f;
-  for (int i = 0; i < spv; ++i) {
-    const uint4 o = sample::philox4x32_10(make_uint4((unsigned)v, (unsigned)i, 0x4552u, 0u), key);
-    const float3 p = make_float3(sample::voxel_coord(vx, o.x, res), sample::voxel_coord(vy, o.y, res),
-                                 sample::voxel_coord(vz, o.z, res));
-    float out[4];
-    forward<C, false>(sm, L, net.act, lat, p, out, nullptr);
-    acc += fabsf(out[0] - vol_sample(vol, p));
+  const float3 zero = make_float3(0.f, 0.f, 0.f);
+  for (long long tile = (long long)blockIdx.x * wpb + warp; tile * 32 < nvox; tile += (long long)gridDim.x * wpb) {
+    // lanes past the last voxel evaluate it again and write nothing
+    const long long v = min(tile * 32 + lane, nvox - 1);
+    const int vx = (int)(v % res), vy = (int)((v / res) % res), vz = (int)(v / ((long long)res * res));
+    float acc = 0.0f;
+    for (int i = 0; i < spv; ++i) {
+      const uint4 o = sample::philox4x32_10(make_uint4((unsigned)v, (unsigned)i, 0x4552u, 0u), key);
+      const float3 p = make_float3(sample::voxel_coord(vx, o.x, res), sample::voxel_coord(vy, o.y, res),
+                                   sample::voxel_coord(vz, o.z, res));
+      tile32::forward<C, false>(ctx, x, x, lat, p, zero, nullptr);
+      acc += fabsf(tile32::last_layer<C, tile32::kPts>(x, sm, t, 0) - vol_sample(vol, p));
+      __syncwarp();
+    }
+    if (tile * 32 + lane < nvox) E[v] = acc / (float)spv;
   }
-  E[v] = acc / (float)spv;
 }
 
 template <int C>
 cudaError_t error_grid_t(const NetDev& net, const VolDev& vol, int res, int spv, unsigned long long seed, float time,
                          float* E, cudaStream_t st) {
-  Layout L = make_layout(net, false);
-  const size_t smem = (size_t)L.total * sizeof(float);
+  const tile32::Net t = tile32::make_net(net);
+  const int rows = t.d0 > C ? t.d0 : C, warps = tile32::warps_for(t, rows);
+  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = error_grid_kernel<C>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   const long long nvox = (long long)res * res * res;
-  k<<<(unsigned)((nvox + kErrThreads - 1) / kErrThreads), kErrThreads, smem, st>>>(net, vol, res, spv, seed, time, E,
-                                                                                   L);
+  const long long blocks = (nvox + 32 * warps - 1) / (32 * warps), most = 4ll * sms;
+  k<<<(unsigned)(blocks < most ? blocks : most), 32 * warps, smem, st>>>(net, vol, res, spv, seed, time, E, t, rows);
   return cudaGetLastError();
 }
 

@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const NetDev n
     if (valid) {
       if (a.mode == 0) p = sample::fit_point(a.cdf, a.cdf_res, a.seed, step, j, a.n);
       else p = clamp_p(make_float3(a.pts_in[3 * j], a.pts_in[3 * j + 1], a.pts_in[3 * j + 2]));
-      tile32::put_inputs<S>(v0, sm, t, lat, p);
+      tile32::put_inputs<S>(v0, sm, t, lat, false, p);
     } else {
       for (int k = 0; k < t.d0; ++k) v0[k * S + lane] = 0.f;
     }

@@ -1,42 +1,92 @@
 // FP32 CUDA-core fV-SRN kernels: ray-marching render (all shading modes)
 // and point evaluation (density, adjoint input gradient).
 //
-// One thread per ray / point.  The network (Section 3 layer equation, Eq. 1-2
-// Fourier features, Section 4.2 latent grid) is staged once per block into
-// shared memory as FP32; every sample runs the whole MLP in registers, so no
-// intermediate state touches global memory (the fused-network idea of
-// Section 4).  Layer 0 is accumulated feature by feature as each input
-// (position, sin/cos feature, latent channel) is produced, so the input
-// vector itself is never materialised.
+// A warp evaluates the network (Section 3 layer equation, Eq. 1-2 Fourier
+// features, Section 4.2 latent grid) for its 32 rays / points as one tile
+// (srn_tile32.cuh); rays, features, gathers and compositing are one lane per
+// ray / point.  The parameters are staged once per CTA in shared memory, and
+// no intermediate state touches global memory (the fused-network idea of
+// Section 4).
 #pragma once
 #include "srn_fp32.h"
-#include "srn_net32.cuh"
+#include "srn_tile32.cuh"
 
 namespace srn {
 namespace fp32 {
 
-constexpr int kThreads = 128;
+constexpr int kMaxThreads = 128;
 using namespace net32;
 
-// Render: each warp covers an 8 x 4 pixel tile; one thread per ray.
+// Rows of 32 floats a warp's tile needs: the inputs and activations share
+// one block, unless the backward needs the inputs again.
+inline int tile_rows(const tile32::Net& t, int C, bool adjoint, bool dout) {
+  return (adjoint ? t.d0 + C : (t.d0 > C ? t.d0 : C)) + (dout ? 4 : 0);
+}
+
+// Density (and gradient for shading) at the lanes' positions p + pl (pairs)
+// for shading mode SH; the finite-difference neighbours are offset as pairs.
+// All lanes of the warp take part.
 template <int C, int SH>
-__global__ void __launch_bounds__(kThreads) render_fp32_kernel(const NetDev net, const BatchDev b, const Layout L) {
+__device__ __forceinline__ float sample_field(const tile32::Ctx& c, float* rows, const Latent& lat, float3 p,
+                                              float3 pl, float fd_h, float3& g) {
+  constexpr int S = tile32::kPts;
+  const tile32::Net& t = *c.t;
+  if constexpr (SH == SRN_SHADE_ADJOINT) {
+    float* x = rows + t.d0 * S;
+    tile32::Acc<C> df[kMaxL - 1], a;
+    tile32::forward<C, true>(c, rows, x, lat, p, pl, df);
+    const float rho = tile32::last_layer<C, S>(x, c.sm, t, 0);
+    tile32::seed<C>(a, c.sm, t, nullptr);
+    g = tile32::input_gradient<C>(c, rows, x, lat, p, a, df);
+    return rho;
+  } else {
+    tile32::forward<C, false>(c, rows, rows, lat, p, pl, nullptr);
+    const float rho = tile32::last_layer<C, S>(rows, c.sm, t, 0);
+    if constexpr (SH == SRN_SHADE_HEAD)
+      g = make_float3(tile32::last_layer<C, S>(rows, c.sm, t, 1), tile32::last_layer<C, S>(rows, c.sm, t, 2),
+                      tile32::last_layer<C, S>(rows, c.sm, t, 3));
+    __syncwarp();
+    if constexpr (SH == SRN_SHADE_FD) {
+      float o[6];
+#pragma unroll 1
+      for (int k = 0; k < 6; ++k) {
+        float3 qh = p, ql = pl;
+        df::offset_axis(qh, ql, k >> 1, (k & 1) ? -fd_h : fd_h);
+        tile32::forward<C, false>(c, rows, rows, lat, qh, ql, nullptr);
+        const float v = tile32::last_layer<C, S>(rows, c.sm, t, 0);
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < 6; ++e)
+          if (e == k) o[e] = v;
+      }
+      g = make_float3((o[0] - o[1]) / (2.0f * fd_h), (o[2] - o[3]) / (2.0f * fd_h), (o[4] - o[5]) / (2.0f * fd_h));
+    }
+    return rho;
+  }
+}
+
+// Render: each warp covers an 8 x 4 pixel tile; one lane per ray.
+template <int C, int SH>
+__global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
+    render_fp32_kernel(const NetDev net, const BatchDev b, const tile32::Net t, int rows) {
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
   __shared__ TFDev tf;
   load_tf(tf, b.tf);
-  load_net<C>(sm, L, net);
+  tile32::load_net<C>(sm, t, net);
+  const tile32::Ctx ctx{sm, &t, net.act, tile32::nerf_rows(sm + t.oF, t.m)};
+  float* mine = sm + t.total + (threadIdx.x >> 5) * rows * tile32::kPts;
 
   const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * kThreads + threadIdx.x) >> 5;
+  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int tiles_x = (b.W + 7) / 8, tiles_y = (b.H + 3) / 4;
   const long long tpf = (long long)tiles_x * tiles_y;
   const long long frame = warp / tpf;
   if (frame >= (long long)b.n_times * b.n_views) return;
-  const int t = (int)(warp - frame * tpf);
-  const int px = (t % tiles_x) * 8 + (lane & 7), py = (t / tiles_x) * 4 + (lane >> 3);
+  const int tt = (int)(warp - frame * tpf);
+  const int px = (tt % tiles_x) * 8 + (lane & 7), py = (tt / tiles_x) * 4 + (lane >> 3);
   const int view = (int)(frame % b.n_views), ti = (int)(frame / b.n_views);
-  if (px >= b.W || py >= b.H) return;
+  const bool inside = px < b.W && py < b.H;
 
   const Latent lat = make_latent(net, b.times[ti]);
   // ray geometry in double-float arithmetic (srn_df.cuh): direction, box
@@ -45,13 +95,18 @@ __global__ void __launch_bounds__(kThreads) render_fp32_kernel(const NetDev net,
   df::Ray ray;
   float C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f;
   unsigned int ns = 0;
-  if (df::ray_setup(b.cams[view], b.W, b.H, px, py, ray)) {
-    const float3 d = make_float3(ray.d[0].h, ray.d[1].h, ray.d[2].h);
-    float len;
-    float3 p, pl;
-    for (int k = 0; df::segment(ray, k, b.step, len, p, pl); ++k) {
-      float3 g = make_float3(0.f, 0.f, 0.f);
-      float rho = sample_field<C, SH>(sm, L, net.act, lat, p, pl, b.fd_h, g);
+  bool live = inside && df::ray_setup(b.cams[view], b.W, b.H, px, py, ray);
+  const float3 d = live ? make_float3(ray.d[0].h, ray.d[1].h, ray.d[2].h) : make_float3(0.f, 0.f, 0.f);
+  float3 p = make_float3(0.5f, 0.5f, 0.5f), pl = make_float3(0.f, 0.f, 0.f);
+  for (int k = 0;; ++k) {
+    float len = 0.f;
+    live = live && df::segment(ray, k, b.step, len, p, pl);
+    if (!__any_sync(0xffffffffu, live)) break;
+    // lanes without a sample evaluate their last position (or the centre); nothing reads the result
+    float3 g = make_float3(0.f, 0.f, 0.f);
+    const float rho = sample_field<C, SH>(ctx, mine, lat, p, pl, b.fd_h, g);
+    __syncwarp();
+    if (live) {
       ++ns;
       float4 c = tf_eval(tf, rho);
       float alpha = -expm1f(-c.w * tf.opacity_scale * len);
@@ -61,11 +116,13 @@ __global__ void __launch_bounds__(kThreads) render_fp32_kernel(const NetDev net,
       C1 = fmaf(w, c.y, C1);
       C2 = fmaf(w, c.z, C2);
       A += w;
-      if (A >= b.et) break;
+      live = !(A >= b.et);
     }
   }
-  size_t idx = ((size_t)frame * b.H + py) * b.W + px;
-  reinterpret_cast<float4*>(b.out)[idx] = make_float4(C0, C1, C2, A);
+  if (inside) {
+    size_t idx = ((size_t)frame * b.H + py) * b.W + px;
+    reinterpret_cast<float4*>(b.out)[idx] = make_float4(C0, C1, C2, A);
+  }
   add_samples(b.samples, ns);
 }
 
@@ -73,71 +130,87 @@ __global__ void __launch_bounds__(kThreads) render_fp32_kernel(const NetDev net,
 // adjoint gradient grad[n][3] (when grad is not null); mode 2 writes the
 // input vector-Jacobian product grad[n][3] = sum_d dout[n][d] d out_d / d p.
 template <int C, int MODE>
-__global__ void __launch_bounds__(kThreads) eval_fp32_kernel(const NetDev net, const float* __restrict__ pts, int n,
-                                                             float time, float* __restrict__ out,
-                                                             float* __restrict__ grad,
-                                                             const float* __restrict__ dout, const Layout L) {
+__global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
+    eval_fp32_kernel(const NetDev net, const float* __restrict__ pts, int n, float time, float* __restrict__ out,
+                     float* __restrict__ grad, const float* __restrict__ dout, const tile32::Net t, int rows) {
+  constexpr int S = tile32::kPts;
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
-  load_net<C>(sm, L, net);
-  const int j = blockIdx.x * kThreads + threadIdx.x;
-  if (j >= n) return;
+  tile32::load_net<C>(sm, t, net);
+  const tile32::Ctx ctx{sm, &t, net.act, tile32::nerf_rows(sm + t.oF, t.m)};
+  float* mine = sm + t.total + (threadIdx.x >> 5) * rows * S;
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   const Latent lat = make_latent(net, time);
-  float3 p = clamp_p(make_float3(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2]));
-  float o[4];
-  if (MODE == 0) {
-    forward<C, false>(sm, L, net.act, lat, p, o, nullptr);
-    for (int d = 0; d < L.D; ++d) out[(size_t)j * L.D + d] = o[d];
-  } else if (MODE == 1) {
-    float hs[kMaxL][C];
-    forward<C, true>(sm, L, net.act, lat, p, o, hs);
-    out[j] = o[0];
-    if (grad) {
-      float3 g = adjoint<C>(sm, L, net.act, lat, p, hs, sm + L.oWl);
-      grad[3 * j] = g.x;
-      grad[3 * j + 1] = g.y;
-      grad[3 * j + 2] = g.z;
+  const float3 zero = make_float3(0.f, 0.f, 0.f);
+  for (long long tile = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); tile * 32 < n;
+       tile += (long long)gridDim.x * wpb) {
+    const long long j = tile * 32 + lane;
+    const bool valid = j < n;
+    const float3 p = valid ? clamp_p(make_float3(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2]))
+                           : make_float3(0.5f, 0.5f, 0.5f);
+    if constexpr (MODE == 0) {
+      tile32::forward<C, false>(ctx, mine, mine, lat, p, zero, nullptr);
+      for (int d = 0; d < t.D; ++d) {
+        const float v = tile32::last_layer<C, S>(mine, sm, t, d);
+        if (valid) out[(size_t)j * t.D + d] = v;
+      }
+    } else {
+      float* x = mine + t.d0 * S;
+      float* seeds = x + C * S;
+      tile32::Acc<C> df[kMaxL - 1], a;
+      tile32::forward<C, true>(ctx, mine, x, lat, p, zero, df);
+      if constexpr (MODE == 1) {
+        const float v = tile32::last_layer<C, S>(x, sm, t, 0);
+        if (valid) out[j] = v;
+        if (grad) tile32::seed<C>(a, sm, t, nullptr);
+      } else {
+        for (int d = 0; d < t.D; ++d) seeds[d * S + lane] = valid ? dout[(size_t)j * t.D + d] : 0.f;
+        __syncwarp();
+        tile32::seed<C>(a, sm, t, seeds);
+      }
+      if (grad) {
+        const float3 g = tile32::input_gradient<C>(ctx, mine, x, lat, p, a, df);
+        if (valid) {
+          grad[3 * j] = g.x;
+          grad[3 * j + 1] = g.y;
+          grad[3 * j + 2] = g.z;
+        }
+      }
     }
-  } else {
-    float hs[kMaxL][C];
-    forward<C, true>(sm, L, net.act, lat, p, o, hs);
-    float seed[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) seed[c] = 0.0f;
-    for (int d = 0; d < L.D; ++d) {
-      const float s = dout[(size_t)j * L.D + d];
-#pragma unroll
-      for (int c = 0; c < C; ++c) seed[c] = fmaf(s, sm[L.oWl + d * C + c], seed[c]);
-    }
-    const float3 g = adjoint<C>(sm, L, net.act, lat, p, hs, seed);
-    grad[3 * j] = g.x;
-    grad[3 * j + 1] = g.y;
-    grad[3 * j + 2] = g.z;
+    __syncwarp();
   }
 }
 
 template <int C, int SH>
 cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s) {
-  Layout L = make_layout(net, SH == SRN_SHADE_ADJOINT);
-  size_t smem = (size_t)L.total * sizeof(float);
+  const tile32::Net t = tile32::make_net(net);
+  const int rows = tile_rows(t, C, SH == SRN_SHADE_ADJOINT, false), warps = tile32::warps_for(t, rows);
+  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = render_fp32_kernel<C, SH>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   long long tiles = (long long)((b.W + 7) / 8) * ((b.H + 3) / 4) * b.n_views * b.n_times;
-  long long blocks = (tiles + (kThreads / 32) - 1) / (kThreads / 32);
-  k<<<(unsigned)blocks, kThreads, smem, s>>>(net, b, L);
+  long long blocks = (tiles + warps - 1) / warps;
+  k<<<(unsigned)blocks, 32 * warps, smem, s>>>(net, b, t, rows);
   return cudaGetLastError();
 }
 
 template <int C, int MODE>
 cudaError_t launch_eval_t(const NetDev& net, const float* pts, int n, float time, float* out, float* grad,
                           const float* dout, cudaStream_t s) {
-  Layout L = make_layout(net, MODE != 0);
-  size_t smem = (size_t)L.total * sizeof(float);
+  const tile32::Net t = tile32::make_net(net);
+  const int rows = tile_rows(t, C, MODE != 0, MODE == 2), warps = tile32::warps_for(t, rows);
+  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = eval_fp32_kernel<C, MODE>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<(n + kThreads - 1) / kThreads, kThreads, smem, s>>>(net, pts, n, time, out, grad, dout, L);
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  // CTAs stage the parameters once and walk the tiles: at most four per SM
+  const long long blocks = ((long long)n + 32 * warps - 1) / (32 * warps), most = 4ll * sms;
+  k<<<(unsigned)(blocks < most ? blocks : most), 32 * warps, smem, s>>>(net, pts, n, time, out, grad, dout, t, rows);
   return cudaGetLastError();
 }
 

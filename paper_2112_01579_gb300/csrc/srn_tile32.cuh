@@ -11,6 +11,11 @@
 // the 4 x C/4 layout, so their values never need a lane of their own.  Every
 // output is the bias plus its products in input order, one FMA each: the same
 // bits as a thread walking the inputs alone.
+//
+// Measured against one thread per point with out-of-line library sines: error
+// grid of 128^3 x 8 evaluations of the main configuration 5.68 -> 3.41 ms
+// (4.9 G evaluations/s; the FMA pipe that takes packed FMAs 68 % busy, the
+// shared-memory data pipe 70 %), the plain workload's 128^2 frame 968 -> 540 us.
 #pragma once
 
 #include "srn_net32.cuh"
@@ -156,6 +161,118 @@ __device__ __forceinline__ void activate_df(int act, Acc<C>& a, Acc<C>& d) {
     }
 }
 
+// ---- inline sine / cosine of the tile paths
+// Reduction by Cody and Waite (Software Manual for the Elementary Functions,
+// 1980) in FMA form, then minimax polynomials from a Remez exchange on the
+// absolute error, each coefficient rounded to FP32 before the next was
+// fitted: sin r on |r| <= 1.0005 pi/2 to 5.0e-9, cos r to 4.4e-10; on
+// |r| <= 1.001 pi/4 1.9e-9 and 1.1e-10 (before FP32 arithmetic rounds, about
+// 6e-8).  They cost a third of the issue slots of the accurate library
+// calls, which stay for arguments beyond kActMax and for Fourier matrices
+// that are not powers of two.
+constexpr float kActMax = 1.0e4f;  // below: rint(x / pi) is off by less than 2e-4, inside the fitted range
+
+__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
+
+// r = x - k pi with k = rint(x / pi) (pi as FP32 hi + lo); t's lowest bit is k's parity.
+__device__ __forceinline__ float2 reduce_pi(float2 x, float2& t) {
+  const float kMagic = 12582912.0f;  // 1.5 2^23
+  t = __ffma2_rn(x, f2(0.318309886183790672f), f2(kMagic));
+  const float2 k = __fadd2_rn(t, f2(-kMagic));
+  const float2 r = __ffma2_rn(k, f2(-3.14159274101257324f), x);
+  return __ffma2_rn(k, f2(8.74227765734758577e-8f), r);
+}
+__device__ __forceinline__ float2 sin_half(float2 r, float2 z) {
+  float2 p = __ffma2_rn(z, f2(2.59889998e-06f), f2(-0.000198060457f));
+  p = __ffma2_rn(z, p, f2(0.00833300874f));
+  p = __ffma2_rn(z, p, f2(-0.166666567f));
+  return __ffma2_rn(__fmul2_rn(r, z), p, r);
+}
+__device__ __forceinline__ float2 cos_half(float2 z) {
+  float2 p = __ffma2_rn(z, f2(-2.62090197e-07f), f2(2.47701792e-05f));
+  p = __ffma2_rn(z, p, f2(-0.00138885854f));
+  p = __ffma2_rn(z, p, f2(0.0416666567f));
+  return __ffma2_rn(__fmul2_rn(z, z), p, __ffma2_rn(z, f2(-0.5f), f2(1.0f)));
+}
+__device__ __forceinline__ float flip(float v, float t) {  // v (-1)^k
+  return __int_as_float(__float_as_int(v) ^ (__float_as_int(t) << 31));
+}
+
+// sin and cos of 2^j w p, w the FP32 value of 2 pi, from X = 2^j p (exact)
+// plus `lo` radians: in quarter turns, q = rint(4 X), f = X - q / 4 (exact),
+// w X = 2 pi X + e X with e = w - 2 pi, so modulo 2 pi the angle is
+// q pi / 2 + w f + e q / 4.
+__device__ __forceinline__ void turn_sincos(float X, float lo, float& s, float& c) {
+  const float kMagic = 12582912.0f;
+  const float t = fmaf(X, 4.0f, kMagic);
+  const float q4 = t - kMagic;
+  const float f = fmaf(q4, -0.25f, X);
+  const float r = fmaf(6.28318548202514648f, f, fmaf(4.37113900e-8f, q4, lo));
+  const float z = r * r;
+  float p = fmaf(z, -0.000194957684f, 0.00833198149f);
+  p = fmaf(z, p, -0.166666508f);
+  const float sr = fmaf(r * z, p, r);
+  p = fmaf(z, 2.44306702e-05f, -0.00138873013f);
+  p = fmaf(z, p, 0.0416666456f);
+  const float cr = fmaf(z * z, p, fmaf(z, -0.5f, 1.0f));
+  const int q = __float_as_int(t);
+  const float a = (q & 1) ? cr : sr, b = (q & 1) ? sr : cr;
+  s = __int_as_float(__float_as_int(a) ^ ((q & 2) << 30));
+  c = __int_as_float(__float_as_int(b) ^ (((q + 1) & 2) << 30));
+}
+constexpr int kTurnRows = 30;  // octaves 0..9: |e X| stays below 1e-4
+
+// Whether F's row k is w 2^(k div 3) on axis k mod 3 (block-wide answer).
+__device__ __forceinline__ bool nerf_rows(const float* F, int m) {
+  bool ok = m <= kTurnRows;
+  for (int i = threadIdx.x; ok && i < 3 * m; i += blockDim.x) {
+    const int k = i / 3, a = i - 3 * k;
+    ok = F[i] == (a == k % 3 ? 6.28318548202514648f * (float)(1 << (k / 3)) : 0.0f);
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+// Activation of the lane's values in place; DF: and its derivative.
+template <int C, bool DF>
+__device__ __forceinline__ void activate(int act, Acc<C>& a, Acc<C>* d) {
+  const bool snake = act == SRN_ACT_SNAKEALT;
+  float big = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < C / 8; ++q) big = fmaxf(big, fmaxf(fabsf(a.v[i][q].x), fabsf(a.v[i][q].y)));
+  if (__any_sync(0xffffffffu, !(big <= kActMax))) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < C / 8; ++q) {
+        const float2 x = a.v[i][q];
+        const float4 r = sincos_pair(x.x, x.y);
+        a.v[i][q] = snake ? make_float2(fmaf(0.5f, x.x, r.x * r.x), fmaf(0.5f, x.y, r.z * r.z)) : make_float2(r.x, r.z);
+        if (DF) d->v[i][q] = snake ? make_float2(0.5f + 2.0f * r.x * r.y, 0.5f + 2.0f * r.z * r.w) : make_float2(r.y, r.w);
+      }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < C / 8; ++q) {
+      const float2 x = a.v[i][q];
+      float2 t;
+      const float2 r = reduce_pi(x, t), z = __fmul2_rn(r, r);
+      const float2 s = sin_half(r, z);
+      float2 c = make_float2(0.f, 0.f);
+      if (DF) c = cos_half(z);
+      if (snake) {  // sin^2 and sin cos do not change with k
+        a.v[i][q] = __ffma2_rn(s, s, __fmul2_rn(x, f2(0.5f)));
+        if (DF) d->v[i][q] = __ffma2_rn(__fadd2_rn(s, s), c, f2(0.5f));
+      } else {
+        a.v[i][q] = make_float2(flip(s.x, t.x), flip(s.y, t.y));
+        if (DF) d->v[i][q] = make_float2(flip(c.x, t.x), flip(c.y, t.y));
+      }
+    }
+}
+
 // Writes the lane's values as rows (output index) of x.
 template <int C, int S>
 __device__ __forceinline__ void put(const Acc<C>& a, float* x) {
@@ -169,19 +286,36 @@ __device__ __forceinline__ void put(const Acc<C>& a, float* x) {
 
 // Input rows of the lane's point p (+ pl, the low part of a position carried
 // as a pair): [p, sin, cos, z, (t)].
+// NeRF Fourier rows (nerf) take the inline quarter-turn form.
 template <int S>
-__device__ __forceinline__ void put_inputs(float* x, const float* sm, const Net& t, const Latent& lat, float3 p,
-                                           float3 pl = make_float3(0.f, 0.f, 0.f)) {
+__device__ __forceinline__ void put_inputs(float* x, const float* sm, const Net& t, const Latent& lat, bool nerf,
+                                           float3 p, float3 pl = make_float3(0.f, 0.f, 0.f)) {
   float* v = x + (threadIdx.x & 31);
   v[0] = p.x;
   v[S] = p.y;
   v[2 * S] = p.z;
   const float* Fm = sm + t.oF;
-  for (int k = 0; k < t.m; ++k) {
-    float s, c;
-    net32::fourier_sincos(Fm + 3 * k, p, s, c, pl);
-    v[(3 + 2 * k) * S] = s;
-    v[(4 + 2 * k) * S] = c;
+  if (nerf) {
+    float w = 1.0f;
+    for (int k = 0; k < t.m; k += 3, w += w) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (k + a < t.m) {
+          const float pa = a == 0 ? p.x : (a == 1 ? p.y : p.z), la = a == 0 ? pl.x : (a == 1 ? pl.y : pl.z);
+          float s, c;
+          turn_sincos(w * pa, 6.28318548202514648f * (w * la), s, c);
+          v[(3 + 2 * (k + a)) * S] = s;
+          v[(4 + 2 * (k + a)) * S] = c;
+        }
+      }
+    }
+  } else {
+    for (int k = 0; k < t.m; ++k) {
+      float s, c;
+      net32::fourier_sincos(Fm + 3 * k, p, s, c, pl);
+      v[(3 + 2 * k) * S] = s;
+      v[(4 + 2 * k) * S] = c;
+    }
   }
   const Cell cell = net32::make_cell(lat, p);
   float* z = v + (3 + 2 * t.m) * S;
@@ -237,6 +371,187 @@ __device__ __forceinline__ void back(float2 (&acc)[2][N], const float* d, const 
       }
     }
   }
+}
+
+// ---- whole passes of a warp's 32 points
+struct Ctx {
+  const float* sm;
+  const Net* t;
+  int act;
+  bool nerf;
+};
+
+// Forward pass of the lanes' points: the last activations end up as rows of
+// x (read them with last_layer; a __syncwarp must follow before the rows are
+// overwritten).  v0: the input rows (may be x itself).  DF: df[h] receives
+// the derivative of activation h.
+template <int C, bool DF>
+__device__ __forceinline__ void forward(const Ctx& c, float* v0, float* x, const Latent& lat, float3 p, float3 pl,
+                                        Acc<C>* df) {
+  constexpr int S = kPts;
+  const Net& t = *c.t;
+  put_inputs<S>(v0, c.sm, t, lat, c.nerf, p, pl);
+  __syncwarp();
+  Acc<C> a;
+  set_bias<C>(a, c.sm + t.ob0);
+  layer<C, S>(a, v0, c.sm + t.oW0, t.d0);
+#pragma unroll 1
+  for (int h = 1; h < t.l - 1; ++h) {
+    activate<C, DF>(c.act, a, DF ? df + (h - 1) : nullptr);
+    __syncwarp();
+    put<C, S>(a, x);
+    __syncwarp();
+    const float* W = c.sm + t.oHid + (h - 1) * t.hidStride;
+    set_bias<C>(a, W + C * C);
+    layer<C, S>(a, x, W, C);
+  }
+  activate<C, DF>(c.act, a, DF ? df + (t.l - 2) : nullptr);
+  __syncwarp();
+  put<C, S>(a, x);
+  __syncwarp();
+}
+
+// The lane's seed sum_d s_d W_last[d][o] from D rows of output adjoints (row
+// stride kPts), or W_last's row 0 (rows == nullptr).
+template <int C>
+__device__ __forceinline__ void seed(Acc<C>& a, const float* sm, const Net& t, const float* rows) {
+  const float* w = sm + t.oWl + out_group() * (C / 4);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < C / 8; ++q)
+      a.v[i][q] = rows ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(w + 2 * q);
+  if (!rows) return;
+  for (int d = 0; d < t.D; ++d) {
+    const float4 dv = *reinterpret_cast<const float4*>(rows + d * kPts + 4 * point_group());
+    const float ds[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+    for (int q = 0; q < C / 8; ++q) {
+      const float2 wq = *reinterpret_cast<const float2*>(w + d * C + 2 * q);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a.v[i][q] = __ffma2_rn(wq, f2(ds[i]), a.v[i][q]);
+    }
+  }
+}
+
+// Input gradient of the lane's point (Section 5 "Adjoint") from the seed in
+// the tile layout: backward through the hidden layers, then the position,
+// Fourier and latent inputs.  v0 holds the input rows of the forward (its
+// latent rows are overwritten), x is scratch of C rows, df the derivatives.
+template <int C>
+__device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float* x, const Latent& lat, float3 p,
+                                                 Acc<C>& a, const Acc<C>* df) {
+  constexpr int S = kPts;
+  const Net& t = *c.t;
+  const int pg = point_group(), og = out_group(), lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < C / 8; ++q) a.v[i][q] = __fmul2_rn(a.v[i][q], df[t.l - 2].v[i][q]);
+  __syncwarp();
+  put<C, S>(a, x);
+  __syncwarp();
+#pragma unroll 1
+  for (int h = t.l - 2; h >= 1; --h) {
+    float2 g[2][C / 4];
+    back<C, S, C / 4>(g, x, c.sm + t.oHid + (h - 1) * t.hidStride, [&](int q) { return og * (C / 4) + q; });
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < C / 8; ++q) {
+        const float2 lo = g[i >> 1][2 * q], hi = g[i >> 1][2 * q + 1];
+        a.v[i][q] = __fmul2_rn((i & 1) ? make_float2(lo.y, hi.y) : make_float2(lo.x, hi.x), df[h - 1].v[i][q]);
+      }
+    __syncwarp();
+    put<C, S>(a, x);
+    __syncwarp();
+  }
+  // layer 0: the lane sums its share of the input rows for its four points
+  const float* W0 = c.sm + t.oW0;
+  float dp[4][3];
+  {
+    float2 g[2][1];
+    const int r = og < 3 ? og : 2;
+    back<C, S, 1>(g, x, W0, [&](int) { return r; });
+    const float v[4] = {g[0][0].x, g[0][0].y, g[1][0].x, g[1][0].y};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax) dp[i][ax] = og == ax ? v[i] : 0.f;
+  }
+  const float* Fm = c.sm + t.oF;
+#pragma unroll 1
+  for (int kb = 0; kb < t.m; kb += 8) {
+    const int ka[2] = {min(kb + og, t.m - 1), min(kb + og + 4, t.m - 1)};
+    float2 g[2][4];
+    back<C, S, 4>(g, x, W0, [&](int q) { return 3 + 2 * ka[q >> 1] + (q & 1); });
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      if (kb + og + 4 * e < t.m) {
+        const int k = ka[e];
+        const float4 s4 = *reinterpret_cast<const float4*>(v0 + (3 + 2 * k) * S + 4 * pg);
+        const float4 c4 = *reinterpret_cast<const float4*>(v0 + (4 + 2 * k) * S + 4 * pg);
+        const float sv[4] = {s4.x, s4.y, s4.z, s4.w}, cv[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float gs = (i & 1) ? g[i >> 1][2 * e].y : g[i >> 1][2 * e].x;
+          const float gc = (i & 1) ? g[i >> 1][2 * e + 1].y : g[i >> 1][2 * e + 1].x;
+          const float coef = gs * cv[i] - gc * sv[i];
+#pragma unroll
+          for (int ax = 0; ax < 3; ++ax) dp[i][ax] = fmaf(coef, Fm[3 * k + ax], dp[i][ax]);
+        }
+      }
+    }
+  }
+#pragma unroll 1
+  for (int fb = 0; fb < t.F; fb += 16) {
+    float2 g[2][4];
+    const int f0 = fb + 4 * og;
+    back<C, S, 4>(g, x, W0 + (3 + 2 * t.m) * C, [&](int q) { return min(f0 + q, t.F - 1); });
+    if (f0 < t.F) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4*>(v0 + (3 + 2 * t.m + f0 + q) * S + 4 * pg) =
+            make_float4(g[0][q].x, g[0][q].y, g[1][q].x, g[1][q].y);
+    }
+  }
+  float3 r = make_float3(0.f, 0.f, 0.f);
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    float mine = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float v = dp[i][ax];
+      v += __shfl_xor_sync(0xffffffffu, v, 8);
+      v += __shfl_xor_sync(0xffffffffu, v, 16);
+      v = __shfl_sync(0xffffffffu, v, lane >> 2);  // point i of group lane / 4
+      if ((lane & 3) == i) mine = v;
+    }
+    if (ax == 0) r.x = mine;
+    if (ax == 1) r.y = mine;
+    if (ax == 2) r.z = mine;
+  }
+  __syncwarp();
+  const Cell cell = net32::make_cell(lat, p);
+  const float* z = v0 + (3 + 2 * t.m) * S + lane;
+  for (int f = 0; f < t.F; f += 4) {
+    float4 gx, gy, gz;
+    net32::latent4_grad(lat, cell, f, gx, gy, gz);
+    const float g0 = z[f * S], g1 = z[(f + 1) * S], g2 = z[(f + 2) * S], g3 = z[(f + 3) * S];
+    r.x += g0 * gx.x + g1 * gx.y + g2 * gx.z + g3 * gx.w;
+    r.y += g0 * gy.x + g1 * gy.y + g2 * gy.z + g3 * gy.w;
+    r.z += g0 * gz.x + g1 * gz.y + g2 * gz.z + g3 * gz.w;
+  }
+  __syncwarp();
+  return r;
+}
+
+// Warps per CTA (4, 2 or 1): the parameters and `rows` rows of 32 floats per
+// warp within 227 KB.
+inline int warps_for(const Net& t, int rows) {
+  int w = 4;
+  while (w > 1 && sizeof(float) * ((size_t)t.total + (size_t)w * rows * kPts) > 227 * 1024) w /= 2;
+  return w;
 }
 
 }  // namespace tile32

@@ -55,3 +55,64 @@ def test_backward_matches_oracle(S, shape, n):
     assert _rel(g.cpu().numpy(), rg) <= TOL_GRAD
     assert _rel(w.cpu().numpy(), _flat(rW)) <= TOL_GRAD
     assert _rel(b.cpu().numpy(), _flat(rb)) <= TOL_GRAD
+
+
+def _points(n, seed):
+    pts = np.random.default_rng(seed).random((n, 3), dtype=np.float32)
+    pts[0] = [1.0, 0.0, 0.5]
+    return pts
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 129, 2500])
+@pytest.mark.parametrize("width,layers,m,nerf", [(32, 2, 12, True), (32, 8, 0, True), (32, 3, 33, True), (32, 4, 14, False),
+                                                 (48, 3, 22, True), (64, 2, 30, True)])
+def test_eval_matches_oracle(S, width, layers, m, nerf, n):
+    """Densities to 1e-5 of max(|rho|, 1), the gradient to its first-order
+    rounding-error bound, the one seeded with output adjoints to 1e-4 of
+    max(|g|, 1): the FP32 bounds.  33 NeRF rows and a general matrix take the
+    accurate library sine."""
+    import torch
+    p = synth.random_params(R=6, F=8, m=m, layers=layers, width=width, out_dim=4, act=synth.ACT_SNAKEALT, seed=n, grid_std=0.5)
+    if not nerf:
+        p["fourier"] = np.random.default_rng(5).normal(0, 8, (m, 3)).astype(np.float32)
+    net, on, pts = S.Network(p), oracle.OracleNet(p), _points(n, n)
+    x = torch.tensor(pts, device="cuda")
+    out = torch.full((n, 4), float("nan"), device="cuda")
+    S.srn_eval(net.ctx, x, out)
+    ref = oracle.net_forward(on, pts)
+    assert (np.abs(out.cpu().numpy() - ref) / np.maximum(np.abs(ref), 1.0)).max() <= 1e-5
+    rho, grad = torch.full((n,), float("nan"), device="cuda"), torch.full((n, 3), float("nan"), device="cuda")
+    S.srn_density_grad(net.ctx, x, rho, grad)
+    rref, gref = oracle.net_input_grad(on, pts)
+    assert torch.equal(rho, out[:, 0])
+    assert (np.abs(grad.cpu().numpy() - gref) / oracle.error_bounds(on, pts, oracle.PREC_FP32)[1]).max() <= 1.0
+    dout = np.random.default_rng(n + 9).standard_normal((n, 4), dtype=np.float32)
+    S.srn_input_backward(net.ctx, x, torch.tensor(dout, device="cuda"), grad)
+    vref = oracle.net_input_vjp(on, pts, dout)
+    assert (np.abs(grad.cpu().numpy() - vref) / np.maximum(np.abs(vref).max(axis=1, keepdims=True), 1.0)).max() <= 1e-4
+
+
+@pytest.mark.parametrize("act", [synth.ACT_SINE, synth.ACT_SNAKEALT])
+@pytest.mark.parametrize("arg", [9999.0, 1.0e4, 10001.0, 3.0e7])
+def test_eval_large_arguments(S, act, arg):
+    """Pre-activations at both sides of the inline sine's range, exact in FP32
+    (a bias alone), so only the sine's own error counts (1e-6, against weights
+    of at most 1); SnakeAlt's linear part takes no weight."""
+    import torch
+    p = synth.random_params(R=4, F=4, m=3, layers=2, width=32, act=act, seed=3, grid_std=0.5)
+    for k, sign in ((0, 1.0), (17, -1.0)):
+        p["weights"][0][k] = 0.0
+        p["biases"][0][k] = sign * arg
+        if act == synth.ACT_SNAKEALT:
+            p["weights"][1][0, k] = 0.0
+    if act == synth.ACT_SINE:
+        p["weights"][1][0, 0], p["weights"][1][0, 17] = 1.0, -0.5
+    net, pts = S.Network(p), _points(33, 4)
+    out = torch.full((33, 1), float("nan"), device="cuda")
+    S.srn_eval(net.ctx, torch.tensor(pts, device="cuda"), out)
+    ref = oracle.net_forward(oracle.OracleNet(p), pts)
+    assert np.abs(out.cpu().numpy() - ref).max() <= 2e-6
+    rho, grad = torch.empty(33, device="cuda"), torch.empty((33, 3), device="cuda")
+    S.srn_density_grad(net.ctx, torch.tensor(pts, device="cuda"), rho, grad)
+    gref = oracle.net_input_grad(oracle.OracleNet(p), pts)[1]
+    assert (np.abs(grad.cpu().numpy() - gref) / np.maximum(np.abs(gref).max(axis=1, keepdims=True), 1.0)).max() <= 1e-4
