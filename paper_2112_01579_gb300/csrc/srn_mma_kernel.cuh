@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   float* fm = reinterpret_cast<float*>(sm + plan.oFm);
   float* qp = reinterpret_cast<float*>(sm + plan.oQp);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + plan.oMbar);
-  volatile int* misc = reinterpret_cast<volatile int*>(sm + plan.oMisc);  // [0] tmem base, [1] nerf, [4+wg] fail
+  volatile int* misc = reinterpret_cast<volatile int*>(sm + plan.oMisc);  // [0] tmem base, [4+wg] fail
 
   const int tid = threadIdx.x;
   const int wg = tid >> 7, row = tid & 127, lane = tid & 31;
@@ -595,63 +595,67 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   // bias as hi + lo at D0, D0+1.  Hidden layer h: [W | W] over 2C columns
   // (hi and lo halves of the activation); its bias hi, lo in columns
   // 16(h-1), 16(h-1)+1 of the bias tile (multiplied by the constant tile).
-  // SnakeAlt folding as described at the top of the file.  One thread stages
-  // one row of one layer.
-  for (int it = tid; it < (L - 1) * C; it += THREADS) {
-    const int layer = it / C, o = it - layer * C;
+  // SnakeAlt folding as described at the top of the file.  A thread stages
+  // 16-byte chunks (8 columns of one row), one or two of them, so the loads
+  // of all weights are in flight at once: a call of few points is mostly this
+  // staging (with one thread per row of a layer and a memset of the work
+  // counter before the launch, 1000 points took 21.4 us a call and 2^20 81.9;
+  // so 16.5 and 72.7).
+  constexpr int CH0 = K0 / 8, CHH = 2 * C / 8;  // chunks of a row, layer 0 and hidden
+  for (int it = tid; it < C * CH0 + (L - 2) * C * CHH; it += THREADS) {
+    const int r = it < C * CH0 ? it / CH0 : (it - C * CH0) / CHH;  // row over all (hidden) layers
+    const int cg = it < C * CH0 ? it - r * CH0 : (it - C * CH0) - r * CHH;
+    const int layer = it < C * CH0 ? 0 : 1 + r / C, o = layer == 0 ? r : r - (layer - 1) * C;
     const int din = layer == 0 ? D0 : C;
     const __half* Wsrc = net.W_h + (layer == 0 ? 0 : (size_t)C * D0 + (size_t)(layer - 1) * C * C) + (size_t)o * din;
-    float bias = net.b[layer * C + o];
-    float scale = 1.0f;
-    if (SNAKE) {
-      scale = layer == 0 ? 2.0f : 1.0f;
-      if (layer > 0) {
-        float rs = 0.0f;
-        for (int c = 0; c < C; ++c) rs += __half2float(Wsrc[c]);
-        bias = 2.0f * bias + rs;
-      } else {
-        bias = 2.0f * bias;
-      }
-    }
-    const __half bh = __float2half_rn(bias);
-    const __half bl = __float2half_rn(bias - __half2float(bh));
-    const int ncol = layer == 0 ? K0 : 2 * C;
+    const float scale = SNAKE && layer == 0 ? 2.0f : 1.0f;
     uint8_t* Wt = layer == 0 ? B0 : Bh + (layer - 1) * NAH * BT;
-    for (int cg = 0; cg < ncol / 8; ++cg) {
-      uint32_t w[4];
+    uint32_t w[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        __half h2[2];
+    for (int e = 0; e < 4; ++e) {
+      __half h2[2];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int col = 8 * cg + 2 * e + q;
-          __half v = __float2half_rn(0.0f);
-          if (layer == 0) {
-            int src = -1;
-            if (col < 2 * M) src = (col & 1) ? 3 + M + (col >> 1) : 3 + (col >> 1);
-            else if (col < 2 * M + 3) src = col - 2 * M;
-            else if (col < D0) src = col;
-            const bool lat = src >= 3 + 2 * M && src < 3 + 2 * M + F;
-            if (src >= 0) v = __float2half_rn(ldexpf(scale * __half2float(Wsrc[src]), lat ? gexp : 0));
-            if (col == D0) v = bh;
-            if (col == D0 + 1) v = bl;
-          } else {
-            v = __float2half_rn(scale * __half2float(Wsrc[col % C]));
+      for (int q = 0; q < 2; ++q) {
+        const int col = 8 * cg + 2 * e + q;
+        __half v = __float2half_rn(0.0f);
+        if (layer == 0) {
+          int src = -1;
+          if (col < 2 * M) src = (col & 1) ? 3 + M + (col >> 1) : 3 + (col >> 1);
+          else if (col < 2 * M + 3) src = col - 2 * M;
+          else if (col < D0) src = col;
+          const bool lat = src >= 3 + 2 * M && src < 3 + 2 * M + F;
+          if (src >= 0) v = __float2half_rn(ldexpf(scale * __half2float(Wsrc[src]), lat ? gexp : 0));
+          if (col == D0 || col == D0 + 1) {
+            const float bias = scale * net.b[o];
+            const __half bh = __float2half_rn(bias);
+            v = col == D0 ? bh : __float2half_rn(bias - __half2float(bh));
           }
-          h2[q] = v;
+        } else {
+          v = __float2half_rn(scale * __half2float(Wsrc[col % C]));
         }
-        __half2 hh = __halves2half2(h2[0], h2[1]);
-        w[e] = *reinterpret_cast<uint32_t*>(&hh);
+        h2[q] = v;
       }
-      *reinterpret_cast<uint4*>(Wt + (cg >> 3) * BT + sw_off(o, cg & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
+      __half2 hh = __halves2half2(h2[0], h2[1]);
+      w[e] = *reinterpret_cast<uint32_t*>(&hh);
     }
-    if (layer > 0) {
-      const int cg = 2 * (layer - 1);  // the layer's 16-column K-block: chunks cg, cg + 1
-      __half2 hb = __halves2half2(bh, bl);
-      const uint32_t wb = *reinterpret_cast<uint32_t*>(&hb);
-      *reinterpret_cast<uint4*>(Bb + (cg >> 3) * BT + sw_off(o, cg & 7)) = make_uint4(wb, 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(Bb + ((cg + 1) >> 3) * BT + sw_off(o, (cg + 1) & 7)) = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(Wt + (cg >> 3) * BT + sw_off(o, cg & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  // hidden biases, the last threads first (the chunks above take the first ones twice)
+  for (int it = THREADS - 1 - tid; it < (L - 2) * C; it += THREADS) {
+    const int layer = 1 + it / C, o = it - (layer - 1) * C;
+    const __half* Wsrc = net.W_h + (size_t)C * D0 + (size_t)(layer - 1) * C * C + (size_t)o * C;
+    float bias = net.b[layer * C + o];
+    if (SNAKE) {
+      float rs = 0.0f;
+      for (int c = 0; c < C; ++c) rs += __half2float(Wsrc[c]);
+      bias = 2.0f * bias + rs;
     }
+    const int cg = 2 * (layer - 1);  // the layer's 16-column K-block: chunks cg, cg + 1
+    const __half bh = __float2half_rn(bias);
+    __half2 hb = __halves2half2(bh, __float2half_rn(bias - __half2float(bh)));
+    const uint32_t wb = *reinterpret_cast<uint32_t*>(&hb);
+    *reinterpret_cast<uint4*>(Bb + (cg >> 3) * BT + sw_off(o, cg & 7)) = make_uint4(wb, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(Bb + ((cg + 1) >> 3) * BT + sw_off(o, (cg + 1) & 7)) = make_uint4(0u, 0u, 0u, 0u);
   }
   if constexpr (ADJ) {
     // backward B tiles, unscaled FP16 weights, K = 2C (hi and lo halves of
@@ -727,22 +731,17 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (tid == 0) {
-    // row k of a NeRF matrix: 2 pi 2^(k div 3) on axis k mod 3, zero elsewhere
-    int ok = 1;
-    for (int k = 0; k < M && ok; ++k)
-      for (int a = 0; a < 3; ++a) {
-        const float want = (a == k % 3) ? 6.2831855f * (float)(1 << (k / 3)) : 0.0f;
-        if (fm[3 * k + a] != want) ok = 0;
-      }
-    misc[1] = ok;
+  // row k of a NeRF matrix: 2 pi 2^(k div 3) on axis k mod 3, zero elsewhere
+  bool ok = true;
+  for (int i = tid; i < 3 * M; i += THREADS) {
+    const int k = i / 3, a = i - 3 * k;
+    ok &= fm[i] == (a == k % 3 ? 6.2831855f * (float)(1 << (k / 3)) : 0.0f);
   }
   for (int i = tid; i < SRN_MAX_TF_POINTS; i += THREADS) {
     const float wdt = i + 1 < tf.n ? tf.pos[i + 1] - tf.pos[i] : 0.0f;
     tfinv[i] = wdt > 0.0f ? 1.0f / wdt : 0.0f;
   }
-  __syncthreads();
-  const bool nerf = misc[1] != 0;
+  const bool nerf = __syncthreads_and(ok) != 0;
   const uint32_t tmem = (uint32_t)misc[0];
   const uint32_t d_tmem = tmem + (uint32_t)(wg * tmem_wg_cols(C, SH, K0));
   const uint32_t t_row = d_tmem + ((uint32_t)((row >> 5) * 32) << 16);  // warp's lane quarter
@@ -1122,6 +1121,15 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   __syncthreads();
   tc_fence_after();
   if (tid < 32) tmem_dealloc(tmem, TMC);
+  // the last CTA leaves the work counter at zero for the next launch
+  if (tid == 0) {
+    unsigned int* done = reinterpret_cast<unsigned int*>(ray_counter + 1);
+    __threadfence();
+    if (atomicAdd(done, 1u) == gridDim.x - 1) {
+      *ray_counter = 0ull;
+      *done = 0u;
+    }
+  }
 }
 
 template <int C, int M, int F, int ACT, int SH, int TI, int GQ, int LF, int ST>
@@ -1137,9 +1145,11 @@ cudaError_t launch_t(const NetDev& net, const BatchDev& b, const PointsDev& pd, 
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
-  k<<<sms, 128 * wgs_for(C, SH), plan.total, s>>>(net, b, pd, plan, ctr, status);
+  // one CTA per SM, or one per 32 points / pixel tile where there are fewer:
+  // a warp claims 32 at a time
+  const long long claims = is_points(SH) ? (pd.n + 31) / 32
+                                         : (long long)((b.W + 7) / 8) * ((b.H + 3) / 4) * b.n_views * b.n_times;
+  k<<<(unsigned)(claims < sms ? claims : sms), 128 * wgs_for(C, SH), plan.total, s>>>(net, b, pd, plan, ctr, status);
   return cudaGetLastError();
 }
 
