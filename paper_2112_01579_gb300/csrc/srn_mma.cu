@@ -35,7 +35,8 @@ int mma_smem_bytes(const NetDev& n, int shading) {
 }  // namespace
 
 bool render_mma_supported(const NetDev& n, int shading) {
-  if (n.l < 2 || n.l > 8) return false;
+  // depths the interface takes: eight layers at width 32, six at 48, seven at 64
+  if (n.l < 2 || n.l > (n.c == 48 ? 6 : (n.c == 64 ? 7 : 8))) return false;
   // adjoint: backward MMAs, at most four layers (two stashed derivative
   // blocks in TMEM), no time input, FP16 grid; the gradient is that of
   // output 0, so the 4-output head is taken too
