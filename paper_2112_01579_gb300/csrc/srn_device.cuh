@@ -122,6 +122,34 @@ __device__ __forceinline__ void load_tf(TFDev& dst, const TFDev& src) {
   }
 }
 
+__device__ __forceinline__ void load_tf_segments(TFSeg& t, const TFDev& tf) {
+  for (int i = threadIdx.x; i < SRN_MAX_TF_POINTS; i += blockDim.x) {
+    const int n = tf.n;
+    const float above = __uint_as_float(__float_as_uint(fmaxf(tf.pos[0], 0.0f)) + 1u);  // next float above pos[0]
+    const float start = i + 1 < n ? fmaxf(tf.pos[i + 1], tf.pos[0] < 0.0f ? tf.pos[0] : above) : INFINITY;
+    reinterpret_cast<float*>(t.bound)[i] = start;
+    const float wdt = i + 1 < n ? tf.pos[i + 1] - tf.pos[i] : 0.0f;
+    t.seg[i] = make_float2(tf.pos[i], wdt > 0.0f ? 1.0f / wdt : 0.0f);
+    const float4 a = tf.rgba[i], b = tf.rgba[i + 1 < n ? i + 1 : i];
+    t.colour[i] = a;
+    t.diff[i] = make_float4(b.x - a.x, b.y - a.y, b.z - a.z, b.w - a.w);
+  }
+}
+
+// quads: groups of four bounds that hold a finite one.
+__device__ __forceinline__ float4 tf_segment_eval(const TFSeg& t, int quads, float rho) {
+  const float x = clamp01f(rho);
+  int i = 0;
+  for (int q = 0; q < quads; ++q) {
+    const float4 b = t.bound[q];
+    i += (x >= b.x) + (x >= b.y) + (x >= b.z) + (x >= b.w);
+  }
+  const float2 s = t.seg[i];
+  const float f = __saturatef((x - s.x) * s.y);
+  const float4 a = t.colour[i], d = t.diff[i];
+  return make_float4(fmaf(f, d.x, a.x), fmaf(f, d.y, a.y), fmaf(f, d.z, a.z), fmaf(f, d.w, a.w));
+}
+
 // Trilinear interpolation of a dense float32 volume [nz][ny][nx].
 __device__ __forceinline__ float vol_sample(const VolDev& v, float3 p) {
   int ix, iy, iz;

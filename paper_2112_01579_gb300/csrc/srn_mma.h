@@ -56,7 +56,7 @@ struct PointsDev {
 
 // ---------------------------------------------------------------- layout
 struct SmemPlan {
-  int oOne, oB0, oBh, oBb, oBhT, oB0T, oWl, oTF, oTFinv, oFm, oQp, oMbar, oMisc, total;
+  int oOne, oB0, oBh, oBb, oBhT, oB0T, oWl, oTF, oFm, oQp, oMbar, oMisc, total;
 };
 
 // Shared memory for hidden width C and WGS warpgroups: the weights (B tiles,
@@ -78,9 +78,8 @@ inline SmemPlan make_plan(const NetDev& n, int C, int WGS, bool adjoint = false)
   s.oB0T = o; if (adjoint) o += NAH * (NA0 * 64) * 128;    // adjoint: [W_0^T | W_0^T], K0 rows
   s.oWl = o; o += (n.D * C + 4) * 4;
   o = (o + 15) & ~15;
-  s.oTF = o; o += (int)sizeof(TFDev);
+  s.oTF = o; o += (int)sizeof(TFSeg);
   o = (o + 15) & ~15;
-  s.oTFinv = o; o += SRN_MAX_TF_POINTS * 4;
   s.oFm = o; o += ((3 * n.m + 3) & ~3) * 4 + 16;
   s.oQp = o; o += 2 * 32 * 4;
   o = (o + 7) & ~7;

@@ -227,21 +227,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&w)[8])
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Transfer function with precomputed reciprocal segment widths (same
-// segments and lerp as the shared tf_eval).
-__device__ __forceinline__ float4 tf_eval_inv(const TFDev& tf, const float* inv, float rho) {
-  const float x = clamp01f(rho);
-  const int n = tf.n;
-  if (x <= tf.pos[0]) return tf.rgba[0];
-  if (x >= tf.pos[n - 1]) return tf.rgba[n - 1];
-  int i = 0;
-  while (i < n - 2 && x >= tf.pos[i + 1]) ++i;
-  const float f = (x - tf.pos[i]) * inv[i];
-  const float4 a = tf.rgba[i], b = tf.rgba[i + 1];
-  return make_float4(fmaf(f, b.x - a.x, a.x), fmaf(f, b.y - a.y, a.y), fmaf(f, b.z - a.z, a.z),
-                     fmaf(f, b.w - a.w, a.w));
-}
-
 struct RayLat {
   int g0, g1;     // element offsets of the bracketing keyframe grids (g1 < 0: single grid)
   float w0, w1;   // time weights
@@ -569,8 +554,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   uint8_t* BhT = sm + plan.oBhT;
   uint8_t* B0T = sm + plan.oB0T;
   float* wl = reinterpret_cast<float*>(sm + plan.oWl);
-  TFDev& tf = *reinterpret_cast<TFDev*>(sm + plan.oTF);
-  float* tfinv = reinterpret_cast<float*>(sm + plan.oTFinv);
+  TFSeg& tf = *reinterpret_cast<TFSeg*>(sm + plan.oTF);
   float* fm = reinterpret_cast<float*>(sm + plan.oFm);
   float* qp = reinterpret_cast<float*>(sm + plan.oQp);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + plan.oMbar);
@@ -710,7 +694,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
       for (int i = tid; i < 2 * F; i += THREADS)  // [lo + 128 step, step] per channel (latent_q)
         qp[i] = ldexpf((i & 1) ? net.grid_qp[i] : fmaf(128.0f, net.grid_qp[i + 1], net.grid_qp[i]), -gexp);
   }
-  load_tf(tf, b.tf);
+  load_tf_segments(tf, b.tf);
   // the constant tile has ones in columns 0 and 1 of every row (the bias MMA
   // of the hidden layers)
   if (wg == 0) {
@@ -736,10 +720,6 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   for (int i = tid; i < 3 * M; i += THREADS) {
     const int k = i / 3, a = i - 3 * k;
     ok &= fm[i] == (a == k % 3 ? 6.2831855f * (float)(1 << (k / 3)) : 0.0f);
-  }
-  for (int i = tid; i < SRN_MAX_TF_POINTS; i += THREADS) {
-    const float wdt = i + 1 < tf.n ? tf.pos[i + 1] - tf.pos[i] : 0.0f;
-    tfinv[i] = wdt > 0.0f ? 1.0f / wdt : 0.0f;
   }
   const bool nerf = __syncthreads_and(ok) != 0;
   const uint32_t tmem = (uint32_t)misc[0];
@@ -1092,8 +1072,8 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
       if (sample_done) {
         ++ns;
         overflow |= !(fabsf(rho_c) < INFINITY);
-        float4 c = tf_eval_inv(tf, tfinv, rho_c);
-        const float alpha = 1.0f - __expf(-c.w * tf.opacity_scale * len);
+        float4 c = tf_segment_eval(tf, (b.tf.n + 2) / 4, rho_c);
+        const float alpha = 1.0f - __expf(-c.w * b.tf.opacity_scale * len);
         if (SH != SRN_SHADE_NONE) shade(c, g, d);
         const float w = (1.0f - Acc) * alpha;
         C0 = fmaf(w, c.x, C0);
