@@ -3,6 +3,18 @@
 // quality comparisons (Section 4 / 6).  Same ray march, transfer function,
 // compositing and shading as the network renderer; density = trilinear
 // interpolation of the volume.
+//
+// One thread per ray, 32 pixels a warp.  Bound by issue slots and by the L1
+// data pipe at once (a warp's corner load takes one wavefront per cache line
+// it touches), so both are kept low: the sample position is carried in voxel
+// units (one FMA per axis), offsets are 32 bits where the volume has fewer
+// than 2^31 voxels, the interpolation is seven nested lerps, the transfer
+// function's segment comes from counting control points out of two 16-byte
+// loads, and the corner values stay in registers while a ray stays in its
+// cell (two samples in five at half a voxel a step).  A 1024^2 frame of a
+// 256^3 volume: 1426 -> 1065 us; without the kept corners 1132, and pixel
+// tiles chosen per view to cross the fewest rows gained nothing.
+
 #include "srn_device.cuh"
 
 namespace srn {
@@ -10,11 +22,53 @@ namespace {
 
 constexpr int kThreads = 128;
 
-template <bool FD>
+// The cell a ray is in and its corner values.
+template <class I>
+struct Cell {
+  I at;
+  float c[8];
+};
+
+// Trilinear density at voxel coordinates g (vertex i at coordinate i).
+template <class I, bool CACHED>
+__device__ __forceinline__ float sample(const VolDev& v, I sy, I sz, float3 g, Cell<I>& k) {
+  const int ix = min(max(__float2int_rd(g.x), 0), v.nx - 2), iy = min(max(__float2int_rd(g.y), 0), v.ny - 2),
+            iz = min(max(__float2int_rd(g.z), 0), v.nz - 2);
+  const float fx = g.x - (float)ix, fy = g.y - (float)iy, fz = g.z - (float)iz;
+  const I at = (I)iz * sz + (I)iy * sy + (I)ix;
+  if (!CACHED || at != k.at) {
+    k.at = at;
+    k.c[0] = __ldg(v.vol + at); k.c[1] = __ldg(v.vol + at + 1);
+    k.c[2] = __ldg(v.vol + at + sy); k.c[3] = __ldg(v.vol + at + sy + 1);
+    k.c[4] = __ldg(v.vol + at + sz); k.c[5] = __ldg(v.vol + at + sz + 1);
+    k.c[6] = __ldg(v.vol + at + sz + sy); k.c[7] = __ldg(v.vol + at + sz + sy + 1);
+  }
+  const float x0 = fmaf(fx, k.c[1] - k.c[0], k.c[0]), x1 = fmaf(fx, k.c[3] - k.c[2], k.c[2]);
+  const float x2 = fmaf(fx, k.c[5] - k.c[4], k.c[4]), x3 = fmaf(fx, k.c[7] - k.c[6], k.c[6]);
+  const float y0 = fmaf(fy, x1 - x0, x0), y1 = fmaf(fy, x3 - x2, x2);
+  return fmaf(fz, y1 - y0, y0);
+}
+
+// 1 - exp(-x), x >= 0: the series below 1/4 (the first term left out is
+// 5e-8 of the value there), where 1 - exp would cancel; steps are short, so
+// that is nearly every sample.
+__device__ __forceinline__ float opacity(float x) {
+  if (x < 0.25f) {
+    float p = fmaf(x, -1.0f / 720.0f, 1.0f / 120.0f);
+    p = fmaf(x, p, -1.0f / 24.0f);
+    p = fmaf(x, p, 1.0f / 6.0f);
+    p = fmaf(x, p, -0.5f);
+    return fmaf(x * x, p, x);
+  }
+  return 1.0f - expf(-x);
+}
+
+template <bool FD, class I>
 __global__ void __launch_bounds__(kThreads) dvr_dense_kernel(const VolDev v, const BatchDev b) {
-  __shared__ TFDev tf;
-  load_tf(tf, b.tf);
+  __shared__ TFSeg tf;
+  load_tf_segments(tf, b.tf);
   __syncthreads();
+  const int quads = (b.tf.n + 2) / 4;  // n - 1 bounds
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int tiles_x = (b.W + 7) / 8, tiles_y = (b.H + 3) / 4;
@@ -31,34 +85,42 @@ __global__ void __launch_bounds__(kThreads) dvr_dense_kernel(const VolDev v, con
   float C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f;
   unsigned int ns = 0;
   float t0, t1;
-  const float hx = 1.0f / (float)(v.nx - 1), hy = 1.0f / (float)(v.ny - 1), hz = 1.0f / (float)(v.nz - 1);
   if (box_intersect(o, d, t0, t1)) {
-    for (int k = 0;; ++k) {
-      float ta = fmaf((float)k, b.step, t0);
-      if (ta >= t1) break;
-      float tb = fminf(fmaf((float)(k + 1), b.step, t0), t1);
-      float len = tb - ta, tm = 0.5f * (ta + tb);
-      float3 p = make_float3(clamp01f(fmaf(tm, d.x, o.x) + 0.5f), clamp01f(fmaf(tm, d.y, o.y) + 0.5f),
-                             clamp01f(fmaf(tm, d.z, o.z) + 0.5f));
-      float rho = vol_sample(v, p);
+    const I sy = (I)v.nx, sz = (I)v.nx * (I)v.ny;
+    const float mx = (float)(v.nx - 1), my = (float)(v.ny - 1), mz = (float)(v.nz - 1);
+    const float3 gd = make_float3(d.x * mx, d.y * my, d.z * mz);
+    const float3 go = make_float3((o.x + 0.5f) * mx, (o.y + 0.5f) * my, (o.z + 0.5f) * mz);
+    const float scale = b.tf.opacity_scale;
+    Cell<I> cell, side;
+    cell.at = ~(I)0;
+    float ta = t0;
+    for (int k = 1; ta < t1; ++k) {
+      const float tb = fminf(fmaf((float)k, b.step, t0), t1);
+      const float len = tb - ta, tm = 0.5f * (ta + tb);
+      const float3 g = make_float3(fminf(fmaxf(fmaf(tm, gd.x, go.x), 0.0f), mx),
+                                   fminf(fmaxf(fmaf(tm, gd.y, go.y), 0.0f), my),
+                                   fminf(fmaxf(fmaf(tm, gd.z, go.z), 0.0f), mz));
+      const float rho = sample<I, true>(v, sy, sz, g, cell);
       ++ns;
-      float4 c = tf_eval(tf, rho);
-      float alpha = 1.0f - expf(-c.w * tf.opacity_scale * len);
+      float4 c = tf_segment_eval(tf, quads, rho);
+      const float alpha = opacity(scale * c.w * len);
       if (FD) {
-        float3 g;
-        g.x = (vol_sample(v, make_float3(clamp01f(p.x + hx), p.y, p.z)) -
-               vol_sample(v, make_float3(clamp01f(p.x - hx), p.y, p.z))) / (2.0f * hx);
-        g.y = (vol_sample(v, make_float3(p.x, clamp01f(p.y + hy), p.z)) -
-               vol_sample(v, make_float3(p.x, clamp01f(p.y - hy), p.z))) / (2.0f * hy);
-        g.z = (vol_sample(v, make_float3(p.x, p.y, clamp01f(p.z + hz))) -
-               vol_sample(v, make_float3(p.x, p.y, clamp01f(p.z - hz)))) / (2.0f * hz);
-        shade(c, g, d);
+        // central differences one voxel apart, clamped to the volume
+        float3 n;
+        n.x = 0.5f * mx * (sample<I, false>(v, sy, sz, make_float3(fminf(g.x + 1.0f, mx), g.y, g.z), side) -
+                           sample<I, false>(v, sy, sz, make_float3(fmaxf(g.x - 1.0f, 0.0f), g.y, g.z), side));
+        n.y = 0.5f * my * (sample<I, false>(v, sy, sz, make_float3(g.x, fminf(g.y + 1.0f, my), g.z), side) -
+                           sample<I, false>(v, sy, sz, make_float3(g.x, fmaxf(g.y - 1.0f, 0.0f), g.z), side));
+        n.z = 0.5f * mz * (sample<I, false>(v, sy, sz, make_float3(g.x, g.y, fminf(g.z + 1.0f, mz)), side) -
+                           sample<I, false>(v, sy, sz, make_float3(g.x, g.y, fmaxf(g.z - 1.0f, 0.0f)), side));
+        shade(c, n, d);
       }
-      float w = (1.0f - A) * alpha;
+      const float w = (1.0f - A) * alpha;
       C0 = fmaf(w, c.x, C0);
       C1 = fmaf(w, c.y, C1);
       C2 = fmaf(w, c.z, C2);
       A += w;
+      ta = tb;
       if (A >= b.et) break;
     }
   }
@@ -70,12 +132,16 @@ __global__ void __launch_bounds__(kThreads) dvr_dense_kernel(const VolDev v, con
 }  // namespace
 
 cudaError_t launch_dvr_dense(const VolDev& v, const BatchDev& b, cudaStream_t s) {
-  long long tiles = (long long)((b.W + 7) / 8) * ((b.H + 3) / 4) * b.n_views * b.n_times;
-  long long blocks = (tiles + (kThreads / 32) - 1) / (kThreads / 32);
-  if (b.shading == SRN_SHADE_NONE)
-    dvr_dense_kernel<false><<<(unsigned)blocks, kThreads, 0, s>>>(v, b);
-  else
-    dvr_dense_kernel<true><<<(unsigned)blocks, kThreads, 0, s>>>(v, b);
+  const long long tiles = (long long)((b.W + 7) / 8) * ((b.H + 3) / 4) * b.n_views * b.n_times;
+  const unsigned blocks = (unsigned)((tiles + (kThreads / 32) - 1) / (kThreads / 32));
+  const bool small = (long long)v.nx * v.ny < (1ll << 31) && (long long)v.nx * v.ny * v.nz < (1ll << 31);
+  if (b.shading == SRN_SHADE_NONE) {
+    if (small) dvr_dense_kernel<false, unsigned int><<<blocks, kThreads, 0, s>>>(v, b);
+    else dvr_dense_kernel<false, unsigned long long><<<blocks, kThreads, 0, s>>>(v, b);
+  } else {
+    if (small) dvr_dense_kernel<true, unsigned int><<<blocks, kThreads, 0, s>>>(v, b);
+    else dvr_dense_kernel<true, unsigned long long><<<blocks, kThreads, 0, s>>>(v, b);
+  }
   return cudaGetLastError();
 }
 
