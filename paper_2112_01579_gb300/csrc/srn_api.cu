@@ -862,8 +862,9 @@ size_t carve_static(FitScratch& s, const NetDev& net, int n, unsigned char* base
   s.key_alt = (unsigned int*)take(sizeof(unsigned int) * nn);
   s.idx = (unsigned int*)take(sizeof(unsigned int) * nn);
   s.idx_alt = (unsigned int*)take(sizeof(unsigned int) * nn);
-  s.radix_bins = 256;  // two 8-bit passes: the smaller histogram keeps the static area's batch
-  const size_t hist_n = 256 * ((nn + 2047) / 2048);
+  s.radix_bins = 256;  // 8-bit digits: the smaller histogram keeps the static area's batch
+  s.sort_items = static_sort_items();
+  const size_t hist_n = 256 * ((nn + s.sort_items - 1) / s.sort_items);
   s.hist = (unsigned int*)take(sizeof(unsigned int) * (hist_n + hist_n / 8192 + 1));
   s.digit_totals = (unsigned int*)take(sizeof(unsigned int) * 256);
   s.cell_start = (unsigned int*)take(sizeof(unsigned int) * (s.n_cells + 1));

@@ -13,14 +13,15 @@
 //      (Two-layer width-32 density networks take the tensor-core point
 //      kernel of srn_fit_mma.cu instead; other networks of up to four layers
 //      and 48 inputs the tiled kernel, fit_tile_kernel.)
-//   2. stable LSD radix sort of (cell, point) pairs, one 9-bit pass for up to
-//      512 cells, else 8-bit digits: per-block per-warp digit counts, a scan
-//      per digit over the blocks, stable scatter (which adds the digits'
-//      prefix and, for one pass, writes the cell offsets).
-//   3. latent-grid gradient without floating-point atomics: dense cells (many
-//      points per cell) sum w_corner(p) * dz per (cell, corner) in one block
-//      per cell, then each vertex adds its <= 8 partials; sparse cells use one
-//      warp per vertex over its cells' points in sorted order.  Fixed orders
+//   2. stable radix sort of (cell, point) pairs: up to 512 cells one 9-bit
+//      pass; up to 2^18 cells a pass over the leading eight bits, then one
+//      block per leading digit; else 8-bit digits from the lowest.  A pass is
+//      per-block per-warp digit counts, a scan per digit over the blocks and a
+//      stable scatter (which adds the digits' prefix and, for one pass, writes
+//      the cell offsets).
+//   3. latent-grid gradient without floating-point atomics: sums of
+//      w_corner(p) * dz per (cell, corner), a block per dense cell or a warp
+//      per sparse one, then each vertex adds its <= 8 partials.  Fixed orders
 //      and butterflies throughout, so the gradient is bit-reproducible.
 //   4. fixed-order reduction of the CTA partials (weights, biases, loss), in
 //      the same launch as the vertex gather.
@@ -41,7 +42,10 @@ using namespace net32;
 
 constexpr int kFitThreads = 128;
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 2048;  // keys per sort block: 8 warps x 8 rounds x 32
+// Keys per sort block: 8 warps x 4 or 8 rounds x 32.  Blocks of 1024 fill the
+// SMs from 2^18 points; larger sets and the static area (whose histogram
+// bounds its batch) take 2048.
+constexpr int kSortItems = 2048, kSortItemsSmall = 1024;
 
 __device__ __forceinline__ float sgnf(float x) { return x > 0.f ? 1.f : (x < 0.f ? -1.f : 0.f); }
 
@@ -604,39 +608,77 @@ cudaError_t launch_fit_tile(const NetDev& net, const PointArgs& pa, int grid, cu
 }
 
 // ---------------------------------------------------------------- radix sort
-// Digit counts of one sort block (8 warps x 8 rounds x 32 keys) per warp:
-// equal digits within a round are grouped with __match_any_sync.  NB bins.
-template <int NB>
-__device__ __forceinline__ void warp_digit_counts(const unsigned int* __restrict__ keys, int n, int shift,
-                                                  unsigned int (*cnt)[NB]) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int base = blockIdx.x * kSortItems + w * 256;
+// A warp's keys of one sort block (ROUNDS x 32, all loads in flight at once);
+// `end`: first index past the keys.
+template <int ROUNDS>
+__device__ __forceinline__ void load_keys(const unsigned int* __restrict__ keys, int base, int end,
+                                          unsigned int (&k)[ROUNDS]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
+  for (int r = 0; r < ROUNDS; ++r) {
     const int i = base + r * 32 + lane;
-    const bool valid = i < n;
-    const unsigned int d = valid ? (keys[i] >> shift) & (unsigned)(NB - 1) : 0xFFFFFFFFu;
+    k[r] = i < end ? keys[i] : 0u;
+  }
+}
+
+// Digit counts of the warp's keys: equal digits within a round are grouped
+// with __match_any_sync.  NB bins.
+template <int NB, int ROUNDS>
+__device__ __forceinline__ void warp_digit_counts(const unsigned int (&k)[ROUNDS], int base, int end, int shift,
+                                                  unsigned int* cnt) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) {
+    const bool valid = base + r * 32 + lane < end;
+    const unsigned int d = valid ? (k[r] >> shift) & (unsigned)(NB - 1) : 0xFFFFFFFFu;
     const unsigned int peers = __match_any_sync(0xffffffffu, d);
-    if (valid && lane == __ffs(peers) - 1) cnt[w][d] += __popc(peers);
+    if (valid && lane == __ffs(peers) - 1) cnt[d] += __popc(peers);
+    __syncwarp();
+  }
+}
+
+// Stable scatter of the warp's keys and values from cnt[d], the position of
+// the warp's next key of digit d.
+template <int NB, int ROUNDS>
+__device__ __forceinline__ void warp_scatter(const unsigned int (&k)[ROUNDS], const unsigned int (&v)[ROUNDS], int base,
+                                             int end, int shift, unsigned int* cnt, unsigned int* __restrict__ kout,
+                                             unsigned int* __restrict__ vout) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) {
+    const bool valid = base + r * 32 + lane < end;
+    const unsigned int d = valid ? (k[r] >> shift) & (unsigned)(NB - 1) : 0xFFFFFFFFu;
+    const unsigned int peers = __match_any_sync(0xffffffffu, d);
+    const unsigned int rank = __popc(peers & ((1u << lane) - 1u));
+    if (valid) {
+      const unsigned int pos = cnt[d] + rank;
+      if (kout) kout[pos] = k[r];
+      vout[pos] = v[r];
+    }
+    __syncwarp();
+    if (valid && lane == __ffs(peers) - 1) cnt[d] += __popc(peers);
     __syncwarp();
   }
 }
 
 // hist[d * nblocks + block] = count of digit d in the block (digit-major, so
 // one exclusive scan gives every (digit, block) its output offset).
-template <int NB>
+template <int NB, int ROUNDS>
 __global__ void __launch_bounds__(kSortThreads) sort_hist_kernel(const unsigned int* __restrict__ keys, int n,
                                                                  int shift, unsigned int* __restrict__ hist,
                                                                  int nblocks) {
   __shared__ unsigned int cnt[8][NB];
+  const int w = threadIdx.x >> 5, base = blockIdx.x * (ROUNDS * kSortThreads) + w * (ROUNDS * 32);
+  unsigned int k[ROUNDS];
+  load_keys<ROUNDS>(keys, base, n, k);
   for (int i = threadIdx.x; i < 8 * NB; i += kSortThreads) (&cnt[0][0])[i] = 0;
   __syncthreads();
-  warp_digit_counts<NB>(keys, n, shift, cnt);
+  warp_digit_counts<NB, ROUNDS>(k, base, n, shift, cnt[w]);
   __syncthreads();
   for (int d = threadIdx.x; d < NB; d += kSortThreads) {
     unsigned int t = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) t += cnt[w][d];
+    for (int q = 0; q < 8; ++q) t += cnt[q][d];
     hist[(size_t)d * nblocks + blockIdx.x] = t;
   }
 }
@@ -767,7 +809,7 @@ __global__ void __launch_bounds__(kDigitThreads) digit_scan_kernel(unsigned int*
   if (tid == kDigitThreads - 1) totals[blockIdx.x] = before + x;
 }
 
-template <int NB>
+template <int NB, int ROUNDS>
 __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const unsigned int* __restrict__ kin,
                                                                     const unsigned int* __restrict__ vin,
                                                                     unsigned int* __restrict__ kout,
@@ -779,6 +821,10 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const unsign
   __shared__ unsigned int cnt[8][NB];
   __shared__ unsigned int dbase[NB];  // keys of all smaller digits (0 when `scanned` is already global)
   __shared__ unsigned int wpart[kSortThreads / 32];
+  const int w = threadIdx.x >> 5, base = blockIdx.x * (ROUNDS * kSortThreads) + w * (ROUNDS * 32);
+  unsigned int key[ROUNDS], val[ROUNDS];
+  load_keys<ROUNDS>(kin, base, n, key);
+  load_keys<ROUNDS>(vin, base, n, val);
   if (totals) {
     // exclusive scan of the digit totals, NB / kSortThreads consecutive digits per thread
     constexpr int PER = NB / kSortThreads;
@@ -814,36 +860,103 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const unsign
   if (cell_start && blockIdx.x == 0)
     for (int c = threadIdx.x; c <= n_cells; c += kSortThreads)
       cell_start[c] = c < NB ? dbase[c] + scanned[(size_t)c * nblocks] : (unsigned int)n;
-  warp_digit_counts<NB>(kin, n, shift, cnt);
+  warp_digit_counts<NB, ROUNDS>(key, base, n, shift, cnt[w]);
   __syncthreads();
   for (int d = threadIdx.x; d < NB; d += kSortThreads) {
-    unsigned int base = dbase[d] + scanned[(size_t)d * nblocks + blockIdx.x];
+    unsigned int at = dbase[d] + scanned[(size_t)d * nblocks + blockIdx.x];
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      const unsigned int c = cnt[w][d];
-      cnt[w][d] = base;
-      base += c;
+    for (int q = 0; q < 8; ++q) {
+      const unsigned int c = cnt[q][d];
+      cnt[q][d] = at;
+      at += c;
     }
   }
   __syncthreads();
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int base = blockIdx.x * kSortItems + w * 256;
+  warp_scatter<NB, ROUNDS>(key, val, base, n, shift, cnt[w], kout, vout);
+}
+
+// Second half of the sort when the leading eight bits of the cell index are
+// in order: one block per leading digit sorts its keys (about n / 256, in
+// chunks of 2048) by the remaining LOW bits in shared memory, stable, and
+// writes the starts of its cells.  In place of a second histogram, scan and
+// scatter over all keys and a pass for the cell starts.
+template <int LOW>
+__global__ void __launch_bounds__(kSortThreads) bucket_sort_kernel(const unsigned int* __restrict__ kin,
+                                                                   const unsigned int* __restrict__ vin,
+                                                                   unsigned int* __restrict__ vout, int n,
+                                                                   int low_bits, unsigned int* __restrict__ cell_start,
+                                                                   long long n_cells,
+                                                                   const unsigned int* __restrict__ totals) {
+  constexpr int NB = 1 << LOW, PER = NB / kSortThreads, ROUNDS = 8;
+  __shared__ unsigned int cnt[8][NB];
+  __shared__ unsigned int next[NB];  // count, then next position of each bin
+  __shared__ unsigned int wpart[kSortThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // keys of the smaller leading digits
+  const unsigned int mine = totals[tid];
+  unsigned int before = tid < (int)blockIdx.x ? mine : 0u;
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int i = base + r * 32 + lane;
-    const bool valid = i < n;
-    const unsigned int k = valid ? kin[i] : 0u;
-    const unsigned int d = valid ? (k >> shift) & (unsigned)(NB - 1) : 0xFFFFFFFFu;
-    const unsigned int peers = __match_any_sync(0xffffffffu, d);
-    const unsigned int rank = __popc(peers & ((1u << lane) - 1u));
-    if (valid) {
-      const unsigned int pos = cnt[w][d] + rank;
-      kout[pos] = k;
-      vout[pos] = vin[i];
+  for (int off = 16; off > 0; off >>= 1) before += __shfl_xor_sync(0xffffffffu, before, off);
+  if (lane == 0) wpart[w] = before;
+  for (int i = tid; i < NB; i += kSortThreads) next[i] = 0u;
+  __syncthreads();
+  unsigned int first = 0u;
+#pragma unroll
+  for (int q = 0; q < kSortThreads / 32; ++q) first += wpart[q];
+  const int b0 = (int)first, b1 = b0 + (int)totals[blockIdx.x];
+  const unsigned int mask = (1u << low_bits) - 1u;
+  for (int i = b0 + tid; i < b1; i += kSortThreads) atomicAdd(&next[kin[i] & mask], 1u);
+  __syncthreads();
+  // exclusive scan of the bins, PER consecutive ones per thread
+  unsigned int v[PER], t = 0u;
+#pragma unroll
+  for (int e = 0; e < PER; ++e) {
+    v[e] = next[tid * PER + e];
+    t += v[e];
+  }
+  unsigned int x = t;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned int y = __shfl_up_sync(0xffffffffu, x, off);
+    if (lane >= off) x += y;
+  }
+  if (lane == 31) wpart[w] = x;
+  __syncthreads();
+  unsigned int run = first + x - t;
+  for (int q = 0; q < w; ++q) run += wpart[q];
+#pragma unroll
+  for (int e = 0; e < PER; ++e) {
+    const int bin = tid * PER + e;
+    const long long cell = ((long long)blockIdx.x << low_bits) + bin;
+    if (bin <= (int)mask && cell < n_cells) cell_start[cell] = run;
+    next[bin] = run;
+    run += v[e];
+  }
+  if (blockIdx.x == 0 && tid == 0) cell_start[n_cells] = (unsigned int)n;
+  for (int c0 = b0; c0 < b1; c0 += ROUNDS * kSortThreads) {
+    const int base = c0 + w * (ROUNDS * 32);
+    unsigned int key[ROUNDS], val[ROUNDS];
+    load_keys<ROUNDS>(kin, base, b1, key);
+    load_keys<ROUNDS>(vin, base, b1, val);
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) key[r] &= mask;
+    for (int i = tid; i < 8 * NB; i += kSortThreads) (&cnt[0][0])[i] = 0u;
+    __syncthreads();
+    warp_digit_counts<NB, ROUNDS>(key, base, b1, 0, cnt[w]);
+    __syncthreads();
+    for (int d = tid; d < NB; d += kSortThreads) {
+      unsigned int at = next[d];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const unsigned int c = cnt[q][d];
+        cnt[q][d] = at;
+        at += c;
+      }
+      next[d] = at;
     }
-    __syncwarp();
-    if (valid && lane == __ffs(peers) - 1) cnt[w][d] += __popc(peers);
-    __syncwarp();
+    __syncthreads();
+    warp_scatter<NB, ROUNDS>(key, val, base, b1, 0, cnt[w], nullptr, vout);
+    __syncthreads();
   }
 }
 
@@ -993,6 +1106,74 @@ __global__ void __launch_bounds__(256) cell_corner_kernel(const float* __restric
   if (lane == 0) {
 #pragma unroll
     for (int f = 0; f < F; ++f) part[((size_t)cell * 8 + c) * F + f] = acc[f];
+  }
+}
+
+// Sparse cells (few points per cell): one warp per cell.  A lane owns one
+// corner and four channels (F = 16: 8 x 4 lanes; narrower vectors leave lane
+// groups that take every second or fourth point, wider ones give a lane two
+// channel groups), the points' cell coordinates are computed one point per
+// lane and handed round, and a point's dz row is read once per warp instead
+// of once per vertex.  The corner sums go to part[cell][corner][F], summed per
+// vertex by vertex_gather_block as for dense cells.  Bound by the latency of
+// three dependent loads per cell (offsets, point index, point); a warp per
+// vertex over its eight cells, with its butterfly over 32 mostly idle lanes,
+// took 57 us for 32^3 vertices whatever the number of points.
+template <int F>
+__global__ void __launch_bounds__(256) cell_warp_kernel(const float* __restrict__ pts, const float* __restrict__ dz,
+                                                        const unsigned int* __restrict__ sidx,
+                                                        const unsigned int* __restrict__ start, int R,
+                                                        long long n_cells, float* __restrict__ part) {
+  constexpr int QL = F >= 16 ? 4 : F / 4;      // lanes per corner
+  constexpr int QN = F / (4 * QL);             // channel groups per lane
+  constexpr int G = 32 / (8 * QL);             // points side by side
+  const long long cell = ((long long)blockIdx.x * 256 + threadIdx.x) >> 5;
+  if (cell >= n_cells) return;
+  const int lane = threadIdx.x & 31, g = lane / (8 * QL), c = (lane / QL) & 7, q = lane % QL;
+  const int s0 = (int)start[cell], s1 = (int)start[cell + 1];
+  float4 acc[QN];
+#pragma unroll
+  for (int e = 0; e < QN; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int base = s0; base < s1; base += 32) {
+    const int cnt = min(32, s1 - base);
+    int j = 0, i;
+    float fx = 0.f, fy = 0.f, fz = 0.f;
+    if (lane < cnt) {
+      j = (int)sidx[base + lane];
+      cell_coord(pts[3 * (size_t)j], R, i, fx);
+      cell_coord(pts[3 * (size_t)j + 1], R, i, fy);
+      cell_coord(pts[3 * (size_t)j + 2], R, i, fz);
+    }
+#pragma unroll 4
+    for (int k = 0; k < cnt; k += G) {
+      const int src = k + g;  // lanes past cnt hold zeros; their weight is cleared below
+      const int jk = __shfl_sync(0xffffffffu, j, src);
+      const float x = __shfl_sync(0xffffffffu, fx, src), y = __shfl_sync(0xffffffffu, fy, src),
+                  z = __shfl_sync(0xffffffffu, fz, src);
+      if (G == 1 || src < cnt) {
+        const float w = ((c & 1) ? x : 1.0f - x) * ((c & 2) ? y : 1.0f - y) * ((c & 4) ? z : 1.0f - z);
+        const float4* row = reinterpret_cast<const float4*>(dz + (size_t)jk * F) + q;
+#pragma unroll
+        for (int e = 0; e < QN; ++e) {
+          const float4 v = row[e * QL];
+          acc[e].x = fmaf(w, v.x, acc[e].x);
+          acc[e].y = fmaf(w, v.y, acc[e].y);
+          acc[e].z = fmaf(w, v.z, acc[e].z);
+          acc[e].w = fmaf(w, v.w, acc[e].w);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < QN; ++e) {
+#pragma unroll
+    for (int off = 8 * QL; off < 32; off <<= 1) {
+      acc[e].x += __shfl_xor_sync(0xffffffffu, acc[e].x, off);
+      acc[e].y += __shfl_xor_sync(0xffffffffu, acc[e].y, off);
+      acc[e].z += __shfl_xor_sync(0xffffffffu, acc[e].z, off);
+      acc[e].w += __shfl_xor_sync(0xffffffffu, acc[e].w, off);
+    }
+    if (g == 0) reinterpret_cast<float4*>(part + ((size_t)cell * 8 + c) * F)[q + e * QL] = acc[e];
   }
 }
 
@@ -1152,6 +1333,51 @@ int sm_count() {
   return n > 0 ? n : 1;
 }
 
+// Latent-grid gradient and the reduction of the weight partials: per-cell
+// corner sums (a block per cell from 32 points a cell on average, where a
+// cell's points are worth staging in shared memory, else a warp per cell),
+// then the sums of each vertex.  Without the per-cell array (the static
+// scratch area, grids whose array would pass kMaxCellPart bytes) a warp per
+// vertex gathers from the points.
+constexpr size_t kMaxCellPart = (size_t)256 << 20;
+
+template <int F>
+void launch_grid_grad(const FitScratch& s, const GradArgs& ga, const ReduceArgs& ra, int rblocks, int n,
+                      cudaStream_t st) {
+  const long long n_vert = (long long)ga.R * ga.R * ga.R;
+  if (!s.cell_part) {
+    const int gblocks = (int)((n_vert * 32 + 255) / 256);
+    grad_tail_kernel<F, false><<<gblocks + rblocks, 256, 0, st>>>(ga, gblocks, ra, s.flag);
+    return;
+  }
+  const long long cells = (long long)s.n_cells;
+  if ((size_t)n >= 32 * s.n_cells)
+    cell_corner_kernel<F><<<(unsigned)cells, 256, 0, st>>>(ga.pts, ga.dz, ga.sidx, ga.start, ga.R, cells, s.cell_part);
+  else
+    cell_warp_kernel<F><<<(unsigned)((cells + 7) / 8), 256, 0, st>>>(ga.pts, ga.dz, ga.sidx, ga.start, ga.R, cells,
+                                                                     s.cell_part);
+  const int vb = (int)((n_vert * F + 255) / 256);
+  grad_tail_kernel<F, true><<<vb + rblocks, 256, 0, st>>>(ga, vb, ra, s.flag);
+}
+
+template <int ROUNDS>
+void launch_hist(int dbits, int nblocks, const unsigned int* k, int n, int shift, unsigned int* hist, cudaStream_t st) {
+  if (dbits == 9) sort_hist_kernel<512, ROUNDS><<<nblocks, kSortThreads, 0, st>>>(k, n, shift, hist, nblocks);
+  else sort_hist_kernel<256, ROUNDS><<<nblocks, kSortThreads, 0, st>>>(k, n, shift, hist, nblocks);
+}
+
+template <int ROUNDS>
+void launch_scatter(int dbits, int nblocks, const unsigned int* k, const unsigned int* v, unsigned int* ko,
+                    unsigned int* vo, int n, int shift, const unsigned int* hist, unsigned int* cs, int n_cells,
+                    const unsigned int* totals, cudaStream_t st) {
+  if (dbits == 9)
+    sort_scatter_kernel<512, ROUNDS><<<nblocks, kSortThreads, 0, st>>>(k, v, ko, vo, n, shift, hist, nblocks, cs,
+                                                                       n_cells, totals);
+  else
+    sort_scatter_kernel<256, ROUNDS><<<nblocks, kSortThreads, 0, st>>>(k, v, ko, vo, n, shift, hist, nblocks, cs,
+                                                                       n_cells, totals);
+}
+
 // Steps 1-4 shared by the fit and the backward.  Writes the grid gradient
 // (all keyframes) to dgrid, weights / biases to dW / db, the loss (fit) to
 // loss.
@@ -1200,20 +1426,24 @@ cudaError_t run_backward(FitScratch& s, const NetDev& net, PointArgs pa, float* 
   unsigned int *k_in = s.key, *v_in = s.idx, *k_out = s.key_alt, *v_out = s.idx_alt;
   int bits = 1;
   while (((size_t)1 << bits) < s.n_cells) ++bits;
-  const int nblocks = (n + kSortItems - 1) / kSortItems;
-  // 9-bit digits when the cell index fits one (one pass for grids up to 8^3
-  // cells), else 8-bit digits
-  const int dbits = s.radix_bins == 512 && bits <= 9 ? 9 : 8;
+  const bool small_blocks = s.sort_items == kSortItemsSmall;
+  const int nblocks = (n + s.sort_items - 1) / s.sort_items;
+  // up to 512 cells: one pass with 9-bit digits; up to 2^18 cells: the leading
+  // eight bits, then each leading digit's keys in one block (18 bits leave ten,
+  // 32 KB of counters); else 8-bit digits from the lowest
+  const bool one_pass = s.radix_bins == 512 && bits <= 9;
+  const bool buckets = !one_pass && bits > 9 && bits <= 18 && nblocks <= kDigitThreads * kDigitPer;
+  const int dbits = one_pass ? 9 : 8;
   const int hist_m = (1 << dbits) * nblocks;
   const int nseg = (hist_m + kScanTile - 1) / kScanTile;  // one 8192-value tile per scan block
-  unsigned int* seg_sums = s.hist + (size_t)s.radix_bins * (size_t)((s.max_points + kSortItems - 1) / kSortItems);
+  unsigned int* seg_sums = s.hist + (size_t)s.radix_bins * (size_t)((s.max_points + s.sort_items - 1) / s.sort_items);
   bool starts_done = false;
-  for (int shift = 0; shift < bits && n > 0; shift += dbits) {
+  for (int shift = buckets ? bits - 8 : 0; shift < bits && n > 0; shift += dbits) {
     // a single pass leaves the cell starts to the scatter kernel
-    unsigned int* cs = (shift == 0 && dbits >= bits) ? s.cell_start : nullptr;
-    starts_done = cs != nullptr;
-    if (dbits == 9) sort_hist_kernel<512><<<nblocks, kSortThreads, 0, st>>>(k_in, n, shift, s.hist, nblocks);
-    else sort_hist_kernel<256><<<nblocks, kSortThreads, 0, st>>>(k_in, n, shift, s.hist, nblocks);
+    unsigned int* cs = one_pass ? s.cell_start : nullptr;
+    starts_done = one_pass || buckets;
+    if (small_blocks) launch_hist<4>(dbits, nblocks, k_in, n, shift, s.hist, st);
+    else launch_hist<8>(dbits, nblocks, k_in, n, shift, s.hist, st);
     const unsigned int* totals = nullptr;
     if (nblocks <= kDigitThreads * kDigitPer) {
       // one block per digit; the scatter kernel adds the digits' prefix
@@ -1226,15 +1456,23 @@ cudaError_t run_backward(FitScratch& s, const NetDev& net, PointArgs pa, float* 
     } else {
       scan_kernel<<<1, kScanThreads, 0, st>>>(s.hist, hist_m, hist_m, nullptr);
     }
-    if (dbits == 9)
-      sort_scatter_kernel<512><<<nblocks, kSortThreads, 0, st>>>(k_in, v_in, k_out, v_out, n, shift, s.hist, nblocks,
-                                                                 cs, (int)s.n_cells, totals);
+    if (small_blocks)
+      launch_scatter<4>(dbits, nblocks, k_in, v_in, k_out, v_out, n, shift, s.hist, cs, (int)s.n_cells, totals, st);
     else
-      sort_scatter_kernel<256><<<nblocks, kSortThreads, 0, st>>>(k_in, v_in, k_out, v_out, n, shift, s.hist,
-                                                                 nblocks, cs, (int)s.n_cells, totals);
+      launch_scatter<8>(dbits, nblocks, k_in, v_in, k_out, v_out, n, shift, s.hist, cs, (int)s.n_cells, totals, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     std::swap(k_in, k_out);
     std::swap(v_in, v_out);
+    if (buckets) {
+      if (bits <= 16)
+        bucket_sort_kernel<8><<<256, kSortThreads, 0, st>>>(k_in, v_in, v_out, n, bits - 8, s.cell_start,
+                                                            (long long)s.n_cells, totals);
+      else
+        bucket_sort_kernel<10><<<256, kSortThreads, 0, st>>>(k_in, v_in, v_out, n, bits - 8, s.cell_start,
+                                                             (long long)s.n_cells, totals);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      std::swap(v_in, v_out);
+    }
   }
   if (!starts_done) cell_start_kernel<<<(n + 1 + 255) / 256, 256, 0, st>>>(k_in, n, s.cell_start, (int)s.n_cells);
   // grid gradient: the gathers below write every vertex of the two bracketing
@@ -1261,44 +1499,16 @@ cudaError_t run_backward(FitScratch& s, const NetDev& net, PointArgs pa, float* 
   const float w0 = net.nkey > 1 ? 1.0f - f : 1.0f, w1 = f;
   float* g0 = dgrid + (size_t)k0 * gsz;
   float* g1 = net.nkey > 1 ? g0 + gsz : nullptr;
-  const long long n_vert = (long long)net.R * net.R * net.R;
   const int ne = nW + nb;
   const ReduceArgs ra{s.part, n_cta, nW, nb, dW, db, loss, 1.0f / (float)n};
   const int rblocks = (ne + 1 + 31) / 32;
   if (n > 0) {
     const GradArgs ga{s.pts, s.dz, v_in, s.cell_start, s.cell_part, net.R, w0, w1, g0, g1};
-    const bool dense_cells = s.cell_part && (size_t)n >= 32 * s.n_cells;
-    if (dense_cells) {
-      const long long nw = (long long)s.n_cells * 8;
-      const unsigned int cb = (unsigned int)((nw * 32 + 255) / 256);
-      const int vb = (int)((n_vert * net.F + 255) / 256);
-      switch (net.F) {
-        case 4:
-          cell_corner_kernel<4><<<cb, 256, 0, st>>>(s.pts, s.dz, v_in, s.cell_start, net.R, (long long)s.n_cells,
-                                                    s.cell_part);
-          grad_tail_kernel<4, true><<<vb + rblocks, 256, 0, st>>>(ga, vb, ra, s.flag);
-          break;
-        case 8:
-          cell_corner_kernel<8><<<cb, 256, 0, st>>>(s.pts, s.dz, v_in, s.cell_start, net.R, (long long)s.n_cells,
-                                                    s.cell_part);
-          grad_tail_kernel<8, true><<<vb + rblocks, 256, 0, st>>>(ga, vb, ra, s.flag);
-          break;
-        case 16:
-          cell_corner_kernel<16><<<cb, 256, 0, st>>>(s.pts, s.dz, v_in, s.cell_start, net.R, (long long)s.n_cells,
-                                                     s.cell_part);
-          grad_tail_kernel<16, true><<<vb + rblocks, 256, 0, st>>>(ga, vb, ra, s.flag);
-          break;
-        default:
-          cell_corner_kernel<32><<<cb, 256, 0, st>>>(s.pts, s.dz, v_in, s.cell_start, net.R, (long long)s.n_cells,
-                                                     s.cell_part);
-          grad_tail_kernel<32, true><<<vb + rblocks, 256, 0, st>>>(ga, vb, ra, s.flag);
-      }
-    } else {
-      const int gblocks = (int)((n_vert * 32 + 255) / 256);
-      if (net.F == 8) grad_tail_kernel<8, false><<<gblocks + rblocks, 256, 0, st>>>(ga, gblocks, ra, s.flag);
-      else if (net.F == 16) grad_tail_kernel<16, false><<<gblocks + rblocks, 256, 0, st>>>(ga, gblocks, ra, s.flag);
-      else if (net.F == 4) grad_tail_kernel<4, false><<<gblocks + rblocks, 256, 0, st>>>(ga, gblocks, ra, s.flag);
-      else grad_tail_kernel<32, false><<<gblocks + rblocks, 256, 0, st>>>(ga, gblocks, ra, s.flag);
+    switch (net.F) {
+      case 4: launch_grid_grad<4>(s, ga, ra, rblocks, n, st); break;
+      case 8: launch_grid_grad<8>(s, ga, ra, rblocks, n, st); break;
+      case 16: launch_grid_grad<16>(s, ga, ra, rblocks, n, st); break;
+      default: launch_grid_grad<32>(s, ga, ra, rblocks, n, st);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   } else {
@@ -1320,7 +1530,8 @@ cudaError_t fit_scratch_alloc(FitScratch& s, const NetDev& net, int max_points) 
   s.n_grid = net_grid_count(net);
   s.max_cta = std::min(4 * sm_count(), (max_points + kFitThreads - 1) / kFitThreads);
   const size_t n = (size_t)max_points;
-  const size_t nsb = (n + kSortItems - 1) / kSortItems;
+  s.sort_items = max_points <= kSortItemsSmall * kDigitThreads * kDigitPer ? kSortItemsSmall : kSortItems;
+  const size_t nsb = (n + s.sort_items - 1) / s.sort_items;
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void** p, size_t bytes) {
     if (e == cudaSuccess) e = cudaMalloc(p, bytes < 16 ? 16 : bytes);
@@ -1345,7 +1556,8 @@ cudaError_t fit_scratch_alloc(FitScratch& s, const NetDev& net, int max_points) 
   // wait, SRN_ERR_TIMEOUT) still sorts and gathers inside the buffers
   for (unsigned int* q : {s.key, s.key_alt, s.idx, s.idx_alt})
     if (e == cudaSuccess) e = cudaMemset(q, 0, sizeof(unsigned int) * n);
-  if ((size_t)max_points >= 32 * s.n_cells) alloc((void**)&s.cell_part, sizeof(float) * s.n_cells * 8 * net.F);
+  const size_t part_bytes = sizeof(float) * s.n_cells * 8 * net.F;
+  if ((size_t)max_points >= 32 * s.n_cells || part_bytes <= kMaxCellPart) alloc((void**)&s.cell_part, part_bytes);
   return e;
 }
 
@@ -1357,6 +1569,8 @@ void fit_scratch_free(FitScratch& s) {
     if (p) cudaFree(p);
   memset(&s, 0, sizeof(s));
 }
+
+int static_sort_items() { return kSortItems; }
 
 int sort_bins(size_t n_cells) { return n_cells <= 512 ? 512 : 256; }
 

@@ -13,6 +13,7 @@ struct FitScratch {
   size_t n_entries;        // weights + biases
   size_t n_grid;           // latent-grid entries over all keyframes
   int radix_bins;          // 256 (8-bit digits) or 512 (one 9-bit pass for up to 512 cells)
+  int sort_items;          // keys per sort block (1024 or 2048)
   float* pts;              // [n][3] positions (clamped) of the current step
   float* dz;               // [n][F] adjoint of the latent vector
   unsigned int* key;       // [n] cell of each point, and radix ping-pong
@@ -25,7 +26,8 @@ struct FitScratch {
   float* part;             // [max_cta][n_entries + 1] per-CTA weight-gradient / loss partials
   float* grads;            // [n_grid + n_entries] gradient of one step (grid | weights | biases)
   unsigned int* flag;      // non-finite flag of the current step
-  float* cell_part;        // [n_cells][8][F] per-(cell, corner) partials (small grids; may be null)
+  float* cell_part;        // [n_cells][8][F] per-(cell, corner) partials (null in the static area and for the
+                           // largest grids)
 };
 
 struct FitArgs {
@@ -55,6 +57,8 @@ struct FitArgs {
 bool fit_supported(const NetDev& net);
 // Radix bins of the cell sort: 512 (one 9-bit pass) for up to 512 cells, else 256.
 int sort_bins(size_t n_cells);
+// Keys per sort block of the static scratch area.
+int static_sort_items();
 cudaError_t fit_scratch_alloc(FitScratch& s, const NetDev& net, int max_points);
 void fit_scratch_free(FitScratch& s);
 cudaError_t launch_backward(FitScratch& s, const NetDev& net, const float* pts, int n, float time, const float* dout,
