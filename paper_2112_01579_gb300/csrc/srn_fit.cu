@@ -1047,7 +1047,7 @@ __device__ __forceinline__ void grid_grad_block(const GradArgs& a, int block, un
 // sums w_corner_c(p) * dz over the cell's points (sorted order, lane-strided,
 // fixed butterfly) into part[cell][c][F]; vertex_gather_block then adds the
 // <= 8 partials of each vertex in a fixed order.  The block stages the cell's
-// points (position, dz) in shared memory 256 at a time, so each point is
+// points (place in the cell, dz) in shared memory 256 at a time, so each point is
 // gathered from global memory once instead of once per corner; lane l still
 // takes points l, l + 32, ... in order, so the sums are those of a warp
 // reading global memory directly.
@@ -1069,25 +1069,37 @@ __global__ void __launch_bounds__(256) cell_corner_kernel(const float* __restric
 #pragma unroll
   for (int f = 0; f < F; ++f) acc[f] = 0.f;
   const int s0 = (int)start[cell], s1 = (int)start[cell + 1];
+  // a thread's point of the next chunk is loaded while this one is summed
+  // (its index one chunk earlier still)
+  const int tid = threadIdx.x;
+  int j = s0 + tid < s1 ? (int)sidx[s0 + tid] : 0;
+  float3 q = make_float3(0.f, 0.f, 0.f);
+  float4 z[F / 4];
+  auto fetch = [&](bool any) {
+    if (!any) return;
+    q = make_float3(pts[3 * (size_t)j], pts[3 * (size_t)j + 1], pts[3 * (size_t)j + 2]);
+    const float4* zz = reinterpret_cast<const float4*>(dz + (size_t)j * F);
+#pragma unroll
+    for (int f = 0; f < F / 4; ++f) z[f] = zz[f];
+  };
+  fetch(s0 + tid < s1);
+  j = s0 + kChunk + tid < s1 ? (int)sidx[s0 + kChunk + tid] : 0;
   for (int base = s0; base < s1; base += kChunk) {
     const int cnt = min(kChunk, s1 - base);
     __syncthreads();
-    for (int i = threadIdx.x; i < cnt; i += 256) {
-      const int j = (int)sidx[base + i];
-      sp[i][0] = pts[3 * (size_t)j];
-      sp[i][1] = pts[3 * (size_t)j + 1];
-      sp[i][2] = pts[3 * (size_t)j + 2];
-      const float4* zz = reinterpret_cast<const float4*>(dz + (size_t)j * F);
+    if (tid < cnt) {
+      int i;
+      cell_coord(q.x, R, i, sp[tid][0]);
+      cell_coord(q.y, R, i, sp[tid][1]);
+      cell_coord(q.z, R, i, sp[tid][2]);
 #pragma unroll
-      for (int f = 0; f < F / 4; ++f) sz[i][f] = zz[f];
+      for (int f = 0; f < F / 4; ++f) sz[tid][f] = z[f];
     }
     __syncthreads();
+    fetch(base + kChunk + tid < s1);
+    j = base + 2 * kChunk + tid < s1 ? (int)sidx[base + 2 * kChunk + tid] : 0;
     for (int i = lane; i < cnt; i += 32) {
-      int ix, iy, iz;
-      float fx, fy, fz;
-      cell_coord(sp[i][0], R, ix, fx);
-      cell_coord(sp[i][1], R, iy, fy);
-      cell_coord(sp[i][2], R, iz, fz);
+      const float fx = sp[i][0], fy = sp[i][1], fz = sp[i][2];
       const float w = (dx ? fx : 1.0f - fx) * (dy ? fy : 1.0f - fy) * (dzz ? fz : 1.0f - fz);
 #pragma unroll
       for (int f = 0; f < F; f += 4) {
@@ -1227,8 +1239,10 @@ __device__ __forceinline__ void reduce_parts_block(const ReduceArgs& a, int bloc
   const int ne = nW + nb;
   const int r0 = (int)((long long)n_cta * w / 8), r1 = (int)((long long)n_cta * (w + 1) / 8);
   float s = 0.f;
-  if (e <= ne)
+  if (e <= ne) {
+#pragma unroll 16  // the loads in flight together; the sum stays in row order
     for (int c = r0; c < r1; ++c) s += part[(size_t)c * (ne + 1) + e];
+  }
   acc[w][lane] = s;
   __syncthreads();
   if (w == 0 && e <= ne) {

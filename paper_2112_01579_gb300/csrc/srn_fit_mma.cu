@@ -114,37 +114,38 @@ __global__ void __launch_bounds__(128 * kFitWGS, 1)
   // ---- stage the FP32 master weights of layer 0 split into FP16 hi + lo.
   // B0 row o: blocks [W hi | W hi | W lo] of 64 columns in the input tile's
   // order; block 0 also carries the bias hi / lo in columns D0, D0+1.
-  for (int r = tid; r < C; r += 128 * kFitWGS) {
-    for (int cg = 0; cg < 24; ++cg) {
-      uint32_t w[4];
+  // A thread stages 16-byte chunks, one or two of them, so that all loads are
+  // in flight at once (one thread per row walked 24 chunks one after another).
+  for (int it = tid; it < C * 24; it += 128 * kFitWGS) {
+    const int r = it / 24, cg = it - r * 24;
+    uint32_t w[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint32_t hh[2];
+    for (int e = 0; e < 4; ++e) {
+      uint32_t hh[2];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int col = 8 * cg + 2 * e + q;
-          const int blk = col >> 6, c = col & 63;
-          int src = -1;
-          if (c < 2 * M) src = (c & 1) ? 3 + M + (c >> 1) : 3 + (c >> 1);
-          else if (c < 2 * M + 3) src = c - 2 * M;
-          else if (c < D0) src = c;
-          float v = 0.0f;
-          if (src >= 0) {
-            const float wv = net.W[(size_t)r * D0 + src];
-            const float wh = __half2float(__float2half_rn(wv));
-            v = blk < 2 ? wh : wv - wh;
-          }
-          if (blk == 0 && (c == D0 || c == D0 + 1)) {
-            const float bias = net.b[r];
-            const float bh = __half2float(__float2half_rn(bias));
-            v = c == D0 ? bh : bias - bh;
-          }
-          hh[q] = h16(v);
+      for (int q = 0; q < 2; ++q) {
+        const int col = 8 * cg + 2 * e + q;
+        const int blk = col >> 6, c = col & 63;
+        int src = -1;
+        if (c < 2 * M) src = (c & 1) ? 3 + M + (c >> 1) : 3 + (c >> 1);
+        else if (c < 2 * M + 3) src = c - 2 * M;
+        else if (c < D0) src = c;
+        float v = 0.0f;
+        if (src >= 0) {
+          const float wv = net.W[(size_t)r * D0 + src];
+          const float wh = __half2float(__float2half_rn(wv));
+          v = blk < 2 ? wh : wv - wh;
         }
-        w[e] = hh[0] | (hh[1] << 16);
+        if (blk == 0 && (c == D0 || c == D0 + 1)) {
+          const float bias = net.b[r];
+          const float bh = __half2float(__float2half_rn(bias));
+          v = c == D0 ? bh : bias - bh;
+        }
+        hh[q] = h16(v);
       }
-      *reinterpret_cast<uint4*>(B0 + (cg >> 3) * (32 * 128) + sw_off(r, cg & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
+      w[e] = hh[0] | (hh[1] << 16);
     }
+    *reinterpret_cast<uint4*>(B0 + (cg >> 3) * (32 * 128) + sw_off(r, cg & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
   }
   for (int i = tid; i < F * C; i += 128 * kFitWGS) {
     const int f = i / C, o = i - f * C;
@@ -158,15 +159,11 @@ __global__ void __launch_bounds__(128 * kFitWGS, 1)
     mbar_init(smem_u32(&mbar[wg]), 1);
     misc[4 + wg] = 0;
   }
-  if (tid == 0) {
-    // row k of a NeRF matrix (Eq. 2): 2 pi 2^(k div 3) on axis k mod 3, zero elsewhere
-    int ok = 1;
-    for (int k = 0; k < M && ok; ++k)
-      for (int ax = 0; ax < 3; ++ax) {
-        const float want = (ax == k % 3) ? 6.2831855f * (float)(1 << (k / 3)) : 0.0f;
-        if (net.fourier[3 * k + ax] != want) ok = 0;
-      }
-    misc[2] = ok;
+  // row k of a NeRF matrix (Eq. 2): 2 pi 2^(k div 3) on axis k mod 3, zero elsewhere
+  bool ok = true;
+  for (int i = tid; i < 3 * M; i += 128 * kFitWGS) {
+    const int k = i / 3, ax = i - 3 * k;
+    ok &= net.fourier[i] == (ax == k % 3 ? 6.2831855f * (float)(1 << (k / 3)) : 0.0f);
   }
   if (tid < 32) {
     tmem_alloc(smem_u32((const void*)&misc[0]), kFitTmemCols);
@@ -174,7 +171,7 @@ __global__ void __launch_bounds__(128 * kFitWGS, 1)
   }
   fence_proxy_async();
   tc_fence_before();
-  __syncthreads();
+  const bool nerf = __syncthreads_and(ok) != 0;
   tc_fence_after();
 
   const uint32_t tmem = (uint32_t)misc[0];
@@ -190,7 +187,6 @@ __global__ void __launch_bounds__(128 * kFitWGS, 1)
   bool failed = false;
 
   const net32::Latent lat = net32::make_latent(net, a.time);
-  const bool nerf = misc[2] != 0;
   const int step = a.step_ptr ? *a.step_ptr : a.step;
   const float inv_n = 1.0f / (float)a.n;
   // delta rows of the weight-gradient MMA are staged times 2^dexp >= n
