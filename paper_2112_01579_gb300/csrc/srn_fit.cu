@@ -286,6 +286,11 @@ __global__ void __launch_bounds__(kFitThreads, 4) fit_point_kernel(const NetDev 
 // 65,537 points of the same network through autograd 434 -> 312 us.
 constexpr int kTileStride = 36;  // floats per row: eight rows' 16-byte loads hit distinct banks
 constexpr int kTileMaxIn = 48;   // inputs of layer 0: 16 threads x 3 entries
+// Points with a residual below this are decided by the accurate functions:
+// inline and library sines move a density by 2e-7 at most on networks of the
+// workloads' shapes.  A converged fit (residuals around 0.01) has a few
+// hundred such points in 2^18.
+constexpr float kSignBand = 4.0e-6f;
 
 // acc[i][j] += sum over the CTA's points of d[o_i][p] v[r_j][p], o_i = tid % 8
 // + 8 i, r_j = tid / 8 + 16 j (rows past `rows` repeat the last one; their
@@ -366,12 +371,14 @@ __device__ __forceinline__ void store_dz(const float* d, const float* Wz, float*
 }
 
 template <int NL>
-__global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const NetDev net, const PointArgs a,
-                                                                  const tile32::Net t, int wfloats) {
+__global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_constant__ NetDev net,
+                                                                  const __grid_constant__ PointArgs a,
+                                                                  const __grid_constant__ tile32::Net t, int wfloats) {
   constexpr int C = 32, S = kTileStride, NH = NL - 1;  // NH activations per point
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
   tile32::load_net<C>(sm, t, net);
+  const bool nerf = tile32::nerf_rows(sm + t.oF, t.m);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* base0 = sm + t.total;                // first warp's rows
   float* v0 = base0 + warp * wfloats;         // layer inputs, then NH blocks of activation rows, then dout
@@ -382,6 +389,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const NetDev n
   const Latent lat = make_latent(net, a.time);
   const float inv_n = 1.0f / (float)a.n;
   const int D = t.D, nchunks = (a.n + kFitThreads - 1) / kFitThreads;
+  const int mode = net.act == SRN_ACT_SNAKEALT ? 1 : 0;
 
   float g0[4][3], gh[NL > 2 ? NL - 2 : 1][4][2], gb[NH], gl[4], gbl = 0.f, loss_acc = 0.f;
 #pragma unroll
@@ -402,16 +410,18 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const NetDev n
     if (valid) {
       if (a.mode == 0) p = sample::fit_point(a.cdf, a.cdf_res, a.seed, step, j, a.n);
       else p = clamp_p(make_float3(a.pts_in[3 * j], a.pts_in[3 * j + 1], a.pts_in[3 * j + 2]));
-      tile32::put_inputs<S>(v0, sm, t, lat, false, p);
+    }
+    // ---- forward: activations to shared memory, their derivatives kept
+    if (valid) {
+      tile32::put_inputs<S, false>(v0, sm, t, lat, nerf, p);
     } else {
       for (int k = 0; k < t.d0; ++k) v0[k * S + lane] = 0.f;
     }
     __syncwarp();
-    // ---- forward: activations to shared memory, their derivatives kept
     tile32::Acc<C> x, df[NH];
     tile32::set_bias<C>(x, sm + t.ob0);
     tile32::layer<C, S>(x, v0, sm + t.oW0, t.d0);
-    tile32::activate_df<C>(net.act, x, df[0]);
+    tile32::activate_call<C>(mode, x, df[0]);
     tile32::put<C, S>(x, act0);
     __syncwarp();
 #pragma unroll
@@ -419,20 +429,21 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const NetDev n
       const float* W = sm + t.oHid + (h - 1) * t.hidStride;
       tile32::set_bias<C>(x, W + C * C);
       tile32::layer<C, S>(x, act0 + (h - 1) * C * S, W, C);
-      tile32::activate_df<C>(net.act, x, df[h]);
+      tile32::activate_call<C>(mode, x, df[h]);
       tile32::put<C, S>(x, act0 + h * C * S);
       __syncwarp();
     }
     const float* alast = act0 + (NH - 1) * C * S;
     float dout[4] = {0.f, 0.f, 0.f, 0.f};
     if (a.mode == 0) {
-      float out[4];
+      float out[4], want[4];
 #pragma unroll
-      for (int dd = 0; dd < 4; ++dd) out[dd] = dd < D ? tile32::last_layer<C, S>(alast, sm, t, dd) : 0.f;
+      for (int dd = 0; dd < 4; ++dd) {
+        out[dd] = dd < D ? tile32::last_layer<C, S>(alast, sm, t, dd) : 0.f;
+        want[dd] = 0.f;
+      }
       if (valid) {
-        const float r = out[0] - vol_sample(a.vol, p);
-        loss_acc += fabsf(r);
-        dout[0] = sgnf(r) * inv_n;
+        want[0] = vol_sample(a.vol, p);
         if (D == 4) {
           const float hh[3] = {1.0f / (float)(a.vol.nx - 1), 1.0f / (float)(a.vol.ny - 1),
                                1.0f / (float)(a.vol.nz - 1)};
@@ -442,10 +453,33 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const NetDev n
             if (ax == 0) { pp.x = clamp01f(p.x + hh[0]); pm.x = clamp01f(p.x - hh[0]); }
             if (ax == 1) { pp.y = clamp01f(p.y + hh[1]); pm.y = clamp01f(p.y - hh[1]); }
             if (ax == 2) { pp.z = clamp01f(p.z + hh[2]); pm.z = clamp01f(p.z - hh[2]); }
-            const float g = (vol_sample(a.vol, pp) - vol_sample(a.vol, pm)) / (2.0f * hh[ax]);
-            const float ra = out[1 + ax] - a.gs * g;
+            want[1 + ax] = a.gs * ((vol_sample(a.vol, pp) - vol_sample(a.vol, pm)) / (2.0f * hh[ax]));
+          }
+        }
+      }
+      // the sign of a residual decides a point's whole gradient: a point with
+      // one within kSignBand of zero takes its outputs from the accurate
+      // functions
+      bool close = false;
+#pragma unroll
+      for (int dd = 0; dd < 4; ++dd) close |= valid && dd < D && fabsf(out[dd] - want[dd]) < kSignBand;
+      for (unsigned int m = __ballot_sync(0xffffffffu, close); m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const float3 q = make_float3(__shfl_sync(0xffffffffu, p.x, src), __shfl_sync(0xffffffffu, p.y, src),
+                                     __shfl_sync(0xffffffffu, p.z, src));
+        const float4 o = tile32::accurate_point(sm, t, net.act, lat, q, sdout);
+        if (lane == src) out[0] = o.x, out[1] = o.y, out[2] = o.z, out[3] = o.w;
+      }
+      if (valid) {
+        const float r = out[0] - want[0];
+        loss_acc += fabsf(r);
+        dout[0] = sgnf(r) * inv_n;
+        if (D == 4) {
+#pragma unroll
+          for (int dd = 1; dd < 4; ++dd) {
+            const float ra = out[dd] - want[dd];
             loss_acc += a.gw * fabsf(ra);
-            dout[1 + ax] = a.gw * sgnf(ra) * inv_n;
+            dout[dd] = a.gw * sgnf(ra) * inv_n;
           }
         }
       }

@@ -146,21 +146,6 @@ static __device__ __noinline__ float4 sincos_pair(float x0, float x1) {
   return r;
 }
 
-// Activation of the lane's values in place, and its derivative.
-template <int C>
-__device__ __forceinline__ void activate_df(int act, Acc<C>& a, Acc<C>& d) {
-  const bool snake = act == SRN_ACT_SNAKEALT;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int q = 0; q < C / 8; ++q) {
-      const float2 x = a.v[i][q];
-      const float4 r = sincos_pair(x.x, x.y);
-      a.v[i][q] = snake ? make_float2(fmaf(0.5f, x.x, r.x * r.x), fmaf(0.5f, x.y, r.z * r.z)) : make_float2(r.x, r.z);
-      d.v[i][q] = snake ? make_float2(0.5f + 2.0f * r.x * r.y, 0.5f + 2.0f * r.z * r.w) : make_float2(r.y, r.w);
-    }
-}
-
 // ---- inline sine / cosine of the tile paths
 // Reduction by Cody and Waite (Software Manual for the Elementary Functions,
 // 1980) in FMA form, then minimax polynomials from a Remez exchange on the
@@ -232,6 +217,62 @@ __device__ __forceinline__ bool nerf_rows(const float* F, int m) {
   return __syncthreads_and(ok) != 0;
 }
 
+// Activation values of four arguments, and their derivatives.  mode: bit 0
+// SnakeAlt, bit 1 by the library functions.
+struct Quad {
+  float4 a, d;
+};
+__device__ __forceinline__ Quad act_quad(float4 x, int mode) {
+  Quad r;
+  if ((mode & 2) || !(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))) <= kActMax)) {
+    const float4 p = sincos_pair(x.x, x.y), q = sincos_pair(x.z, x.w);
+    if (mode & 1) {
+      r.a = make_float4(fmaf(0.5f, x.x, p.x * p.x), fmaf(0.5f, x.y, p.z * p.z), fmaf(0.5f, x.z, q.x * q.x),
+                        fmaf(0.5f, x.w, q.z * q.z));
+      r.d = make_float4(0.5f + 2.0f * p.x * p.y, 0.5f + 2.0f * p.z * p.w, 0.5f + 2.0f * q.x * q.y,
+                        0.5f + 2.0f * q.z * q.w);
+    } else {
+      r.a = make_float4(p.x, p.z, q.x, q.z);
+      r.d = make_float4(p.y, p.w, q.y, q.w);
+    }
+    return r;
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float2 v = h ? make_float2(x.z, x.w) : make_float2(x.x, x.y);
+    float2 t, a, d;
+    const float2 e = reduce_pi(v, t), z = __fmul2_rn(e, e), s = sin_half(e, z), c = cos_half(z);
+    if (mode & 1) {  // sin^2 and sin cos do not change with k
+      a = __ffma2_rn(s, s, __fmul2_rn(v, f2(0.5f)));
+      d = __ffma2_rn(__fadd2_rn(s, s), c, f2(0.5f));
+    } else {
+      a = make_float2(flip(s.x, t.x), flip(s.y, t.y));
+      d = make_float2(flip(c.x, t.x), flip(c.y, t.y));
+    }
+    if (h) r.a.z = a.x, r.a.w = a.y, r.d.z = d.x, r.d.w = d.y;
+    else r.a.x = a.x, r.a.y = a.y, r.d.x = d.x, r.d.y = d.y;
+  }
+  return r;
+}
+// Out of line: a kernel that activates several unrolled layers would not fit
+// the instruction cache with the code inlined at every value.
+static __device__ __noinline__ Quad act_quad_call(float4 x, int mode) { return act_quad(x, mode); }
+
+// Activation and derivative of the lane's values by act_quad_call.
+template <int C>
+__device__ __forceinline__ void activate_call(int mode, Acc<C>& a, Acc<C>& d) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < C / 8; q += 2) {
+      const Quad r = act_quad_call(make_float4(a.v[i][q].x, a.v[i][q].y, a.v[i][q + 1].x, a.v[i][q + 1].y), mode);
+      a.v[i][q] = make_float2(r.a.x, r.a.y);
+      a.v[i][q + 1] = make_float2(r.a.z, r.a.w);
+      d.v[i][q] = make_float2(r.d.x, r.d.y);
+      d.v[i][q + 1] = make_float2(r.d.z, r.d.w);
+    }
+}
+
 // Activation of the lane's values in place; DF: and its derivative.
 template <int C, bool DF>
 __device__ __forceinline__ void activate(int act, Acc<C>& a, Acc<C>* d) {
@@ -284,13 +325,36 @@ __device__ __forceinline__ void put(const Acc<C>& a, float* x) {
   }
 }
 
+// Channels f0 .. f0 + N - 1 of the latent vector at p as rows of z; all 8 N / 4
+// loads (twice that with two keyframes) can be in flight at once.
+template <int S, int N>
+__device__ __forceinline__ void put_latent(float* z, const Latent& lat, float3 p, int f0 = 0) {
+  const Cell cell = net32::make_cell(lat, p);
+  float4 q[N / 4];
+#pragma unroll
+  for (int f = 0; f < N / 4; ++f) q[f] = net32::latent4(lat, cell, f0 + 4 * f);
+#pragma unroll
+  for (int f = 0; f < N / 4; ++f) {
+    z[(4 * f) * S] = q[f].x;
+    z[(4 * f + 1) * S] = q[f].y;
+    z[(4 * f + 2) * S] = q[f].z;
+    z[(4 * f + 3) * S] = q[f].w;
+  }
+}
+
 // Input rows of the lane's point p (+ pl, the low part of a position carried
 // as a pair): [p, sin, cos, z, (t)].
-// NeRF Fourier rows (nerf) take the inline quarter-turn form.
-template <int S>
+// NeRF Fourier rows (nerf) take the inline quarter-turn form.  AHEAD: the
+// latent gather first, so that its loads are in flight during the features
+// (kernels with registers to spare: error grid 3.41 -> 3.37 ms; the fit's
+// point kernel spills and loses 5 %).
+template <int S, bool AHEAD = true>
 __device__ __forceinline__ void put_inputs(float* x, const float* sm, const Net& t, const Latent& lat, bool nerf,
                                            float3 p, float3 pl = make_float3(0.f, 0.f, 0.f)) {
   float* v = x + (threadIdx.x & 31);
+  float* z = v + (3 + 2 * t.m) * S;
+  if (AHEAD && t.F == 16) put_latent<S, 16>(z, lat, p);
+  else if (AHEAD && t.F == 8) put_latent<S, 8>(z, lat, p);
   v[0] = p.x;
   v[S] = p.y;
   v[2 * S] = p.z;
@@ -317,15 +381,8 @@ __device__ __forceinline__ void put_inputs(float* x, const float* sm, const Net&
       v[(4 + 2 * k) * S] = c;
     }
   }
-  const Cell cell = net32::make_cell(lat, p);
-  float* z = v + (3 + 2 * t.m) * S;
-  for (int f = 0; f < t.F; f += 4) {
-    const float4 q = net32::latent4(lat, cell, f);
-    z[f * S] = q.x;
-    z[(f + 1) * S] = q.y;
-    z[(f + 2) * S] = q.z;
-    z[(f + 3) * S] = q.w;
-  }
+  if (!AHEAD || (t.F != 16 && t.F != 8))
+    for (int f = 0; f < t.F; f += 4) put_latent<S, 4>(z + f * S, lat, p, f);
   if (t.ti) z[t.F * S] = lat.tin;
 }
 
@@ -344,6 +401,67 @@ __device__ __forceinline__ float last_layer(const float* x, const float* sm, con
     s3 = fmaf(w4.w, v[(o + 3) * S], s3);
   }
   return sm[t.obl + dd] + ((s0 + s1) + (s2 + s3));
+}
+
+// Outputs of one point (the same p in all lanes) by the accurate functions,
+// the whole warp on it: a lane per Fourier row, latent channel and output
+// neuron, so one point takes about a microsecond; the products in the order
+// of the tile passes.  x: 112 floats of scratch.  Out of line and with its
+// arguments by value: it is for rare use, and the caller keeps its registers.
+static __device__ __noinline__ float4 accurate_point(const float* sm, const Net t, int act, const Latent lat, float3 p,
+                                                     float* x) {
+  constexpr int C = 32;
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  if (lane < 3) x[lane] = lane == 0 ? p.x : (lane == 1 ? p.y : p.z);
+  for (int k = lane; k < t.m; k += 32) {
+    float s, c;
+    net32::fourier_sincos(sm + t.oF + 3 * k, p, s, c);
+    x[3 + 2 * k] = s;
+    x[4 + 2 * k] = c;
+  }
+  const Cell cell = net32::make_cell(lat, p);
+  for (int f = 4 * lane; f < t.F; f += 128) {
+    const float4 q = net32::latent4(lat, cell, f);
+    float* z = x + 3 + 2 * t.m + f;
+    z[0] = q.x;
+    z[1] = q.y;
+    z[2] = q.z;
+    z[3] = q.w;
+  }
+  if (t.ti && lane == 0) x[3 + 2 * t.m + t.F] = lat.tin;
+  __syncwarp();
+  const float* W = sm + t.oW0;
+  const float* in = x;
+  float h = sm[t.ob0 + lane];
+  int K = t.d0;
+  for (int layer = 1;; ++layer) {
+#pragma unroll 8
+    for (int k = 0; k < K; ++k) h = fmaf(W[k * C + lane], in[k], h);
+    const float s = sinf(h);
+    float* next = x + 48 + (layer & 1) * C;
+    next[lane] = act == SRN_ACT_SNAKEALT ? fmaf(0.5f, h, s * s) : s;
+    __syncwarp();
+    in = next;
+    if (layer == t.l - 1) break;
+    W = sm + t.oHid + (layer - 1) * t.hidStride;
+    h = W[C * C + lane];
+    K = C;
+  }
+  // lane 4 d + r: the r-th of the four interleaved sums of output d
+  float sum = 0.f;
+  const int d = lane >> 2, r = lane & 3;
+  if (d < t.D)
+    for (int o = r; o < C; o += 4) sum = fmaf(sm[t.oWl + d * C + o], in[o], sum);
+  float out[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float s0 = __shfl_sync(0xffffffffu, sum, 4 * k), s1 = __shfl_sync(0xffffffffu, sum, 4 * k + 1),
+                s2 = __shfl_sync(0xffffffffu, sum, 4 * k + 2), s3 = __shfl_sync(0xffffffffu, sum, 4 * k + 3);
+    out[k] = k < t.D ? sm[t.obl + k] + ((s0 + s1) + (s2 + s3)) : 0.f;
+  }
+  __syncwarp();
+  return make_float4(out[0], out[1], out[2], out[3]);
 }
 
 // acc[q][j] (points 2q, 2q + 1 of the lane; N weight rows) = sum over the C
