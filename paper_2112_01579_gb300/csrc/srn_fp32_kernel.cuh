@@ -65,10 +65,15 @@ __device__ __forceinline__ float sample_field(const tile32::Ctx& c, float* rows,
   }
 }
 
-// Render: each warp covers an 8 x 4 pixel tile; one lane per ray.
+// Render: a warp takes 32 / K rays, K consecutive samples of each at a time
+// (K = 1, 2, 4, 8; K lanes per ray, pixel tiles of 8 x 4, 4 x 4, 4 x 2,
+// 2 x 2).  The samples of a ray only meet in the compositing, which runs in
+// order over the K lanes; samples past the one that ends the ray are dropped
+// (at most K - 1 a ray).  Large images take K = 1; small ones have too few
+// rays to fill the chip, and their time is a ray's chain of samples.
 template <int C, int SH>
 __global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
-    render_fp32_kernel(const NetDev net, const BatchDev b, const tile32::Net t, int rows) {
+    render_fp32_kernel(const NetDev net, const BatchDev b, const tile32::Net t, int rows, int log2k) {
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
   __shared__ TFDev tf;
@@ -77,14 +82,15 @@ __global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
   const tile32::Ctx ctx{sm, &t, net.act, tile32::nerf_rows(sm + t.oF, t.m)};
   float* mine = sm + t.total + (threadIdx.x >> 5) * rows * tile32::kPts;
 
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, K = 1 << log2k;
+  const int lw = log2k == 0 ? 3 : (log2k == 3 ? 1 : 2), lh = 5 - log2k - lw;  // log2 of the pixel tile's sides
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int tiles_x = (b.W + 7) / 8, tiles_y = (b.H + 3) / 4;
+  const int tiles_x = (b.W + (1 << lw) - 1) >> lw, tiles_y = (b.H + (1 << lh) - 1) >> lh;
   const long long tpf = (long long)tiles_x * tiles_y;
   const long long frame = warp / tpf;
   if (frame >= (long long)b.n_times * b.n_views) return;
-  const int tt = (int)(warp - frame * tpf);
-  const int px = (tt % tiles_x) * 8 + (lane & 7), py = (tt / tiles_x) * 4 + (lane >> 3);
+  const int tt = (int)(warp - frame * tpf), ray_id = lane >> log2k, off = lane & (K - 1);
+  const int px = ((tt % tiles_x) << lw) + (ray_id & ((1 << lw) - 1)), py = ((tt / tiles_x) << lh) + (ray_id >> lw);
   const int view = (int)(frame % b.n_views), ti = (int)(frame / b.n_views);
   const bool inside = px < b.W && py < b.H;
 
@@ -95,31 +101,47 @@ __global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
   df::Ray ray;
   float C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f;
   unsigned int ns = 0;
-  bool live = inside && df::ray_setup(b.cams[view], b.W, b.H, px, py, ray);
+  bool live = inside && df::ray_setup(b.cams[view], b.W, b.H, px, py, ray);  // the same in a ray's K lanes
   const float3 d = live ? make_float3(ray.d[0].h, ray.d[1].h, ray.d[2].h) : make_float3(0.f, 0.f, 0.f);
   float3 p = make_float3(0.5f, 0.5f, 0.5f), pl = make_float3(0.f, 0.f, 0.f);
-  for (int k = 0;; ++k) {
+  for (int k = off;; k += K) {
     float len = 0.f;
-    live = live && df::segment(ray, k, b.step, len, p, pl);
-    if (!__any_sync(0xffffffffu, live)) break;
+    const bool have = live && df::segment(ray, k, b.step, len, p, pl);
+    if (!__any_sync(0xffffffffu, have)) break;
     // lanes without a sample evaluate their last position (or the centre); nothing reads the result
     float3 g = make_float3(0.f, 0.f, 0.f);
     const float rho = sample_field<C, SH>(ctx, mine, lat, p, pl, b.fd_h, g);
     __syncwarp();
-    if (live) {
-      ++ns;
-      float4 c = tf_eval(tf, rho);
-      float alpha = -expm1f(-c.w * tf.opacity_scale * len);
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (have) {
+      c = tf_eval(tf, rho);
+      c.w = -expm1f(-c.w * tf.opacity_scale * len);
       if (SH != SRN_SHADE_NONE) shade(c, g, d);
-      float w = (1.0f - A) * alpha;
-      C0 = fmaf(w, c.x, C0);
-      C1 = fmaf(w, c.y, C1);
-      C2 = fmaf(w, c.z, C2);
-      A += w;
-      live = !(A >= b.et);
+    }
+    for (int i = 0; i < K; ++i) {
+      const int src = (lane & ~(K - 1)) + i;
+      float4 v = c;
+      bool any = have;
+      if (K > 1) {
+        v.x = __shfl_sync(0xffffffffu, c.x, src);
+        v.y = __shfl_sync(0xffffffffu, c.y, src);
+        v.z = __shfl_sync(0xffffffffu, c.z, src);
+        v.w = __shfl_sync(0xffffffffu, c.w, src);
+        any = __shfl_sync(0xffffffffu, (int)have, src) != 0;
+      }
+      live = live && any;  // the ray's last segment is behind it
+      if (live) {
+        ns += off == 0;
+        const float w = (1.0f - A) * v.w;
+        C0 = fmaf(w, v.x, C0);
+        C1 = fmaf(w, v.y, C1);
+        C2 = fmaf(w, v.z, C2);
+        A += w;
+        live = !(A >= b.et);
+      }
     }
   }
-  if (inside) {
+  if (inside && off == 0) {
     size_t idx = ((size_t)frame * b.H + py) * b.W + px;
     reinterpret_cast<float4*>(b.out)[idx] = make_float4(C0, C1, C2, A);
   }
@@ -189,9 +211,21 @@ cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s
   auto k = render_fp32_kernel<C, SH>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  long long tiles = (long long)((b.W + 7) / 8) * ((b.H + 3) / 4) * b.n_views * b.n_times;
-  long long blocks = (tiles + warps - 1) / warps;
-  k<<<(unsigned)blocks, 32 * warps, smem, s>>>(net, b, t, rows);
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  // samples of a ray per warp: double while that leaves at most the warps the
+  // SMs hold at once (16 each; beyond, the dropped samples only cost)
+  int log2k = 0;
+  long long tiles = 0;
+  for (;; ++log2k) {
+    const int lw = log2k == 0 ? 3 : (log2k == 3 ? 1 : 2), lh = 5 - log2k - lw;
+    tiles = (long long)((b.W + (1 << lw) - 1) >> lw) * ((b.H + (1 << lh) - 1) >> lh) * b.n_views * b.n_times;
+    if (log2k == 3 || 2 * tiles > 16ll * sms) break;
+  }
+  const long long blocks = (tiles + warps - 1) / warps;
+  k<<<(unsigned)blocks, 32 * warps, smem, s>>>(net, b, t, rows, log2k);
   return cudaGetLastError();
 }
 
