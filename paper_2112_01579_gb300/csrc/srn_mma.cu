@@ -75,8 +75,7 @@ cudaError_t launch_render_mma(const NetDev& n, const BatchDev& b, unsigned long 
   if (n.m == 14 && n.F == 16) {
     // the four-layer SnakeAlt networks of the inference and shading workloads:
     // layer loop unrolled, output count fixed and, for a single latent grid,
-    // no time blend in the gather (the adjoint keeps the generic kernel, whose
-    // register allocation spills less there)
+    // no time blend in the gathers
     if (n.act == SRN_ACT_SNAKEALT && n.l == 4) {
       const PointsDev pd{};
       const bool st = n.nkey == 1;
@@ -85,6 +84,8 @@ cudaError_t launch_render_mma(const NetDev& n, const BatchDev& b, unsigned long 
                   : launch_t<32, 14, 16, SRN_ACT_SNAKEALT, SRN_SHADE_NONE, 0, 0, 4, 0>(n, b, pd, ctr, status, s);
       if (st && n.D == 1 && b.shading == SRN_SHADE_FD)
         return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, SRN_SHADE_FD, 0, 0, 4, 1>(n, b, pd, ctr, status, s);
+      if (st && n.D == 1 && b.shading == SRN_SHADE_ADJOINT)
+        return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, SRN_SHADE_ADJOINT, 0, 0, 4, 1>(n, b, pd, ctr, status, s);
       if (st && n.D == 4 && b.shading == SRN_SHADE_HEAD)
         return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, SRN_SHADE_HEAD, 0, 0, 4, 1>(n, b, pd, ctr, status, s);
     }

@@ -132,6 +132,17 @@ __device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uin
       : "memory");
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                : "memory");
@@ -166,6 +177,9 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   d |= (uint64_t)2u << 61;              // SWIZZLE_128B
   return d;
 }
+
+// A descriptor moved by `bytes` (a multiple of 16; addresses stay below 2^18).
+__device__ __forceinline__ uint64_t desc_at(uint64_t d, uint32_t bytes) { return d + (uint64_t)(bytes >> 4); }
 
 // Instruction descriptor: kind::f16, A = B = FP16, D = FP32, both K-major,
 // M = 128, N = the layer's output width.
@@ -484,7 +498,7 @@ __device__ __forceinline__ void tmem_st_row(uint32_t taddr, const float (&v)[C])
 // (trilinear in p inside the cell chosen by cell_coord, time-blended):
 // sum over corners and keyframes of w_time (gz . g_corner) grad w_corner(p),
 // with d f / d p = R - 1 per axis.
-template <int F>
+template <int F, int ST>
 __device__ __forceinline__ float3 latent_grad_h(const __half* __restrict__ G, int R, const RayLat& rl, float3 p,
                                                 const float* gz) {
   int ix, iy, iz;
@@ -501,9 +515,9 @@ __device__ __forceinline__ float3 latent_grad_h(const __half* __restrict__ G, in
     const float wx = dx ? fx : 1.0f - fx, wy = dy ? fy : 1.0f - fy, wz = dz ? fz : 1.0f - fz;
     const int off = base + dx * sx + dy * sy + dz * sz;
 #pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-      const int gb = kk ? rl.g1 : rl.g0;
-      if (kk && gb < 0) break;
+    for (int kk = 0; kk < (ST ? 1 : 2); ++kk) {
+      const int gb = ST ? 0 : (kk ? rl.g1 : rl.g0);
+      if (!ST && kk && gb < 0) break;
       float dot = 0.0f;
 #pragma unroll
       for (int c = 0; c < F; c += 8) {
@@ -516,7 +530,7 @@ __device__ __forceinline__ float3 latent_grad_h(const __half* __restrict__ G, in
           dot = fmaf(gz[c + 2 * e + 1], v.y, dot);
         }
       }
-      dot *= kk ? rl.w1 : rl.w0;
+      if (!ST) dot *= kk ? rl.w1 : rl.w0;
       g.x = fmaf(dot, (dx ? wy : -wy) * wz, g.x);
       g.y = fmaf(dot, wx * (dy ? wz : -wz), g.y);
       g.z = fmaf(dot, wx * (dz ? wy : -wy), g.z);
@@ -561,7 +575,12 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   volatile int* misc = reinterpret_cast<volatile int*>(sm + plan.oMisc);  // [0] tmem base, [4+wg] fail
 
   const int tid = threadIdx.x;
-  const int wg = tid >> 7, row = tid & 127, lane = tid & 31;
+  // the warp's index by a broadcast is known to be uniform, so addresses made
+  // from it stay in uniform registers: 3 % of a frame; point evaluation is
+  // 12 % slower that way (81 against 72 us for 2^20 points)
+  const int warp_id = POINTS ? tid >> 5 : __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int wg = warp_id >> 2, row = tid & 127, lane = tid & 31;
+  const bool issuer = (warp_id & 3) == 0;  // the warp whose elected lane issues its warpgroup's MMAs
   // LF > 0: a network of LF layers and D = 1 output (4 for the gradient
   // head), both fixed at compile time (the layer loop unrolls, the output
   // loop has its exact trip count); the dispatch picks such an instantiation
@@ -730,9 +749,9 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   // takes the place of the consumed derivative stash)
   constexpr int ACOL = C;
   const uint32_t a_tmem = d_tmem + ACOL, t_a = t_row + ACOL;
-  const uint32_t b0_addr = smem_u32(B0), bh_addr = smem_u32(Bh), bb_addr = smem_u32(Bb);
-  const uint32_t one_addr = smem_u32(sm + plan.oOne);
-  const uint32_t bht_addr = smem_u32(BhT), b0t_addr = smem_u32(B0T);
+  const uint64_t b0_desc = sw128_desc(smem_u32(B0)), bh_desc = sw128_desc(smem_u32(Bh)),
+                 bb_desc = sw128_desc(smem_u32(Bb)), one_desc = sw128_desc(smem_u32(sm + plan.oOne));
+  const uint64_t bht_desc = sw128_desc(smem_u32(BhT)), b0t_desc = sw128_desc(smem_u32(B0T));
   const uint32_t mb = smem_u32(&mbar[wg]);
   const int bar_id = 1 + wg;
 
@@ -841,12 +860,12 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
     tc_fence_before();
     const bool any = bar_red_or(bar_id, 128, active && !failed);
     if (!any || misc[4 + wg]) break;
-    if (row == 0 && !b.stall_test) {  // stall_test: no MMA, no commit, nothing in flight
+    if (issuer && !b.stall_test && elect_one()) {  // stall_test: no MMA, no commit, nothing in flight
       tc_fence_after();
 #pragma unroll
       for (int kk = 0; kk < K0 / 16; ++kk) {
         const uint32_t ka = ((16 * kk) >> 6), kb = ((16 * kk) & 63) * 2;
-        mma_f16_ta(d_tmem, a_tmem + 8 * kk, sw128_desc(b0_addr + ka * BT + kb), IDESC, kk > 0);
+        mma_f16_ta(d_tmem, a_tmem + 8 * kk, desc_at(b0_desc, ka * BT + kb), IDESC, kk > 0);
       }
       mma_commit(mb);
     }
@@ -892,18 +911,17 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
           }
         }
         tc_fence_before();
-        bar_sync(bar_id, 128);
-        if (misc[4 + wg]) { stop = true; break; }
-        if (row == 0) {
+        if (bar_red_or(bar_id, 128, failed)) { stop = true; break; }
+        if (issuer && elect_one()) {
           tc_fence_after();
-          const uint32_t bw = bh_addr + layer * NAH * BT;
+          const uint64_t bw = desc_at(bh_desc, layer * NAH * BT);
           const uint32_t kbias = 16 * layer;  // this layer's K-block of the bias tile
-          mma_f16(d_tmem, sw128_desc(one_addr), sw128_desc(bb_addr + (kbias >> 6) * BT + (kbias & 63) * 2), IDESC,
+          mma_f16(d_tmem, one_desc, desc_at(bb_desc, (kbias >> 6) * BT + (kbias & 63) * 2), IDESC,
                   0u);
 #pragma unroll
           for (int kk = 0; kk < 2 * C / 16; ++kk) {
             const uint32_t ka = ((16 * kk) >> 6), kb = ((16 * kk) & 63) * 2;
-            mma_f16_ta(d_tmem, a_tmem + 8 * kk, sw128_desc(bw + ka * BT + kb), IDESC, 1u);
+            mma_f16_ta(d_tmem, a_tmem + 8 * kk, desc_at(bw, ka * BT + kb), IDESC, 1u);
           }
           mma_commit(mb);
         }
@@ -950,18 +968,17 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
           tmem_wait_st();
         }
         tc_fence_before();
-        bar_sync(bar_id, 128);
-        if (misc[4 + wg]) { stop = true; break; }
-        if (row == 0) {
+        if (bar_red_or(bar_id, 128, failed)) { stop = true; break; }
+        if (issuer && elect_one()) {
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < 2 * C / 16; ++kk) {
             const uint32_t ka = ((16 * kk) >> 6), kb = ((16 * kk) & 63) * 2;
             const uint32_t ad = d_tmem + acol + 8 * kk;
             if (h >= 1)
-              mma_f16_ta(d_tmem, ad, sw128_desc(bht_addr + (h - 1) * NAH * BT + ka * BT + kb), IDESC, kk > 0);
+              mma_f16_ta(d_tmem, ad, desc_at(bht_desc, (h - 1) * NAH * BT + ka * BT + kb), IDESC, kk > 0);
             else
-              mma_f16_ta(d_tmem, ad, sw128_desc(b0t_addr + ka * (K0 * 128) + kb), idesc_n(K0), kk > 0);
+              mma_f16_ta(d_tmem, ad, desc_at(b0t_desc, ka * (K0 * 128) + kb), idesc_n(K0), kk > 0);
           }
           mma_commit(mb);
         }
@@ -1020,7 +1037,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
                 gp.z = fmaf(coef, fm[3 * kq + 2], gp.z);
               }
             }
-            float3 gl = latent_grad_h<F>(net.grid_h, net.R, rl, qs, gv + 2 * M + 3);
+            float3 gl = latent_grad_h<F, ST>(net.grid_h, net.R, rl, qs, gv + 2 * M + 3);
             gl = make_float3(gl.x * gscale, gl.y * gscale, gl.z * gscale);  // grid_h = G 2^-gexp
             gadj = make_float3(gp.x + gl.x, gp.y + gl.y, gp.z + gl.z);
           }

@@ -116,3 +116,22 @@ def test_eval_large_arguments(S, act, arg):
     S.srn_density_grad(net.ctx, torch.tensor(pts, device="cuda"), rho, grad)
     gref = oracle.net_input_grad(oracle.OracleNet(p), pts)[1]
     assert (np.abs(grad.cpu().numpy() - gref) / np.maximum(np.abs(gref).max(axis=1, keepdims=True), 1.0)).max() <= 1e-4
+
+
+@pytest.mark.parametrize("width,m,most", [(32, 14, 8), (48, 22, 6), (64, 30, 7)])
+def test_fp16_depths(S, width, m, most):
+    """The depths the FP16 path takes at each width, and the next one refused."""
+    import torch
+    for layers in {most, min(most + 1, 8)}:
+        p = synth.to_half_exact(synth.random_params(R=3, F=16, m=m, layers=layers, width=width, act=synth.ACT_SNAKEALT, seed=layers))
+        net, pts = S.Network(p, precision=S.SRN_PREC_FP16), _points(200, 1)
+        out = torch.full((200, 1), float("nan"), device="cuda")
+        if layers > most:
+            with pytest.raises(S.SrnError) as e:
+                S.srn_eval(net.ctx, torch.tensor(pts, device="cuda"), out)
+            assert e.value.status == S.SRN_ERR_UNSUPPORTED
+            continue
+        S.srn_eval(net.ctx, torch.tensor(pts, device="cuda"), out)
+        on = oracle.OracleNet(p)
+        bound = oracle.error_bounds(on, pts, oracle.PREC_FP16, grad=False)[0]
+        assert (np.abs(out.cpu().numpy() - oracle.net_forward(on, pts)) / bound).max() <= 1.0
