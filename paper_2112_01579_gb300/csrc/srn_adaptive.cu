@@ -20,11 +20,10 @@ namespace {
 
 using namespace net32;
 
-constexpr int kErrThreads = 128;
 constexpr int kCdfThreads = kCdfBlock / 2;  // two weights per thread
 
 template <int C>
-__global__ void __launch_bounds__(kErrThreads, C == 32 ? 4 : 2)
+__global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     error_grid_kernel(const NetDev net, const VolDev vol, int res, int spv, unsigned long long seed, float time,
                       float* __restrict__ E, const tile32::Net t, int rows) {
   extern __shared__ float4 smem4[];
@@ -58,17 +57,17 @@ template <int C>
 cudaError_t error_grid_t(const NetDev& net, const VolDev& vol, int res, int spv, unsigned long long seed, float time,
                          float* E, cudaStream_t st) {
   const tile32::Net t = tile32::make_net(net);
-  const int rows = t.d0 > C ? t.d0 : C, warps = tile32::warps_for(t, rows);
-  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
-  auto k = error_grid_kernel<C>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const long long nvox = (long long)res * res * res;
-  const long long blocks = (nvox + 32 * warps - 1) / (32 * warps), most = 4ll * sms;
+  const long long tiles = ((long long)res * res * res + 31) / 32;
+  const int rows = t.d0 > C ? t.d0 : C, warps = tile32::warps_for(t, C, rows, tiles, sms);
+  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
+  auto k = error_grid_kernel<C>;
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const long long blocks = (tiles + warps - 1) / warps, most = (long long)(tile32::max_warps(C) / warps) * sms;
   k<<<(unsigned)(blocks < most ? blocks : most), 32 * warps, smem, st>>>(net, vol, res, spv, seed, time, E, t, rows);
   return cudaGetLastError();
 }

@@ -14,7 +14,6 @@
 namespace srn {
 namespace fp32 {
 
-constexpr int kMaxThreads = 128;
 using namespace net32;
 
 // Rows of 32 floats a warp's tile needs: the inputs and activations share
@@ -72,7 +71,7 @@ __device__ __forceinline__ float sample_field(const tile32::Ctx& c, float* rows,
 // (at most K - 1 a ray).  Large images take K = 1; small ones have too few
 // rays to fill the chip, and their time is a ray's chain of samples.
 template <int C, int SH>
-__global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
+__global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     render_fp32_kernel(const NetDev net, const BatchDev b, const tile32::Net t, int rows, int log2k) {
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
@@ -152,7 +151,7 @@ __global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
 // adjoint gradient grad[n][3] (when grad is not null); mode 2 writes the
 // input vector-Jacobian product grad[n][3] = sum_d dout[n][d] d out_d / d p.
 template <int C, int MODE>
-__global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
+__global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     eval_fp32_kernel(const NetDev net, const float* __restrict__ pts, int n, float time, float* __restrict__ out,
                      float* __restrict__ grad, const float* __restrict__ dout, const tile32::Net t, int rows) {
   constexpr int S = tile32::kPts;
@@ -206,13 +205,8 @@ __global__ void __launch_bounds__(kMaxThreads, C == 32 ? 4 : 2)
 template <int C, int SH>
 cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s) {
   const tile32::Net t = tile32::make_net(net);
-  const int rows = tile_rows(t, C, SH == SRN_SHADE_ADJOINT, false), warps = tile32::warps_for(t, rows);
-  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
-  auto k = render_fp32_kernel<C, SH>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   // samples of a ray per warp: double while that leaves at most the warps the
@@ -224,6 +218,11 @@ cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s
     tiles = (long long)((b.W + (1 << lw) - 1) >> lw) * ((b.H + (1 << lh) - 1) >> lh) * b.n_views * b.n_times;
     if (log2k == 3 || 2 * tiles > 16ll * sms) break;
   }
+  const int rows = tile_rows(t, C, SH == SRN_SHADE_ADJOINT, false), warps = tile32::warps_for(t, C, rows, 0, sms);
+  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
+  auto k = render_fp32_kernel<C, SH>;
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   const long long blocks = (tiles + warps - 1) / warps;
   k<<<(unsigned)blocks, 32 * warps, smem, s>>>(net, b, t, rows, log2k);
   return cudaGetLastError();
@@ -233,17 +232,18 @@ template <int C, int MODE>
 cudaError_t launch_eval_t(const NetDev& net, const float* pts, int n, float time, float* out, float* grad,
                           const float* dout, cudaStream_t s) {
   const tile32::Net t = tile32::make_net(net);
-  const int rows = tile_rows(t, C, MODE != 0, MODE == 2), warps = tile32::warps_for(t, rows);
-  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
-  auto k = eval_fp32_kernel<C, MODE>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  // CTAs stage the parameters once and walk the tiles: at most four per SM
-  const long long blocks = ((long long)n + 32 * warps - 1) / (32 * warps), most = 4ll * sms;
+  const long long tiles = ((long long)n + 31) / 32;
+  const int rows = tile_rows(t, C, MODE != 0, MODE == 2), warps = tile32::warps_for(t, C, rows, tiles, sms);
+  const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
+  auto k = eval_fp32_kernel<C, MODE>;
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // CTAs stage the parameters once and walk the tiles: as many as an SM holds
+  const long long blocks = (tiles + warps - 1) / warps, most = (long long)(tile32::max_warps(C) / warps) * sms;
   k<<<(unsigned)(blocks < most ? blocks : most), 32 * warps, smem, s>>>(net, pts, n, time, out, grad, dout, t, rows);
   return cudaGetLastError();
 }
