@@ -152,8 +152,8 @@ static __device__ __noinline__ float4 sincos_pair(float x0, float x1) {
 // Reduction by Cody and Waite (Software Manual for the Elementary Functions,
 // 1980) in FMA form, then minimax polynomials from a Remez exchange on the
 // absolute error, each coefficient rounded to FP32 before the next was
-// fitted: sin r on |r| <= 1.0005 pi/2 to 5.0e-9, cos r to 4.4e-10; on
-// |r| <= 1.001 pi/4 1.9e-9 and 1.1e-10 (before FP32 arithmetic rounds, about
+// fitted: sin r on |r| <= 1.0005 pi/2 to 5.0e-9; on
+// |r| <= 1.001 pi/4 sin to 1.9e-9 and cos to 1.1e-10 (before FP32 arithmetic rounds, about
 // 6e-8).  They cost a third of the issue slots of the accurate library
 // calls, which stay for arguments beyond kActMax and for Fourier matrices
 // that are not powers of two.
@@ -175,11 +175,12 @@ __device__ __forceinline__ float2 sin_half(float2 r, float2 z) {
   p = __ffma2_rn(z, p, f2(-0.166666567f));
   return __ffma2_rn(__fmul2_rn(r, z), p, r);
 }
-__device__ __forceinline__ float2 cos_half(float2 z) {
-  float2 p = __ffma2_rn(z, f2(-2.62090197e-07f), f2(2.47701792e-05f));
-  p = __ffma2_rn(z, p, f2(-0.00138885854f));
-  p = __ffma2_rn(z, p, f2(0.0416666567f));
-  return __ffma2_rn(__fmul2_rn(z, z), p, __ffma2_rn(z, f2(-0.5f), f2(1.0f)));
+// cos r = sin(pi / 2 - |r|): a polynomial in r would lose the relative
+// precision near the cosine's zero.
+__device__ __forceinline__ float2 cos_half(float2 r) {
+  const float2 a = make_float2(fabsf(r.x), fabsf(r.y));
+  const float2 h = __fadd2_rn(__ffma2_rn(a, f2(-1.0f), f2(1.57079637050628662f)), f2(-4.37113883e-8f));
+  return sin_half(h, __fmul2_rn(h, h));
 }
 __device__ __forceinline__ float flip(float v, float t) {  // v (-1)^k
   return __int_as_float(__float_as_int(v) ^ (__float_as_int(t) << 31));
@@ -243,7 +244,7 @@ __device__ __forceinline__ Quad act_quad(float4 x, int mode) {
   for (int h = 0; h < 2; ++h) {
     const float2 v = h ? make_float2(x.z, x.w) : make_float2(x.x, x.y);
     float2 t, a, d;
-    const float2 e = reduce_pi(v, t), z = __fmul2_rn(e, e), s = sin_half(e, z), c = cos_half(z);
+    const float2 e = reduce_pi(v, t), z = __fmul2_rn(e, e), s = sin_half(e, z), c = cos_half(e);
     if (mode & 1) {  // sin^2 and sin cos do not change with k
       a = __ffma2_rn(s, s, __fmul2_rn(v, f2(0.5f)));
       d = __ffma2_rn(__fadd2_rn(s, s), c, f2(0.5f));
@@ -305,7 +306,7 @@ __device__ __forceinline__ void activate(int act, Acc<C>& a, Acc<C>* d) {
       const float2 r = reduce_pi(x, t), z = __fmul2_rn(r, r);
       const float2 s = sin_half(r, z);
       float2 c = make_float2(0.f, 0.f);
-      if (DF) c = cos_half(z);
+      if (DF) c = cos_half(r);
       if (snake) {  // sin^2 and sin cos do not change with k
         a.v[i][q] = __ffma2_rn(s, s, __fmul2_rn(x, f2(0.5f)));
         if (DF) d->v[i][q] = __ffma2_rn(__fadd2_rn(s, s), c, f2(0.5f));
@@ -468,27 +469,39 @@ static __device__ __noinline__ float4 accurate_point(const float* sm, const Net 
 
 // acc[q][j] (points 2q, 2q + 1 of the lane; N weight rows) = sum over the C
 // entries o of d (rows of S floats) of W[row j][o]: the product with the
-// transposed layer, entries ascending.  row(j) gives the lane's weight rows.
-template <int C, int S, int N, class Row>
+// transposed layer, in PARTS sums of C / PARTS consecutive entries.  row(j)
+// gives the lane's weight rows.
+template <int C, int S, int N, int PARTS = 1, class Row>
 __device__ __forceinline__ void back(float2 (&acc)[2][N], const float* d, const float* W, Row row) {
   const float* dp = d + 4 * point_group();
 #pragma unroll
   for (int j = 0; j < N; ++j) acc[0][j] = acc[1][j] = make_float2(0.f, 0.f);
-#pragma unroll 2
-  for (int o = 0; o < C; o += 4) {
-    float4 x[4];
+#pragma unroll 1
+  for (int part = 0; part < PARTS; ++part) {
+    float2 s[2][N];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) x[e] = *reinterpret_cast<const float4*>(dp + (o + e) * S);
+    for (int j = 0; j < N; ++j) s[0][j] = s[1][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int o = part * (C / PARTS); o < (part + 1) * (C / PARTS); o += 4) {
+      float4 x[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] = *reinterpret_cast<const float4*>(dp + (o + e) * S);
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const float4 w = *reinterpret_cast<const float4*>(W + row(j) * C + o);
+        const float ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 ww = make_float2(ws[e], ws[e]);
+          s[0][j] = __ffma2_rn(make_float2(x[e].x, x[e].y), ww, s[0][j]);
+          s[1][j] = __ffma2_rn(make_float2(x[e].z, x[e].w), ww, s[1][j]);
+        }
+      }
+    }
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      const float4 w = *reinterpret_cast<const float4*>(W + row(j) * C + o);
-      const float ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 ww = make_float2(ws[e], ws[e]);
-        acc[0][j] = __ffma2_rn(make_float2(x[e].x, x[e].y), ww, acc[0][j]);
-        acc[1][j] = __ffma2_rn(make_float2(x[e].z, x[e].w), ww, acc[1][j]);
-      }
+      acc[0][j] = PARTS == 1 ? s[0][j] : __fadd2_rn(acc[0][j], s[0][j]);
+      acc[1][j] = PARTS == 1 ? s[1][j] : __fadd2_rn(acc[1][j], s[1][j]);
     }
   }
 }
@@ -554,6 +567,39 @@ __device__ __forceinline__ void seed(Acc<C>& a, const float* sm, const Net& t, c
   }
 }
 
+// l += gradient with respect to the cell coordinates of sum_f g_f z_f over N
+// channels from f0 (g_f in rows of z): per corner the product of g with the
+// corner's values, times the derivative of its weight.
+template <int S, int N>
+__device__ __forceinline__ void latent_vjp(float3& l, const float* z, const Latent& lat, const Cell& c, int f0) {
+  float g[N];
+#pragma unroll
+  for (int f = 0; f < N; ++f) g[f] = z[f * S];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
+    const float wx = dx ? c.fx : 1.0f - c.fx, wy = dy ? c.fy : 1.0f - c.fy, wz = dz ? c.fz : 1.0f - c.fz;
+    const int at = c.base + dx * c.sx + dy * c.sy + dz * c.sz + f0;
+    float dot = 0.f;
+#pragma unroll
+    for (int f = 0; f < N; f += 4) {
+      float4 v = __ldg(reinterpret_cast<const float4*>(lat.g0 + at + f));
+      if (lat.g1) {
+        const float4 h = __ldg(reinterpret_cast<const float4*>(lat.g1 + at + f));
+        v = make_float4(lat.tw0 * v.x + lat.tw1 * h.x, lat.tw0 * v.y + lat.tw1 * h.y, lat.tw0 * v.z + lat.tw1 * h.z,
+                        lat.tw0 * v.w + lat.tw1 * h.w);
+      }
+      dot = fmaf(g[f], v.x, dot);
+      dot = fmaf(g[f + 1], v.y, dot);
+      dot = fmaf(g[f + 2], v.z, dot);
+      dot = fmaf(g[f + 3], v.w, dot);
+    }
+    l.x = fmaf(dot, (dx ? wy : -wy) * wz, l.x);
+    l.y = fmaf(dot, wx * (dy ? wz : -wz), l.y);
+    l.z = fmaf(dot, wx * (dz ? wy : -wy), l.z);
+  }
+}
+
 // Input gradient of the lane's point (Section 5 "Adjoint") from the seed in
 // the tile layout: backward through the hidden layers, then the position,
 // Fourier and latent inputs.  v0 holds the input rows of the forward (its
@@ -592,7 +638,7 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
   {
     float2 g[2][1];
     const int r = og < 3 ? og : 2;
-    back<C, S, 1>(g, x, W0, [&](int) { return r; });
+    back<C, S, 1, 4>(g, x, W0, [&](int) { return r; });
     const float v[4] = {g[0][0].x, g[0][0].y, g[1][0].x, g[1][0].y};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -604,7 +650,7 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
   for (int kb = 0; kb < t.m; kb += 8) {
     const int ka[2] = {min(kb + og, t.m - 1), min(kb + og + 4, t.m - 1)};
     float2 g[2][4];
-    back<C, S, 4>(g, x, W0, [&](int q) { return 3 + 2 * ka[q >> 1] + (q & 1); });
+    back<C, S, 4, 4>(g, x, W0, [&](int q) { return 3 + 2 * ka[q >> 1] + (q & 1); });
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       if (kb + og + 4 * e < t.m) {
@@ -627,7 +673,7 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
   for (int fb = 0; fb < t.F; fb += 16) {
     float2 g[2][4];
     const int f0 = fb + 4 * og;
-    back<C, S, 4>(g, x, W0 + (3 + 2 * t.m) * C, [&](int q) { return min(f0 + q, t.F - 1); });
+    back<C, S, 4, 4>(g, x, W0 + (3 + 2 * t.m) * C, [&](int q) { return min(f0 + q, t.F - 1); });
     if (f0 < t.F) {
 #pragma unroll
       for (int q = 0; q < 4; ++q)
@@ -652,16 +698,16 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
     if (ax == 2) r.z = mine;
   }
   __syncwarp();
-  const Cell cell = net32::make_cell(lat, p);
   const float* z = v0 + (3 + 2 * t.m) * S + lane;
-  for (int f = 0; f < t.F; f += 4) {
-    float4 gx, gy, gz;
-    net32::latent4_grad(lat, cell, f, gx, gy, gz);
-    const float g0 = z[f * S], g1 = z[(f + 1) * S], g2 = z[(f + 2) * S], g3 = z[(f + 3) * S];
-    r.x += g0 * gx.x + g1 * gx.y + g2 * gx.z + g3 * gx.w;
-    r.y += g0 * gy.x + g1 * gy.y + g2 * gy.z + g3 * gy.w;
-    r.z += g0 * gz.x + g1 * gz.y + g2 * gz.z + g3 * gz.w;
+  const Cell cell = net32::make_cell(lat, p);
+  float3 l = make_float3(0.f, 0.f, 0.f);
+  if (t.F == 16) {
+    latent_vjp<S, 16>(l, z, lat, cell, 0);
+  } else {
+    for (int f = 0; f < t.F; f += 4) latent_vjp<S, 4>(l, z + f * S, lat, cell, f);
   }
+  const float scale = (float)(lat.R - 1);
+  r = make_float3(fmaf(scale, l.x, r.x), fmaf(scale, l.y, r.y), fmaf(scale, l.z, r.z));
   __syncwarp();
   return r;
 }
