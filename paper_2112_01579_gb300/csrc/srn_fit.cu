@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kFitThreads, 4) fit_point_kernel(const NetDev 
 // neither sines nor Fourier features are evaluated twice.  Fit step of the
 // main configuration (32^3 x 16, four layers) at 2^18 points: 876 -> 375 us;
 // 65,537 points of the same network through autograd 434 -> 312 us.
-constexpr int kTileStride = 36;  // floats per row: eight rows' 16-byte loads hit distinct banks
+constexpr int kTileStride = 36;  // floats per adjoint row: eight rows' 16-byte loads hit distinct banks
 constexpr int kTileMaxIn = 48;   // inputs of layer 0: 16 threads x 3 entries
 // Points with a residual below this are decided by the accurate functions:
 // inline and library sines move a density by 2e-7 at most on networks of the
@@ -296,12 +296,14 @@ constexpr float kSignBand = 4.0e-6f;
 // + 8 i, r_j = tid / 8 + 16 j (rows past `rows` repeat the last one; their
 // sums are never stored).  d and v are the first warp's rows, `wstride`
 // floats apart per warp.
-template <int NJ>
+// VS: floats per row of v (rows a quarter-warp reads together are one row, so
+// v needs no padding).
+template <int NJ, int VS>
 __device__ __forceinline__ void outer_sum(float (&acc)[4][NJ], const float* d, const float* v, int wstride, int rows) {
   const int og = threadIdx.x & 7, jg = threadIdx.x >> 3;
   int vr[NJ];
 #pragma unroll
-  for (int j = 0; j < NJ; ++j) vr[j] = min(jg + 16 * j, rows - 1) * kTileStride;
+  for (int j = 0; j < NJ; ++j) vr[j] = min(jg + 16 * j, rows - 1) * VS;
 #pragma unroll 1
   for (int w = 0; w < kFitThreads / 32; ++w) {
     const float* dw = d + w * wstride + og * kTileStride;
@@ -311,7 +313,7 @@ __device__ __forceinline__ void outer_sum(float (&acc)[4][NJ], const float* d, c
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < NJ; ++j) s[i][j] = make_float2(0.f, 0.f);
-#pragma unroll 2
+#pragma unroll
     for (int p = 0; p < 32; p += 4) {
       float4 dd[4], vv[NJ];
 #pragma unroll
@@ -358,7 +360,7 @@ template <int F>
 __device__ __forceinline__ void store_dz(const float* d, const float* Wz, float* dz, int j0, int n) {
   const int pg = tile32::point_group(), og = tile32::out_group();
   float2 acc[2][F / 4];
-  tile32::back<32, kTileStride, F / 4>(acc, d, Wz, [&](int f) { return og * (F / 4) + f; });
+  tile32::back<32, kTileStride, F / 4, 4>(acc, d, Wz, [&](int f) { return og * (F / 4) + f; });
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int j = j0 + 4 * pg + i;
@@ -375,6 +377,10 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
                                                                   const __grid_constant__ PointArgs a,
                                                                   const __grid_constant__ tile32::Net t, int wfloats) {
   constexpr int C = 32, S = kTileStride, NH = NL - 1;  // NH activations per point
+  constexpr int VS = 32;  // floats per input row
+  // four layers: the first activation's derivatives wait in shared memory (a
+  // lane's own 32 values), which leaves registers for loads in flight
+  constexpr bool PARK = NL == 4;
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
   tile32::load_net<C>(sm, t, net);
@@ -382,8 +388,9 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* base0 = sm + t.total;                // first warp's rows
   float* v0 = base0 + warp * wfloats;         // layer inputs, then NH blocks of activation rows, then dout
-  float* act0 = v0 + t.d0 * S;
+  float* act0 = v0 + t.d0 * VS;
   float* sdout = act0 + NH * C * S;
+  float4* parked = reinterpret_cast<float4*>(sdout + 4 * S) + lane;
   const int pg = tile32::point_group(), og = tile32::out_group();
   const int step = a.step_ptr ? *a.step_ptr : a.step;
   const Latent lat = make_latent(net, a.time);
@@ -413,15 +420,23 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
     }
     // ---- forward: activations to shared memory, their derivatives kept
     if (valid) {
-      tile32::put_inputs<S, false>(v0, sm, t, lat, nerf, p);
+      tile32::put_inputs<VS>(v0, sm, t, lat, nerf, p);
     } else {
-      for (int k = 0; k < t.d0; ++k) v0[k * S + lane] = 0.f;
+      for (int k = 0; k < t.d0; ++k) v0[k * VS + lane] = 0.f;
     }
     __syncwarp();
     tile32::Acc<C> x, df[NH];
     tile32::set_bias<C>(x, sm + t.ob0);
-    tile32::layer<C, S>(x, v0, sm + t.oW0, t.d0);
+    tile32::layer<C, VS>(x, v0, sm + t.oW0, t.d0);
     tile32::activate_call<C>(mode, x, df[0]);
+    if (PARK) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < C / 8; q += 2)
+          parked[(2 * i + q / 2) * 32] =
+              make_float4(df[0].v[i][q].x, df[0].v[i][q].y, df[0].v[i][q + 1].x, df[0].v[i][q + 1].y);
+    }
     tile32::put<C, S>(x, act0);
     __syncwarp();
 #pragma unroll
@@ -436,12 +451,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
     const float* alast = act0 + (NH - 1) * C * S;
     float dout[4] = {0.f, 0.f, 0.f, 0.f};
     if (a.mode == 0) {
-      float out[4], want[4];
-#pragma unroll
-      for (int dd = 0; dd < 4; ++dd) {
-        out[dd] = dd < D ? tile32::last_layer<C, S>(alast, sm, t, dd) : 0.f;
-        want[dd] = 0.f;
-      }
+      float out[4], want[4] = {0.f, 0.f, 0.f, 0.f};
       if (valid) {
         want[0] = vol_sample(a.vol, p);
         if (D == 4) {
@@ -457,6 +467,8 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
           }
         }
       }
+#pragma unroll
+      for (int dd = 0; dd < 4; ++dd) out[dd] = dd < D ? tile32::last_layer<C, S>(alast, sm, t, dd) : 0.f;
       // the sign of a residual decides a point's whole gradient: a point with
       // one within kSignBand of zero takes its outputs from the accurate
       // functions
@@ -527,11 +539,21 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
 #pragma unroll
     for (int h = NH - 1; h >= 1; --h) {
       const float* dh = act0 + h * C * S;
-      outer_sum<2>(gh[h - 1], base0 + t.d0 * S + h * C * S, base0 + t.d0 * S + (h - 1) * C * S, wfloats, C);
+      outer_sum<2, S>(gh[h - 1], base0 + t.d0 * VS + h * C * S, base0 + t.d0 * VS + (h - 1) * C * S, wfloats, C);
       gb[h] += row_sum(dh + lane * S);
       float2 g[2][C / 4];
       tile32::back<C, S, C / 4>(g, dh, sm + t.oHid + (h - 1) * t.hidStride,
                                 [&](int q) { return og * (C / 4) + q; });
+      if (PARK && h == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int q = 0; q < C / 8; q += 2) {
+            const float4 v = parked[(2 * i + q / 2) * 32];
+            df[0].v[i][q] = make_float2(v.x, v.y);
+            df[0].v[i][q + 1] = make_float2(v.z, v.w);
+          }
+      }
       __syncthreads();  // block h - 1's activations are read
       float* dn = act0 + (h - 1) * C * S + og * (C / 4) * S + 4 * pg;
 #pragma unroll
@@ -543,7 +565,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
       __syncthreads();
     }
     // ---- layer 0, the latent adjoint and the point's cell
-    outer_sum<3>(g0, base0 + t.d0 * S, base0, wfloats, t.d0);
+    outer_sum<3, VS>(g0, base0 + t.d0 * VS, base0, wfloats, t.d0);
     gb[0] += row_sum(act0 + lane * S);
     {
       const float* Wz = sm + t.oW0 + (3 + 2 * t.m) * C;
@@ -613,8 +635,11 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
   }
 }
 
-// Rows of one warp's tile in floats (inputs, activations, output adjoints).
-int fit_tile_floats(const NetDev& net) { return (net_d0(net) + (net.l - 1) * 32 + 4) * kTileStride; }
+// One warp's tile in floats (input rows, activation rows, output adjoints,
+// four layers: parked derivatives).
+int fit_tile_floats(const NetDev& net) {
+  return net_d0(net) * 32 + ((net.l - 1) * 32 + 4) * kTileStride + (net.l == 4 ? 32 * 32 : 0);
+}
 size_t fit_tile_smem(const NetDev& net) {
   return sizeof(float) * ((size_t)tile32::make_net(net).total + (size_t)(kFitThreads / 32) * fit_tile_floats(net));
 }
