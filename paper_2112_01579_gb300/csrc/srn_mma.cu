@@ -1,8 +1,6 @@
 // Dispatch of the FP16 tensor-core render / point evaluation: which network
 // shapes and shading modes have a kernel variant, and which variant runs.
 // The kernel itself is in srn_mma_kernel.cuh.
-#include <string.h>
-
 #include "srn_mma.h"
 
 namespace srn {
@@ -13,11 +11,18 @@ using mma::PointsDev;
 
 namespace {
 
+const BatchDev kNoBatch{};  // of the point modes, which take no batch
+
 template <int C, int M, int F, int ACT>
 cudaError_t dispatch_shading(const NetDev& net, const BatchDev& b, unsigned long long* ctr, unsigned int* st,
                              cudaStream_t s) {
   switch (b.shading) {
-    case SRN_SHADE_NONE: return launch_t<C, M, F, ACT, SRN_SHADE_NONE, 0, 0>(net, b, PointsDev{}, ctr, st, s);
+    case SRN_SHADE_NONE:
+      // a single latent grid: no time blend in the gather (SnakeAlt networks,
+      // the ones rendered unshaded at depths other than four)
+      if constexpr (ACT == SRN_ACT_SNAKEALT && F == 16)
+        if (net.nkey == 1) return launch_t<C, M, F, ACT, SRN_SHADE_NONE, 0, 0, 0, 1>(net, b, PointsDev{}, ctr, st, s);
+      return launch_t<C, M, F, ACT, SRN_SHADE_NONE, 0, 0>(net, b, PointsDev{}, ctr, st, s);
     case SRN_SHADE_FD: return launch_t<C, M, F, ACT, SRN_SHADE_FD, 0, 0>(net, b, PointsDev{}, ctr, st, s);
     case SRN_SHADE_ADJOINT: return launch_t<C, M, F, ACT, SRN_SHADE_ADJOINT, 0, 0>(net, b, PointsDev{}, ctr, st, s);
     default: return launch_t<C, M, F, ACT, SRN_SHADE_HEAD, 0, 0>(net, b, PointsDev{}, ctr, st, s);
@@ -102,9 +107,7 @@ bool eval_mma_supported(const NetDev& n) { return render_mma_supported(n, SRN_SH
 cudaError_t launch_eval_mma(const NetDev& n, const float* pts, long long count, float time, float* out,
                             unsigned long long* ctr, unsigned int* status, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
-  BatchDev b;
-  memset(&b, 0, sizeof(b));
-  b.tf.n = 2;
+  const BatchDev& b = kNoBatch;
   PointsDev pd{pts, out, count, time, nullptr};
   if (n.ti) return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 1, 0>(n, b, pd, ctr, status, s);
   if (n.gq) return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 1>(n, b, pd, ctr, status, s);
@@ -128,12 +131,12 @@ bool density_grad_mma_supported(const NetDev& n) { return render_mma_supported(n
 cudaError_t launch_density_grad_mma(const NetDev& n, const float* pts, long long count, float time, float* rho,
                                     float* grad, unsigned long long* ctr, unsigned int* status, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
-  BatchDev b;
-  memset(&b, 0, sizeof(b));
-  b.tf.n = 2;
+  const BatchDev& b = kNoBatch;
   PointsDev pd{pts, rho, count, time, grad};
   if (n.c == 48) return launch_t<48, 22, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s);
   if (n.c == 64) return launch_t<64, 30, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s);
+  if (n.m == 14 && n.F == 16 && n.act == SRN_ACT_SNAKEALT && n.l == 4 && n.D == 1 && n.nkey == 1)
+    return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0, 4, 1>(n, b, pd, ctr, status, s);
   if (n.m == 14 && n.F == 16)
     return n.act == SRN_ACT_SNAKEALT
                ? launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s)

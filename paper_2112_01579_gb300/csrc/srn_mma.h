@@ -54,6 +54,23 @@ struct PointsDev {
   float* grad;       // kPointsAdj: d rho / d p [n][3], or null
 };
 
+// What the point modes take in place of a batch of frames: the same names
+// without the cameras, times and transfer function, 7 KB of kernel arguments
+// that a call of few points would wait for.
+struct PointsBatch {
+  CamDev cams[1];
+  float times[1];
+  int n_views, n_times, W, H;
+  float step, et, fd_h;
+  struct {
+    int n;
+    float opacity_scale;
+  } tf;
+  float* out;
+  unsigned long long* samples;
+  int stall_test;
+};
+
 // ---------------------------------------------------------------- layout
 struct SmemPlan {
   int oOne, oB0, oBh, oBb, oBhT, oB0T, oWl, oTF, oFm, oQp, oMbar, oMisc, total;

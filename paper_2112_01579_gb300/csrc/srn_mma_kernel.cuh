@@ -44,6 +44,8 @@
 #pragma once
 #include <string.h>
 
+#include <type_traits>
+
 #include "srn_device.cuh"
 #include "srn_mma.h"
 
@@ -542,7 +544,7 @@ __device__ __forceinline__ float3 latent_grad_h(const __half* __restrict__ G, in
 
 template <int C, int M, int F, int ACT, int SH, int TI, int GQ, int LF, int ST>
 __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
-    render_mma_kernel(const NetDev net, const BatchDev b, const PointsDev pd, const SmemPlan plan,
+    render_mma_kernel(const NetDev net, const std::conditional_t<is_points(SH), PointsBatch, BatchDev> b, const PointsDev pd, const SmemPlan plan,
                       unsigned long long* __restrict__ ray_counter, unsigned int* __restrict__ status) {
   constexpr int WGS = wgs_for(C, SH), THREADS = 128 * WGS;
   constexpr int D0 = 3 + 2 * M + F + TI;
@@ -713,7 +715,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
       for (int i = tid; i < 2 * F; i += THREADS)  // [lo + 128 step, step] per channel (latent_q)
         qp[i] = ldexpf((i & 1) ? net.grid_qp[i] : fmaf(128.0f, net.grid_qp[i + 1], net.grid_qp[i]), -gexp);
   }
-  load_tf_segments(tf, b.tf);
+  if constexpr (!POINTS) load_tf_segments(tf, b.tf);
   // the constant tile has ones in columns 0 and 1 of every row (the bias MMA
   // of the hidden layers)
   if (wg == 0) {
@@ -782,17 +784,31 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
     rl.tin = pd.time;
   }
 
+  // Points are taken by the warp's place in the grid, then a grid stride on,
+  // without round trips to the counter (1000 points 16.5 -> 12.3 us).  Rays go
+  // by the counter: they differ in length, and the choice at run time costs
+  // the march 2 % (registers).
+  uint32_t place = 32u * (blockIdx.x + gridDim.x * (unsigned)(tid >> 5));
   while (true) {
     // ---- refill: a warp whose lanes are all done claims the next 32 rays
     // (one 8 x 4 pixel tile), so its lanes march neighbouring rays together
     while (true) {
-      const bool need = !__any_sync(0xffffffffu, active) && !exhausted && !failed;
+      bool need = !__any_sync(0xffffffffu, active) && !exhausted && !failed;
+      if (POINTS && (long long)place >= n_rays) {
+        exhausted = exhausted || need;
+        need = false;
+      }
       const unsigned int mask = __ballot_sync(0xffffffffu, need);
       if (mask == 0) break;
       unsigned long long base = 0;
-      const int leader = __ffs(mask) - 1;
-      if (lane == leader) base = atomicAdd(ray_counter, (unsigned long long)__popc(mask));
-      base = __shfl_sync(0xffffffffu, base, leader);
+      if constexpr (POINTS) {
+        base = place;
+        place += gridDim.x * THREADS;
+      } else {
+        const int leader = __ffs(mask) - 1;
+        if (lane == leader) base = atomicAdd(ray_counter, (unsigned long long)__popc(mask));
+        base = __shfl_sync(0xffffffffu, base, leader);
+      }
       if (need) {
         const long long r = (long long)base + __popc(mask & ((1u << lane) - 1u));
         if (r >= n_rays) {
@@ -996,12 +1012,15 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
 #pragma unroll
           for (int j = 0; j < C; ++j) dl[j] = g[j] * dv[j];
         } else {
-          float gv[K0];
-          tmem_ld_row<K0>(t_row, gv);
+          // in two parts, so that half the registers hold it at a time: the
+          // Fourier and position columns with what shares their last 16, then
+          // the rest of the latent columns
+          constexpr int P1 = (2 * M + 3 + 15) / 16 * 16, P2 = (2 * M + 3 + F - P1 + 15) / 16 * 16;
+          float gv[P1], gl[F];
+          tmem_ld_row<P1>(t_row, gv);
+          float3 gp = make_float3(gv[2 * M], gv[2 * M + 1], gv[2 * M + 2]);
           if (active) {
-            // position columns, then the Fourier features (d sin e = cos e F_k,
-            // d cos e = -sin e F_k), then the latent vector
-            float3 gp = make_float3(gv[2 * M], gv[2 * M + 1], gv[2 * M + 2]);
+            // the Fourier features: d sin e = cos e F_k, d cos e = -sin e F_k
             if (nerf) {
               constexpr int kReseed = M > 15 ? 4 : 64;
               constexpr float kW = 6.28318548202514648f, kWErr = 1.74845560252379070e-7f;
@@ -1037,9 +1056,19 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
                 gp.z = fmaf(coef, fm[3 * kq + 2], gp.z);
               }
             }
-            float3 gl = latent_grad_h<F, ST>(net.grid_h, net.R, rl, qs, gv + 2 * M + 3);
-            gl = make_float3(gl.x * gscale, gl.y * gscale, gl.z * gscale);  // grid_h = G 2^-gexp
-            gadj = make_float3(gp.x + gl.x, gp.y + gl.y, gp.z + gl.z);
+          }
+#pragma unroll
+          for (int c = 0; c < F; ++c)
+            if (2 * M + 3 + c < P1) gl[c] = gv[2 * M + 3 + c];
+          float g2[P2];
+          tmem_ld_row<P2>(t_row + P1, g2);
+#pragma unroll
+          for (int c = 0; c < F; ++c)
+            if (2 * M + 3 + c >= P1) gl[c] = g2[2 * M + 3 + c - P1];
+          if (active) {
+            const float3 l = latent_grad_h<F, ST>(net.grid_h, net.R, rl, qs, gl);
+            // grid_h = G 2^-gexp
+            gadj = make_float3(fmaf(l.x, gscale, gp.x), fmaf(l.y, gscale, gp.y), fmaf(l.z, gscale, gp.z));
           }
         }
       }
@@ -1146,7 +1175,9 @@ cudaError_t launch_t(const NetDev& net, const BatchDev& b, const PointsDev& pd, 
   // a warp claims 32 at a time
   const long long claims = is_points(SH) ? (pd.n + 31) / 32
                                          : (long long)((b.W + 7) / 8) * ((b.H + 3) / 4) * b.n_views * b.n_times;
-  k<<<(unsigned)(claims < sms ? claims : sms), 128 * wgs_for(C, SH), plan.total, s>>>(net, b, pd, plan, ctr, status);
+  const unsigned grid = (unsigned)(claims < sms ? claims : sms);
+  if constexpr (is_points(SH)) k<<<grid, 128 * wgs_for(C, SH), plan.total, s>>>(net, PointsBatch{}, pd, plan, ctr, status);
+  else k<<<grid, 128 * wgs_for(C, SH), plan.total, s>>>(net, b, pd, plan, ctr, status);
   return cudaGetLastError();
 }
 
