@@ -115,14 +115,23 @@ def _check(st):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_current = None
 
 
 def _stream(stream):
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    """The cudaStream_t of ``stream``, or of torch's current stream: the raw
+    handle, without a Stream object (0.4 us a call instead of 3.4)."""
+    global _current
+    if stream is not None:
+        return stream.cuda_stream
+    if _current is None:
+        import torch
+        torch.cuda.current_stream()  # initialises CUDA
+        _current = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+    return _current[0](_current[1]())
 
 
 def _cams(cams):
