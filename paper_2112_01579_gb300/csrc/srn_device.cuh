@@ -5,6 +5,16 @@
 
 namespace srn {
 
+// 32 bytes (address a multiple of 32) through the read-only path in one load.
+// A gather whose lanes hit different lines takes one L1 wavefront per lane and
+// load, so rows of 32 bytes or more cost half of what 16-byte loads do.
+__device__ __forceinline__ void ldg32(const void* p, uint4& a, uint4& b) {
+  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+      : "l"(p));
+}
+__device__ __forceinline__ bool aligned32(const void* p) { return ((unsigned long long)p & 31ull) == 0; }
+
 __device__ __forceinline__ float clamp01f(float x) { return fminf(fmaxf(x, 0.0f), 1.0f); }
 
 // Pinhole ray through the centre of pixel (px, py) in FP32 from the camera

@@ -257,7 +257,11 @@ struct RayLat {
 // relative) moves z_c by at most 2^-11 sum_k w_k |G_kc|, about as much as the
 // FP16 rounding of z itself for the A tile.
 // ST: one latent grid (no keyframes), known at compile time: no time blend.
-template <int F, int ST>
+// WIDE: 32-byte loads (grid rows of 32 bytes, aligned), for points that do not
+// share cells: a warp's lanes then hit 32 lines whatever the load's width, and
+// the L1 takes a wavefront per line and load (2^20 random points 70.0 -> 61.6
+// us; rays of one tile share cells, where the width makes no difference).
+template <int F, int ST, bool WIDE = false>
 __device__ __forceinline__ void latent_h(const __half* __restrict__ G, int R, const RayLat& rl, float3 p,
                                          float (&z)[F]) {
   int ix, iy, iz;
@@ -280,9 +284,11 @@ __device__ __forceinline__ void latent_h(const __half* __restrict__ G, int R, co
       if (!ST && kk && g < 0) break;
       const __half wh = __float2half_rn(ST ? w : w * (kk ? rl.w1 : rl.w0));
       const uint16_t wb = *reinterpret_cast<const uint16_t*>(&wh);
+      uint4 wide[2];
+      if constexpr (WIDE) ldg32(G + g + off, wide[0], wide[1]);
 #pragma unroll
       for (int c = 0; c < F; c += 8) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4*>(G + g + off + c));
+        const uint4 q = WIDE ? wide[(c / 8) & 1] : __ldg(reinterpret_cast<const uint4*>(G + g + off + c));
         const uint32_t qq[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -365,16 +371,22 @@ __device__ __forceinline__ void latent_q(const uint8_t* __restrict__ Q, const fl
 // reads.  Values are packed to FP16 pairs
 // and stored to the thread's TMEM row 16 at a time as they are produced; the
 // whole warp takes part (tcgen05.st is warp-collective), lanes without a
-// sample write a row nothing reads.
-template <int M, int F, int K0, int TI, int GQ, int ST>
+// sample write a row nothing reads.  SCATTERED: points of no common cell.
+template <int M, int F, int K0, int TI, int GQ, int ST, bool SCATTERED>
 __device__ __forceinline__ void write_input_row(uint32_t t_a, float3 p, bool nerf, const float* fm,
                                                 const __half* G, const uint8_t* Q, const float* qp, int R,
                                                 const RayLat& rl) {
   constexpr int D0 = 3 + 2 * M + F + TI;
   static_assert(M >= 3, "the NeRF recurrence needs the three base rows");
   float z[F];
-  if constexpr (GQ != 0) latent_q<F, ST>(Q, qp, R, rl, p, z);
-  else latent_h<F, ST>(G, R, rl, p, z);
+  if constexpr (GQ != 0) {
+    latent_q<F, ST>(Q, qp, R, rl, p, z);
+  } else if constexpr (SCATTERED && F == 16) {
+    if (aligned32(G)) latent_h<F, ST, true>(G, R, rl, p, z);
+    else latent_h<F, ST>(G, R, rl, p, z);
+  } else {
+    latent_h<F, ST>(G, R, rl, p, z);
+  }
   uint32_t w[8];
   int nw = 0, col = 0;
   auto emit = [&](float a, float b) {
@@ -870,7 +882,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
       qs = q;
     }
     if (__any_sync(0xffffffffu, active && !failed)) {
-      write_input_row<M, F, K0, TI, GQ, ST>(t_a, qs, nerf, fm, net.grid_h, net.grid_q, qp, net.R, rl);
+      write_input_row<M, F, K0, TI, GQ, ST, POINTS>(t_a, qs, nerf, fm, net.grid_h, net.grid_q, qp, net.R, rl);
       tmem_wait_st();
     }
     tc_fence_before();

@@ -42,3 +42,54 @@ def test_grid_gradient(S, R, F, n, crowd):
     again = torch.empty_like(g)
     S.srn_backward(net.ctx, torch.tensor(pts, device="cuda"), torch.tensor(dout, device="cuda"), again, w, b)
     assert torch.equal(g, again)  # fixed orders: the same bits on every run
+
+
+def _shifted(t):
+    """A copy of t that starts 16 bytes behind a 512-byte boundary."""
+    import torch
+    k = 16 // t.element_size()
+    v = torch.empty(t.numel() + k, dtype=t.dtype, device=t.device)[k:]
+    v.copy_(t.reshape(-1))
+    assert v.data_ptr() % 32 == 16
+    return v
+
+
+@pytest.mark.parametrize("F,m,layers,act,keys", [(8, 12, 2, synth.ACT_SINE, 1), (16, 14, 2, synth.ACT_SNAKEALT, 1),
+                                                 (16, 14, 4, synth.ACT_SNAKEALT, 1), (16, 14, 4, synth.ACT_SNAKEALT, 3),
+                                                 (32, 6, 3, synth.ACT_SNAKEALT, 1), (4, 6, 3, synth.ACT_SINE, 1)])
+def test_grids_off_a_32_byte_boundary(S, F, m, layers, act, keys):
+    """Grids are 16-byte aligned by contract; those that are not 32-byte
+    aligned take narrower gathers and give the same bits."""
+    import torch
+    p = synth.random_params(R=6, F=F, m=m, layers=layers, width=32, act=act, seed=F + layers, grid_std=0.5, n_keyframes=keys)
+    rng = np.random.default_rng(8)
+    pts = torch.tensor(rng.random((400, 3), dtype=np.float32), device="cuda")
+    dout = torch.tensor(rng.standard_normal((400, 1), dtype=np.float32), device="cuda")
+    vol = torch.tensor(rng.random((9, 8, 7), dtype=np.float32), device="cuda")
+    t = 0.5 if keys > 1 else 0.0
+    got = []
+    for shift in (False, True):
+        net = S.Network(p, max_fit_points=400, adam=True)
+        grid = _shifted(net.grid) if shift else net.grid
+        prm = net._params()
+        prm.grid = grid.data_ptr()
+        S.srn_set_params(net.ctx, prm)
+        out, grad, err, loss = (torch.zeros(n, device="cuda") for n in (400, 1200, 125, 1))
+        S.srn_density_grad(net.ctx, pts, out, grad, time=t)
+        vjp, dg, dw, db = torch.empty_like(grad), torch.empty_like(net.grid), torch.empty_like(net.weights), torch.empty_like(net.biases)
+        S.srn_input_backward(net.ctx, pts, dout, vjp, time=t)
+        S.srn_backward(net.ctx, pts, dout, dg, dw, db, time=t)
+        S.srn_error_grid(net.ctx, vol, 5, 2, 3, err, time=t)
+        S.srn_fit_step(net.ctx, vol, 400, 5, 0, loss, time=t)
+        half = S.Network(p, precision=S.SRN_PREC_FP16) if (F, m) in ((8, 12), (16, 14)) else None
+        rho = torch.zeros((400, 1), device="cuda")
+        if half is not None:
+            prm = half._params()
+            grid_h = _shifted(half.grid_h) if shift else half.grid_h
+            prm.grid_h = grid_h.data_ptr()
+            S.srn_set_params(half.ctx, prm)
+            S.srn_eval(half.ctx, pts, rho, time=t)
+        torch.cuda.synchronize()
+        got.append([x.clone() for x in (out, grad, vjp, dg, dw, db, err, loss, grid, net.weights, net.biases, rho)])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
