@@ -26,9 +26,9 @@
 //   (C -> D) runs on the CUDA cores in FP32.
 // * SnakeAlt(x) = 0.5 x + sin^2 x = (x - cos 2x + 1) / 2 (Eq. 3).  Every MMA
 //   layer is staged to produce u = 2x (weights and bias doubled, which is
-//   exact in FP16), the epilogue hands a = u / 2 - cos u = 2 SnakeAlt(x) - 1
-//   to the next layer, and the factor 1/2 and the shift 1/2 are folded into
-//   that layer's weights and bias: the doubled next layer then simply uses W
+//   exact in FP16), the epilogue hands cos u - u / 2 = 1 - 2 SnakeAlt(x)
+//   to the next layer, and the factor -1/2 and the shift 1/2 are folded into
+//   that layer's weights and bias: the doubled next layer then simply uses -W
 //   and 2b + sum_j W_j.
 // * Rays are claimed dynamically from a work counter, a warp at a time: when
 //   every lane's ray has terminated (box exit or opacity >= threshold), the
@@ -212,12 +212,15 @@ __device__ __forceinline__ void split_h2(float a0, float a1, uint32_t& hi, uint3
   lo = pack_h2(r0, r1);
 }
 
-// Activation value handed to the next layer from the accumulator value: sin(x)
-// for the sine network; for SnakeAlt the accumulator holds u = 2x and the
-// value is u / 2 - cos u = 2 SnakeAlt(x) - 1.
-template <int ACT>
-__device__ __forceinline__ float act_fold(float acc) {
-  return ACT == SRN_ACT_SNAKEALT ? fmaf(0.5f, acc, -__cosf(acc)) : __sinf(acc);
+// Activation values handed to the next layer from two accumulator values:
+// sin(x) for the sine network; for SnakeAlt the accumulator holds u = 2x and
+// the value is cos u - u / 2 = 1 - 2 SnakeAlt(x) (the next layer's weights
+// carry the minus sign; with PACK one packed FMA does two).
+template <int ACT, bool PACK>
+__device__ __forceinline__ float2 act_fold(float x, float y) {
+  if (ACT != SRN_ACT_SNAKEALT) return make_float2(__sinf(x), __sinf(y));
+  if (PACK) return __ffma2_rn(make_float2(x, y), make_float2(-0.5f, -0.5f), make_float2(__cosf(x), __cosf(y)));
+  return make_float2(fmaf(-0.5f, x, __cosf(x)), fmaf(-0.5f, y, __cosf(y)));
 }
 
 // Byte offset of 16-byte chunk cg (= column / 8) of row r in a tile of
@@ -600,6 +603,13 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   // loop has its exact trip count); the dispatch picks such an instantiation
   // only for such a network
   constexpr int DF = SH == SRN_SHADE_HEAD ? 4 : 1;
+  // The activations and the last layer in packed FMAs (two channels each)
+  // where that was faster: the single-grid width-32 march without shading or
+  // with the adjoint gradient (main configuration, 1024^2: 8.61 -> 8.36 ms;
+  // 512^2 shaded: 13.66 -> 13.32 ms).  Elsewhere the register pairs cost as
+  // much as they save or more: keyframes 6.30 -> 6.38 ms, width 48 2.89 ->
+  // 2.91, gradient head 3.98 -> 4.04, points with gradient 166 -> 169 us.
+  constexpr bool PACK = ST == 1 && C == 32 && (SH == SRN_SHADE_NONE || SH == SRN_SHADE_ADJOINT);
   const int L = LF > 0 ? LF : net.l;
   const int D = LF > 0 ? DF : net.D;
   // the FP16 latent grid holds G 2^-gexp: the latent columns' layer-0 weights
@@ -648,7 +658,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
             v = col == D0 ? bh : __float2half_rn(bias - __half2float(bh));
           }
         } else {
-          v = __float2half_rn(scale * __half2float(Wsrc[col % C]));
+          v = __float2half_rn((SNAKE ? -1.0f : 1.0f) * __half2float(Wsrc[col % C]));  // see act_fold
         }
         h2[q] = v;
       }
@@ -712,7 +722,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   {
     // last layer on the CUDA cores: folded like the hidden layers
     const __half* Wl = net.W_h + (size_t)C * D0 + (size_t)(L - 2) * C * C;
-    for (int i = tid; i < D * C; i += THREADS) wl[i] = (SNAKE ? 0.5f : 1.0f) * __half2float(Wl[i]);
+    for (int i = tid; i < D * C; i += THREADS) wl[i] = (SNAKE ? -0.5f : 1.0f) * __half2float(Wl[i]);
     if (tid < D) {
       float bias = net.b[(L - 1) * C + tid];
       if (SNAKE) {
@@ -923,7 +933,8 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
             uint32_t hi[8], lo[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              split_h2(act_fold<ACT>(x[16 * j + 2 * e]), act_fold<ACT>(x[16 * j + 2 * e + 1]), hi[e], lo[e]);
+              const float2 a = act_fold<ACT, PACK>(x[16 * j + 2 * e], x[16 * j + 2 * e + 1]);
+              split_h2(a.x, a.y, hi[e], lo[e]);
             }
             tmem_st8(t_a + 8 * j, hi);
             tmem_st8(t_a + C / 2 + 8 * j, lo);
@@ -934,7 +945,12 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
             // backward: SnakeAlt' = 0.5 + sin(2x) (the accumulator holds 2x); sin' = cos
             float dv[C];
 #pragma unroll
-            for (int j = 0; j < C; ++j) dv[j] = SNAKE ? 0.5f + __sinf(x[j]) : __cosf(x[j]);
+            for (int j = 0; j < C; j += 2) {
+              const float2 p = SNAKE ? __fadd2_rn(make_float2(0.5f, 0.5f), make_float2(__sinf(x[j]), __sinf(x[j + 1])))
+                                     : make_float2(__cosf(x[j]), __cosf(x[j + 1]));
+              dv[j] = p.x;
+              dv[j + 1] = p.y;
+            }
             tmem_st_row<C>(t_row + NACC + C * layer, dv);
           }
         }
@@ -954,22 +970,33 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
           mma_commit(mb);
         }
       } else if (!failed) {
-        float a[C];
+        float2 a[C / 2];
 #pragma unroll
-        for (int j = 0; j < C; ++j) a[j] = act_fold<ACT>(x[j]);
+        for (int j = 0; j < C / 2; ++j) a[j] = act_fold<ACT, PACK>(x[2 * j], x[2 * j + 1]);
 #pragma unroll
         for (int dd = 0; dd < 4; ++dd) {
           if (dd < D) {
-            float sacc = wl[D * C + dd];
+            if constexpr (PACK) {  // two sums per output
+              float2 sacc = make_float2(wl[D * C + dd], 0.0f);
 #pragma unroll
-            for (int j = 0; j < C; ++j) sacc = fmaf(wl[dd * C + j], a[j], sacc);
-            out[dd] = sacc;
+              for (int j = 0; j < C / 2; j += 2) {
+                const float4 w = *reinterpret_cast<const float4*>(wl + dd * C + 2 * j);
+                sacc = __ffma2_rn(make_float2(w.x, w.y), a[j], sacc);
+                sacc = __ffma2_rn(make_float2(w.z, w.w), a[j + 1], sacc);
+              }
+              out[dd] = sacc.x + sacc.y;
+            } else {
+              float sacc = wl[D * C + dd];
+#pragma unroll
+              for (int j = 0; j < C / 2; ++j) sacc = fmaf(wl[dd * C + 2 * j + 1], a[j].y, fmaf(wl[dd * C + 2 * j], a[j].x, sacc));
+              out[dd] = sacc;
+            }
           }
         }
         if constexpr (ADJ) {
-          // d out / d x of the last hidden layer; wl holds W / 2 for SnakeAlt
+          // d out / d x of the last hidden layer; wl holds -W / 2 for SnakeAlt
 #pragma unroll
-          for (int j = 0; j < C; ++j) dl[j] = SNAKE ? wl[j] * fmaf(2.0f, __sinf(x[j]), 1.0f) : wl[j] * __cosf(x[j]);
+          for (int j = 0; j < C; ++j) dl[j] = SNAKE ? -wl[j] * fmaf(2.0f, __sinf(x[j]), 1.0f) : wl[j] * __cosf(x[j]);
         }
       }
     }
@@ -1018,11 +1045,16 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
         tc_fence_after();
         if (failed) continue;
         if (h >= 1) {
+          // packed here and where dv is made: 512^2 shaded 13.32 -> 12.93 ms
           float g[C], dv[C];
           tmem_ld_row<C>(t_row, g);
           tmem_ld_row<C>(t_row + NACC + C * (h - 1), dv);
 #pragma unroll
-          for (int j = 0; j < C; ++j) dl[j] = g[j] * dv[j];
+          for (int j = 0; j < C; j += 2) {
+            const float2 p = __fmul2_rn(make_float2(g[j], g[j + 1]), make_float2(dv[j], dv[j + 1]));
+            dl[j] = p.x;
+            dl[j + 1] = p.y;
+          }
         } else {
           // in two parts, so that half the registers hold it at a time: the
           // Fourier and position columns with what shares their last 16, then
