@@ -4,9 +4,11 @@
 // Design (GB300-first restatement of the fused TensorCore network of
 // Section 4.1):
 // * A CTA holds 7 (6 with finite-difference shading), 4 or 3 warpgroups for
-//   hidden width 32, 48 or 64 (what shared memory and registers allow).  Each
-//   warpgroup owns a tile of 128 rays, one per thread; thread i of the warpgroup is row i of the MMA operand A and
-//   TMEM lane i of the accumulator, so the per-ray work (ray stepping,
+//   hidden width 32, 48 or 64 (what registers allow: 72, 128 and 168 a
+//   thread; one more warpgroup at widths 48 and 64 spills and is 3 % slower).
+//   Each warpgroup owns a tile of 128 rays, one per thread; thread i of the
+//   warpgroup is row i of the MMA operand A and TMEM lane i of the
+//   accumulator, so the per-ray work (ray stepping,
 //   latent-grid trilinear fetch, Fourier features, transfer function,
 //   compositing, early termination) stays one thread per ray as in the paper,
 //   while the layers run as M=128 x N=C tensor-core MMAs.
@@ -36,7 +38,7 @@
 //   rays in step, so their latent-grid gathers mostly hit the same cells and
 //   the L1 serves a warp's loads in few wavefronts (per-lane refill, which
 //   keeps every lane busy but scatters the lanes over the volume, was 10 %
-//   slower on the config-2 frame).
+//   slower on the main configuration's frame).
 // * Every mbarrier wait is bounded; on timeout the warpgroup stops, records
 //   SRN_ERR_TIMEOUT in the status word and the CTA frees its TMEM.
 // * A non-finite network output (an input or activation beyond the FP16
@@ -605,11 +607,17 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   constexpr int DF = SH == SRN_SHADE_HEAD ? 4 : 1;
   // The activations and the last layer in packed FMAs (two channels each)
   // where that was faster: the single-grid width-32 march without shading or
-  // with the adjoint gradient (main configuration, 1024^2: 8.61 -> 8.36 ms;
-  // 512^2 shaded: 13.66 -> 13.32 ms).  Elsewhere the register pairs cost as
-  // much as they save or more: keyframes 6.30 -> 6.38 ms, width 48 2.89 ->
-  // 2.91, gradient head 3.98 -> 4.04, points with gradient 166 -> 169 us.
+  // with the adjoint gradient (main configuration, 1024^2: 8.61 -> 8.37 ms;
+  // 512^2 shaded, with the packed products of the backward below: 13.68 ->
+  // 12.94 ms).  Elsewhere the register pairs cost as much as they save or
+  // more: keyframes 6.30 -> 6.38 ms, width 48 2.89 -> 2.91.
   constexpr bool PACK = ST == 1 && C == 32 && (SH == SRN_SHADE_NONE || SH == SRN_SHADE_ADJOINT);
+  // The last layer as a sum over the even and one over the odd channels with
+  // 16-byte weight loads, the same at width 32 with and without PACK (every
+  // march of a network gives the same bits); keyframes 6.30 -> 6.25 ms.  One
+  // sum at widths 48 and 64 (the other form: 2.89 -> 2.93 ms) and for points
+  // with gradient (166 -> 170 us for 2^20).
+  constexpr bool SUM2 = C == 32 && SH != kPointsAdj;
   const int L = LF > 0 ? LF : net.l;
   const int D = LF > 0 ? DF : net.D;
   // the FP16 latent grid holds G 2^-gexp: the latent columns' layer-0 weights
@@ -976,19 +984,24 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
 #pragma unroll
         for (int dd = 0; dd < 4; ++dd) {
           if (dd < D) {
-            if constexpr (PACK) {  // two sums per output
+            if constexpr (SUM2) {
               float2 sacc = make_float2(wl[D * C + dd], 0.0f);
 #pragma unroll
               for (int j = 0; j < C / 2; j += 2) {
                 const float4 w = *reinterpret_cast<const float4*>(wl + dd * C + 2 * j);
-                sacc = __ffma2_rn(make_float2(w.x, w.y), a[j], sacc);
-                sacc = __ffma2_rn(make_float2(w.z, w.w), a[j + 1], sacc);
+                if (PACK) {
+                  sacc = __ffma2_rn(make_float2(w.x, w.y), a[j], sacc);
+                  sacc = __ffma2_rn(make_float2(w.z, w.w), a[j + 1], sacc);
+                } else {
+                  sacc = make_float2(fmaf(w.x, a[j].x, sacc.x), fmaf(w.y, a[j].y, sacc.y));
+                  sacc = make_float2(fmaf(w.z, a[j + 1].x, sacc.x), fmaf(w.w, a[j + 1].y, sacc.y));
+                }
               }
               out[dd] = sacc.x + sacc.y;
             } else {
               float sacc = wl[D * C + dd];
 #pragma unroll
-              for (int j = 0; j < C / 2; ++j) sacc = fmaf(wl[dd * C + 2 * j + 1], a[j].y, fmaf(wl[dd * C + 2 * j], a[j].x, sacc));
+              for (int j = 0; j < C; ++j) sacc = fmaf(wl[dd * C + j], (j & 1) ? a[j / 2].y : a[j / 2].x, sacc);
               out[dd] = sacc;
             }
           }
@@ -1045,7 +1058,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
         tc_fence_after();
         if (failed) continue;
         if (h >= 1) {
-          // packed here and where dv is made: 512^2 shaded 13.32 -> 12.93 ms
+          // packed here and where dv is made: 512^2 shaded 13.3 -> 12.9 ms
           float g[C], dv[C];
           tmem_ld_row<C>(t_row, g);
           tmem_ld_row<C>(t_row + NACC + C * (h - 1), dv);
