@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kFitThreads, 4) fit_point_kernel(const NetDev 
     if (valid) {
       if (a.mode == 0) p = sample::fit_point(a.cdf, a.cdf_res, a.seed, step, j, a.n);
       else p = clamp_p(make_float3(a.pts_in[3 * j], a.pts_in[3 * j + 1], a.pts_in[3 * j + 2]));
-      forward<C, true>(sm, L, net.act, lat, p, out, hs);
+      forward<C>(sm, L, net.act, lat, p, out, hs);
       if (a.mode == 0) {
         const float r = out[0] - vol_sample(a.vol, p);
         loss_acc += fabsf(r);
@@ -282,8 +282,9 @@ __global__ void __launch_bounds__(kFitThreads, 4) fit_point_kernel(const NetDev 
 // layer's adjoint rows take the place of its activations once the gradient
 // that needs them is done), the activation derivatives in registers, so
 // neither sines nor Fourier features are evaluated twice.  Fit step of the
-// main configuration (32^3 x 16, four layers) at 2^18 points: 876 -> 375 us;
-// 65,537 points of the same network through autograd 434 -> 312 us.
+// main configuration (32^3 x 16, four layers) at 2^18 points: 876 -> 302 us
+// (with the sort and gather below); 65,537 points of the same network through
+// autograd 434 -> 261 us.
 constexpr int kTileStride = 36;  // floats per adjoint row: eight rows' 16-byte loads hit distinct banks
 constexpr int kTileMaxIn = 48;   // inputs of layer 0: 16 threads x 3 entries
 // Points with a residual below this are decided by the accurate functions:
@@ -1458,7 +1459,7 @@ cudaError_t run_backward(FitScratch& s, const NetDev& net, PointArgs pa, float* 
                          float* loss, cudaStream_t st, unsigned int* mma_status = nullptr) {
   const int n = pa.n;
   const int nW = (int)(net_weight_count(net)), nb = (int)net_bias_count(net);
-  Layout L = make_layout(net, true);
+  Layout L = make_layout(net);
   // odd row stride: per-thread rows written at the same column hit distinct banks
   const int dstride = ((net_d0(net) > net.c ? net_d0(net) : net.c) + 1) | 1;
   pa.dstride = dstride;

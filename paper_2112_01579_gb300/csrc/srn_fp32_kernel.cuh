@@ -8,6 +8,7 @@
 // no intermediate state touches global memory (the fused-network idea of
 // Section 4).
 #pragma once
+#include "srn_df.cuh"
 #include "srn_fp32.h"
 #include "srn_tile32.cuh"
 

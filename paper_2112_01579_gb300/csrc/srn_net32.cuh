@@ -1,11 +1,10 @@
-// FP32 network device code shared by the render / eval kernels and the fit
-// kernels: shared-memory staging of the parameters, the forward pass
-// (Section 3 layer equation, Eq. 1-2 Fourier features, Section 4.2 latent
-// grid) and the adjoint input gradient (Section 5 "Adjoint").
+// FP32 network device code, one thread per point: the latent gather (Section
+// 4.2) and the Fourier features (Eq. 1-2) that all FP32 kernels share, and the
+// shared-memory staging and forward pass (Section 3 layer equation) of the fit
+// point kernel for networks the tiled kernel does not take.
 #pragma once
 
 #include "srn_device.cuh"
-#include "srn_df.cuh"
 
 namespace srn {
 namespace net32 {
@@ -16,19 +15,17 @@ constexpr int kMaxL = 8;  // deepest network the FP32 kernels stash for the adjo
 struct Layout {
   int d0, l, D, m, F, ti;
   int oF, oW0T, ob0, oHid, hidStride, oWl, obl, total;
-  int rowmajor;
 };
 
-inline Layout make_layout(const NetDev& n, bool rowmajor) {
+inline Layout make_layout(const NetDev& n) {
   Layout L;
   const int C = n.c;
   L.d0 = net_d0(n); L.l = n.l; L.D = n.D; L.m = n.m; L.F = n.F; L.ti = n.ti;
-  L.rowmajor = rowmajor ? 1 : 0;
   int o = 0;
   L.oF = o; o += ((3 * n.m + 3) / 4) * 4;
   L.oW0T = o; o += L.d0 * C;
   L.ob0 = o; o += C;
-  L.oHid = o; L.hidStride = C * C + C + (rowmajor ? C * C : 0);
+  L.oHid = o; L.hidStride = 2 * C * C + C;
   o += (n.l - 2) * L.hidStride;
   L.oWl = o; o += n.D * C;
   L.obl = o; o += 4;
@@ -56,7 +53,7 @@ __device__ void load_net(float* sm, const Layout& L, const NetDev& n) {
     for (int i = tid; i < C * C; i += nt) {
       int o = i / C, j = i - o * C;
       base[j * C + o] = W[i];
-      if (L.rowmajor) base[C * C + C + i] = W[i];
+      base[C * C + C + i] = W[i];
     }
     for (int i = tid; i < C; i += nt) base[C * C + i] = bb[i];
     W += C * C;
@@ -98,7 +95,7 @@ __device__ __forceinline__ float dotrow(const float* __restrict__ row, const flo
   return (s0 + s1) + (s2 + s3);
 }
 
-// Eq. 3 SnakeAlt(x) = 0.5 x + sin^2 x, or sin(x); and their derivatives.
+// Eq. 3 SnakeAlt(x) = 0.5 x + sin^2 x, or sin(x); and the derivatives.
 // Out-of-line sin / cos: the accurate functions carry a large argument-
 // reduction path, and inlined once per hidden unit of the unrolled layers
 // they overflow the instruction cache (the fit kernel stalled mostly on
@@ -122,15 +119,6 @@ __device__ __forceinline__ void act_and_df(int act, float x, float& a, float& d)
     d = c;
   }
 }
-__device__ __forceinline__ float act_df(int act, float x) {
-  if (act == SRN_ACT_SNAKEALT) {
-    float s, c;
-    sincosf(x, &s, &c);
-    return 0.5f + 2.0f * s * c;
-  }
-  return cosf(x);
-}
-
 // Latent grid source of one frame: z = tw0 G_k0(p) + tw1 G_k0+1(p).
 struct Latent {
   const float* g0;
@@ -194,30 +182,6 @@ __device__ __forceinline__ float4 latent4(const Latent& lat, const Cell& c, int 
   return z;
 }
 
-// Gradient w.r.t. p of channels f..f+3 of the latent vector; gx/gy/gz hold
-// d z_{f+i} / d p_x etc.
-__device__ __forceinline__ void latent4_grad(const Latent& lat, const Cell& c, int f, float4& gx, float4& gy,
-                                             float4& gz) {
-  gx = gy = gz = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float s = (float)(lat.R - 1);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
-    float wx = dx ? c.fx : 1.0f - c.fx, wy = dy ? c.fy : 1.0f - c.fy, wz = dz ? c.fz : 1.0f - c.fz;
-    float ax = (dx ? s : -s) * wy * wz, ay = wx * (dy ? s : -s) * wz, az = wx * wy * (dz ? s : -s);
-    int off = c.base + dx * c.sx + dy * c.sy + dz * c.sz + f;
-    float4 g = __ldg(reinterpret_cast<const float4*>(lat.g0 + off));
-    if (lat.g1) {
-      float4 h = __ldg(reinterpret_cast<const float4*>(lat.g1 + off));
-      g = make_float4(lat.tw0 * g.x + lat.tw1 * h.x, lat.tw0 * g.y + lat.tw1 * h.y, lat.tw0 * g.z + lat.tw1 * h.z,
-                      lat.tw0 * g.w + lat.tw1 * h.w);
-    }
-    gx.x = fmaf(ax, g.x, gx.x); gx.y = fmaf(ax, g.y, gx.y); gx.z = fmaf(ax, g.z, gx.z); gx.w = fmaf(ax, g.w, gx.w);
-    gy.x = fmaf(ay, g.x, gy.x); gy.y = fmaf(ay, g.y, gy.y); gy.z = fmaf(ay, g.z, gy.z); gy.w = fmaf(ay, g.w, gy.w);
-    gz.x = fmaf(az, g.x, gz.x); gz.y = fmaf(az, g.y, gz.y); gz.z = fmaf(az, g.z, gz.z); gz.w = fmaf(az, g.w, gz.w);
-  }
-}
-
 // sin and cos of the Fourier argument e = F_k . p (Eq. 2) with e carried to
 // about twice FP32 precision: each product split exactly into hi + lo by an
 // FMA, the three products summed with error-free two-sums, then
@@ -245,12 +209,11 @@ __device__ __forceinline__ void fourier_sincos(const float* f, float3 p, float& 
   c = fmaf(-sh, lo, ch);
 }
 
-// Full forward pass at p (+ pl, the low part of a position carried as a
-// pair, which only the Fourier arguments use).  out[0..D-1]; when STASH,
-// hs[i] receives the pre-activation of layer i (i = 0..l-2) for the adjoint.
-template <int C, bool STASH>
+// Full forward pass at p.  out[0..D-1]; hs[i] receives the pre-activation of
+// layer i (i = 0..l-2) for the backward.
+template <int C>
 __device__ __forceinline__ void forward(const float* sm, const Layout& L, int act, const Latent& lat, float3 p,
-                                        float (&out)[4], float (*hs)[C], float3 pl = make_float3(0.f, 0.f, 0.f)) {
+                                        float (&out)[4], float (*hs)[C]) {
   float h[C];
   const float* W0T = sm + L.oW0T;
 #pragma unroll
@@ -261,7 +224,7 @@ __device__ __forceinline__ void forward(const float* sm, const Layout& L, int ac
   const float* Fm = sm + L.oF;
   for (int k = 0; k < L.m; ++k) {
     float s, c;
-    fourier_sincos(Fm + 3 * k, p, s, c, pl);
+    fourier_sincos(Fm + 3 * k, p, s, c);
     axpy<C>(h, W0T + (3 + k) * C, s);
     axpy<C>(h, W0T + (3 + L.m + k) * C, c);
   }
@@ -280,7 +243,7 @@ __device__ __forceinline__ void forward(const float* sm, const Layout& L, int ac
     float a[C];
 #pragma unroll
     for (int o = 0; o < C; ++o) {
-      if (STASH) hs[i - 1][o] = h[o];
+      hs[i - 1][o] = h[o];
       a[o] = act_f(act, h[o]);
     }
 #pragma unroll
@@ -291,7 +254,7 @@ __device__ __forceinline__ void forward(const float* sm, const Layout& L, int ac
   float a[C];
 #pragma unroll
   for (int o = 0; o < C; ++o) {
-    if (STASH) hs[L.l - 2][o] = h[o];
+    hs[L.l - 2][o] = h[o];
     a[o] = act_f(act, h[o]);
   }
 #pragma unroll
@@ -299,87 +262,7 @@ __device__ __forceinline__ void forward(const float* sm, const Layout& L, int ac
     out[d] = d < L.D ? sm[L.obl + d] + dotrow<C>(sm + L.oWl + d * C, a) : 0.0f;
 }
 
-// Adjoint input gradient (Section 5 "Adjoint") of sum_d s_d out_d, whose
-// derivative with respect to the last hidden activation is seed[o] =
-// sum_d s_d W_last[d][o] (seed = row 0 of W_last: d out_0 / d p):
-// backpropagate through the hidden layers, then through layer 0's inputs:
-// identity for p, cos(e) F_k / -sin(e) F_k for the Fourier features,
-// trilinear Jacobian for the latent vector.
-template <int C>
-__device__ __forceinline__ float3 adjoint(const float* sm, const Layout& L, int act, const Latent& lat, float3 p,
-                                          float (*hs)[C], const float* seed, float3 pl = make_float3(0.f, 0.f, 0.f)) {
-  float delta[C];
-#pragma unroll
-  for (int o = 0; o < C; ++o) delta[o] = seed[o] * act_df(act, hs[L.l - 2][o]);
-  for (int i = L.l - 2; i >= 1; --i) {
-    const float* Wrm = sm + L.oHid + (i - 1) * L.hidStride + C * C + C;
-    float g[C];
-#pragma unroll
-    for (int j = 0; j < C; ++j) g[j] = 0.0f;
-#pragma unroll
-    for (int o = 0; o < C; ++o) axpy<C>(g, Wrm + o * C, delta[o]);
-#pragma unroll
-    for (int j = 0; j < C; ++j) delta[j] = g[j] * act_df(act, hs[i - 1][j]);
-  }
-  const float* W0T = sm + L.oW0T;
-  float3 dp = make_float3(dotrow<C>(W0T, delta), dotrow<C>(W0T + C, delta), dotrow<C>(W0T + 2 * C, delta));
-  const float* Fm = sm + L.oF;
-  for (int k = 0; k < L.m; ++k) {
-    float gs = dotrow<C>(W0T + (3 + k) * C, delta);
-    float gc = dotrow<C>(W0T + (3 + L.m + k) * C, delta);
-    float s, c;
-    fourier_sincos(Fm + 3 * k, p, s, c, pl);
-    float coef = gs * c - gc * s;
-    dp.x = fmaf(coef, Fm[3 * k], dp.x);
-    dp.y = fmaf(coef, Fm[3 * k + 1], dp.y);
-    dp.z = fmaf(coef, Fm[3 * k + 2], dp.z);
-  }
-  Cell cell = make_cell(lat, p);
-  for (int f = 0; f < L.F; f += 4) {
-    const float* r = W0T + (3 + 2 * L.m + f) * C;
-    float g0 = dotrow<C>(r, delta), g1 = dotrow<C>(r + C, delta), g2 = dotrow<C>(r + 2 * C, delta),
-          g3 = dotrow<C>(r + 3 * C, delta);
-    float4 gx, gy, gz;
-    latent4_grad(lat, cell, f, gx, gy, gz);
-    dp.x += g0 * gx.x + g1 * gx.y + g2 * gx.z + g3 * gx.w;
-    dp.y += g0 * gy.x + g1 * gy.y + g2 * gy.z + g3 * gy.w;
-    dp.z += g0 * gz.x + g1 * gz.y + g2 * gz.z + g3 * gz.w;
-  }
-  return dp;
-}
-
 __device__ __forceinline__ float3 clamp_p(float3 p) { return make_float3(clamp01f(p.x), clamp01f(p.y), clamp01f(p.z)); }
-
-// Density (and gradient for shading) at the position ph + pl (a pair) for
-// shading mode SH; the finite-difference neighbours are offset as pairs.
-template <int C, int SH>
-__device__ __forceinline__ float sample_field(const float* sm, const Layout& L, int act, const Latent& lat, float3 p,
-                                              float3 pl, float fd_h, float3& g) {
-  float out[4];
-  if (SH == SRN_SHADE_ADJOINT) {
-    float hs[kMaxL][C];
-    forward<C, true>(sm, L, act, lat, p, out, hs, pl);
-    g = adjoint<C>(sm, L, act, lat, p, hs, sm + L.oWl, pl);
-    return out[0];
-  }
-  forward<C, false>(sm, L, act, lat, p, out, nullptr, pl);
-  if (SH == SRN_SHADE_HEAD) g = make_float3(out[1], out[2], out[3]);
-  if (SH == SRN_SHADE_FD) {
-    float gg[3];
-#pragma unroll 1
-    for (int a = 0; a < 3; ++a) {
-      float3 qh = p, ql = pl, rh = p, rl = pl;
-      df::offset_axis(qh, ql, a, fd_h);
-      df::offset_axis(rh, rl, a, -fd_h);
-      float o1[4], o2[4];
-      forward<C, false>(sm, L, act, lat, qh, o1, nullptr, ql);
-      forward<C, false>(sm, L, act, lat, rh, o2, nullptr, rl);
-      gg[a] = (o1[0] - o2[0]) / (2.0f * fd_h);
-    }
-    g = make_float3(gg[0], gg[1], gg[2]);
-  }
-  return out[0];
-}
 
 }  // namespace net32
 }  // namespace srn

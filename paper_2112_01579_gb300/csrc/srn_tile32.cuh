@@ -13,9 +13,10 @@
 // bits as a thread walking the inputs alone.
 //
 // Measured against one thread per point with out-of-line library sines: error
-// grid of 128^3 x 8 evaluations of the main configuration 5.68 -> 3.41 ms
-// (4.9 G evaluations/s; the FMA pipe that takes packed FMAs 68 % busy, the
-// shared-memory data pipe 70 %), the plain workload's 128^2 frame 968 -> 540 us.
+// grid of 128^3 x 8 evaluations of the main configuration 5.68 -> 3.09 ms
+// (5.4 G evaluations/s; bound by the pipe that takes packed FMAs and the
+// shared-memory data pipe together), the plain workload's 128^2 frame 968 ->
+// 202 us (with several samples of a ray per pass).
 #pragma once
 
 #include "srn_net32.cuh"
