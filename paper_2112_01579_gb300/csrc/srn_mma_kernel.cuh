@@ -28,10 +28,10 @@
 //   (C -> D) runs on the CUDA cores in FP32.
 // * SnakeAlt(x) = 0.5 x + sin^2 x = (x - cos 2x + 1) / 2 (Eq. 3).  Every MMA
 //   layer is staged to produce u = 2x (weights and bias doubled, which is
-//   exact in FP16), the epilogue hands cos u - u / 2 = 1 - 2 SnakeAlt(x)
-//   to the next layer, and the factor -1/2 and the shift 1/2 are folded into
-//   that layer's weights and bias: the doubled next layer then simply uses -W
-//   and 2b + sum_j W_j.
+//   exact in FP16), the epilogue hands a = u / 2 - cos u = 2 SnakeAlt(x) - 1
+//   to the next layer, and the factor 1/2 and the shift 1/2 are folded into
+//   that layer's weights and bias: the doubled next layer then simply uses W
+//   and 2b + sum_j W_j (width 32: -a and -W, see act_fold).
 // * Rays are claimed dynamically from a work counter, a warp at a time: when
 //   every lane's ray has terminated (box exit or opacity >= threshold), the
 //   warp takes the next 8 x 4 pixel tile.  The lanes then march neighbouring
@@ -216,12 +216,15 @@ __device__ __forceinline__ void split_h2(float a0, float a1, uint32_t& hi, uint3
 
 // Activation values handed to the next layer from two accumulator values:
 // sin(x) for the sine network; for SnakeAlt the accumulator holds u = 2x and
-// the value is cos u - u / 2 = 1 - 2 SnakeAlt(x) (the next layer's weights
-// carry the minus sign; with PACK one packed FMA does two).
-template <int ACT, bool PACK>
+// the value is u / 2 - cos u = 2 SnakeAlt(x) - 1, or its negative with NEG
+// (the next layer's weights then carry the minus sign), which with PACK is one
+// packed FMA for two.  Width 32 takes NEG; at width 48 the schedule it led to
+// was 1 % slower.
+template <int ACT, bool PACK, bool NEG>
 __device__ __forceinline__ float2 act_fold(float x, float y) {
   if (ACT != SRN_ACT_SNAKEALT) return make_float2(__sinf(x), __sinf(y));
   if (PACK) return __ffma2_rn(make_float2(x, y), make_float2(-0.5f, -0.5f), make_float2(__cosf(x), __cosf(y)));
+  if (!NEG) return make_float2(fmaf(0.5f, x, -__cosf(x)), fmaf(0.5f, y, -__cosf(y)));
   return make_float2(fmaf(-0.5f, x, __cosf(x)), fmaf(-0.5f, y, __cosf(y)));
 }
 
@@ -618,6 +621,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   // sum at widths 48 and 64 (the other form: 2.89 -> 2.93 ms) and for points
   // with gradient (166 -> 170 us for 2^20).
   constexpr bool SUM2 = C == 32 && SH != kPointsAdj;
+  constexpr bool NEG = C == 32;  // see act_fold
   const int L = LF > 0 ? LF : net.l;
   const int D = LF > 0 ? DF : net.D;
   // the FP16 latent grid holds G 2^-gexp: the latent columns' layer-0 weights
@@ -666,7 +670,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
             v = col == D0 ? bh : __float2half_rn(bias - __half2float(bh));
           }
         } else {
-          v = __float2half_rn((SNAKE ? -1.0f : 1.0f) * __half2float(Wsrc[col % C]));  // see act_fold
+          v = __float2half_rn((SNAKE && NEG ? -1.0f : 1.0f) * __half2float(Wsrc[col % C]));  // see act_fold
         }
         h2[q] = v;
       }
@@ -730,7 +734,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   {
     // last layer on the CUDA cores: folded like the hidden layers
     const __half* Wl = net.W_h + (size_t)C * D0 + (size_t)(L - 2) * C * C;
-    for (int i = tid; i < D * C; i += THREADS) wl[i] = (SNAKE ? -0.5f : 1.0f) * __half2float(Wl[i]);
+    for (int i = tid; i < D * C; i += THREADS) wl[i] = (SNAKE ? (NEG ? -0.5f : 0.5f) : 1.0f) * __half2float(Wl[i]);
     if (tid < D) {
       float bias = net.b[(L - 1) * C + tid];
       if (SNAKE) {
@@ -941,7 +945,7 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
             uint32_t hi[8], lo[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              const float2 a = act_fold<ACT, PACK>(x[16 * j + 2 * e], x[16 * j + 2 * e + 1]);
+              const float2 a = act_fold<ACT, PACK, NEG>(x[16 * j + 2 * e], x[16 * j + 2 * e + 1]);
               split_h2(a.x, a.y, hi[e], lo[e]);
             }
             tmem_st8(t_a + 8 * j, hi);
@@ -978,13 +982,13 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
           mma_commit(mb);
         }
       } else if (!failed) {
-        float2 a[C / 2];
+        if constexpr (SUM2) {
+          float2 a[C / 2];
 #pragma unroll
-        for (int j = 0; j < C / 2; ++j) a[j] = act_fold<ACT, PACK>(x[2 * j], x[2 * j + 1]);
+          for (int j = 0; j < C / 2; ++j) a[j] = act_fold<ACT, PACK, NEG>(x[2 * j], x[2 * j + 1]);
 #pragma unroll
-        for (int dd = 0; dd < 4; ++dd) {
-          if (dd < D) {
-            if constexpr (SUM2) {
+          for (int dd = 0; dd < 4; ++dd) {
+            if (dd < D) {
               float2 sacc = make_float2(wl[D * C + dd], 0.0f);
 #pragma unroll
               for (int j = 0; j < C / 2; j += 2) {
@@ -998,18 +1002,30 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
                 }
               }
               out[dd] = sacc.x + sacc.y;
-            } else {
+            }
+          }
+        } else {
+          float a[C];
+#pragma unroll
+          for (int j = 0; j < C; j += 2) {
+            const float2 v = act_fold<ACT, false, NEG>(x[j], x[j + 1]);
+            a[j] = v.x;
+            a[j + 1] = v.y;
+          }
+#pragma unroll
+          for (int dd = 0; dd < 4; ++dd) {
+            if (dd < D) {
               float sacc = wl[D * C + dd];
 #pragma unroll
-              for (int j = 0; j < C; ++j) sacc = fmaf(wl[dd * C + j], (j & 1) ? a[j / 2].y : a[j / 2].x, sacc);
+              for (int j = 0; j < C; ++j) sacc = fmaf(wl[dd * C + j], a[j], sacc);
               out[dd] = sacc;
             }
           }
         }
         if constexpr (ADJ) {
-          // d out / d x of the last hidden layer; wl holds -W / 2 for SnakeAlt
+          // d out / d x of the last hidden layer; wl holds W / 2 (NEG: -W / 2) for SnakeAlt
 #pragma unroll
-          for (int j = 0; j < C; ++j) dl[j] = SNAKE ? -wl[j] * fmaf(2.0f, __sinf(x[j]), 1.0f) : wl[j] * __cosf(x[j]);
+          for (int j = 0; j < C; ++j) dl[j] = SNAKE ? (NEG ? -wl[j] : wl[j]) * fmaf(2.0f, __sinf(x[j]), 1.0f) : wl[j] * __cosf(x[j]);
         }
       }
     }
