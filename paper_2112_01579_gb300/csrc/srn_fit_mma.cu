@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(128 * kFitWGS, 1)
   const uint32_t d_dw = d_acc + 64;                           // dW0 accumulator (64 columns)
   const uint32_t t_row = d_acc + ((uint32_t)(warp * 32) << 16);
   const uint32_t t_dw = d_dw + ((uint32_t)(warp * 32) << 16);
-  const uint32_t af_addr = smem_u32(Af), bt_addr = smem_u32(Bt);
-  const uint32_t b0_addr = smem_u32(B0);
+  const uint64_t af_desc = sw128_desc(smem_u32(Af)), b0_desc = sw128_desc(smem_u32(B0));
+  const uint64_t af_mn_desc = sw128_mn_desc(smem_u32(Af), kTile), bt_mn_desc = sw128_mn_desc(smem_u32(Bt), kTile);
   const uint32_t mb = smem_u32(&mbar[wg]);
   const int bar_id = 1 + wg;
   uint32_t phase = 0;
@@ -284,14 +284,16 @@ __global__ void __launch_bounds__(128 * kFitWGS, 1)
     tc_fence_before();
     bar_sync(bar_id, 128);
     if (misc[4 + wg]) break;
-    if (row == 0 && !a.stall_test) {  // stall_test: no MMA, no commit, nothing in flight
+    // the elected lane issues, from descriptors built once: four steps of 2^18
+    // points 362 -> 344 us against a branch on the thread's row
+    if (warp == 0 && !a.stall_test && elect_one()) {  // stall_test: no MMA, no commit, nothing in flight
       tc_fence_after();
       // K blocks [v hi | v lo | v hi] x [W hi | W hi | W lo]: the third A block is the first
 #pragma unroll
       for (int kk = 0; kk < 12; ++kk) {
         const uint32_t ka = kk >> 2, kb = (kk & 3) * 32;
-        mma_f16(d_acc, sw128_desc(af_addr + (ka == 2 ? 0u : ka) * kTile + kb),
-                sw128_desc(b0_addr + ka * (32 * 128) + kb), idesc_n(32), kk > 0);
+        mma_f16(d_acc, desc_at(af_desc, (ka == 2 ? 0u : ka) * kTile + kb), desc_at(b0_desc, ka * (32 * 128) + kb),
+                idesc_n(32), kk > 0);
       }
       mma_commit(mb);
     }
@@ -365,14 +367,14 @@ __global__ void __launch_bounds__(128 * kFitWGS, 1)
     tc_fence_before();
     bar_sync(bar_id, 128);
     if (misc[4 + wg]) break;
-    if (row == 0) {
+    if (warp == 0 && elect_one()) {
       tc_fence_after();
       // dW0^T += v0^T delta over this tile's points (M = 128: v hi, v lo features; N = 64: delta hi,
       // delta lo; K = 128 points, 16 rows = 2048 bytes per MMA)
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) {
-        mma_f16(d_dw, sw128_mn_desc(af_addr + kk * 2048, kTile), sw128_mn_desc(bt_addr + kk * 2048, kTile),
-                kIdescGrad, (first && kk == 0) ? 0u : 1u);
+        mma_f16(d_dw, desc_at(af_mn_desc, kk * 2048), desc_at(bt_mn_desc, kk * 2048), kIdescGrad,
+                (first && kk == 0) ? 0u : 1u);
       }
       mma_commit(mb);
     }
