@@ -246,7 +246,7 @@ def fit_cfg3(vol, pts, steps=FIT_STEPS, seed=0):
                                                       "frac": tf_ach / pk["bf16_tflops"] if pk.get("bf16_tflops") else None},
                        "gather": {"achieved": gb_ach, "unit": "GB/s", "bytes_per_point": FIT_GATHER_BYTES_PER_POINT,
                                   "hbm_frac": gb_ach / pk["hbm_gbs"] if pk.get("hbm_gbs") else None},
-                       "note": "eight short dependent kernels per step (2-15 us each): launch and tail latency, "
+                       "note": "seven dependent kernels per step (the point kernel about 40 us, the others 3-15): latency, "
                                "not a unit's throughput, set the rate"}
     net.close()
     return res
@@ -713,10 +713,10 @@ SMS, MUFU_PER_SM_CLK, FP32_PER_SM_CLK, MAX_SM_GHZ = 152, 16, 128, 2.07
 # DRAM bytes (read + write) of one 1024^2 frame of the render kernel and of
 # the dense DVR, from the ncu captures summarised in profiles/ (None when the
 # kernel changed after the capture).
-RENDER_DRAM_BYTES = 1174272 + 10240
+RENDER_DRAM_BYTES = 1684224 + 18176
 # Warp instructions per network sample of the render kernel from the same
-# capture (smsp__inst_executed.sum 8.19375e9 over 2.08797e8 samples).
-WARP_INST_PER_SAMPLE = 8.19375e9 / 2.08797e8
+# capture (smsp__inst_executed.sum 7.2486e9 over 2.10e8 samples).
+WARP_INST_PER_SAMPLE = 7.2486e9 / 2.10e8
 # Algorithmic work of one plain-workload fit step per point: forward 2 (35 x 32
 # + 32) FLOP, weight gradients the same again, the backward through the
 # output layer (2 x 32), the latent-input gradient (2 x 32 x 8) and its
@@ -725,7 +725,8 @@ WARP_INST_PER_SAMPLE = 8.19375e9 / 2.08797e8
 FIT_FLOP_PER_POINT = 2 * (35 * 32 + 32) * 2 + 2 * 32 + 2 * 32 * 8 + 8 * 8 * 2
 FIT_GATHER_BYTES_PER_POINT = 32
 DENSE_DRAM_BYTES = 67166208 + 9174016
-DENSE_L1_WAVEFRONT_PCT = 88.3  # l1tex__data_pipe_lsu_wavefronts, % of peak, same capture
+DENSE_L1_WAVEFRONT_PCT = 59.3  # l1tex__data_pipe_lsu_wavefronts, % of peak
+DENSE_ISSUE_PCT = 82.5  # smsp__issue_active, % of peak, same capture
 # L1 load bandwidth of one SM (bytes per clock) for the gather roofline of
 # dense DVR (unit count; the peak is derived, not measured).
 L1_BYTES_PER_SM_CLK = 128
@@ -741,12 +742,13 @@ def dense_roofline(samples, ms_total, frames, vol_bytes):
     peak = SMS * L1_BYTES_PER_SM_CLK * MAX_SM_GHZ
     hbm = peaks().get("hbm_gbs")
     vol_gbs = vol_bytes * frames / secs / 1e9
-    return {"bound": "l1", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+    return {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": DENSE_DRAM_BYTES, "kernel": "dvr_dense_kernel", "per_sample_bytes": DENSE_GATHER_BYTES,
             "peak_source": "152 SMs x 128 B/clk x 2.07 GHz (unit counts)",
             "l1_data_wavefronts_pct": DENSE_L1_WAVEFRONT_PCT,
-            "l1_note": "ncu: the L1 data pipe is 88 % busy with the wavefronts of the scattered 4-byte corner "
-                       "gathers (several cache lines per warp load), which is what bounds the kernel",
+            "issue_active_pct": DENSE_ISSUE_PCT,
+            "l1_note": "ncu: 82 % of the issue slots are taken and the L1 data pipe is 59 % busy with the wavefronts "
+                       "of the scattered 4-byte corner gathers; the fraction here is against the L1 gather roofline",
             "hbm_floor": {"achieved": vol_gbs, "peak": hbm, "unit": "GB/s",
                           "frac": vol_gbs / hbm if hbm else None,
                           "note": "the volume read once per frame, against MEASURED_PEAKS.json hbm_gbs"}}
