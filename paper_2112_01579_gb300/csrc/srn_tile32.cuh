@@ -713,16 +713,21 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
   return r;
 }
 
-// Warps per CTA of a tile kernel over `tiles` tiles.  One CTA of 16 warps (8
-// at widths 48 and 64: what registers allow an SM) where that many tiles per
-// SM wait, so that the parameters are in shared memory once and the rest stays
-// L1 for the gathers; CTAs of 4 for fewer tiles, which then spread over all
-// SMs; less where the parameters and `rows` rows of 32 floats per warp pass
-// 227 KB.  Error grid of 128^3 x 8: 3.37 -> 3.09 ms.
+// Warps per CTA of a tile kernel over `tiles` tiles (0: not known).  One CTA
+// of 16 warps (8 at widths 48 and 64: what registers allow an SM) where that
+// many tiles per SM wait, so that the parameters are in shared memory once and
+// the rest stays L1 for the gathers (error grid of 128^3 x 8: 3.37 -> 3.09
+// ms).  Fewer tiles: one CTA per SM that holds its share, so that every tile
+// is in the first wave (CTAs of 4, of which shared memory held three per SM,
+// left a second wave nearly empty: 60,000 points of the main network 31.3 -> 26.6
+// us, with gradient 57.5 -> 45.1 us); not under 4 warps, which then
+// spread over as many SMs as there are tiles for.  Less where the parameters
+// and `rows` rows of 32 floats per warp pass 227 KB.
 constexpr int max_warps(int C) { return C == 32 ? 16 : 8; }
 inline int warps_for(const Net& t, int C, int rows, long long tiles, int sms) {
-  int w = tiles >= (long long)max_warps(C) * sms ? max_warps(C) : 4;
-  while (w > 1 && sizeof(float) * ((size_t)t.total + (size_t)w * rows * kPts) > 227 * 1024) w /= 2;
+  const long long share = (tiles + sms - 1) / sms;
+  int w = share >= max_warps(C) ? max_warps(C) : (share > 4 ? (int)share : 4);
+  while (w > 1 && sizeof(float) * ((size_t)t.total + (size_t)w * rows * kPts) > 227 * 1024) --w;
   return w;
 }
 

@@ -135,3 +135,26 @@ def test_fp16_depths(S, width, m, most):
         on = oracle.OracleNet(p)
         bound = oracle.error_bounds(on, pts, oracle.PREC_FP16, grad=False)[0]
         assert (np.abs(out.cpu().numpy() - oracle.net_forward(on, pts)) / bound).max() <= 1.0
+
+
+@pytest.mark.parametrize("width,per_sm,extra", [(32, 4, 1), (32, 5, -31), (32, 13, 7), (32, 16, 0), (32, 16, 1), (64, 4, 33), (64, 8, 0)])
+def test_calls_between_one_wave_and_many(S, width, per_sm, extra):
+    """Point calls whose tiles give each SM one CTA of 4 to 16 warps (a tile
+    each), at the edges of that range: the same bits as the points in calls of
+    1000, each point being evaluated by itself."""
+    import torch
+    p = synth.random_params(R=5, F=16, m=14 if width == 32 else 30, layers=4, width=width, act=synth.ACT_SNAKEALT, seed=per_sm,
+                            grid_std=0.5)
+    n = 32 * per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    net = S.Network(p)
+    pts = torch.tensor(_points(n, 6), device="cuda")
+    dout = torch.randn((n, 1), generator=torch.Generator(device="cuda").manual_seed(n), device="cuda")
+    whole, parts = ([torch.full(s, float("nan"), device="cuda") for s in ((n, 1), (n,), (n, 3), (n, 3))] for _ in range(2))
+    for bufs, size in ((whole, n), (parts, 1000)):
+        for i in range(0, n, size):
+            out, rho, grad, vjp = (b[i : i + size] for b in bufs)
+            S.srn_eval(net.ctx, pts[i : i + size], out)
+            S.srn_density_grad(net.ctx, pts[i : i + size], rho, grad)
+            S.srn_input_backward(net.ctx, pts[i : i + size], dout[i : i + size], vjp)
+    for a, b in zip(whole, parts):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
