@@ -196,6 +196,11 @@ srn_status srn_sync_half(srn_ctx* ctx, void* stream);
  * activations exceed that renders non-finite densities, which the FP16 path
  * records as SRN_ERR_NONFINITE (reported by srn_sync_status); the FP32 path
  * evaluates such networks.
+ * FP16 renders of one context share a work counter, cleared at the start of
+ * each: two of them whose work overlaps on the GPU (different streams) spoil
+ * each other's frames, so serialize them or use a context each.  Later
+ * frames are not touched, and srn_eval / srn_density_grad may overlap with
+ * renders and with each other.
  */
 srn_status srn_render(srn_ctx* ctx, const srn_camera* cams, int n_views, const float* times, int n_times,
                       const srn_tf* tf, const srn_render_desc* desc, float* rgba_dev,

@@ -22,12 +22,10 @@ struct srn_ctx {
   srn_params prm;
   int device;
   // device words: [0] status (SRN_OK / SRN_ERR_NONFINITE / ...), [1] graph step
-  // index, [2..3] render work counter, [4] CTAs of the render that have
-  // finished, [5] FP16 latent-grid scale exponent, [6] scratch of its
-  // computation (bits of max |grid|)
+  // index, [2..3] render work counter, [4] FP16 latent-grid scale exponent,
+  // [5] scratch of its computation (bits of max |grid|)
   unsigned int* status;
-  unsigned long long* ray_counter;  // persistent-render work counter (8-byte aligned), then the finished CTAs;
-                                    // both zero between launches (the kernel's last CTA resets them)
+  unsigned long long* ray_counter;  // persistent-render work counter (8-byte aligned), cleared before every render
   FitScratch fit;             // scratch of srn_fit_step / srn_backward
   // Section 6.2 adaptive distribution (srn_fit_set_sampling)
   unsigned long long* cdf = nullptr;   // [cdf_cap] exclusive prefix sums of the voxel weights
@@ -135,17 +133,17 @@ NetDev make_net(const srn_ctx* ctx) {
   n.gq = c.grid_u8;
   n.grid_q = reinterpret_cast<const uint8_t*>(ctx->prm.grid_q);
   n.grid_qp = ctx->prm.grid_qp;
-  n.grid_exp = ctx->status ? reinterpret_cast<const int*>(ctx->status + 5) : nullptr;
+  n.grid_exp = ctx->status ? reinterpret_cast<const int*>(ctx->status + 4) : nullptr;
   for (int k = 0; k < SRN_MAX_KEYFRAMES; ++k) n.key_times[k] = k < c.n_keyframes ? c.key_times[k] : 0.0f;
   return n;
 }
 
 // FP16 copies of the FP32 masters: the latent grid with its power-of-two
-// scale (exponent into status[5]), the weights as they are, the 8-bit grid.
+// scale (exponent into status[4]), the weights as they are, the 8-bit grid.
 cudaError_t write_half_copies(srn_ctx* ctx, cudaStream_t s) {
   const NetDev n = make_net(ctx);
   cudaError_t e = launch_grid_to_half_scaled(n.grid, (__half*)ctx->prm.grid_h, net_grid_count(n),
-                                             reinterpret_cast<int*>(ctx->status + 5), s);
+                                             reinterpret_cast<int*>(ctx->status + 4), s);
   if (e == cudaSuccess) e = launch_to_half(n.W, (__half*)ctx->prm.weights_h, net_weight_count(n), s);
   if (e == cudaSuccess && ctx->cfg.grid_u8)
     e = launch_quantize_grid(n.grid, net_grid_count(n) / n.F, n.F, (uint8_t*)ctx->prm.grid_q, ctx->prm.grid_qp, s);
@@ -363,7 +361,7 @@ srn_status srn_eval(srn_ctx* ctx, const float* pts_dev, int n, float time, float
   cudaError_t e;
   if (ctx->cfg.precision == SRN_PREC_FP16) {
     if (!eval_mma_supported(net)) return fail(SRN_ERR_UNSUPPORTED, "FP16 tensor-core eval does not implement this shape");
-    e = launch_eval_mma(net, pts_dev, n, time, out_dev, ctx->ray_counter, ctx->status, (cudaStream_t)stream);
+    e = launch_eval_mma(net, pts_dev, n, time, out_dev, ctx->status, (cudaStream_t)stream);
   } else {
     e = launch_eval_fp32(net, pts_dev, n, time, out_dev, nullptr, 0, (cudaStream_t)stream);
   }
@@ -381,8 +379,7 @@ srn_status srn_density_grad(srn_ctx* ctx, const float* pts_dev, int n, float tim
   if (ctx->cfg.precision == SRN_PREC_FP16) {
     if (!density_grad_mma_supported(net))
       return fail(SRN_ERR_UNSUPPORTED, "the FP16 tensor-core adjoint does not implement this shape");
-    e = launch_density_grad_mma(net, pts_dev, n, time, rho_dev, grad_dev, ctx->ray_counter, ctx->status,
-                                (cudaStream_t)stream);
+    e = launch_density_grad_mma(net, pts_dev, n, time, rho_dev, grad_dev, ctx->status, (cudaStream_t)stream);
   } else {
     e = launch_eval_fp32(net, pts_dev, n, time, rho_dev, grad_dev, 1, (cudaStream_t)stream);
   }
@@ -453,7 +450,7 @@ srn_status make_fit_args(srn_ctx* ctx, const float* volume_dev, const int dims[3
   a.status = ctx->status;
   a.grid_h = reinterpret_cast<__half*>(ctx->prm.grid_h);
   a.weights_h = reinterpret_cast<__half*>(ctx->prm.weights_h);
-  a.grid_exp = reinterpret_cast<const int*>(ctx->status + 5);
+  a.grid_exp = reinterpret_cast<const int*>(ctx->status + 4);
   a.adam_m = ctx->prm.adam_m;
   a.adam_v = ctx->prm.adam_v;
   a.grid = ctx->prm.grid;

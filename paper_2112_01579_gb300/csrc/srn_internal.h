@@ -100,13 +100,12 @@ cudaError_t launch_render_mma(const NetDev& net, const BatchDev& b, unsigned lon
 bool render_mma_supported(const NetDev& net, int shading);
 bool eval_mma_supported(const NetDev& net);
 cudaError_t launch_eval_mma(const NetDev& net, const float* pts, long long n, float time, float* out,
-                            unsigned long long* ray_counter, unsigned int* status, cudaStream_t s);
+                            unsigned int* status, cudaStream_t s);
 // Density and adjoint input gradient at n points on the tensor cores (the
 // render's adjoint MMAs; width 32, density output, at most four layers).
 bool density_grad_mma_supported(const NetDev& net);
 cudaError_t launch_density_grad_mma(const NetDev& net, const float* pts, long long n, float time, float* rho,
-                                    float* grad, unsigned long long* ray_counter, unsigned int* status,
-                                    cudaStream_t s);
+                                    float* grad, unsigned int* status, cudaStream_t s);
 
 // Conversions and small utilities.
 cudaError_t launch_to_half(const float* src, __half* dst, size_t n, cudaStream_t s);

@@ -105,23 +105,23 @@ bool eval_mma_supported(const NetDev& n) { return render_mma_supported(n, SRN_SH
 
 // Network output at n points with the tensor-core layers (mode kPoints).
 cudaError_t launch_eval_mma(const NetDev& n, const float* pts, long long count, float time, float* out,
-                            unsigned long long* ctr, unsigned int* status, cudaStream_t s) {
+                            unsigned int* status, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
   const BatchDev& b = kNoBatch;
   PointsDev pd{pts, out, count, time, nullptr};
-  if (n.ti) return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 1, 0>(n, b, pd, ctr, status, s);
-  if (n.gq) return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 1>(n, b, pd, ctr, status, s);
-  if (n.c == 48) return launch_t<48, 22, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, ctr, status, s);
-  if (n.c == 64) return launch_t<64, 30, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, ctr, status, s);
+  if (n.ti) return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 1, 0>(n, b, pd, nullptr, status, s);
+  if (n.gq) return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 1>(n, b, pd, nullptr, status, s);
+  if (n.c == 48) return launch_t<48, 22, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, nullptr, status, s);
+  if (n.c == 64) return launch_t<64, 30, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, nullptr, status, s);
   if (n.m == 14 && n.F == 16) {
     if (n.act == SRN_ACT_SNAKEALT && n.l == 4 && n.D == 1)
-      return n.nkey == 1 ? launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0, 4, 1>(n, b, pd, ctr, status, s)
-                         : launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0, 4, 0>(n, b, pd, ctr, status, s);
-    return n.act == SRN_ACT_SNAKEALT ? launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, ctr, status, s)
-                                     : launch_t<32, 14, 16, SRN_ACT_SINE, kPoints, 0, 0>(n, b, pd, ctr, status, s);
+      return n.nkey == 1 ? launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0, 4, 1>(n, b, pd, nullptr, status, s)
+                         : launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0, 4, 0>(n, b, pd, nullptr, status, s);
+    return n.act == SRN_ACT_SNAKEALT ? launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, nullptr, status, s)
+                                     : launch_t<32, 14, 16, SRN_ACT_SINE, kPoints, 0, 0>(n, b, pd, nullptr, status, s);
   }
-  return n.act == SRN_ACT_SNAKEALT ? launch_t<32, 12, 8, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, ctr, status, s)
-                                   : launch_t<32, 12, 8, SRN_ACT_SINE, kPoints, 0, 0>(n, b, pd, ctr, status, s);
+  return n.act == SRN_ACT_SNAKEALT ? launch_t<32, 12, 8, SRN_ACT_SNAKEALT, kPoints, 0, 0>(n, b, pd, nullptr, status, s)
+                                   : launch_t<32, 12, 8, SRN_ACT_SINE, kPoints, 0, 0>(n, b, pd, nullptr, status, s);
 }
 
 bool density_grad_mma_supported(const NetDev& n) { return render_mma_supported(n, SRN_SHADE_ADJOINT); }
@@ -129,20 +129,20 @@ bool density_grad_mma_supported(const NetDev& n) { return render_mma_supported(n
 // Density and adjoint input gradient at n points (mode kPointsAdj): the
 // forward and backward MMAs of the adjoint-shaded render without the march.
 cudaError_t launch_density_grad_mma(const NetDev& n, const float* pts, long long count, float time, float* rho,
-                                    float* grad, unsigned long long* ctr, unsigned int* status, cudaStream_t s) {
+                                    float* grad, unsigned int* status, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
   const BatchDev& b = kNoBatch;
   PointsDev pd{pts, rho, count, time, grad};
-  if (n.c == 48) return launch_t<48, 22, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s);
-  if (n.c == 64) return launch_t<64, 30, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s);
+  if (n.c == 48) return launch_t<48, 22, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, nullptr, status, s);
+  if (n.c == 64) return launch_t<64, 30, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, nullptr, status, s);
   if (n.m == 14 && n.F == 16 && n.act == SRN_ACT_SNAKEALT && n.l == 4 && n.D == 1 && n.nkey == 1)
-    return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0, 4, 1>(n, b, pd, ctr, status, s);
+    return launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0, 4, 1>(n, b, pd, nullptr, status, s);
   if (n.m == 14 && n.F == 16)
     return n.act == SRN_ACT_SNAKEALT
-               ? launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s)
-               : launch_t<32, 14, 16, SRN_ACT_SINE, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s);
-  return n.act == SRN_ACT_SNAKEALT ? launch_t<32, 12, 8, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s)
-                                   : launch_t<32, 12, 8, SRN_ACT_SINE, kPointsAdj, 0, 0>(n, b, pd, ctr, status, s);
+               ? launch_t<32, 14, 16, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, nullptr, status, s)
+               : launch_t<32, 14, 16, SRN_ACT_SINE, kPointsAdj, 0, 0>(n, b, pd, nullptr, status, s);
+  return n.act == SRN_ACT_SNAKEALT ? launch_t<32, 12, 8, SRN_ACT_SNAKEALT, kPointsAdj, 0, 0>(n, b, pd, nullptr, status, s)
+                                   : launch_t<32, 12, 8, SRN_ACT_SINE, kPointsAdj, 0, 0>(n, b, pd, nullptr, status, s);
 }
 
 }  // namespace srn

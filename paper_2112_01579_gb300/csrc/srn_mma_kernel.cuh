@@ -819,7 +819,8 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   }
 
   // Points are taken by the warp's place in the grid, then a grid stride on,
-  // without round trips to the counter (1000 points 16.5 -> 12.3 us).  Rays go
+  // without round trips to the counter (1000 points 16.5 -> 12.3 us), so point
+  // calls of one context may overlap on several streams.  Rays go
   // by the counter: they differ in length, and the choice at run time costs
   // the march 2 % (registers).
   uint32_t place = 32u * (blockIdx.x + gridDim.x * (unsigned)(tid >> 5));
@@ -1220,15 +1221,6 @@ __global__ void __launch_bounds__(128 * wgs_for(C, SH), 1)
   __syncthreads();
   tc_fence_after();
   if (tid < 32) tmem_dealloc(tmem, TMC);
-  // the last CTA leaves the work counter at zero for the next launch
-  if (tid == 0) {
-    unsigned int* done = reinterpret_cast<unsigned int*>(ray_counter + 1);
-    __threadfence();
-    if (atomicAdd(done, 1u) == gridDim.x - 1) {
-      *ray_counter = 0ull;
-      *done = 0u;
-    }
-  }
 }
 
 template <int C, int M, int F, int ACT, int SH, int TI, int GQ, int LF, int ST>
@@ -1249,8 +1241,15 @@ cudaError_t launch_t(const NetDev& net, const BatchDev& b, const PointsDev& pd, 
   const long long claims = is_points(SH) ? (pd.n + 31) / 32
                                          : (long long)((b.W + 7) / 8) * ((b.H + 3) / 4) * b.n_views * b.n_times;
   const unsigned grid = (unsigned)(claims < sms ? claims : sms);
-  if constexpr (is_points(SH)) k<<<grid, 128 * wgs_for(C, SH), plan.total, s>>>(net, PointsBatch{}, pd, plan, ctr, status);
-  else k<<<grid, 128 * wgs_for(C, SH), plan.total, s>>>(net, b, pd, plan, ctr, status);
+  if constexpr (is_points(SH)) {
+    k<<<grid, 128 * wgs_for(C, SH), plan.total, s>>>(net, PointsBatch{}, pd, plan, ctr, status);
+  } else {
+    // Cleared here and not by the launch before: what overlapping calls of
+    // one context leave in the counter reaches no later frame.
+    e = cudaMemsetAsync(ctr, 0, sizeof(*ctr), s);
+    if (e != cudaSuccess) return e;
+    k<<<grid, 128 * wgs_for(C, SH), plan.total, s>>>(net, b, pd, plan, ctr, status);
+  }
   return cudaGetLastError();
 }
 
