@@ -219,7 +219,8 @@ cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s
     tiles = (long long)((b.W + (1 << lw) - 1) >> lw) * ((b.H + (1 << lh) - 1) >> lh) * b.n_views * b.n_times;
     if (log2k == 3 || 2 * tiles > 16ll * sms) break;
   }
-  const int rows = tile_rows(t, C, SH == SRN_SHADE_ADJOINT, false), warps = tile32::warps_for(t, C, rows, 0, sms);
+  const int rows = tile_rows(t, C, SH == SRN_SHADE_ADJOINT, false);
+  const int warps = tile32::warps_for(t, C, rows, 0, sms, (int)sizeof(TFDev));
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = render_fp32_kernel<C, SH>;
   e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -722,12 +722,14 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
 // left a second wave nearly empty: 60,000 points of the main network 31.3 -> 26.6
 // us, with gradient 57.5 -> 45.1 us); not under 4 warps, which then
 // spread over as many SMs as there are tiles for.  Less where the parameters
-// and `rows` rows of 32 floats per warp pass 227 KB.
+// and `rows` rows of 32 floats per warp pass the 227 KB a CTA may have, of
+// which the kernel's own static shared memory is a part.
 constexpr int max_warps(int C) { return C == 32 ? 16 : 8; }
-inline int warps_for(const Net& t, int C, int rows, long long tiles, int sms) {
+constexpr int max_dynamic(int static_bytes) { return 227 * 1024 - static_bytes; }
+inline int warps_for(const Net& t, int C, int rows, long long tiles, int sms, int static_bytes = 0) {
   const long long share = (tiles + sms - 1) / sms;
   int w = share >= max_warps(C) ? max_warps(C) : (share > 4 ? (int)share : 4);
-  while (w > 1 && sizeof(float) * ((size_t)t.total + (size_t)w * rows * kPts) > 227 * 1024) --w;
+  while (w > 1 && sizeof(float) * ((size_t)t.total + (size_t)w * rows * kPts) > (size_t)max_dynamic(static_bytes)) --w;
   return w;
 }
 

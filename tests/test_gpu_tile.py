@@ -158,3 +158,32 @@ def test_calls_between_one_wave_and_many(S, width, per_sm, extra):
             S.srn_input_backward(net.ctx, pts[i : i + size], dout[i : i + size], vjp)
     for a, b in zip(whole, parts):
         assert torch.equal(a, b) and torch.isfinite(a).all()
+
+
+# (width, layers, latent channels, Fourier rows, outputs, shading): more than 128 inputs, where a render's CTA takes all
+# the shared memory an SM gives one but the transfer function's
+WIDE_INPUT = [(64, 7, 32, 57, 4, 1), (64, 8, 8, 79, 4, 0), (64, 8, 32, 110, 1, 0), (32, 8, 4, 124, 1, 0)]
+
+
+@pytest.mark.parametrize("width,layers,F,m,D,shading", WIDE_INPUT)
+def test_render_of_wide_inputs(S, width, layers, F, m, D, shading):
+    """The image against the oracle.  With the transfer function of slope 1
+    and extinction 4 rho over rays of at most 1.74, a density error e moves a
+    pixel by at most (2 4 1.74 + 1) e < 16 e; e is twice the largest FP32
+    bound of 2000 points.  Shading adds its own bound."""
+    import torch
+    p = synth.random_params(R=4, F=F, m=m, layers=layers, width=width, out_dim=D, act=synth.ACT_SNAKEALT, seed=m, grid_std=0.5)
+    p["fourier"] = np.random.default_rng(6).normal(0, 6, (m, 3)).astype(np.float32)
+    net, on = S.Network(p), oracle.OracleNet(p)
+    tf = dict(pos=np.asarray([0.0, 1.0], np.float32), rgba=np.asarray([[0, 0, 0, 0], [1, 1, 1, 1]], np.float32), opacity_scale=4.0)
+    otf, cams = oracle.OracleTF(tf["pos"], tf["rgba"], 4.0), synth.orbit_cameras(1)
+    out = torch.full((1, 1, 12, 17, 4), float("nan"), device="cuda")
+    S.srn_render(net.ctx, cams, tf, S.render_desc(17, 12, 1 / 24, 2.0, shading), out)
+    tol = 16 * 2 * float(oracle.error_bounds(on, _points(2000, 7), oracle.PREC_FP32, grad=False)[0].max())
+    if shading:
+        ref, bound = oracle.render_shade_bound(on, cams, otf, 17, 12, 1 / 24, 2.0, shading, oracle.PREC_FP32)
+        err, lim = np.abs(out.cpu().numpy() - ref).max(axis=-1).ravel(), tol + np.asarray(bound).ravel()
+    else:
+        ref, _, _ = oracle.render(on, cams, otf, 17, 12, 1 / 24, 2.0)
+        err, lim = np.abs(out.cpu().numpy() - ref).max(axis=-1).ravel(), tol
+    assert tol < 1e-2 and (err <= lim).all(), (err.max(), tol)
