@@ -65,7 +65,7 @@ cudaError_t error_grid_t(const NetDev& net, const VolDev& vol, int res, int spv,
   const int rows = t.d0 > C ? t.d0 : C, warps = tile32::warps_for(t, C, rows, tiles, sms);
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = error_grid_kernel<C>;
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = tile32::allow_dynamic(k);
   if (e != cudaSuccess) return e;
   const long long blocks = (tiles + warps - 1) / warps, most = (long long)(tile32::max_warps(C) / warps) * sms;
   k<<<(unsigned)(blocks < most ? blocks : most), 32 * warps, smem, st>>>(net, vol, res, spv, seed, time, E, t, rows);

@@ -656,7 +656,7 @@ template <int NL>
 cudaError_t fit_tile_t(const NetDev& net, const PointArgs& pa, int grid, cudaStream_t st) {
   auto k = fit_tile_kernel<NL>;
   const size_t smem = fit_tile_smem(net);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = tile32::allow_dynamic(k);
   if (e != cudaSuccess) return e;
   k<<<grid, kFitThreads, smem, st>>>(net, pa, tile32::make_net(net), fit_tile_floats(net));
   return cudaGetLastError();

@@ -223,7 +223,7 @@ cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s
   const int warps = tile32::warps_for(t, C, rows, 0, sms, (int)sizeof(TFDev));
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = render_fp32_kernel<C, SH>;
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = tile32::allow_dynamic(k, (int)sizeof(TFDev));
   if (e != cudaSuccess) return e;
   const long long blocks = (tiles + warps - 1) / warps;
   k<<<(unsigned)blocks, 32 * warps, smem, s>>>(net, b, t, rows, log2k);
@@ -242,7 +242,7 @@ cudaError_t launch_eval_t(const NetDev& net, const float* pts, int n, float time
   const int rows = tile_rows(t, C, MODE != 0, MODE == 2), warps = tile32::warps_for(t, C, rows, tiles, sms);
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = eval_fp32_kernel<C, MODE>;
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = tile32::allow_dynamic(k);
   if (e != cudaSuccess) return e;
   // CTAs stage the parameters once and walk the tiles: as many as an SM holds
   const long long blocks = (tiles + warps - 1) / warps, most = (long long)(tile32::max_warps(C) / warps) * sms;

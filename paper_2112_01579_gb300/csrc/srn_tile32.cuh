@@ -726,6 +726,14 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
 // which the kernel's own static shared memory is a part.
 constexpr int max_warps(int C) { return C == 32 ? 16 : 8; }
 constexpr int max_dynamic(int static_bytes) { return 227 * 1024 - static_bytes; }
+// Lets kernel k have as much shared memory as there is.  Not what the call at
+// hand needs: that follows the number of points, and a second host thread
+// with a smaller call of the same network would lower the limit between this
+// thread's setting and its launch, which is then refused.
+template <class K>
+cudaError_t allow_dynamic(K k, int static_bytes = 0) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dynamic(static_bytes));
+}
 inline int warps_for(const Net& t, int C, int rows, long long tiles, int sms, int static_bytes = 0) {
   const long long share = (tiles + sms - 1) / sms;
   int w = share >= max_warps(C) ? max_warps(C) : (share > 4 ? (int)share : 4);

@@ -1,5 +1,8 @@
-"""One context used from two streams: calls that share nothing give the bits of
-serial calls, and no call leaves anything behind that a later one trips over."""
+"""One context used from two streams, and one network from two host threads:
+calls that share nothing give the bits of serial calls, and no call leaves
+anything behind that a later one trips over."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -66,3 +69,40 @@ def test_overlapping_calls_of_one_fp16_context(S, overlap):
         for o in out:
             for a, b in zip(o, ref):
                 assert torch.equal(a, b)
+
+
+def test_two_threads_one_network(S):
+    """Large and small FP32 batches of one network from two host threads: the
+    CTA, and with it the shared memory a launch asks for, follows the batch."""
+    import torch
+    net = S.Network(H.cfg2_params(seed=6, R=8))
+    rng = np.random.default_rng(2)
+    vol = torch.tensor(rng.random((9, 8, 7), dtype=np.float32), device="cuda")
+    sizes, errors = [60000, 50], []
+    pts = [torch.tensor(rng.random((n, 3), dtype=np.float32), device="cuda") for n in sizes]
+    out = [[torch.empty((n, 1), device="cuda"), torch.empty((n, 3), device="cuda")] for n in sizes]
+    err = [torch.empty(r ** 3, device="cuda") for r in (40, 4)]
+
+    def calls(k, reps, stream):
+        try:
+            for _ in range(reps):
+                S.srn_eval(net.ctx, pts[k], out[k][0], stream=stream)
+                S.srn_density_grad(net.ctx, pts[k], out[k][0], out[k][1], stream=stream)
+                S.srn_error_grid(net.ctx, vol, 40 if k == 0 else 4, 1, 3, err[k], stream=stream)
+        except S.SrnError as e:
+            errors.append(str(e))
+
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for k in range(2):
+        calls(k, 1, streams[k])
+    torch.cuda.synchronize()
+    want = [x.clone() for x in (*out[0], *out[1], *err)]
+    threads = [threading.Thread(target=calls, args=(k, 3000, streams[k])) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors[:2]
+    for a, b in zip(want, (*out[0], *out[1], *err)):
+        assert torch.equal(a, b)
