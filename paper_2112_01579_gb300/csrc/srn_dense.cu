@@ -29,7 +29,9 @@ struct Cell {
   float c[8];
 };
 
-// Trilinear density at voxel coordinates g (vertex i at coordinate i).
+// Trilinear density at voxel coordinates g (vertex i at coordinate i).  The
+// lerps are (1 - f) a + f b and not a + f (b - a): infinite or very large
+// voxels next to each other or to small ones keep their values.
 template <class I, bool CACHED>
 __device__ __forceinline__ float sample(const VolDev& v, I sy, I sz, float3 g, Cell<I>& k) {
   const int ix = min(max(__float2int_rd(g.x), 0), v.nx - 2), iy = min(max(__float2int_rd(g.y), 0), v.ny - 2),
@@ -43,10 +45,11 @@ __device__ __forceinline__ float sample(const VolDev& v, I sy, I sz, float3 g, C
     k.c[4] = __ldg(v.vol + at + sz); k.c[5] = __ldg(v.vol + at + sz + 1);
     k.c[6] = __ldg(v.vol + at + sz + sy); k.c[7] = __ldg(v.vol + at + sz + sy + 1);
   }
-  const float x0 = fmaf(fx, k.c[1] - k.c[0], k.c[0]), x1 = fmaf(fx, k.c[3] - k.c[2], k.c[2]);
-  const float x2 = fmaf(fx, k.c[5] - k.c[4], k.c[4]), x3 = fmaf(fx, k.c[7] - k.c[6], k.c[6]);
-  const float y0 = fmaf(fy, x1 - x0, x0), y1 = fmaf(fy, x3 - x2, x2);
-  return fmaf(fz, y1 - y0, y0);
+  const float ex = 1.0f - fx, ey = 1.0f - fy, ez = 1.0f - fz;
+  const float x0 = fmaf(fx, k.c[1], ex * k.c[0]), x1 = fmaf(fx, k.c[3], ex * k.c[2]);
+  const float x2 = fmaf(fx, k.c[5], ex * k.c[4]), x3 = fmaf(fx, k.c[7], ex * k.c[6]);
+  const float y0 = fmaf(fy, x1, ey * x0), y1 = fmaf(fy, x3, ey * x2);
+  return fmaf(fz, y1, ez * y0);
 }
 
 // 1 - exp(-x), x >= 0: the series below 1/4 (the first term left out is

@@ -1,0 +1,53 @@
+"""Dense DVR at values outside the usual range: infinite and very large voxels."""
+import numpy as np
+import pytest
+
+from paper_2112_01579_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def S():
+    from paper_2112_01579_gb300 import build
+    build.build()
+    from paper_2112_01579_gb300 import srn
+    return srn
+
+
+def _tf(pos, rgba, scale):
+    return dict(pos=np.asarray(pos, np.float32), rgba=np.asarray(rgba, np.float32), opacity_scale=scale)
+
+
+def _dense(S, vol, cams, tf, w=60, h=44, step=1 / 64, et=0.99, shading=0):
+    import torch
+    out = torch.full((len(cams), h, w, 4), float("nan"), device="cuda")
+    S.srn_dvr_dense(torch.as_tensor(vol, dtype=torch.float32, device="cuda").contiguous(), cams, tf,
+                    S.render_desc(w, h, step, et, shading), out)
+    torch.cuda.synchronize()
+    return out.cpu().numpy()
+
+
+# one colour above 0.9: a density that interpolation rounds to just below 1 looks like 1
+CAPPED = _tf([0.0, 0.5, 0.9, 1.0], [[0, 0, 0, 0], [0.2, 0.7, 0.4, 0.01], [0.9, 0.5, 0.1, 0.05], [0.9, 0.5, 0.1, 0.05]], 20.0)
+
+
+def test_infinite_voxels_are_opaque(S):
+    """+Inf between +Inf is +Inf, the density 1 after the clamp."""
+    cams = synth.orbit_cameras(3)
+    inf, one = (np.full((9, 10, 11), v, np.float32) for v in (np.inf, 1.0))
+    want = _dense(S, one, cams, CAPPED)
+    assert want[..., 3].max() > 0.3
+    assert np.array_equal(_dense(S, inf, cams, CAPPED), want)
+
+
+def test_infinite_slab_beside_finite_voxels(S):
+    """A slab of +Inf looks like one of 1e30: every weight that is not zero
+    takes either of them past 1."""
+    cams = synth.orbit_cameras(3)
+    vol = synth.blobs_volume(24, 6, seed=3).numpy().copy()
+    big, inf = vol.copy(), vol.copy()
+    big[8:14], inf[8:14] = 1e30, np.inf
+    want = _dense(S, big, cams, CAPPED)
+    assert not np.array_equal(want, _dense(S, vol, cams, CAPPED))
+    assert np.array_equal(_dense(S, inf, cams, CAPPED), want)
