@@ -36,7 +36,9 @@ template <class I, bool CACHED>
 __device__ __forceinline__ float sample(const VolDev& v, I sy, I sz, float3 g, Cell<I>& k) {
   const int ix = min(max(__float2int_rd(g.x), 0), v.nx - 2), iy = min(max(__float2int_rd(g.y), 0), v.ny - 2),
             iz = min(max(__float2int_rd(g.z), 0), v.nz - 2);
-  const float fx = g.x - (float)ix, fy = g.y - (float)iy, fz = g.z - (float)iz;
+  // saturated: a coordinate outside the volume (the rounding of a ray from
+  // far away) takes the value at the face, in no more instructions
+  const float fx = __saturatef(g.x - (float)ix), fy = __saturatef(g.y - (float)iy), fz = __saturatef(g.z - (float)iz);
   const I at = (I)iz * sz + (I)iy * sy + (I)ix;
   if (!CACHED || at != k.at) {
     k.at = at;
@@ -100,8 +102,9 @@ __global__ void __launch_bounds__(kThreads) dvr_dense_kernel(const VolDev v, con
     for (float k = 1.0f; ta < t1; k += 1.0f) {
       const float tb = fminf(fmaf(k, b.step, t0), t1);
       const float len = tb - ta, tm = 0.5f * (ta + tb);
-      // no clamp: inside the box up to rounding, and the cell index is limited
-      const float3 g = make_float3(fmaf(tm, gd.x, go.x), fmaf(tm, gd.y, go.y), fmaf(tm, gd.z, go.z));
+      // inside the box up to rounding; sample() clamps, the neighbours need it here
+      float3 g = make_float3(fmaf(tm, gd.x, go.x), fmaf(tm, gd.y, go.y), fmaf(tm, gd.z, go.z));
+      if (FD) g = make_float3(fminf(fmaxf(g.x, 0.0f), mx), fminf(fmaxf(g.y, 0.0f), my), fminf(fmaxf(g.z, 0.0f), mz));
       const float rho = sample<I, true>(v, sy, sz, g, cell);
       ++ns;
       float4 c = tf_segment_eval(tf, quads, rho);

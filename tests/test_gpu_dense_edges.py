@@ -1,4 +1,7 @@
-"""Dense DVR at values outside the usual range: infinite and very large voxels."""
+"""Dense DVR at values and views outside the usual range: infinite and very
+large voxels, an eye far from the box."""
+import math
+
 import numpy as np
 import pytest
 
@@ -51,3 +54,24 @@ def test_infinite_slab_beside_finite_voxels(S):
     want = _dense(S, big, cams, CAPPED)
     assert not np.array_equal(want, _dense(S, vol, cams, CAPPED))
     assert np.array_equal(_dense(S, inf, cams, CAPPED), want)
+
+
+@pytest.mark.parametrize("shading", [0, 2])
+@pytest.mark.parametrize("distance", [3.0, 1e4, 1e5])
+def test_far_eye_does_not_extrapolate(S, shading, distance):
+    """Interpolation stays between the voxels' values whatever the rounding of
+    the sample position: nothing outside [0.4, 0.6] is seen.  The outer layer
+    differs from the next one, so a position past it would show."""
+    rng = np.random.default_rng(4)
+    vol = np.where(rng.random((40, 48, 64)) < 0.5, 0.4, 0.6).astype(np.float32)
+    vol[0], vol[-1], vol[:, 0], vol[:, -1], vol[:, :, 0], vol[:, :, -1] = (0.6,) * 6
+    vol[1], vol[-2], vol[:, 1], vol[:, -2], vol[:, :, 1], vol[:, :, -2] = (0.4,) * 6
+    vol[0], vol[-1], vol[:, 0], vol[:, -1], vol[:, :, 0], vol[:, :, -1] = (0.6,) * 6
+    marker = _tf([0.0, 0.38, 0.39, 0.61, 0.62, 1.0], [[1, 1, 1, 1]] * 2 + [[0, 0, 0, 0]] * 2 + [[1, 1, 1, 1]] * 2, 500.0)
+    d = np.array([0.5, 0.4, 0.77]) / np.linalg.norm([0.5, 0.4, 0.77])
+    cams = [dict(eye=list(distance * d), target=[0.0, 0.0, 0.0], up=[0.0, 1.0, 0.0], fovy=2 * math.atan(0.8 / distance))]
+    got = _dense(S, vol, cams, marker, 120, 90, 1 / 256, 2.0, shading)
+    assert not got.any(), float(np.abs(got).max())
+    # the view does hit the volume
+    seen = _dense(S, vol, cams, _tf([0.0, 1.0], [[1, 1, 1, 1]] * 2, 20.0), 120, 90, 1 / 256, 2.0, shading)
+    assert seen[..., 3].max() > 0.9
