@@ -54,11 +54,11 @@ __device__ __forceinline__ float sample(const VolDev& v, I sy, I sz, float3 g, C
   return fmaf(fz, y1, ez * y0);
 }
 
-// 1 - exp(-x), x >= 0: the series below 1/4 (the first term left out is
+// 1 - exp(-x): the series for |x| below 1/4 (the first term left out is
 // 5e-8 of the value there), where 1 - exp would cancel; steps are short, so
-// that is nearly every sample.
+// that is nearly every sample.  x is negative where a control point's alpha is.
 __device__ __forceinline__ float opacity(float x) {
-  if (x < 0.25f) {
+  if (fabsf(x) < 0.25f) {
     float p = fmaf(x, -1.0f / 720.0f, 1.0f / 120.0f);
     p = fmaf(x, p, -1.0f / 24.0f);
     p = fmaf(x, p, 1.0f / 6.0f);

@@ -1,11 +1,13 @@
 """Dense DVR at values and views outside the usual range: infinite and very
-large voxels, an eye far from the box."""
+large voxels, an eye far from the box, negative control values."""
 import math
 
 import numpy as np
 import pytest
 
+import oracle
 from paper_2112_01579_gb300 import synth
+from tests import helpers as H
 
 pytestmark = pytest.mark.gpu
 
@@ -75,3 +77,16 @@ def test_far_eye_does_not_extrapolate(S, shading, distance):
     # the view does hit the volume
     seen = _dense(S, vol, cams, _tf([0.0, 1.0], [[1, 1, 1, 1]] * 2, 20.0), 120, 90, 1 / 256, 2.0, shading)
     assert seen[..., 3].max() > 0.9
+
+
+@pytest.mark.parametrize("alpha,step", [(-0.4, 0.5), (-0.01, 0.05), (0.4, 0.5)])
+def test_negative_alpha_follows_the_exponential(S, alpha, step):
+    """1 - exp(-x) for either sign of x.  Constant volume, so the density is
+    0.5 to rounding and only the opacity counts: |x| <= 4 a sample to 2^-21
+    (product and exponential), at most 40 samples, each factor of the
+    transmittance off by 2^-21 (1 + |x|): 5e-5 of the largest value."""
+    tf = _tf([0.0, 1.0], [[0.8, 0.5, 0.3, alpha]] * 2, 20.0)
+    cams, vol = synth.orbit_cameras(2), np.full((8, 8, 8), 0.5, np.float32)
+    got = _dense(S, vol, cams, tf, 40, 30, step, 2.0)
+    ref, _, _ = oracle.dvr_dense(vol, cams, H.oracle_tf(tf), 40, 30, step, 2.0)
+    assert np.abs(got - ref).max() <= 5e-5 * max(1.0, np.abs(ref).max())
