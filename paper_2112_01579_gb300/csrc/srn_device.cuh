@@ -1,6 +1,8 @@
 // Device helpers shared by the render, eval and dense-DVR kernels.
 #pragma once
 
+#include <float.h>
+
 #include "srn_internal.h"
 
 namespace srn {
@@ -132,6 +134,13 @@ __device__ __forceinline__ void load_tf(TFDev& dst, const TFDev& src) {
   }
 }
 
+// b - a, finite: tf_segment_eval multiplies it by 0 at the ends of a segment,
+// and a control point of infinite alpha (opaque) must not turn into NaN there.
+__device__ __forceinline__ float tf_difference(float a, float b) {
+  const float d = b - a;
+  return a == b ? 0.0f : (isinf(d) ? copysignf(FLT_MAX, d) : d);
+}
+
 __device__ __forceinline__ void load_tf_segments(TFSeg& t, const TFDev& tf) {
   for (int i = threadIdx.x; i < SRN_MAX_TF_POINTS; i += blockDim.x) {
     const int n = tf.n;
@@ -142,7 +151,8 @@ __device__ __forceinline__ void load_tf_segments(TFSeg& t, const TFDev& tf) {
     t.seg[i] = make_float2(tf.pos[i], wdt > 0.0f ? 1.0f / wdt : 0.0f);
     const float4 a = tf.rgba[i], b = tf.rgba[i + 1 < n ? i + 1 : i];
     t.colour[i] = a;
-    t.diff[i] = make_float4(b.x - a.x, b.y - a.y, b.z - a.z, b.w - a.w);
+    t.diff[i] = make_float4(tf_difference(a.x, b.x), tf_difference(a.y, b.y), tf_difference(a.z, b.z),
+                            tf_difference(a.w, b.w));
   }
 }
 

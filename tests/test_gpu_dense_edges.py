@@ -1,5 +1,6 @@
-"""Dense DVR at values and views outside the usual range: infinite and very
-large voxels, an eye far from the box, negative control values."""
+"""Dense DVR and the transfer function at values and views outside the usual
+range: infinite and very large voxels, an eye far from the box, negative and
+infinite control values."""
 import math
 
 import numpy as np
@@ -90,3 +91,29 @@ def test_negative_alpha_follows_the_exponential(S, alpha, step):
     got = _dense(S, vol, cams, tf, 40, 30, step, 2.0)
     ref, _, _ = oracle.dvr_dense(vol, cams, H.oracle_tf(tf), 40, 30, step, 2.0)
     assert np.abs(got - ref).max() <= 5e-5 * max(1.0, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("path", ["dense", "fp16"])
+@pytest.mark.parametrize("where", ["last", "flat", "second"])
+def test_infinite_alpha_is_opaque(S, path, where):
+    """A control point of infinite alpha stops the ray at its colour; a point
+    before it keeps its own."""
+    import torch
+    alphas = dict(last=[0.0, 0.1, 0.2, np.inf], flat=[0.0, 0.1, np.inf, np.inf], second=[0.0, np.inf, np.inf, np.inf])[where]
+    colour = [[0.1, 0.2, 0.3], [0.5, 0.4, 0.3], [0.6, 0.2, 0.9], [0.3, 0.8, 0.7]]
+    tfs = [_tf([0.2, 0.4, 0.6, 0.8], [c + [min(a, top)] for c, a in zip(colour, alphas)], 20.0) for top in (np.inf, 1e30)]
+    cams = synth.orbit_cameras(2)
+    if path == "dense":
+        vol = synth.blobs_volume(24, 6, seed=5).numpy()
+        got, want = (_dense(S, vol, cams, tf) for tf in tfs)
+    else:
+        net = S.Network(synth.to_half_exact(H.cfg2_params(seed=8, R=8)), precision=S.SRN_PREC_FP16)
+        imgs = []
+        for tf in tfs:
+            out = torch.full((1, 2, 44, 60, 4), float("nan"), device="cuda")
+            S.srn_render(net.ctx, cams, tf, S.render_desc(60, 44, 1 / 64, 0.99), out)
+            torch.cuda.synchronize()
+            imgs.append(out.cpu().numpy())
+        got, want = imgs
+    assert want[..., 3].max() == 1.0
+    assert np.array_equal(got, want)
