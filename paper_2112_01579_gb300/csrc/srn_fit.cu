@@ -1191,18 +1191,148 @@ __global__ void __launch_bounds__(256) cell_corner_kernel(const float* __restric
 // three dependent loads per cell (offsets, point index, point); a warp per
 // vertex over its eight cells, with its butterfly over 32 mostly idle lanes,
 // took 57 us for 32^3 vertices whatever the number of points.
+//
+// Points may crowd: a cell of more than kLongCell points is left to all eight
+// warps of its CTA (one warp on 2^18 points of one cell: 32 ms; so 3.3).
+constexpr int kLongCell = 96;
+
+constexpr int kCellPass = 16;  // points a warp brings to shared memory at a time
+
+// Corner sums of a crowded cell's points, the rows of dz through shared memory
+// so that a pass has one wait for all of them.
 template <int F>
-__global__ void __launch_bounds__(256) cell_warp_kernel(const float* __restrict__ pts, const float* __restrict__ dz,
-                                                        const unsigned int* __restrict__ sidx,
-                                                        const unsigned int* __restrict__ start, int R,
-                                                        long long n_cells, float* __restrict__ part) {
+struct CellSum {
+  static constexpr int QL = F >= 16 ? 4 : F / 4;  // lanes per corner
+  static constexpr int QN = F / (4 * QL);         // channel groups per lane
+  static constexpr int G = 32 / (8 * QL);         // points side by side
+  static constexpr int LR = F / 4;                // lanes per row of dz
+  static constexpr int P = kCellPass, NR = P * LR >= 32 ? P * LR / 32 : 1;  // row loads of a lane
+  float4 acc[QN];
+
+  // acc = the corner sums of the points base .. base + P - 1, then `stride`
+  // on, up to s1.  Each P are summed first, so that the rounding error does
+  // not grow with the length of one chain.  place, rows: the warp's P entries.
+  __device__ __forceinline__ void run(const float* __restrict__ pts, const float* __restrict__ dz,
+                                      const unsigned int* __restrict__ sidx, int R, int base, int s1, int stride,
+                                      float4* place, float4 (*rows)[LR]) {
+    const int lane = threadIdx.x & 31, g = lane / (8 * QL), c = (lane / QL) & 7, q = lane % QL;
+    const float wx = (c & 1) ? 1.f : -1.f, wy = (c & 2) ? 1.f : -1.f, wz = (c & 4) ? 1.f : -1.f;
+    const float ox = (c & 1) ? 0.f : 1.f, oy = (c & 2) ? 0.f : 1.f, oz = (c & 4) ? 0.f : 1.f;
+#pragma unroll
+    for (int e = 0; e < QN; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    int j = lane < P && base + lane < s1 ? (int)sidx[base + lane] : 0;
+#pragma unroll 1
+    for (; base < s1; base += stride) {
+      const int cnt = min(P, s1 - base);
+      float4 v[NR];
+#pragma unroll
+      for (int e = 0; e < NR; ++e) {
+        const int src = e * (32 / LR) + lane / LR, jk = __shfl_sync(0xffffffffu, j, src);
+        if (src < cnt) v[e] = reinterpret_cast<const float4*>(dz + (size_t)jk * F)[lane % LR];
+      }
+      if (lane < cnt) {
+        int i;
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        cell_coord(pts[3 * (size_t)j], R, i, f.x);
+        cell_coord(pts[3 * (size_t)j + 1], R, i, f.y);
+        cell_coord(pts[3 * (size_t)j + 2], R, i, f.z);
+        place[lane] = f;
+      }
+      j = lane < P && base + stride + lane < s1 ? (int)sidx[base + stride + lane] : 0;
+#pragma unroll
+      for (int e = 0; e < NR; ++e) {
+        const int src = e * (32 / LR) + lane / LR;
+        if (src < cnt) rows[src][lane % LR] = v[e];
+      }
+      __syncwarp();
+      float4 a[QN];
+#pragma unroll
+      for (int e = 0; e < QN; ++e) a[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int k = g; k < cnt; k += G) {
+        const float4 f = place[k];
+        const float w = fmaf(wx, f.x, ox) * fmaf(wy, f.y, oy) * fmaf(wz, f.z, oz);
+#pragma unroll
+        for (int e = 0; e < QN; ++e) {
+          const float4 x = rows[k][q + e * QL];
+          a[e].x = fmaf(w, x.x, a[e].x);
+          a[e].y = fmaf(w, x.y, a[e].y);
+          a[e].z = fmaf(w, x.z, a[e].z);
+          a[e].w = fmaf(w, x.w, a[e].w);
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int e = 0; e < QN; ++e) {
+        acc[e].x += a[e].x;
+        acc[e].y += a[e].y;
+        acc[e].z += a[e].z;
+        acc[e].w += a[e].w;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < QN; ++e)
+#pragma unroll
+      for (int off = 8 * QL; off < 32; off <<= 1) {
+        acc[e].x += __shfl_xor_sync(0xffffffffu, acc[e].x, off);
+        acc[e].y += __shfl_xor_sync(0xffffffffu, acc[e].y, off);
+        acc[e].z += __shfl_xor_sync(0xffffffffu, acc[e].z, off);
+        acc[e].w += __shfl_xor_sync(0xffffffffu, acc[e].w, off);
+      }
+  }
+  // The sums as rows [8 corners][F] of out.
+  __device__ __forceinline__ void store(float* out) const {
+    const int lane = threadIdx.x & 31;
+    if (lane >= 8 * QL) return;
+    float4* o = reinterpret_cast<float4*>(out + (lane / QL) * F) + lane % QL;
+#pragma unroll
+    for (int e = 0; e < QN; ++e) o[e * QL] = acc[e];
+  }
+};
+
+// The crowded cells of a CTA (bits of `crowded`; lane l holds the first point
+// of cell l and of the next one), by all its warps.
+template <int F>
+__device__ __noinline__ void crowded_cells(const float* __restrict__ pts, const float* __restrict__ dz,
+                                           const unsigned int* __restrict__ sidx, int R, long long cell0, int at,
+                                           int end, unsigned int crowded, float* __restrict__ part) {
+  __shared__ float4 place[8][kCellPass], rows[8][kCellPass][F / 4];
+  const int warp = threadIdx.x >> 5;
+  for (unsigned int left = crowded; left; left &= left - 1) {
+    const int w = __ffs(left) - 1;
+    const int c0 = __shfl_sync(0xffffffffu, at, w), c1 = __shfl_sync(0xffffffffu, end, w);
+    CellSum<F> sum;
+    sum.run(pts, dz, sidx, R, c0 + kCellPass * warp, c1, 8 * kCellPass, place[warp], rows[warp]);
+    sum.store(reinterpret_cast<float*>(rows[warp]));  // a warp's rows hold twice its sums
+    __syncthreads();
+    for (int i = threadIdx.x; i < 8 * F; i += 256) {
+      float t = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) t += reinterpret_cast<const float*>(rows[k])[i];
+      part[(size_t)(cell0 + w) * 8 * F + i] = t;
+    }
+    __syncthreads();
+  }
+}
+
+template <int F>
+__global__ void __launch_bounds__(256, 6)
+    cell_warp_kernel(const float* __restrict__ pts, const float* __restrict__ dz, const unsigned int* __restrict__ sidx,
+                     const unsigned int* __restrict__ start, int R, long long n_cells, float* __restrict__ part) {
   constexpr int QL = F >= 16 ? 4 : F / 4;      // lanes per corner
   constexpr int QN = F / (4 * QL);             // channel groups per lane
   constexpr int G = 32 / (8 * QL);             // points side by side
-  const long long cell = ((long long)blockIdx.x * 256 + threadIdx.x) >> 5;
-  if (cell >= n_cells) return;
   const int lane = threadIdx.x & 31, g = lane / (8 * QL), c = (lane / QL) & 7, q = lane % QL;
-  const int s0 = (int)start[cell], s1 = (int)start[cell + 1];
+  const int warp = threadIdx.x >> 5;
+  const long long cell0 = (long long)blockIdx.x * 8, cell = cell0 + warp;
+  // every warp reads the offsets of the CTA's cells, so that all know without
+  // a barrier which ones are crowded
+  const int at = lane < 9 ? (int)start[min(cell0 + lane, n_cells)] : 0;
+  const int end = __shfl_down_sync(0xffffffffu, at, 1);
+  const unsigned int crowded = __ballot_sync(0xffffffffu, lane < 8 && end - at > kLongCell);
+  if (crowded) crowded_cells<F>(pts, dz, sidx, R, cell0, at, end, crowded, part);
+  if (cell >= n_cells || (crowded >> warp & 1u)) return;
+  const int s0 = __shfl_sync(0xffffffffu, at, warp), s1 = __shfl_sync(0xffffffffu, end, warp);
   float4 acc[QN];
 #pragma unroll
   for (int e = 0; e < QN; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);

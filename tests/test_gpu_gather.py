@@ -93,3 +93,78 @@ def test_grids_off_a_32_byte_boundary(S, F, m, layers, act, keys):
         got.append([x.clone() for x in (out, grad, vjp, dg, dw, db, err, loss, grid, net.weights, net.biases, rho)])
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+def _crowd(kind, n, k, R, seed):
+    """n points, k of them in one place below the middle: a `cell`, the cells
+    of one leading `digit` of the cell index (three rows of a z layer at R =
+    33), or `two` cells a half of the grid apart; the others above the middle."""
+    rng = np.random.default_rng(seed)
+    pts, h = rng.random((n, 3), dtype=np.float32), 1.0 / (R - 1)
+    u = 0.02 + 0.96 * pts[:k].astype(np.float64)
+    pts[k:, 2] = 0.5 + 0.5 * pts[k:, 2]
+    if kind == "cell":
+        pts[:k] = (u + [2, 1, 1]) * h
+    elif kind == "two":
+        u[::2, 2] += R // 2
+        pts[:k] = (u + [1, 2, 0]) * h
+    else:
+        pts[:k] = np.stack([u[:, 0] * (R - 1), u[:, 1] * 3 + R // 2, u[:, 2] + R // 3], 1) * h
+    return rng.permutation(np.clip(pts, 0.0, 1.0), axis=0).astype(np.float32)
+
+
+@pytest.mark.parametrize("R,F,n,k,kind", [(5, 16, 1900, 1800, "cell"), (10, 8, 20000, 18000, "cell"), (10, 8, 131073, 65536, "cell"),
+                                          (10, 4, 131073, 65537, "cell"), (17, 32, 20000, 18000, "two"),
+                                          (33, 16, 131072, 131000, "cell"), (33, 16, 300001, 270000, "cell"),
+                                          (33, 8, 140000, 131072, "digit"), (33, 4, 300000, 270000, "two"),
+                                          (42, 4, 140000, 120000, "digit"), (65, 8, 20000, 18000, "cell"),
+                                          (65, 4, 180000, 160000, "two")])
+def test_crowded_points(S, R, F, n, k, kind):
+    """Cells of more points than a warp takes and leading digits of more keys
+    than a block sorts: whole at the limit and cut one past it, segments full
+    and not, up to 27 of them, one and two cut digits, eight and ten low bits,
+    and what the static scratch holds of it."""
+    import torch
+    p = synth.random_params(R=R, F=F, m=3, layers=2, width=32, act=synth.ACT_SINE, seed=R, grid_std=0.5)
+    net, rng = S.Network(p, max_fit_points=n), np.random.default_rng(n)
+    pts, dout = _crowd(kind, n, k, R, n), rng.standard_normal((n, 1), dtype=np.float32)
+    x, d = torch.tensor(pts, device="cuda"), torch.tensor(dout, device="cuda")
+    rg = np.asarray(oracle.net_backward(oracle.OracleNet(p), pts, dout)[2]).ravel()
+    g, w, b = (torch.full_like(t, float("nan")) for t in (net.grid, net.weights, net.biases))
+    S.srn_backward(net.ctx, x, d, g, w, b)
+    assert np.abs(g.cpu().numpy() - rg).max() <= TOL_GRAD * np.abs(rg).max()
+    again = torch.full_like(g, float("nan"))
+    S.srn_backward(net.ctx, x, d, again, w, b)
+    assert torch.equal(g, again)
+    if n * F <= 1200000:
+        S.srn_backward_static(net.cfg, net._params(), x, d, again, w, b)
+        assert np.abs(again.cpu().numpy() - rg).max() <= TOL_GRAD * np.abs(rg).max()
+
+
+@pytest.mark.parametrize("kind,F,m,most", [("cell", 16, 14, 20), ("two", 16, 14, 20)])
+def test_crowded_points_take_their_share_of_the_chip(S, kind, F, m, most):
+    """2^18 points of a two-layer network, all in one cell or pair of cells,
+    against the evenly spread batch: within 20 times (a warp per vertex over
+    the points of its cells takes 19 times, one warp on all points of a cell
+    196)."""
+    import torch
+    n = 1 << 18
+    p = synth.random_params(R=33, F=F, m=m, layers=2, width=32, act=synth.ACT_SNAKEALT, seed=1, grid_std=0.5)
+    net = S.Network(p, max_fit_points=n)
+    d = torch.randn((n, 1), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    g, w, b = (torch.empty_like(t) for t in (net.grid, net.weights, net.biases))
+
+    def us(pts):
+        x, times = torch.tensor(pts, device="cuda"), []
+        for _ in range(12):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            S.srn_backward(net.ctx, x, d, g, w, b)
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(1e3 * t0.elapsed_time(t1))
+        return sorted(times)[len(times) // 2]
+
+    even, crowded = us(np.random.default_rng(1).random((n, 3), dtype=np.float32)), us(_crowd(kind, n, n, 33, 1))
+    print(f"{kind}: {even:.0f} us evenly spread, {crowded:.0f} us crowded")
+    assert crowded <= most * even
