@@ -862,6 +862,7 @@ size_t carve_static(FitScratch& s, const NetDev& net, int n, unsigned char* base
   s.radix_bins = 256;  // 8-bit digits: the smaller histogram keeps the static area's batch
   s.sort_items = static_sort_items();
   const size_t hist_n = 256 * ((nn + s.sort_items - 1) / s.sort_items);
+  s.hist_len = hist_n;
   s.hist = (unsigned int*)take(sizeof(unsigned int) * (hist_n + hist_n / 8192 + 1));
   s.digit_totals = (unsigned int*)take(sizeof(unsigned int) * 256);
   s.cell_start = (unsigned int*)take(sizeof(unsigned int) * (s.n_cells + 1));

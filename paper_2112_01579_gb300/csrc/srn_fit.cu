@@ -27,6 +27,8 @@
 //      the same launch as the vertex gather.
 //   5. Adam over grid, weights and biases (skipped if anything is not
 //      finite), refreshing the FP16 copies.
+#include <limits.h>
+
 #include <algorithm>
 #include <utility>
 
@@ -936,38 +938,92 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const unsign
 }
 
 // Second half of the sort when the leading eight bits of the cell index are
-// in order: one block per leading digit sorts its keys (about n / 256, in
-// chunks of 2048) by the remaining LOW bits in shared memory, stable, and
-// writes the starts of its cells.  In place of a second histogram, scan and
-// scatter over all keys and a pass for the cell starts.
-template <int LOW>
-__global__ void __launch_bounds__(kSortThreads) bucket_sort_kernel(const unsigned int* __restrict__ kin,
-                                                                   const unsigned int* __restrict__ vin,
-                                                                   unsigned int* __restrict__ vout, int n,
-                                                                   int low_bits, unsigned int* __restrict__ cell_start,
-                                                                   long long n_cells,
-                                                                   const unsigned int* __restrict__ totals) {
-  constexpr int NB = 1 << LOW, PER = NB / kSortThreads, ROUNDS = 8;
-  __shared__ unsigned int cnt[8][NB];
-  __shared__ unsigned int next[NB];  // count, then next position of each bin
+// in order: the keys of a leading digit (about n / 256, in chunks of 2048) are
+// sorted by the remaining LOW bits in shared memory, stable, and the starts of
+// the digit's cells written.  In place of a second histogram, scan and scatter
+// over all keys and a pass for the cell starts.
+//
+// One block on a digit's keys is right where points spread.  Where they may
+// crowd (points a caller gave, or drawn by the error), one block could be left
+// with most of the batch: 2^18 points in one digit took 0.3 ms where the rest
+// of the sort takes 0.02.  From kCutFrom points on, digits of more than
+// kBucketWhole keys are therefore cut into segments: the blocks behind the
+// first 256 count them, bucket_split_kernel scatters each from the counts of
+// all.  Both find their segment from the digits' totals; a block without one
+// ends at once (4 us a step, which evenly drawn points do not pay).
+constexpr int kBucketWhole = 65536, kCutFrom = 2 * kBucketWhole, kSegKeys = 8192, kSegMost = 32;
+
+// Keys of a segment of a digit with `total` keys: 8192 at least, at most 32 segments.
+__host__ __device__ inline int seg_len(int total) {
+  const int each = (total + kSegMost - 1) / kSegMost;
+  return each <= kSegKeys ? kSegKeys : (each + 2047) / 2048 * 2048;
+}
+// At least the segments of n keys, however they fall (a cut digit with t >
+// kBucketWhole keys has at most t / 8192 + 1 <= 9 t / 65536 of them).
+inline int seg_count(int n) { return n <= kCutFrom ? 0 : (int)((long long)n * 9 / 65536); }
+inline int bucket_low(int bits) { return bits <= 16 ? 8 : 10; }  // log2 of the bins of one digit
+
+struct Segment {
+  int digit, first, c0, c1;  // leading digit, its first key, the segment's keys
+  int row0, index, rows;     // count rows of the digit's segments: the first, this one, how many
+};
+
+// Segment `id` of all cut digits (256 threads; the same answer in all, digit < 0: none).
+__device__ __forceinline__ Segment find_segment(const unsigned int* __restrict__ totals, int id) {
+  __shared__ int wsum[2][8];
+  __shared__ Segment found;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int total = (int)totals[tid], len = seg_len(total);
+  const int segs = total > kBucketWhole ? (total + len - 1) / len : 0;
+  if (!__syncthreads_or(segs)) return Segment{-1, 0, 0, 0, 0, 0, 0};  // no digit is cut
+  int a = total, b = segs;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, a, off), z = __shfl_up_sync(0xffffffffu, b, off);
+    if (lane >= off) {
+      a += y;
+      b += z;
+    }
+  }
+  if (lane == 31) {
+    wsum[0][w] = a;
+    wsum[1][w] = b;
+  }
+  if (tid == 0) found.digit = -1;
+  __syncthreads();
+  for (int q = 0; q < w; ++q) {
+    a += wsum[0][q];
+    b += wsum[1][q];
+  }
+  const int first = a - total, row0 = b - segs;
+  if (id >= row0 && id < row0 + segs) {
+    const int c0 = first + (id - row0) * len;
+    found = Segment{tid, first, c0, min(c0 + len, first + total), row0, id - row0, segs};
+  }
+  __syncthreads();
+  return found;
+}
+
+// next[low bits] += counts of the keys c0 .. c1 - 1 (one add per value a warp
+// meets, so that equal keys do not queue up).
+__device__ __forceinline__ void count_low(const unsigned int* __restrict__ kin, int c0, int c1, unsigned int mask,
+                                          unsigned int* next) {
+  for (int base = c0; base < c1; base += kSortThreads) {
+    const int i = base + (int)threadIdx.x;
+    const unsigned int d = i < c1 ? kin[i] & mask : 0xFFFFFFFFu;
+    const unsigned int peers = __match_any_sync(0xffffffffu, d);
+    if (i < c1 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&next[d], (unsigned int)__popc(peers));
+  }
+}
+
+// next[bin] (counts of a whole digit) -> the position of the bin's first key,
+// `first` being the digit's; writes the starts of the digit's cells when asked.
+template <int NB>
+__device__ __forceinline__ void scan_bins(unsigned int* next, unsigned int first, unsigned int mask, int digit,
+                                          int low_bits, long long n_cells, unsigned int* __restrict__ cell_start) {
+  constexpr int PER = NB / kSortThreads;  // consecutive bins of a thread
   __shared__ unsigned int wpart[kSortThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  // keys of the smaller leading digits
-  const unsigned int mine = totals[tid];
-  unsigned int before = tid < (int)blockIdx.x ? mine : 0u;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) before += __shfl_xor_sync(0xffffffffu, before, off);
-  if (lane == 0) wpart[w] = before;
-  for (int i = tid; i < NB; i += kSortThreads) next[i] = 0u;
-  __syncthreads();
-  unsigned int first = 0u;
-#pragma unroll
-  for (int q = 0; q < kSortThreads / 32; ++q) first += wpart[q];
-  const int b0 = (int)first, b1 = b0 + (int)totals[blockIdx.x];
-  const unsigned int mask = (1u << low_bits) - 1u;
-  for (int i = b0 + tid; i < b1; i += kSortThreads) atomicAdd(&next[kin[i] & mask], 1u);
-  __syncthreads();
-  // exclusive scan of the bins, PER consecutive ones per thread
   unsigned int v[PER], t = 0u;
 #pragma unroll
   for (int e = 0; e < PER; ++e) {
@@ -987,22 +1043,31 @@ __global__ void __launch_bounds__(kSortThreads) bucket_sort_kernel(const unsigne
 #pragma unroll
   for (int e = 0; e < PER; ++e) {
     const int bin = tid * PER + e;
-    const long long cell = ((long long)blockIdx.x << low_bits) + bin;
-    if (bin <= (int)mask && cell < n_cells) cell_start[cell] = run;
+    const long long cell = ((long long)digit << low_bits) + bin;
+    if (cell_start && bin <= (int)mask && cell < n_cells) cell_start[cell] = run;
     next[bin] = run;
     run += v[e];
   }
-  if (blockIdx.x == 0 && tid == 0) cell_start[n_cells] = (unsigned int)n;
-  for (int c0 = b0; c0 < b1; c0 += ROUNDS * kSortThreads) {
-    const int base = c0 + w * (ROUNDS * 32);
+}
+
+// Stable scatter of the keys c0 .. c1 - 1 of one digit by their low bits from
+// next[bin], the position of the bin's next key.
+template <int NB>
+__device__ __forceinline__ void scatter_low(const unsigned int* __restrict__ kin, const unsigned int* __restrict__ vin,
+                                            unsigned int* __restrict__ vout, int c0, int c1, unsigned int mask,
+                                            unsigned int (*cnt)[NB], unsigned int* next) {
+  constexpr int ROUNDS = 8;
+  const int tid = threadIdx.x, w = tid >> 5;
+  for (int c = c0; c < c1; c += ROUNDS * kSortThreads) {
+    const int base = c + w * (ROUNDS * 32);
     unsigned int key[ROUNDS], val[ROUNDS];
-    load_keys<ROUNDS>(kin, base, b1, key);
-    load_keys<ROUNDS>(vin, base, b1, val);
+    load_keys<ROUNDS>(kin, base, c1, key);
+    load_keys<ROUNDS>(vin, base, c1, val);
 #pragma unroll
     for (int r = 0; r < ROUNDS; ++r) key[r] &= mask;
     for (int i = tid; i < 8 * NB; i += kSortThreads) (&cnt[0][0])[i] = 0u;
     __syncthreads();
-    warp_digit_counts<NB, ROUNDS>(key, base, b1, 0, cnt[w]);
+    warp_digit_counts<NB, ROUNDS>(key, base, c1, 0, cnt[w]);
     __syncthreads();
     for (int d = tid; d < NB; d += kSortThreads) {
       unsigned int at = next[d];
@@ -1015,9 +1080,98 @@ __global__ void __launch_bounds__(kSortThreads) bucket_sort_kernel(const unsigne
       next[d] = at;
     }
     __syncthreads();
-    warp_scatter<NB, ROUNDS>(key, val, base, b1, 0, cnt[w], nullptr, vout);
+    warp_scatter<NB, ROUNDS>(key, val, base, c1, 0, cnt[w], nullptr, vout);
     __syncthreads();
   }
+}
+
+template <int LOW>
+__global__ void __launch_bounds__(kSortThreads) bucket_sort_kernel(const unsigned int* __restrict__ kin,
+                                                                   const unsigned int* __restrict__ vin,
+                                                                   unsigned int* __restrict__ vout, int n,
+                                                                   int low_bits, unsigned int* __restrict__ cell_start,
+                                                                   long long n_cells,
+                                                                   const unsigned int* __restrict__ totals, int whole,
+                                                                   unsigned int* __restrict__ seg_counts) {
+  constexpr int NB = 1 << LOW;
+  __shared__ unsigned int cnt[8][NB];
+  __shared__ unsigned int next[NB];
+  __shared__ unsigned int wpart[kSortThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const unsigned int mask = (1u << low_bits) - 1u;
+  for (int i = tid; i < NB; i += kSortThreads) next[i] = 0u;
+  if (blockIdx.x >= 256) {
+    const int id = (int)blockIdx.x - 256;
+    const Segment s = find_segment(totals, id);
+    if (s.digit < 0) return;
+    count_low(kin, s.c0, s.c1, mask, next);
+    __syncthreads();
+    for (int i = tid; i < NB; i += kSortThreads) seg_counts[(size_t)id * NB + i] = next[i];
+    return;
+  }
+  // keys of the smaller leading digits
+  unsigned int before = tid < (int)blockIdx.x ? totals[tid] : 0u;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) before += __shfl_xor_sync(0xffffffffu, before, off);
+  if (lane == 0) wpart[w] = before;
+  __syncthreads();
+  unsigned int first = 0u;
+#pragma unroll
+  for (int q = 0; q < kSortThreads / 32; ++q) first += wpart[q];
+  if (blockIdx.x == 0 && tid == 0) cell_start[n_cells] = (unsigned int)n;
+  const int total = (int)totals[blockIdx.x];
+  if (total > whole) return;  // bucket_split_kernel's
+  const int b0 = (int)first, b1 = b0 + total;
+  for (int i = b0 + tid; i < b1; i += kSortThreads) atomicAdd(&next[kin[i] & mask], 1u);
+  __syncthreads();
+  scan_bins<NB>(next, first, mask, (int)blockIdx.x, low_bits, n_cells, cell_start);
+  scatter_low<NB>(kin, vin, vout, b0, b1, mask, cnt, next);
+}
+
+template <int LOW>
+__global__ void __launch_bounds__(kSortThreads) bucket_split_kernel(const unsigned int* __restrict__ kin,
+                                                                    const unsigned int* __restrict__ vin,
+                                                                    unsigned int* __restrict__ vout, int low_bits,
+                                                                    unsigned int* __restrict__ cell_start,
+                                                                    long long n_cells,
+                                                                    const unsigned int* __restrict__ totals,
+                                                                    const unsigned int* __restrict__ seg_counts) {
+  constexpr int NB = 1 << LOW;
+  __shared__ unsigned int cnt[8][NB];
+  __shared__ unsigned int next[NB], before[NB];
+  const int tid = threadIdx.x;
+  const Segment s = find_segment(totals, (int)blockIdx.x);
+  if (s.digit < 0) return;
+  for (int i = tid; i < NB; i += kSortThreads) {
+    unsigned int all = 0u, b = 0u;
+    const unsigned int* row = seg_counts + (size_t)s.row0 * NB + i;
+#pragma unroll 8
+    for (int q = 0; q < s.rows; ++q) {
+      const unsigned int c = row[(size_t)q * NB];
+      all += c;
+      b += q < s.index ? c : 0u;
+    }
+    next[i] = all;
+    before[i] = b;
+  }
+  __syncthreads();
+  const unsigned int mask = (1u << low_bits) - 1u;
+  scan_bins<NB>(next, (unsigned int)s.first, mask, s.digit, low_bits, n_cells, s.index == 0 ? cell_start : nullptr);
+  __syncthreads();
+  for (int i = tid; i < NB; i += kSortThreads) next[i] += before[i];
+  scatter_low<NB>(kin, vin, vout, s.c0, s.c1, mask, cnt, next);
+}
+
+// segs: blocks for the segments of crowded digits (seg_count; 0: no digit is cut).
+template <int LOW>
+void launch_buckets(const unsigned int* kin, const unsigned int* vin, unsigned int* vout, int n, int bits,
+                    unsigned int* cell_start, long long n_cells, const unsigned int* totals, int segs,
+                    unsigned int* seg_counts, cudaStream_t st) {
+  bucket_sort_kernel<LOW><<<256 + segs, kSortThreads, 0, st>>>(kin, vin, vout, n, bits - 8, cell_start, n_cells,
+                                                               totals, segs > 0 ? kBucketWhole : INT_MAX, seg_counts);
+  if (segs > 0)
+    bucket_split_kernel<LOW><<<segs, kSortThreads, 0, st>>>(kin, vin, vout, bits - 8, cell_start, n_cells, totals,
+                                                            seg_counts);
 }
 
 // cell_start[c] = first sorted position with key >= c, for c in [0, n_cells].
@@ -1633,14 +1787,17 @@ cudaError_t run_backward(FitScratch& s, const NetDev& net, PointArgs pa, float* 
   const bool small_blocks = s.sort_items == kSortItemsSmall;
   const int nblocks = (n + s.sort_items - 1) / s.sort_items;
   // up to 512 cells: one pass with 9-bit digits; up to 2^18 cells: the leading
-  // eight bits, then each leading digit's keys in one block (18 bits leave ten,
-  // 32 KB of counters); else 8-bit digits from the lowest
+  // eight bits, then each leading digit's keys by themselves (18 bits leave
+  // ten, 32 KB of counters) where the counts of crowded digits find room (not
+  // in the static area past 2^16 cells); else 8-bit digits from the lowest
   const bool one_pass = s.radix_bins == 512 && bits <= 9;
-  const bool buckets = !one_pass && bits > 9 && bits <= 18 && nblocks <= kDigitThreads * kDigitPer;
+  const int segs = pa.mode == 0 && !pa.cdf ? 0 : seg_count(n);  // evenly drawn points do not crowd
+  const bool buckets = !one_pass && bits > 9 && bits <= 18 && nblocks <= kDigitThreads * kDigitPer &&
+                       ((size_t)segs << bucket_low(bits)) <= s.hist_len;
   const int dbits = one_pass ? 9 : 8;
   const int hist_m = (1 << dbits) * nblocks;
   const int nseg = (hist_m + kScanTile - 1) / kScanTile;  // one 8192-value tile per scan block
-  unsigned int* seg_sums = s.hist + (size_t)s.radix_bins * (size_t)((s.max_points + s.sort_items - 1) / s.sort_items);
+  unsigned int* seg_sums = s.hist + s.hist_len;
   bool starts_done = false;
   for (int shift = buckets ? bits - 8 : 0; shift < bits && n > 0; shift += dbits) {
     // a single pass leaves the cell starts to the scatter kernel
@@ -1668,12 +1825,11 @@ cudaError_t run_backward(FitScratch& s, const NetDev& net, PointArgs pa, float* 
     std::swap(k_in, k_out);
     std::swap(v_in, v_out);
     if (buckets) {
-      if (bits <= 16)
-        bucket_sort_kernel<8><<<256, kSortThreads, 0, st>>>(k_in, v_in, v_out, n, bits - 8, s.cell_start,
-                                                            (long long)s.n_cells, totals);
+      // the histogram's space is free again: the counts of the segments
+      if (bucket_low(bits) == 8)
+        launch_buckets<8>(k_in, v_in, v_out, n, bits, s.cell_start, (long long)s.n_cells, totals, segs, s.hist, st);
       else
-        bucket_sort_kernel<10><<<256, kSortThreads, 0, st>>>(k_in, v_in, v_out, n, bits - 8, s.cell_start,
-                                                             (long long)s.n_cells, totals);
+        launch_buckets<10>(k_in, v_in, v_out, n, bits, s.cell_start, (long long)s.n_cells, totals, segs, s.hist, st);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       std::swap(v_in, v_out);
     }
@@ -1747,8 +1903,11 @@ cudaError_t fit_scratch_alloc(FitScratch& s, const NetDev& net, int max_points) 
   alloc((void**)&s.idx, sizeof(unsigned int) * n);
   alloc((void**)&s.idx_alt, sizeof(unsigned int) * n);
   s.radix_bins = sort_bins(s.n_cells);
-  // radix histograms, then the per-segment sums of their scan
-  alloc((void**)&s.hist, sizeof(unsigned int) * (s.radix_bins * nsb + (s.radix_bins * nsb) / 8192 + 1));
+  // radix histograms, which also hold the counts of crowded digits (of 2^10
+  // bins past 2^16 cells), then the per-segment sums of their scan
+  s.hist_len = s.radix_bins * nsb;
+  if (s.n_cells > 65536) s.hist_len = std::max(s.hist_len, (size_t)seg_count(max_points) << 10);
+  alloc((void**)&s.hist, sizeof(unsigned int) * (s.hist_len + (s.radix_bins * nsb) / 8192 + 1));
   alloc((void**)&s.digit_totals, sizeof(unsigned int) * s.radix_bins);
   alloc((void**)&s.cell_start, sizeof(unsigned int) * (s.n_cells + 1));
   alloc((void**)&s.part, sizeof(float) * (size_t)s.max_cta * (s.n_entries + 1));

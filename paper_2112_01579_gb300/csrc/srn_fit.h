@@ -14,6 +14,7 @@ struct FitScratch {
   size_t n_grid;           // latent-grid entries over all keyframes
   int radix_bins;          // 256 (8-bit digits) or 512 (one 9-bit pass for up to 512 cells)
   int sort_items;          // keys per sort block (1024 or 2048)
+  size_t hist_len;         // entries of hist before the sums of its scan
   float* pts;              // [n][3] positions (clamped) of the current step
   float* dz;               // [n][F] adjoint of the latent vector
   unsigned int* key;       // [n] cell of each point, and radix ping-pong
