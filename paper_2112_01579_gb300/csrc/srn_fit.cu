@@ -338,7 +338,7 @@ __device__ __forceinline__ void outer_sum(float (&acc)[4][NJ], const float* d, c
   }
 }
 
-// Sum of one row's 32 values (times w's, when given), four interleaved sums.
+// Sum of one row's 32 values, and of two rows' products, in four interleaved sums.
 __device__ __forceinline__ float row_sum(const float* r) {
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
   const Latent lat = make_latent(net, a.time);
   const float inv_n = 1.0f / (float)a.n;
   const int D = t.D, nchunks = (a.n + kFitThreads - 1) / kFitThreads;
-  const int mode = net.act == SRN_ACT_SNAKEALT ? 1 : 0;
+  const bool snake = net.act == SRN_ACT_SNAKEALT;
 
   float g0[4][3], gh[NL > 2 ? NL - 2 : 1][4][2], gb[NH], gl[4], gbl = 0.f, loss_acc = 0.f;
 #pragma unroll
@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
     tile32::Acc<C> x, df[NH];
     tile32::set_bias<C>(x, sm + t.ob0);
     tile32::layer<C, VS>(x, v0, sm + t.oW0, t.d0);
-    tile32::activate_call<C>(mode, x, df[0]);
+    tile32::activate_call<C>(snake, x, df[0]);
     if (PARK) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
       const float* W = sm + t.oHid + (h - 1) * t.hidStride;
       tile32::set_bias<C>(x, W + C * C);
       tile32::layer<C, S>(x, act0 + (h - 1) * C * S, W, C);
-      tile32::activate_call<C>(mode, x, df[h]);
+      tile32::activate_call<C>(snake, x, df[h]);
       tile32::put<C, S>(x, act0 + h * C * S);
       __syncwarp();
     }
@@ -648,7 +648,7 @@ size_t fit_tile_smem(const NetDev& net) {
 }
 // Up to four layers: their activation derivatives fit a thread's registers
 // (32 a layer), and with at most 48 inputs two CTAs' rows fit an SM's shared
-// memory (100 KB a CTA).  Deeper or wider-input networks keep
+// memory (113 KB a CTA).  Deeper or wider-input networks keep
 // fit_point_kernel, which stashes in local memory.
 bool fit_tile_supported(const NetDev& net) {
   return net.c == 32 && net.l >= 2 && net.l <= 4 && net_d0(net) <= kTileMaxIn && net.F <= 32;

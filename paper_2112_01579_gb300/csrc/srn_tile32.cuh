@@ -221,16 +221,15 @@ __device__ __forceinline__ bool nerf_rows(const float* F, int m) {
   return __syncthreads_and(ok) != 0;
 }
 
-// Activation values of four arguments, and their derivatives.  mode: bit 0
-// SnakeAlt, bit 1 by the library functions.
+// Activation values of four arguments, and their derivatives.
 struct Quad {
   float4 a, d;
 };
-__device__ __forceinline__ Quad act_quad(float4 x, int mode) {
+__device__ __forceinline__ Quad act_quad(float4 x, bool snake) {
   Quad r;
-  if ((mode & 2) || !(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))) <= kActMax)) {
+  if (!(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))) <= kActMax)) {
     const float4 p = sincos_pair(x.x, x.y), q = sincos_pair(x.z, x.w);
-    if (mode & 1) {
+    if (snake) {
       r.a = make_float4(fmaf(0.5f, x.x, p.x * p.x), fmaf(0.5f, x.y, p.z * p.z), fmaf(0.5f, x.z, q.x * q.x),
                         fmaf(0.5f, x.w, q.z * q.z));
       r.d = make_float4(0.5f + 2.0f * p.x * p.y, 0.5f + 2.0f * p.z * p.w, 0.5f + 2.0f * q.x * q.y,
@@ -246,7 +245,7 @@ __device__ __forceinline__ Quad act_quad(float4 x, int mode) {
     const float2 v = h ? make_float2(x.z, x.w) : make_float2(x.x, x.y);
     float2 t, a, d;
     const float2 e = reduce_pi(v, t), z = __fmul2_rn(e, e), s = sin_half(e, z), c = cos_half(e);
-    if (mode & 1) {  // sin^2 and sin cos do not change with k
+    if (snake) {  // sin^2 and sin cos do not change with k
       a = __ffma2_rn(s, s, __fmul2_rn(v, f2(0.5f)));
       d = __ffma2_rn(__fadd2_rn(s, s), c, f2(0.5f));
     } else {
@@ -260,16 +259,16 @@ __device__ __forceinline__ Quad act_quad(float4 x, int mode) {
 }
 // Out of line: a kernel that activates several unrolled layers would not fit
 // the instruction cache with the code inlined at every value.
-static __device__ __noinline__ Quad act_quad_call(float4 x, int mode) { return act_quad(x, mode); }
+static __device__ __noinline__ Quad act_quad_call(float4 x, bool snake) { return act_quad(x, snake); }
 
 // Activation and derivative of the lane's values by act_quad_call.
 template <int C>
-__device__ __forceinline__ void activate_call(int mode, Acc<C>& a, Acc<C>& d) {
+__device__ __forceinline__ void activate_call(bool snake, Acc<C>& a, Acc<C>& d) {
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int q = 0; q < C / 8; q += 2) {
-      const Quad r = act_quad_call(make_float4(a.v[i][q].x, a.v[i][q].y, a.v[i][q + 1].x, a.v[i][q + 1].y), mode);
+      const Quad r = act_quad_call(make_float4(a.v[i][q].x, a.v[i][q].y, a.v[i][q + 1].x, a.v[i][q + 1].y), snake);
       a.v[i][q] = make_float2(r.a.x, r.a.y);
       a.v[i][q + 1] = make_float2(r.a.z, r.a.w);
       d.v[i][q] = make_float2(r.d.x, r.d.y);
@@ -348,17 +347,16 @@ __device__ __forceinline__ void put_latent(float* z, const Latent& lat, float3 p
 
 // Input rows of the lane's point p (+ pl, the low part of a position carried
 // as a pair): [p, sin, cos, z, (t)].
-// NeRF Fourier rows (nerf) take the inline quarter-turn form.  AHEAD: the
-// latent gather first, so that its loads are in flight during the features
-// (kernels with registers to spare: error grid 3.41 -> 3.37 ms; the fit's
-// point kernel spills and loses 5 %).
-template <int S, bool AHEAD = true>
+// NeRF Fourier rows (nerf) take the inline quarter-turn form.  The latent
+// gather of the usual channel counts goes first, so that its loads are in
+// flight during the features (error grid 3.41 -> 3.37 ms).
+template <int S>
 __device__ __forceinline__ void put_inputs(float* x, const float* sm, const Net& t, const Latent& lat, bool nerf,
                                            float3 p, float3 pl = make_float3(0.f, 0.f, 0.f)) {
   float* v = x + (threadIdx.x & 31);
   float* z = v + (3 + 2 * t.m) * S;
-  if (AHEAD && t.F == 16) put_latent<S, 16>(z, lat, p);
-  else if (AHEAD && t.F == 8) put_latent<S, 8>(z, lat, p);
+  if (t.F == 16) put_latent<S, 16>(z, lat, p);
+  else if (t.F == 8) put_latent<S, 8>(z, lat, p);
   v[0] = p.x;
   v[S] = p.y;
   v[2 * S] = p.z;
@@ -385,7 +383,7 @@ __device__ __forceinline__ void put_inputs(float* x, const float* sm, const Net&
       v[(4 + 2 * k) * S] = c;
     }
   }
-  if (!AHEAD || (t.F != 16 && t.F != 8))
+  if (t.F != 16 && t.F != 8)
     for (int f = 0; f < t.F; f += 4) put_latent<S, 4>(z + f * S, lat, p, f);
   if (t.ti) z[t.F * S] = lat.tin;
 }
