@@ -187,3 +187,36 @@ def test_render_of_wide_inputs(S, width, layers, F, m, D, shading):
         ref, _, _ = oracle.render(on, cams, otf, 17, 12, 1 / 24, 2.0)
         err, lim = np.abs(out.cpu().numpy() - ref).max(axis=-1).ravel(), tol
     assert tol < 1e-2 and (err <= lim).all(), (err.max(), tol)
+
+
+@pytest.mark.parametrize("path", ["density_grad", "backward"])
+@pytest.mark.parametrize("scale", [4.0, 64.0])
+def test_sine_derivative_is_a_cosine_to_a_rounding(S, path, scale):
+    """One sine neuron, arguments exact in FP32 (4913 vertices of a 17^3 grid
+    spell multiples of 2^-10 times scale / 4), weights powers of two, one
+    point per vertex: what comes back is the cosine alone.  Its rms error is
+    at most 1.45 times that of the correctly rounded one (CUDA's own cosine:
+    1.35; sin(pi / 2 - |r|) from a reduced r: 1.8)."""
+    import torch
+    p = synth.random_params(R=17, F=4, m=0, layers=2, width=32, act=synth.ACT_SINE, seed=1)
+    p["grid"] = np.zeros_like(p["grid"])
+    for a in p["weights"] + p["biases"]:
+        a[:] = 0.0
+    p["weights"][0][0, :4] = [scale, scale / 16, scale / 256, 1.0]
+    p["weights"][1][0, 0] = 1.0
+    i = np.arange(17 ** 3)
+    v = np.stack([i % 17, i // 17 % 17, i // 289], 1)
+    pts = (v / 16.0).astype(np.float32)
+    arg = pts.astype(np.float64) @ np.array([scale, scale / 16, scale / 256])
+    want = np.cos(arg)
+    net, x = S.Network(p, max_fit_points=len(i)), torch.tensor(pts, device="cuda")
+    if path == "backward":
+        g, w, b = (torch.empty_like(t) for t in (net.grid, net.weights, net.biases))
+        S.srn_backward(net.ctx, x, torch.ones((len(i), 1), device="cuda"), g, w, b)
+        got = g.cpu().numpy().reshape(-1, 4)[:, 0]  # vertex order is x fastest, as i
+    else:
+        rho, grad = torch.empty(len(i), device="cuda"), torch.empty((len(i), 3), device="cuda")
+        S.srn_density_grad(net.ctx, x, rho, grad)
+        got = grad.cpu().numpy()[:, 0] / scale
+    rms = lambda e: float(np.sqrt(np.mean(e ** 2)))  # noqa: E731
+    assert rms(got - want) <= 1.45 * rms(want.astype(np.float32) - want)
