@@ -375,7 +375,7 @@ __device__ __forceinline__ void store_dz(const float* d, const float* Wz, float*
   }
 }
 
-template <int NL>
+template <int NL, bool SNAKE>
 __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_constant__ NetDev net,
                                                                   const __grid_constant__ PointArgs a,
                                                                   const __grid_constant__ tile32::Net t, int wfloats) {
@@ -399,7 +399,6 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
   const Latent lat = make_latent(net, a.time);
   const float inv_n = 1.0f / (float)a.n;
   const int D = t.D, nchunks = (a.n + kFitThreads - 1) / kFitThreads;
-  const bool snake = net.act == SRN_ACT_SNAKEALT;
 
   float g0[4][3], gh[NL > 2 ? NL - 2 : 1][4][2], gb[NH], gl[4], gbl = 0.f, loss_acc = 0.f;
 #pragma unroll
@@ -431,7 +430,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
     tile32::Acc<C> x, df[NH];
     tile32::set_bias<C>(x, sm + t.ob0);
     tile32::layer<C, VS>(x, v0, sm + t.oW0, t.d0);
-    tile32::activate_call<C>(snake, x, df[0]);
+    tile32::activate_call<C, SNAKE>(x, df[0]);
     if (PARK) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -447,7 +446,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) fit_tile_kernel(const __grid_c
       const float* W = sm + t.oHid + (h - 1) * t.hidStride;
       tile32::set_bias<C>(x, W + C * C);
       tile32::layer<C, S>(x, act0 + (h - 1) * C * S, W, C);
-      tile32::activate_call<C>(snake, x, df[h]);
+      tile32::activate_call<C, SNAKE>(x, df[h]);
       tile32::put<C, S>(x, act0 + h * C * S);
       __syncwarp();
     }
@@ -656,7 +655,9 @@ bool fit_tile_supported(const NetDev& net) {
 
 template <int NL>
 cudaError_t fit_tile_t(const NetDev& net, const PointArgs& pa, int grid, cudaStream_t st) {
-  auto k = fit_tile_kernel<NL>;
+  // an instantiation for each activation: one for both, whose out-of-line
+  // activation holds the code of both, took 8 us more of a 300 us step
+  auto k = net.act == SRN_ACT_SNAKEALT ? fit_tile_kernel<NL, true> : fit_tile_kernel<NL, false>;
   const size_t smem = fit_tile_smem(net);
   cudaError_t e = tile32::allow_dynamic(k);
   if (e != cudaSuccess) return e;

@@ -281,22 +281,20 @@ __device__ __forceinline__ Quad act_quad(float4 x, bool snake) {
   return r;
 }
 // Out of line: a kernel that activates several unrolled layers would not fit
-// the instruction cache with the code inlined at every value.  A function for
-// each activation: one for both took 4 us more of a 300 us fit step.
+// the instruction cache with the code inlined at every value.
 template <bool SNAKE>
 __device__ __noinline__ Quad act_quad_call(float4 x) {
   return act_quad(x, SNAKE);
 }
 
 // Activation and derivative of the lane's values by act_quad_call.
-template <int C>
-__device__ __forceinline__ void activate_call(bool snake, Acc<C>& a, Acc<C>& d) {
+template <int C, bool SNAKE>
+__device__ __forceinline__ void activate_call(Acc<C>& a, Acc<C>& d) {
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int q = 0; q < C / 8; q += 2) {
-      const float4 v = make_float4(a.v[i][q].x, a.v[i][q].y, a.v[i][q + 1].x, a.v[i][q + 1].y);
-      const Quad r = snake ? act_quad_call<true>(v) : act_quad_call<false>(v);
+      const Quad r = act_quad_call<SNAKE>(make_float4(a.v[i][q].x, a.v[i][q].y, a.v[i][q + 1].x, a.v[i][q + 1].y));
       a.v[i][q] = make_float2(r.a.x, r.a.y);
       a.v[i][q + 1] = make_float2(r.a.z, r.a.w);
       d.v[i][q] = make_float2(r.d.x, r.d.y);
