@@ -22,7 +22,7 @@ using namespace net32;
 
 constexpr int kCdfThreads = kCdfBlock / 2;  // two weights per thread
 
-template <int C>
+template <int C, bool WIDE>
 __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     error_grid_kernel(const NetDev net, const VolDev vol, int res, int spv, unsigned long long seed, float time,
                       float* __restrict__ E, const tile32::Net t, int rows) {
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
       const uint4 o = sample::philox4x32_10(make_uint4((unsigned)v, (unsigned)i, 0x4552u, 0u), key);
       const float3 p = make_float3(sample::voxel_coord(vx, o.x, res), sample::voxel_coord(vy, o.y, res),
                                    sample::voxel_coord(vz, o.z, res));
-      tile32::forward<C, false>(ctx, x, x, lat, p, zero, nullptr);
+      tile32::forward<C, false, WIDE>(ctx, x, x, lat, p, zero, nullptr);
       acc += fabsf(tile32::last_layer<C, tile32::kPts>(x, sm, t, 0) - vol_sample(vol, p));
       __syncwarp();
     }
@@ -62,9 +62,9 @@ cudaError_t error_grid_t(const NetDev& net, const VolDev& vol, int res, int spv,
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const long long tiles = ((long long)res * res * res + 31) / 32;
-  const int rows = t.d0 > C ? t.d0 : C, warps = tile32::warps_for(t, C, rows, tiles, sms);
+  const int rows = t.rows > C ? t.rows : C, warps = tile32::warps_for(t, C, rows, tiles, sms);
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
-  auto k = error_grid_kernel<C>;
+  auto k = t.wide ? error_grid_kernel<C, true> : error_grid_kernel<C, false>;
   e = tile32::allow_dynamic(k);
   if (e != cudaSuccess) return e;
   const long long blocks = (tiles + warps - 1) / warps, most = (long long)(tile32::max_warps(C) / warps) * sms;

@@ -20,27 +20,27 @@ using namespace net32;
 // Rows of 32 floats a warp's tile needs: the inputs and activations share
 // one block, unless the backward needs the inputs again.
 inline int tile_rows(const tile32::Net& t, int C, bool adjoint, bool dout) {
-  return (adjoint ? t.d0 + C : (t.d0 > C ? t.d0 : C)) + (dout ? 4 : 0);
+  return (adjoint ? t.rows + C : (t.rows > C ? t.rows : C)) + (dout ? 4 : 0);
 }
 
 // Density (and gradient for shading) at the lanes' positions p + pl (pairs)
 // for shading mode SH; the finite-difference neighbours are offset as pairs.
 // All lanes of the warp take part.
-template <int C, int SH>
+template <int C, int SH, bool WIDE>
 __device__ __forceinline__ float sample_field(const tile32::Ctx& c, float* rows, const Latent& lat, float3 p,
                                               float3 pl, float fd_h, float3& g) {
   constexpr int S = tile32::kPts;
   const tile32::Net& t = *c.t;
   if constexpr (SH == SRN_SHADE_ADJOINT) {
-    float* x = rows + t.d0 * S;
+    float* x = rows + t.rows * S;
     tile32::Acc<C> df[kMaxL - 1], a;
-    tile32::forward<C, true>(c, rows, x, lat, p, pl, df);
+    tile32::forward<C, true, WIDE>(c, rows, x, lat, p, pl, df);
     const float rho = tile32::last_layer<C, S>(x, c.sm, t, 0);
     tile32::seed<C>(a, c.sm, t, nullptr);
-    g = tile32::input_gradient<C>(c, rows, x, lat, p, a, df);
+    g = tile32::input_gradient<C, WIDE>(c, rows, x, lat, p, a, df);
     return rho;
   } else {
-    tile32::forward<C, false>(c, rows, rows, lat, p, pl, nullptr);
+    tile32::forward<C, false, WIDE>(c, rows, rows, lat, p, pl, nullptr);
     const float rho = tile32::last_layer<C, S>(rows, c.sm, t, 0);
     if constexpr (SH == SRN_SHADE_HEAD)
       g = make_float3(tile32::last_layer<C, S>(rows, c.sm, t, 1), tile32::last_layer<C, S>(rows, c.sm, t, 2),
@@ -52,7 +52,7 @@ __device__ __forceinline__ float sample_field(const tile32::Ctx& c, float* rows,
       for (int k = 0; k < 6; ++k) {
         float3 qh = p, ql = pl;
         df::offset_axis(qh, ql, k >> 1, (k & 1) ? -fd_h : fd_h);
-        tile32::forward<C, false>(c, rows, rows, lat, qh, ql, nullptr);
+        tile32::forward<C, false, WIDE>(c, rows, rows, lat, qh, ql, nullptr);
         const float v = tile32::last_layer<C, S>(rows, c.sm, t, 0);
         __syncwarp();
 #pragma unroll
@@ -71,7 +71,7 @@ __device__ __forceinline__ float sample_field(const tile32::Ctx& c, float* rows,
 // order over the K lanes; samples past the one that ends the ray are dropped
 // (at most K - 1 a ray).  Large images take K = 1; small ones have too few
 // rays to fill the chip, and their time is a ray's chain of samples.
-template <int C, int SH>
+template <int C, int SH, bool WIDE>
 __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     render_fp32_kernel(const NetDev net, const BatchDev b, const tile32::Net t, int rows, int log2k) {
   extern __shared__ float4 smem4[];
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     if (!__any_sync(0xffffffffu, have)) break;
     // lanes without a sample evaluate their last position (or the centre); nothing reads the result
     float3 g = make_float3(0.f, 0.f, 0.f);
-    const float rho = sample_field<C, SH>(ctx, mine, lat, p, pl, b.fd_h, g);
+    const float rho = sample_field<C, SH, WIDE>(ctx, mine, lat, p, pl, b.fd_h, g);
     __syncwarp();
     float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
     if (have) {
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
 // Point evaluation: mode 0 writes out[n][D]; mode 1 writes rho[n] and the
 // adjoint gradient grad[n][3] (when grad is not null); mode 2 writes the
 // input vector-Jacobian product grad[n][3] = sum_d dout[n][d] d out_d / d p.
-template <int C, int MODE>
+template <int C, int MODE, bool WIDE>
 __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     eval_fp32_kernel(const NetDev net, const float* __restrict__ pts, int n, float time, float* __restrict__ out,
                      float* __restrict__ grad, const float* __restrict__ dout, const tile32::Net t, int rows) {
@@ -171,16 +171,16 @@ __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
     const float3 p = valid ? clamp_p(make_float3(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2]))
                            : make_float3(0.5f, 0.5f, 0.5f);
     if constexpr (MODE == 0) {
-      tile32::forward<C, false>(ctx, mine, mine, lat, p, zero, nullptr);
+      tile32::forward<C, false, WIDE>(ctx, mine, mine, lat, p, zero, nullptr);
       for (int d = 0; d < t.D; ++d) {
         const float v = tile32::last_layer<C, S>(mine, sm, t, d);
         if (valid) out[(size_t)j * t.D + d] = v;
       }
     } else {
-      float* x = mine + t.d0 * S;
+      float* x = mine + t.rows * S;
       float* seeds = x + C * S;
       tile32::Acc<C> df[kMaxL - 1], a;
-      tile32::forward<C, true>(ctx, mine, x, lat, p, zero, df);
+      tile32::forward<C, true, WIDE>(ctx, mine, x, lat, p, zero, df);
       if constexpr (MODE == 1) {
         const float v = tile32::last_layer<C, S>(x, sm, t, 0);
         if (valid) out[j] = v;
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
         tile32::seed<C>(a, sm, t, seeds);
       }
       if (grad) {
-        const float3 g = tile32::input_gradient<C>(ctx, mine, x, lat, p, a, df);
+        const float3 g = tile32::input_gradient<C, WIDE>(ctx, mine, x, lat, p, a, df);
         if (valid) {
           grad[3 * j] = g.x;
           grad[3 * j + 1] = g.y;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(32 * tile32::max_warps(C), 1)
 
 template <int C, int SH>
 cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s) {
-  const tile32::Net t = tile32::make_net(net);
+  const tile32::Net t = tile32::make_net(net, SH == SRN_SHADE_ADJOINT);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -222,7 +222,7 @@ cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s
   const int rows = tile_rows(t, C, SH == SRN_SHADE_ADJOINT, false);
   const int warps = tile32::warps_for(t, C, rows, 0, sms, (int)sizeof(TFDev));
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
-  auto k = render_fp32_kernel<C, SH>;
+  auto k = t.wide ? render_fp32_kernel<C, SH, true> : render_fp32_kernel<C, SH, false>;
   e = tile32::allow_dynamic(k, (int)sizeof(TFDev));
   if (e != cudaSuccess) return e;
   const long long blocks = (tiles + warps - 1) / warps;
@@ -233,7 +233,7 @@ cudaError_t launch_render_t(const NetDev& net, const BatchDev& b, cudaStream_t s
 template <int C, int MODE>
 cudaError_t launch_eval_t(const NetDev& net, const float* pts, int n, float time, float* out, float* grad,
                           const float* dout, cudaStream_t s) {
-  const tile32::Net t = tile32::make_net(net);
+  const tile32::Net t = tile32::make_net(net, MODE != 0);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -241,12 +241,12 @@ cudaError_t launch_eval_t(const NetDev& net, const float* pts, int n, float time
   const long long tiles = ((long long)n + 31) / 32;
   const int rows = tile_rows(t, C, MODE != 0, MODE == 2), warps = tile32::warps_for(t, C, rows, tiles, sms);
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
-  auto k = eval_fp32_kernel<C, MODE>;
+  auto k = t.wide ? eval_fp32_kernel<C, MODE, true> : eval_fp32_kernel<C, MODE, false>;
   e = tile32::allow_dynamic(k);
   if (e != cudaSuccess) return e;
-  // CTAs stage the parameters once and walk the tiles: as many as an SM holds
-  const long long blocks = (tiles + warps - 1) / warps, most = (long long)(tile32::max_warps(C) / warps) * sms;
-  k<<<(unsigned)(blocks < most ? blocks : most), 32 * warps, smem, s>>>(net, pts, n, time, out, grad, dout, t, rows);
+  // CTAs stage the parameters once and walk the tiles: one per SM, by which warps were counted
+  const long long blocks = (tiles + warps - 1) / warps;
+  k<<<(unsigned)(blocks < sms ? blocks : sms), 32 * warps, smem, s>>>(net, pts, n, time, out, grad, dout, t, rows);
   return cudaGetLastError();
 }
 

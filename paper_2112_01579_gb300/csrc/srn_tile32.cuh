@@ -35,9 +35,24 @@ constexpr int kPts = 32;  // points of a warp's tile
 struct Net {
   int d0, l, D, m, F, ti;
   int oF, oW0, ob0, oHid, hidStride, oWl, obl, total;
+  int rows;   // rows of 32 floats that a warp keeps of its inputs
+  bool wide;  // more inputs than that: see put_block
 };
 
-inline Net make_net(const NetDev& n) {
+// Networks of more than kWideIn inputs run layer 0 in blocks of rows, so that
+// a warp's tile leaves room for others (rows for 235 inputs: six warps an SM).
+// 300,000 points of 4 layers of 32, with all rows -> in blocks (a thread per
+// point): 155 inputs 276 -> 207 us (277), 255 inputs 472 -> 270 (364), 8 layers
+// of 64 and 255 inputs 1480 -> 680 (1776); a 400 x 300 frame of those 24.4 ->
+// 7.3 ms (13.4).  At 127 inputs and less there is nothing to gain.  A gradient
+// evaluates its Fourier rows twice that way; at width 32, where they are the
+// larger part, that pays later (169 inputs 412 -> 495 us, 255 842 -> 705).
+constexpr int kWideIn = 128, kWideInGradient32 = 192;
+constexpr int kBlockFeatures = 32, kBlockChannels = 64;  // Fourier rows, latent channels of a block
+constexpr int kBlockLow = 3 + 2 * kBlockFeatures + 1;    // first of three rows that keep the positions' low parts
+constexpr int kBlockRows = kBlockLow + 3;
+
+inline Net make_net(const NetDev& n, bool gradient = false) {
   Net t;
   const int C = n.c;
   t.d0 = net_d0(n); t.l = n.l; t.D = n.D; t.m = n.m; t.F = n.F; t.ti = n.ti;
@@ -50,6 +65,8 @@ inline Net make_net(const NetDev& n) {
   t.oWl = o; o += n.D * C;
   t.obl = o; o += 4;
   t.total = o;
+  t.wide = t.d0 > (gradient && C == 32 ? kWideInGradient32 : kWideIn);
+  t.rows = t.wide ? kBlockRows : t.d0;
   return t;
 }
 
@@ -412,6 +429,53 @@ __device__ __forceinline__ void put_inputs(float* x, const float* sm, const Net&
   if (t.ti) z[t.F * S] = lat.tin;
 }
 
+// sin and cos of Fourier row k at p + pl.
+__device__ __forceinline__ void feature(const float* Fm, int k, bool nerf, float3 p, float3 pl, float& s, float& c) {
+  if (nerf) {
+    const float w = (float)(1 << (k / 3));
+    const int a = k % 3;
+    const float pa = a == 0 ? p.x : (a == 1 ? p.y : p.z), la = a == 0 ? pl.x : (a == 1 ? pl.y : pl.z);
+    turn_sincos(w * pa, 6.28318548202514648f * (w * la), s, c);
+  } else {
+    net32::fourier_sincos(Fm + 3 * k, p, s, c, pl);
+  }
+}
+
+// The input rows of a wide network from `row` on, as many as a block holds, in
+// the lane's column v; returns how many.  The values are those of put_inputs.
+// Out of line, arguments by value, like all of the wide path: the others keep
+// their registers.
+static __device__ __noinline__ int put_block(float* v, const float* Fm, int m, int F, int ti, bool nerf,
+                                             const Latent lat, float3 p, float3 pl, int row) {
+  constexpr int S = kPts;
+  int n = 0;
+  if (row < 3 + 2 * m) {
+    if (row == 0) {
+      v[0] = p.x;
+      v[S] = p.y;
+      v[2 * S] = p.z;
+      v[kBlockLow * S] = pl.x;
+      v[(kBlockLow + 1) * S] = pl.y;
+      v[(kBlockLow + 2) * S] = pl.z;
+      n = 3;
+    }
+    const int k0 = row == 0 ? 0 : (row - 3) / 2, k1 = min(m, k0 + kBlockFeatures);
+#pragma unroll 2
+    for (int k = k0; k < k1; ++k, n += 2) {
+      float s, c;
+      feature(Fm, k, nerf, p, pl, s, c);
+      v[n * S] = s;
+      v[(n + 1) * S] = c;
+    }
+    return n;
+  }
+  const int f0 = row - 3 - 2 * m, f1 = min(F, f0 + kBlockChannels);
+  for (; f0 + n + 16 <= f1; n += 16) put_latent<S, 16>(v + n * S, lat, p, f0 + n);
+  for (; f0 + n < f1; n += 4) put_latent<S, 4>(v + n * S, lat, p, f0 + n);
+  if (f1 == F && ti) v[n++ * S] = lat.tin;
+  return n;
+}
+
 // Output dd of the lane's point from the last activation rows.
 template <int C, int S>
 __device__ __forceinline__ float last_layer(const float* x, const float* sm, const Net& t, int dd) {
@@ -540,17 +604,29 @@ struct Ctx {
 // Forward pass of the lanes' points: the last activations end up as rows of
 // x (read them with last_layer; a __syncwarp must follow before the rows are
 // overwritten).  v0: the input rows (may be x itself).  DF: df[h] receives
-// the derivative of activation h.
-template <int C, bool DF>
+// the derivative of activation h.  WIDE: for the networks put_block is for, in
+// kernels of their own (the branch alone cost the error grid 2.5 %).
+template <int C, bool DF, bool WIDE>
 __device__ __forceinline__ void forward(const Ctx& c, float* v0, float* x, const Latent& lat, float3 p, float3 pl,
                                         Acc<C>* df) {
   constexpr int S = kPts;
   const Net& t = *c.t;
-  put_inputs<S>(v0, c.sm, t, lat, c.nerf, p, pl);
-  __syncwarp();
   Acc<C> a;
-  set_bias<C>(a, c.sm + t.ob0);
-  layer<C, S>(a, v0, c.sm + t.oW0, t.d0);
+  if constexpr (WIDE) {
+    set_bias<C>(a, c.sm + t.ob0);
+    for (int row = 0; row < t.d0;) {
+      const int n = put_block(v0 + (threadIdx.x & 31), c.sm + t.oF, t.m, t.F, t.ti, c.nerf, lat, p, pl, row);
+      __syncwarp();
+      layer<C, S>(a, v0, c.sm + t.oW0 + row * C, n);
+      row += n;
+      __syncwarp();
+    }
+  } else {
+    put_inputs<S>(v0, c.sm, t, lat, c.nerf, p, pl);
+    __syncwarp();
+    set_bias<C>(a, c.sm + t.ob0);
+    layer<C, S>(a, v0, c.sm + t.oW0, t.d0);
+  }
 #pragma unroll 1
   for (int h = 1; h < t.l - 1; ++h) {
     activate<C, DF>(c.act, a, DF ? df + (h - 1) : nullptr);
@@ -623,11 +699,80 @@ __device__ __forceinline__ void latent_vjp(float3& l, const float* z, const Late
   }
 }
 
+// The second half of input_gradient for a wide network: Fourier rows and
+// latent channels in blocks, the features evaluated again.  Rows 0 to 2 of v0
+// hold the products of the position rows, x the adjoint rows.
+template <int C>
+__device__ __noinline__ float3 wide_gradient(const float* W0, const float* Fm, int m, int F, bool nerf, float* v0,
+                                             const float* x, const Latent lat, float3 p) {
+  constexpr int S = kPts;
+  const int pg = point_group(), og = out_group(), lane = threadIdx.x & 31;
+  __syncwarp();
+  float3 r = make_float3(v0[lane], v0[S + lane], v0[2 * S + lane]);
+  const float3 pl = make_float3(v0[kBlockLow * S + lane], v0[(kBlockLow + 1) * S + lane], v0[(kBlockLow + 2) * S + lane]);
+  for (int k0 = 0; k0 < m; k0 += kBlockFeatures) {
+    const int k1 = min(m, k0 + kBlockFeatures);
+    __syncwarp();
+#pragma unroll 2
+    for (int k = k0; k < k1; ++k) {
+      float s, c;
+      feature(Fm, k, nerf, p, pl, s, c);
+      v0[2 * (k - k0) * S + lane] = s;
+      v0[(2 * (k - k0) + 1) * S + lane] = c;
+    }
+    __syncwarp();
+    for (int kb = k0; kb < k1; kb += 16) {  // four Fourier rows a lane
+      float2 g[2][8];
+      back<C, S, 8, 4>(g, x, W0, [&](int q) { return 3 + 2 * min(kb + 4 * og + (q >> 1), m - 1) + (q & 1); });
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int k = kb + 4 * og + e;
+        if (k < k1) {
+          float4* row = reinterpret_cast<float4*>(v0 + 2 * (k - k0) * S + 4 * pg);
+          const float4 s4 = *row, c4 = *reinterpret_cast<const float4*>(v0 + (2 * (k - k0) + 1) * S + 4 * pg);
+          const float2 s01 = g[0][2 * e], c01 = g[0][2 * e + 1], s23 = g[1][2 * e], c23 = g[1][2 * e + 1];
+          *row = make_float4(s01.x * c4.x - c01.x * s4.x, s01.y * c4.y - c01.y * s4.y, s23.x * c4.z - c23.x * s4.z,
+                             s23.y * c4.w - c23.y * s4.w);
+        }
+      }
+    }
+    __syncwarp();
+    for (int k = k0; k < k1; ++k) {
+      const float coef = v0[2 * (k - k0) * S + lane];
+      r.x = fmaf(coef, Fm[3 * k], r.x);
+      r.y = fmaf(coef, Fm[3 * k + 1], r.y);
+      r.z = fmaf(coef, Fm[3 * k + 2], r.z);
+    }
+  }
+  const Cell cell = net32::make_cell(lat, p);
+  float3 l = make_float3(0.f, 0.f, 0.f);
+  for (int f0 = 0; f0 < F; f0 += kBlockChannels) {
+    const int f1 = min(F, f0 + kBlockChannels);
+    __syncwarp();
+    for (int fb = f0; fb < f1; fb += 32) {  // eight channels a lane
+      float2 g[2][8];
+      const int f = fb + 8 * og;
+      back<C, S, 8, 4>(g, x, W0 + (3 + 2 * m) * C, [&](int q) { return min(f + q, F - 1); });
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (f + q < f1)
+          *reinterpret_cast<float4*>(v0 + (f - f0 + q) * S + 4 * pg) = make_float4(g[0][q].x, g[0][q].y, g[1][q].x, g[1][q].y);
+    }
+    __syncwarp();
+    int f = f0;
+    for (; f + 16 <= f1; f += 16) latent_vjp<S, 16>(l, v0 + (f - f0) * S + lane, lat, cell, f);
+    for (; f < f1; f += 4) latent_vjp<S, 4>(l, v0 + (f - f0) * S + lane, lat, cell, f);
+  }
+  __syncwarp();
+  const float scale = (float)(lat.R - 1);
+  return make_float3(fmaf(scale, l.x, r.x), fmaf(scale, l.y, r.y), fmaf(scale, l.z, r.z));
+}
+
 // Input gradient of the lane's point (Section 5 "Adjoint") from the seed in
 // the tile layout: backward through the hidden layers, then the position,
 // Fourier and latent inputs.  v0 holds the input rows of the forward (all but
 // the cosines are overwritten), x is scratch of C rows, df the derivatives.
-template <int C>
+template <int C, bool WIDE>
 __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float* x, const Latent& lat, float3 p,
                                                  Acc<C>& a, const Acc<C>* df) {
   constexpr int S = kPts;
@@ -666,58 +811,62 @@ __device__ __forceinline__ float3 input_gradient(const Ctx& c, float* v0, float*
     back<C, S, 1, 4>(g, x, W0, [&](int) { return r; });
     if (og < 3) *reinterpret_cast<float4*>(v0 + og * S + 4 * pg) = make_float4(g[0][0].x, g[0][0].y, g[1][0].x, g[1][0].y);
   }
+  if constexpr (WIDE) {
+    return wide_gradient<C>(W0, c.sm + t.oF, t.m, t.F, c.nerf, v0, x, lat, p);
+  } else {
 #pragma unroll 1
-  for (int kb = 0; kb < t.m; kb += 8) {
-    const int ka[2] = {min(kb + og, t.m - 1), min(kb + og + 4, t.m - 1)};
-    float2 g[2][4];
-    back<C, S, 4, 4>(g, x, W0, [&](int q) { return 3 + 2 * ka[q >> 1] + (q & 1); });
+    for (int kb = 0; kb < t.m; kb += 8) {
+      const int ka[2] = {min(kb + og, t.m - 1), min(kb + og + 4, t.m - 1)};
+      float2 g[2][4];
+      back<C, S, 4, 4>(g, x, W0, [&](int q) { return 3 + 2 * ka[q >> 1] + (q & 1); });
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      if (kb + og + 4 * e < t.m) {
-        const int k = ka[e];
-        const float4 s4 = *reinterpret_cast<const float4*>(v0 + (3 + 2 * k) * S + 4 * pg);
-        const float4 c4 = *reinterpret_cast<const float4*>(v0 + (4 + 2 * k) * S + 4 * pg);
-        const float2 s01 = g[0][2 * e], c01 = g[0][2 * e + 1], s23 = g[1][2 * e], c23 = g[1][2 * e + 1];
-        *reinterpret_cast<float4*>(v0 + (3 + 2 * k) * S + 4 * pg) =
-            make_float4(s01.x * c4.x - c01.x * s4.x, s01.y * c4.y - c01.y * s4.y, s23.x * c4.z - c23.x * s4.z,
-                        s23.y * c4.w - c23.y * s4.w);
+      for (int e = 0; e < 2; ++e) {
+        if (kb + og + 4 * e < t.m) {
+          const int k = ka[e];
+          const float4 s4 = *reinterpret_cast<const float4*>(v0 + (3 + 2 * k) * S + 4 * pg);
+          const float4 c4 = *reinterpret_cast<const float4*>(v0 + (4 + 2 * k) * S + 4 * pg);
+          const float2 s01 = g[0][2 * e], c01 = g[0][2 * e + 1], s23 = g[1][2 * e], c23 = g[1][2 * e + 1];
+          *reinterpret_cast<float4*>(v0 + (3 + 2 * k) * S + 4 * pg) =
+              make_float4(s01.x * c4.x - c01.x * s4.x, s01.y * c4.y - c01.y * s4.y, s23.x * c4.z - c23.x * s4.z,
+                          s23.y * c4.w - c23.y * s4.w);
+        }
       }
     }
-  }
 #pragma unroll 1
-  for (int fb = 0; fb < t.F; fb += 16) {
-    float2 g[2][4];
-    const int f0 = fb + 4 * og;
-    back<C, S, 4, 4>(g, x, W0 + (3 + 2 * t.m) * C, [&](int q) { return min(f0 + q, t.F - 1); });
-    if (f0 < t.F) {
+    for (int fb = 0; fb < t.F; fb += 16) {
+      float2 g[2][4];
+      const int f0 = fb + 4 * og;
+      back<C, S, 4, 4>(g, x, W0 + (3 + 2 * t.m) * C, [&](int q) { return min(f0 + q, t.F - 1); });
+      if (f0 < t.F) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<float4*>(v0 + (3 + 2 * t.m + f0 + q) * S + 4 * pg) =
-            make_float4(g[0][q].x, g[0][q].y, g[1][q].x, g[1][q].y);
+        for (int q = 0; q < 4; ++q)
+          *reinterpret_cast<float4*>(v0 + (3 + 2 * t.m + f0 + q) * S + 4 * pg) =
+              make_float4(g[0][q].x, g[0][q].y, g[1][q].x, g[1][q].y);
+      }
     }
-  }
-  __syncwarp();
-  float3 r = make_float3(v0[lane], v0[S + lane], v0[2 * S + lane]);
-  const float* Fm = c.sm + t.oF;
+    __syncwarp();
+    float3 r = make_float3(v0[lane], v0[S + lane], v0[2 * S + lane]);
+    const float* Fm = c.sm + t.oF;
 #pragma unroll 2
-  for (int k = 0; k < t.m; ++k) {
-    const float coef = v0[(3 + 2 * k) * S + lane];
-    r.x = fmaf(coef, Fm[3 * k], r.x);
-    r.y = fmaf(coef, Fm[3 * k + 1], r.y);
-    r.z = fmaf(coef, Fm[3 * k + 2], r.z);
+    for (int k = 0; k < t.m; ++k) {
+      const float coef = v0[(3 + 2 * k) * S + lane];
+      r.x = fmaf(coef, Fm[3 * k], r.x);
+      r.y = fmaf(coef, Fm[3 * k + 1], r.y);
+      r.z = fmaf(coef, Fm[3 * k + 2], r.z);
+    }
+    const float* z = v0 + (3 + 2 * t.m) * S + lane;
+    const Cell cell = net32::make_cell(lat, p);
+    float3 l = make_float3(0.f, 0.f, 0.f);
+    if (t.F == 16) {
+      latent_vjp<S, 16>(l, z, lat, cell, 0);
+    } else {
+      for (int f = 0; f < t.F; f += 4) latent_vjp<S, 4>(l, z + f * S, lat, cell, f);
+    }
+    const float scale = (float)(lat.R - 1);
+    r = make_float3(fmaf(scale, l.x, r.x), fmaf(scale, l.y, r.y), fmaf(scale, l.z, r.z));
+    __syncwarp();
+    return r;
   }
-  const float* z = v0 + (3 + 2 * t.m) * S + lane;
-  const Cell cell = net32::make_cell(lat, p);
-  float3 l = make_float3(0.f, 0.f, 0.f);
-  if (t.F == 16) {
-    latent_vjp<S, 16>(l, z, lat, cell, 0);
-  } else {
-    for (int f = 0; f < t.F; f += 4) latent_vjp<S, 4>(l, z + f * S, lat, cell, f);
-  }
-  const float scale = (float)(lat.R - 1);
-  r = make_float3(fmaf(scale, l.x, r.x), fmaf(scale, l.y, r.y), fmaf(scale, l.z, r.z));
-  __syncwarp();
-  return r;
 }
 
 // Warps per CTA of a tile kernel over `tiles` tiles (0: not known).  One CTA

@@ -239,3 +239,63 @@ def test_position_gradient_rounds_each_fourier_row_once(S, act, most):
         want = oracle.net_input_grad(oracle.OracleNet(p), pts)[1]
         errs.append(np.linalg.norm(grad.cpu().numpy() - want) / np.linalg.norm(want))
     assert np.mean(errs) <= most
+
+
+# (width, layers, latent channels, Fourier rows, outputs, time input, NeRF matrix): inputs at both sides of the line
+# past which layer 0 runs in blocks (128), blocks full and not, with and without Fourier rows
+BLOCKED = [(32, 3, 64, 30, 1, 1, True), (32, 3, 68, 30, 1, 0, True), (32, 2, 200, 0, 4, 0, True), (48, 3, 4, 96, 4, 1, False),
+           (64, 2, 64, 93, 1, 0, False), (64, 8, 32, 110, 1, 0, False), (32, 8, 4, 124, 4, 1, False)]
+
+
+@pytest.mark.parametrize("n", [33, 700])
+@pytest.mark.parametrize("width,layers,F,m,D,ti,nerf", BLOCKED)
+def test_wide_inputs_match_oracle(S, width, layers, F, m, D, ti, nerf, n):
+    """Outputs and density gradient to the FP32 bounds of the oracle's
+    first-order analysis, the gradient seeded with output adjoints to 1e-4 of
+    max(|g|, 1), and the error grid to twice the largest density bound."""
+    import torch
+    p = synth.random_params(R=5, F=F, m=m, layers=layers, width=width, out_dim=D, act=synth.ACT_SNAKEALT, seed=n, grid_std=0.5,
+                            time_input=ti)
+    if not nerf:
+        p["fourier"] = np.random.default_rng(5).normal(0, 6, (m, 3)).astype(np.float32)
+    net, on, pts, t = S.Network(p), oracle.OracleNet(p), _points(n, n), 0.25
+    x = torch.tensor(pts, device="cuda")
+    brho, bgrad = oracle.error_bounds(on, pts, oracle.PREC_FP32, t)
+    out, rho, grad = (torch.full(s, float("nan"), device="cuda") for s in ((n, D), (n,), (n, 3)))
+    S.srn_eval(net.ctx, x, out, time=t)
+    S.srn_density_grad(net.ctx, x, rho, grad, time=t)
+    rref, gref = oracle.net_input_grad(on, pts, t)
+    assert torch.equal(rho, out[:, 0])
+    assert (np.abs(rho.cpu().numpy() - rref) / np.asarray(brho).reshape(n, -1)[:, 0]).max() <= 1.0
+    assert (np.abs(grad.cpu().numpy() - gref) / bgrad).max() <= 1.0
+    dout = np.random.default_rng(n + 9).standard_normal((n, D), dtype=np.float32)
+    S.srn_input_backward(net.ctx, x, torch.tensor(dout, device="cuda"), grad, time=t)
+    vref = oracle.net_input_vjp(on, pts, dout, t)
+    assert (np.abs(grad.cpu().numpy() - vref) / np.maximum(np.abs(vref).max(axis=1, keepdims=True), 1.0)).max() <= 1e-4
+    vol, err = np.random.default_rng(1).random((6, 7, 8), dtype=np.float32), torch.full((6 ** 3,), float("nan"), device="cuda")
+    S.srn_error_grid(net.ctx, torch.tensor(vol, device="cuda"), 6, 2, 3, err, time=t)
+    eref = oracle.error_grid(on, vol, 6, 2, 3, t)
+    assert np.abs(err.cpu().numpy() - eref.ravel()).max() <= 2.0 * float(np.max(brho)) + 1e-6
+
+
+def test_wide_inputs_keep_the_warps_of_an_sm(S):
+    """255 inputs against 127 of the same eight layers of 64: a quarter more
+    arithmetic, and no more than 1.6 times the time (one warp an SM for the
+    rows of all inputs: above 2)."""
+    import torch
+    times = []
+    for m in (46, 110):
+        p = synth.random_params(R=5, F=32, m=m, layers=8, width=64, act=synth.ACT_SNAKEALT, seed=m, grid_std=0.5)
+        p["fourier"] = np.random.default_rng(5).normal(0, 6, (m, 3)).astype(np.float32)
+        net, x, out = S.Network(p), torch.tensor(_points(200000, 1), device="cuda"), torch.empty((200000, 1), device="cuda")
+        each = []
+        for _ in range(9):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            S.srn_eval(net.ctx, x, out)
+            t1.record()
+            torch.cuda.synchronize()
+            each.append(t0.elapsed_time(t1))
+        times.append(sorted(each)[4])
+    print(f"127 inputs {times[0]:.3f} ms, 255 inputs {times[1]:.3f} ms")
+    assert times[1] <= 1.6 * times[0]
