@@ -239,7 +239,13 @@ cudaError_t launch_eval_t(const NetDev& net, const float* pts, int n, float time
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const long long tiles = ((long long)n + 31) / 32;
-  const int rows = tile_rows(t, C, MODE != 0, MODE == 2), warps = tile32::warps_for(t, C, rows, tiles, sms);
+  const int rows = tile_rows(t, C, MODE != 0, MODE == 2);
+  int warps = tile32::warps_for(t, C, rows, tiles, sms);
+  // A gradient gathers each point's corners twice; from 32 channels on the
+  // second time finds them in an L1 that fewer tiles leave larger (300,000
+  // points, two layers: 32 channels 295 -> 260 us, 64 channels 504 -> 389).
+  // Not where that would take a second wave for a few tiles.
+  if (MODE != 0 && t.F >= 32 && warps > 8 && tiles >= 16ll * sms) warps = 8;
   const size_t smem = sizeof(float) * ((size_t)t.total + (size_t)warps * rows * tile32::kPts);
   auto k = t.wide ? eval_fp32_kernel<C, MODE, true> : eval_fp32_kernel<C, MODE, false>;
   e = tile32::allow_dynamic(k);

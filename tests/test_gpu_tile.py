@@ -299,3 +299,27 @@ def test_wide_inputs_keep_the_warps_of_an_sm(S):
         times.append(sorted(each)[4])
     print(f"127 inputs {times[0]:.3f} ms, 255 inputs {times[1]:.3f} ms")
     assert times[1] <= 1.6 * times[0]
+
+
+@pytest.mark.parametrize("F,most", [(32, 2.2), (64, 3.6)])
+def test_gradients_of_many_channels(S, F, most):
+    """300,000 points of a two-layer network of 14 Fourier rows: the gradient
+    with F latent channels against 16 of them.  Twice the gathers and a third
+    more inputs, or four times and twice: a thread per point takes 1.7 and 2.7
+    times as long, four channels a pass through little L1 2.5 and 4.6."""
+    import torch
+    times = []
+    for channels in (16, F):
+        p = synth.random_params(R=12, F=channels, m=14, layers=2, width=32, act=synth.ACT_SNAKEALT, seed=1, grid_std=0.5)
+        net, x = S.Network(p), torch.tensor(_points(300000, 1), device="cuda")
+        rho, grad, each = torch.empty(300000, device="cuda"), torch.empty((300000, 3), device="cuda"), []
+        for _ in range(9):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            S.srn_density_grad(net.ctx, x, rho, grad)
+            t1.record()
+            torch.cuda.synchronize()
+            each.append(t0.elapsed_time(t1))
+        times.append(sorted(each)[4])
+    print(f"16 channels {times[0]:.3f} ms, {F} channels {times[1]:.3f} ms")
+    assert times[1] <= most * times[0]
