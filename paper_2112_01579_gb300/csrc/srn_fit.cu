@@ -289,10 +289,14 @@ __global__ void __launch_bounds__(kFitThreads, 4) fit_point_kernel(const NetDev 
 // autograd 434 -> 261 us.
 constexpr int kTileStride = 36;  // floats per adjoint row: eight rows' 16-byte loads hit distinct banks
 constexpr int kTileMaxIn = 48;   // inputs of layer 0: 16 threads x 3 entries
-// Points with a residual below this are decided by the accurate functions:
-// inline and library sines move a density by 2e-7 at most on networks of the
-// workloads' shapes.  A converged fit (residuals around 0.01) has a few
-// hundred such points in 2^18.
+// Points with a residual below this are decided by the accurate functions.  It
+// holds what inline and library sines move an output by on trained networks of
+// the workloads' shapes (4e-7 at most of 2^18 points, densities and gradient
+// outputs) and at Xavier's weights (1e-6).  With larger weights the two differ
+// by more (twice Xavier's, four layers: 1e-5), and both are as far from 64 bits
+// (1.3e-5 and 1.1e-5 at most, 1.8e-6 rms each): which sign is right is then not
+// decided by either, and a wider band would only cost.  A converged fit
+// (residuals around 0.01) has a few hundred points of 2^18 in it.
 constexpr float kSignBand = 4.0e-6f;
 
 // acc[i][j] += sum over the CTA's points of d[o_i][p] v[r_j][p], o_i = tid % 8
