@@ -167,7 +167,12 @@ const char* srn_last_error(void);
  * Create a context for one network.  Copies *cfg and *params (the pointed-to
  * device arrays are not copied and must outlive the context).  Allocates the
  * device scratch of the fit / backward (sized by cfg->max_fit_points) and a
- * small status word; nothing else allocates later.
+ * small status word; nothing else allocates later.  With max_fit_points > 0
+ * the scratch holds 32 feat (grid_res - 1)^3 bytes of per-cell gradient sums
+ * beside what goes by points and parameters: 15 MB for a 32^3 x 16 grid, 128
+ * MB for 64^3 x 16.  Where they would pass 256 MB or the device has no room,
+ * and there are fewer than 32 points per cell, the context does without: the
+ * grid gradient then takes longer and adds in another order.
  */
 srn_status srn_create(const srn_config* cfg, const srn_params* params, srn_ctx** out);
 

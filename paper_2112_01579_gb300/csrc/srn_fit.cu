@@ -1925,7 +1925,12 @@ cudaError_t fit_scratch_alloc(FitScratch& s, const NetDev& net, int max_points) 
   for (unsigned int* q : {s.key, s.key_alt, s.idx, s.idx_alt})
     if (e == cudaSuccess) e = cudaMemset(q, 0, sizeof(unsigned int) * n);
   const size_t part_bytes = sizeof(float) * s.n_cells * 8 * net.F;
-  if ((size_t)max_points >= 32 * s.n_cells || part_bytes <= kMaxCellPart) alloc((void**)&s.cell_part, part_bytes);
+  if ((size_t)max_points >= 32 * s.n_cells) {
+    alloc((void**)&s.cell_part, part_bytes);
+  } else if (e == cudaSuccess && part_bytes <= kMaxCellPart && cudaMalloc((void**)&s.cell_part, part_bytes) != cudaSuccess) {
+    s.cell_part = nullptr;  // no room: the gradient is gathered per vertex, as for larger grids
+    cudaGetLastError();
+  }
   return e;
 }
 

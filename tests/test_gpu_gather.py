@@ -169,3 +169,27 @@ def test_crowded_points_take_their_share_of_the_chip(S, kind, F, m, most):
     even, crowded = us(np.random.default_rng(1).random((n, 3), dtype=np.float32)), us(_crowd(kind, n, n, 33, 1))
     print(f"{kind}: {even:.0f} us evenly spread, {crowded:.0f} us crowded")
     assert crowded <= most * even
+
+
+@pytest.mark.parametrize("R,F,points,cells_held", [(17, 16, 1000, True), (65, 16, 5000, True), (83, 16, 5000, False), (17, 4, 140000, True)])
+def test_scratch_is_what_the_header_says(S, R, F, points, cells_held):
+    """Device memory of a context: per-cell sums of 32 F (R - 1)^3 bytes up to
+    256 MB, and at most 32 F + 200 bytes a point, three times the parameters
+    and 64 MB of fixed arrays and allocation granularity beside them."""
+    import ctypes
+
+    import torch
+    p = synth.random_params(R=R, F=F, m=3, layers=2, width=32, act=synth.ACT_SINE, seed=1)
+    keep = S.Network(p, max_fit_points=0)  # the parameters, before the count
+    cfg = keep.cfg
+    cfg.max_fit_points = points
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    ctx = S.srn_create(cfg, keep._params())
+    held = before - torch.cuda.mem_get_info()[0]
+    assert isinstance(ctx, ctypes.c_void_p)
+    S.srn_destroy(ctx)
+    cells = 32 * F * (R - 1) ** 3
+    rest = (32 * F + 200) * points + 3 * 4 * keep.grid.numel() + (64 << 20)
+    assert held <= (cells if cells_held else 0) + rest
+    assert held >= (cells if cells_held else 0)
