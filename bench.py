@@ -713,10 +713,10 @@ SMS, MUFU_PER_SM_CLK, FP32_PER_SM_CLK, MAX_SM_GHZ = 152, 16, 128, 2.07
 # DRAM bytes (read + write) of one 1024^2 frame of the render kernel and of
 # the dense DVR, from the ncu captures summarised in profiles/ (None when the
 # kernel changed after the capture).
-RENDER_DRAM_BYTES = 1684224 + 18176
+RENDER_DRAM_BYTES = 1678848 + 20224
 # Warp instructions per network sample of the render kernel from the same
-# capture (smsp__inst_executed.sum 7.2486e9 over 2.10e8 samples).
-WARP_INST_PER_SAMPLE = 7.2486e9 / 2.10e8
+# capture (smsp__inst_executed.sum 7.2514e9 over 2.10e8 samples).
+WARP_INST_PER_SAMPLE = 7.2514e9 / 2.10e8
 # Algorithmic work of one plain-workload fit step per point: forward 2 (35 x 32
 # + 32) FLOP, weight gradients the same again, the backward through the
 # output layer (2 x 32), the latent-input gradient (2 x 32 x 8) and its
@@ -724,9 +724,9 @@ WARP_INST_PER_SAMPLE = 7.2486e9 / 2.10e8
 # 4-byte corners.
 FIT_FLOP_PER_POINT = 2 * (35 * 32 + 32) * 2 + 2 * 32 + 2 * 32 * 8 + 8 * 8 * 2
 FIT_GATHER_BYTES_PER_POINT = 32
-DENSE_DRAM_BYTES = 67166208 + 9174016
-DENSE_L1_WAVEFRONT_PCT = 59.3  # l1tex__data_pipe_lsu_wavefronts, % of peak
-DENSE_ISSUE_PCT = 82.5  # smsp__issue_active, % of peak, same capture
+DENSE_DRAM_BYTES = 67141888 + 8636160
+DENSE_L1_WAVEFRONT_PCT = 61.2  # l1tex__data_pipe_lsu_wavefronts, % of peak
+DENSE_ISSUE_PCT = 83.3  # smsp__issue_active, % of peak, same capture
 # L1 load bandwidth of one SM (bytes per clock) for the gather roofline of
 # dense DVR (unit count; the peak is derived, not measured).
 L1_BYTES_PER_SM_CLK = 128
@@ -747,7 +747,7 @@ def dense_roofline(samples, ms_total, frames, vol_bytes):
             "peak_source": "152 SMs x 128 B/clk x 2.07 GHz (unit counts)",
             "l1_data_wavefronts_pct": DENSE_L1_WAVEFRONT_PCT,
             "issue_active_pct": DENSE_ISSUE_PCT,
-            "l1_note": "ncu: 82 % of the issue slots are taken and the L1 data pipe is 59 % busy with the wavefronts "
+            "l1_note": "ncu: 83 % of the issue slots are taken and the L1 data pipe is 61 % busy with the wavefronts "
                        "of the scattered 4-byte corner gathers; the fraction here is against the L1 gather roofline",
             "hbm_floor": {"achieved": vol_gbs, "peak": hbm, "unit": "GB/s",
                           "frac": vol_gbs / hbm if hbm else None,

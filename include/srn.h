@@ -368,8 +368,9 @@ srn_status srn_lowpass_resample(const float* volume_dev, const int dims[3], int 
  * callers cannot use srn_backward; this entry point needs no context and
  * allocates nothing (no cudaMalloc, cudaFree or allocating library call).
  *
- * It computes exactly what srn_backward computes for the network described
- * by *cfg / *params (same arguments, same outputs, overwritten), using a
+ * It computes what srn_backward computes for the network described by *cfg /
+ * *params (same arguments, same outputs, overwritten; the latent-grid gradient
+ * adds its points in another order, the same on every run), using a
  * fixed device scratch area of SRN_STATIC_SCRATCH_BYTES that every GPU
  * loading the library holds until the process exits.  Limits and rules:
  * - n is limited by that area; the largest n depends on the network shape

@@ -8,11 +8,12 @@
 // data pipe at once (a warp's corner load takes one wavefront per cache line
 // it touches), so both are kept low: the sample position is carried in voxel
 // units (one FMA per axis), offsets are 32 bits where the volume has fewer
-// than 2^31 voxels, the interpolation is seven nested lerps, the transfer
+// than 2^31 voxels, the interpolation is seven nested lerps by two weights (a
+// difference of two voxels would lose infinities), the transfer
 // function's segment comes from counting control points out of two 16-byte
 // loads, and the corner values stay in registers while a ray stays in its
 // cell (two samples in five at half a voxel a step).  A 1024^2 frame of a
-// 256^3 volume: 1427 -> 1051 us; without the kept corners 6 % more, and pixel
+// 256^3 volume: 1427 -> 1062 us; without the kept corners 6 % more, and pixel
 // tiles chosen per view to cross the fewest rows gained nothing.
 
 #include "srn_device.cuh"

@@ -14,8 +14,9 @@
 //      kernel of srn_fit_mma.cu instead; other networks of up to four layers
 //      and 48 inputs the tiled kernel, fit_tile_kernel.)
 //   2. stable radix sort of (cell, point) pairs: up to 512 cells one 9-bit
-//      pass; up to 2^18 cells a pass over the leading eight bits, then one
-//      block per leading digit; else 8-bit digits from the lowest.  A pass is
+//      pass; up to 2^18 cells a pass over the leading eight bits, then each
+//      leading digit by itself (a block, or several where points crowd);
+//      else 8-bit digits from the lowest.  A pass is
 //      per-block per-warp digit counts, a scan per digit over the blocks and a
 //      stable scatter (which adds the digits' prefix and, for one pass, writes
 //      the cell offsets).
@@ -284,9 +285,9 @@ __global__ void __launch_bounds__(kFitThreads, 4) fit_point_kernel(const NetDev 
 // layer's adjoint rows take the place of its activations once the gradient
 // that needs them is done), the activation derivatives in registers, so
 // neither sines nor Fourier features are evaluated twice.  Fit step of the
-// main configuration (32^3 x 16, four layers) at 2^18 points: 876 -> 302 us
+// main configuration (32^3 x 16, four layers) at 2^18 points: 876 -> 305 us
 // (with the sort and gather below); 65,537 points of the same network through
-// autograd 434 -> 261 us.
+// autograd 434 -> 250 us.
 constexpr int kTileStride = 36;  // floats per adjoint row: eight rows' 16-byte loads hit distinct banks
 constexpr int kTileMaxIn = 48;   // inputs of layer 0: 16 threads x 3 entries
 // Points with a residual below this are decided by the accurate functions.  It

@@ -13,7 +13,7 @@
 // bits as a thread walking the inputs alone.
 //
 // Measured against one thread per point with out-of-line library sines: error
-// grid of 128^3 x 8 evaluations of the main configuration 5.68 -> 3.09 ms
+// grid of 128^3 x 8 evaluations of the main configuration 5.68 -> 3.06 ms
 // (5.4 G evaluations/s; bound by the pipe that takes packed FMAs and the
 // shared-memory data pipe together), the plain workload's 128^2 frame 968 ->
 // 202 us (with several samples of a ray per pass).
