@@ -1353,7 +1353,7 @@ __global__ void __launch_bounds__(256) cell_corner_kernel(const float* __restric
 // took 57 us for 32^3 vertices whatever the number of points.
 //
 // Points may crowd: a cell of more than kLongCell points is left to all eight
-// warps of its CTA (one warp on 2^18 points of one cell: 32 ms; so 3.3).
+// warps of its CTA (one warp on 2^18 points of one cell: 32 ms; so 2.2).
 constexpr int kLongCell = 96;
 
 constexpr int kCellPass = 16;  // points a warp brings to shared memory at a time
@@ -1371,47 +1371,56 @@ struct CellSum {
 
   // acc = the corner sums of the points base .. base + P - 1, then `stride`
   // on, up to s1.  Each P are summed first, so that the rounding error does
-  // not grow with the length of one chain.  place, rows: the warp's P entries.
+  // not grow with the length of one chain.  weights (of the eight corners) and
+  // rows: the warp's P entries.
   __device__ __forceinline__ void run(const float* __restrict__ pts, const float* __restrict__ dz,
                                       const unsigned int* __restrict__ sidx, int R, int base, int s1, int stride,
-                                      float4* place, float4 (*rows)[LR]) {
+                                      float4 (*weights)[2], float4 (*rows)[LR]) {
     const int lane = threadIdx.x & 31, g = lane / (8 * QL), c = (lane / QL) & 7, q = lane % QL;
-    const float wx = (c & 1) ? 1.f : -1.f, wy = (c & 2) ? 1.f : -1.f, wz = (c & 4) ? 1.f : -1.f;
-    const float ox = (c & 1) ? 0.f : 1.f, oy = (c & 2) ? 0.f : 1.f, oz = (c & 4) ? 0.f : 1.f;
 #pragma unroll
     for (int e = 0; e < QN; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    int j = lane < P && base + lane < s1 ? (int)sidx[base + lane] : 0;
-#pragma unroll 1
-    for (; base < s1; base += stride) {
-      const int cnt = min(P, s1 - base);
-      float4 v[NR];
+    // a pass's points and rows are loaded while the one before is summed,
+    // their indices one pass earlier still
+    float4 v[NR];
+    float3 at = make_float3(0.f, 0.f, 0.f);
+    int j = index_at(sidx, base, s1);
+    auto fetch = [&](int b) {
 #pragma unroll
       for (int e = 0; e < NR; ++e) {
         const int src = e * (32 / LR) + lane / LR, jk = __shfl_sync(0xffffffffu, j, src);
-        if (src < cnt) v[e] = reinterpret_cast<const float4*>(dz + (size_t)jk * F)[lane % LR];
+        if (src < P && b + src < s1) v[e] = reinterpret_cast<const float4*>(dz + (size_t)jk * F)[lane % LR];
       }
+      if (lane < P && b + lane < s1)
+        at = make_float3(pts[3 * (size_t)j], pts[3 * (size_t)j + 1], pts[3 * (size_t)j + 2]);
+      j = index_at(sidx, b + stride, s1);
+    };
+    fetch(base);
+#pragma unroll 1
+    for (; base < s1; base += stride) {
+      const int cnt = min(P, s1 - base);
       if (lane < cnt) {
         int i;
-        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-        cell_coord(pts[3 * (size_t)j], R, i, f.x);
-        cell_coord(pts[3 * (size_t)j + 1], R, i, f.y);
-        cell_coord(pts[3 * (size_t)j + 2], R, i, f.z);
-        place[lane] = f;
+        float x, y, z;
+        cell_coord(at.x, R, i, x);
+        cell_coord(at.y, R, i, y);
+        cell_coord(at.z, R, i, z);
+        const float u = 1.0f - z, yz[4] = {(1.0f - y) * u, y * u, (1.0f - y) * z, y * z};
+        weights[lane][0] = make_float4((1.0f - x) * yz[0], x * yz[0], (1.0f - x) * yz[1], x * yz[1]);
+        weights[lane][1] = make_float4((1.0f - x) * yz[2], x * yz[2], (1.0f - x) * yz[3], x * yz[3]);
       }
-      j = lane < P && base + stride + lane < s1 ? (int)sidx[base + stride + lane] : 0;
 #pragma unroll
       for (int e = 0; e < NR; ++e) {
         const int src = e * (32 / LR) + lane / LR;
         if (src < cnt) rows[src][lane % LR] = v[e];
       }
       __syncwarp();
+      fetch(base + stride);
       float4 a[QN];
 #pragma unroll
       for (int e = 0; e < QN; ++e) a[e] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
       for (int k = g; k < cnt; k += G) {
-        const float4 f = place[k];
-        const float w = fmaf(wx, f.x, ox) * fmaf(wy, f.y, oy) * fmaf(wz, f.z, oz);
+        const float w = reinterpret_cast<const float*>(weights[k])[c];
 #pragma unroll
         for (int e = 0; e < QN; ++e) {
           const float4 x = rows[k][q + e * QL];
@@ -1440,6 +1449,11 @@ struct CellSum {
         acc[e].w += __shfl_xor_sync(0xffffffffu, acc[e].w, off);
       }
   }
+  // The lane's point of the P from b on.
+  static __device__ __forceinline__ int index_at(const unsigned int* __restrict__ sidx, int b, int s1) {
+    const int i = b + (int)(threadIdx.x & 31);
+    return (threadIdx.x & 31) < P && i < s1 ? (int)sidx[i] : 0;
+  }
   // The sums as rows [8 corners][F] of out.
   __device__ __forceinline__ void store(float* out) const {
     const int lane = threadIdx.x & 31;
@@ -1456,13 +1470,13 @@ template <int F>
 __device__ __noinline__ void crowded_cells(const float* __restrict__ pts, const float* __restrict__ dz,
                                            const unsigned int* __restrict__ sidx, int R, long long cell0, int at,
                                            int end, unsigned int crowded, float* __restrict__ part) {
-  __shared__ float4 place[8][kCellPass], rows[8][kCellPass][F / 4];
+  __shared__ float4 weights[8][kCellPass][2], rows[8][kCellPass][F / 4];
   const int warp = threadIdx.x >> 5;
   for (unsigned int left = crowded; left; left &= left - 1) {
     const int w = __ffs(left) - 1;
     const int c0 = __shfl_sync(0xffffffffu, at, w), c1 = __shfl_sync(0xffffffffu, end, w);
     CellSum<F> sum;
-    sum.run(pts, dz, sidx, R, c0 + kCellPass * warp, c1, 8 * kCellPass, place[warp], rows[warp]);
+    sum.run(pts, dz, sidx, R, c0 + kCellPass * warp, c1, 8 * kCellPass, weights[warp], rows[warp]);
     sum.store(reinterpret_cast<float*>(rows[warp]));  // a warp's rows hold twice its sums
     __syncthreads();
     for (int i = threadIdx.x; i < 8 * F; i += 256) {
